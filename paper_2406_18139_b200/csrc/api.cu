@@ -829,7 +829,7 @@ int build_decode_plan(DecodePlan& dp, const lookm_cache_layout* lay, int n_req, 
     if (!(lay->softmax_scale >= 0.f) || !std::isfinite(lay->softmax_scale)) return LOOKM_ERR_INVALID_ARG;
     const int group = lay->n_q_heads / lay->n_kv_heads;
     dp.n_req = n_req;
-    dp.gt = group % 8 == 0 ? 8 : group % 4 == 0 ? 4 : group % 2 == 0 ? 2 : 1;
+    for (dp.gt = std::min(group, 8); group % dp.gt; --dp.gt) {}    // largest divisor of the group up to 8
     dp.n_pass = group / dp.gt;
     const long long units = (long long)lay->n_kv_heads * dp.n_pass;      // (KV head, pass) per request
     const int sms = decode_sms();

@@ -16,6 +16,8 @@
 // than one split the CTA leaves its partial result in the workspace and a second kernel, chained
 // behind the first, adds the splits in split order.  No CTA waits for another and the order of
 // additions never depends on timing, so results are reproducible bit for bit.
+//
+// Query heads that share a KV head go to decode_mma_kernel below, which has the same structure.
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -61,7 +63,7 @@ struct DecShared {
     float o[kDecWarps][GT][kHeadDim];
 };
 
-// GT query heads of the group are handled per pass over the rows (GT divides the group size).
+// GT query heads of the group are handled per pass over the rows; only GT = 1 is instantiated.
 template <int GT>
 __global__ void __launch_bounds__(kDecThreads)
 decode_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __restrict__ q,
@@ -277,6 +279,256 @@ decode_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// Grouped queries: several query heads attend over the same rows.  With the scalar kernel above the
+// arithmetic (four shuffles and sixteen FMAs per lane, row and head) takes longer than the rows take
+// to arrive, so this one multiplies on the tensor cores (mma.sync m16n8k16; per row it is a
+// bandwidth-bound kernel, far from needing tcgen05's rate):
+//   S = Q K^T   A = query heads, B = sixteen key rows;  O += P V   A = probabilities, B = value rows.
+// The sixteen rows of A hold the GP <= 8 heads of the pass several times over.  In S the copies are
+// equal; in P they are the three bf16 terms of the fp32 probability (24 bits together), so that the
+// product keeps the precision of fp32 probabilities: row r belongs to head r mod GP and term r / GP.
+// With GP = 8 only two terms fit and a second product adds the third.
+// A CTA of four warps takes a split; a warp takes sixteen rows of K and V at a time through a
+// cp.async ring of its own, 16-byte chunks XOR-swizzled so that ldmatrix is free of bank conflicts.
+// The reference of the running softmax moves only when a logit leaves it by 2^8.
+// ---------------------------------------------------------------------------------------------
+constexpr int kMmaThreads = 128;
+constexpr int kMmaWarps = kMmaThreads / 32;
+constexpr int kMmaRows = 16;                         // rows per warp and step
+constexpr int kMmaRing = 3;                          // steps in a warp's ring (all but one in flight)
+constexpr int kMmaStepBytes = 2 * kMmaRows * kDecRowBytes;         // [K|V][row][256 B]
+constexpr int kMmaRingBytes = kMmaWarps * kMmaRing * kMmaStepBytes;
+constexpr float kMmaSlack = 8.f;                     // log2 by which a logit may exceed the reference
+
+__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+    const __nv_bfloat162 b = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&b);
+}
+// Terms `part` (0, 1, 2; else zero) of the bf16 expansions of two fp32 values.
+__device__ __forceinline__ uint32_t bf16_term(float x, float y, int part) {
+    if (part >= 1) { x -= __bfloat162float(__float2bfloat16_rn(x)); y -= __bfloat162float(__float2bfloat16_rn(y)); }
+    if (part >= 2) { x -= __bfloat162float(__float2bfloat16_rn(x)); y -= __bfloat162float(__float2bfloat16_rn(y)); }
+    return part >= 3 ? 0u : pack_bf16(x, y);
+}
+
+template <int GP>
+struct MmaShared {
+    float m[kMmaWarps][GP];
+    float l[kMmaWarps][GP];
+    float o[kMmaWarps][GP][kHeadDim];
+};
+
+// gt <= GP query heads of the group are handled per pass over the rows.
+template <int GP>
+__global__ void __launch_bounds__(kMmaThreads)
+decode_mma_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __restrict__ q,
+                  const __nv_bfloat16* __restrict__ k_new, const __nv_bfloat16* __restrict__ v_new,
+                  __nv_bfloat16* __restrict__ cache_k, __nv_bfloat16* __restrict__ cache_v,
+                  long long stride_row, long long stride_head, int n_q_heads, int n_kv_heads, int group, int gt,
+                  int rows_per_split, float scale_log2, float* __restrict__ parts, float* __restrict__ out) {
+    __shared__ MmaShared<GP> sh;
+    extern __shared__ __align__(128) uint8_t dec_ring[];         // [warp][ring step][K|V][row][256 B, swizzled]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int r = 0;
+    {
+        int lo = 0, hi = batch.n_req - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (batch.r[mid].cta_begin <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
+        }
+        r = lo;
+    }
+    const DecodeReq rq = batch.r[r];
+    const int n_pass = group / gt;
+    const int local = (int)blockIdx.x - rq.cta_begin;            // [head][pass][split]
+    const int split = local % rq.n_splits;
+    const int pass = (local / rq.n_splits) % n_pass;
+    const int h = local / (rq.n_splits * n_pass);
+    const int n_rows = rq.len + 1;                               // cached rows + the new one
+    const int row0 = split * rows_per_split, row1 = min(n_rows, row0 + rows_per_split);
+    const int qh0 = h * group + pass * gt;                       // first query head of this pass
+
+    grid_dependency_wait();
+
+    const long long head_off = (long long)h * stride_head;
+    const __nv_bfloat16* ck = cache_k + rq.begin * stride_row + head_off;
+    const __nv_bfloat16* cv = cache_v + rq.begin * stride_row + head_off;
+    const __nv_bfloat16* nk = k_new + ((long long)rq.index * n_kv_heads + h) * kHeadDim;
+    const __nv_bfloat16* nv = v_new + ((long long)rq.index * n_kv_heads + h) * kHeadDim;
+
+    // Copies of one step: half a warp per row, 16 bytes per lane; rows past the split are zero-filled
+    // (and masked below).  Chunk c of row i goes to chunk c xor (i mod 8).
+    const int l16 = lane & 15, hi_half = lane >> 4;
+    const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(dec_ring) + warp * (kMmaRing * kMmaStepBytes);
+    auto issue = [&](int step) {
+        const int base = row0 + (step * kMmaWarps + warp) * kMmaRows;
+        const uint32_t dst = ring0 + (uint32_t)(step % kMmaRing) * kMmaStepBytes;
+        if (base < row1) {
+#pragma unroll
+            for (int f = 0; f < kMmaRows / 2; ++f) {
+                const int i = 2 * f + hi_half;
+                const int row = base + i;
+                const bool is_new = (row == rq.len);
+                const bool valid = row < row1;
+                const __nv_bfloat16* kp = ((is_new || !valid) ? nk : ck + (long long)row * stride_row) + l16 * 8;
+                const __nv_bfloat16* vp = ((is_new || !valid) ? nv : cv + (long long)row * stride_row) + l16 * 8;
+                const int nbytes = valid ? 16 : 0;
+                const uint32_t at = dst + i * kDecRowBytes + ((l16 ^ (i & 7)) << 4);
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(at), "l"(kp), "r"(nbytes) : "memory");
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                             ::"r"(at + kMmaRows * kDecRowBytes), "l"(vp), "r"(nbytes) : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    const int n_groups = (row1 - row0 + kMmaRows - 1) / kMmaRows;                // of sixteen rows in the split
+    const int n_steps = n_groups > warp ? (n_groups - warp + kMmaWarps - 1) / kMmaWarps : 0;
+#pragma unroll
+    for (int st = 0; st < kMmaRing - 1; ++st) issue(st);
+
+    // Query fragments: A row lane / 4 (and + 8, which is the same head) is head (lane / 4) mod GP.
+    const int head = (lane >> 2) % GP;
+    const int part_lo = (lane >> 2) / GP, part_hi = ((lane >> 2) + 8) / GP;      // terms of this lane's two rows of P
+    uint32_t qa[8][2];
+#pragma unroll
+    for (int kk = 0; kk < 8; ++kk) {
+        const __nv_bfloat16* src = q + ((long long)rq.index * n_q_heads + qh0 + head) * kHeadDim + kk * 16 + (lane & 3) * 2;
+        qa[kk][0] = head < gt ? *reinterpret_cast<const uint32_t*>(src) : 0u;
+        qa[kk][1] = head < gt ? *reinterpret_cast<const uint32_t*>(src + 8) : 0u;
+    }
+    // The appended row (Eq. 2) is also written into the cache by the CTA that owns it on the group's
+    // first pass (nobody reads cache row `len` in this step).
+    if (pass == 0 && rq.len >= row0 && rq.len < row1 && warp == 0) {
+        const __nv_bfloat16* src = (lane < 16 ? nk : nv) + l16 * 8;
+        __nv_bfloat16* dst = (lane < 16 ? cache_k : cache_v) + rq.begin * stride_row + head_off +
+                             (long long)rq.len * stride_row + l16 * 8;
+        *reinterpret_cast<uint4*>(dst) = __ldg(reinterpret_cast<const uint4*>(src));
+    }
+
+    float o[16][4];                                  // feature group j: features 8j + 2 (lane mod 4), + 1; rows lane / 4, + 8
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) o[j][c] = 0.f;
+    float m = -INFINITY, l = 0.f;                    // reference and sum (over this lane's keys) of the head
+    // ldmatrix: matrix i of an x4 is addressed by lanes 8i .. 8i + 7
+    const int mi = lane >> 3, mr = lane & 7;
+    const int k_row = (mi >> 1) * 8 + mr, k_chunk = mi & 1;      // K: (rows 0-7, 8-15) x (chunk, next chunk)
+    const int v_row = (mi & 1) * 8 + mr, v_chunk = mi >> 1;      // V: two row halves of one chunk, then of the next
+
+    for (int st = 0; st < n_steps; ++st) {
+        issue(st + kMmaRing - 1);                    // into the buffer that was consumed one iteration ago
+        asm volatile("cp.async.wait_group %0;" ::"n"(kMmaRing - 1) : "memory");
+        __syncwarp();                                // every lane's copies are visible to the whole warp
+        const int base = row0 + (st * kMmaWarps + warp) * kMmaRows;
+        const uint32_t kbuf = ring0 + (uint32_t)(st % kMmaRing) * kMmaStepBytes;
+        const uint32_t vbuf = kbuf + kMmaRows * kDecRowBytes;
+        float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};           // keys 0-7, 8-15
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) {
+            uint32_t b[4];
+            ldmatrix_x4(b, kbuf + k_row * kDecRowBytes + (((2 * kk + k_chunk) ^ (k_row & 7)) << 4));
+            mma_bf16(s[0], qa[kk][0], qa[kk][0], qa[kk][1], qa[kk][1], b[0], b[1]);
+            mma_bf16(s[1], qa[kk][0], qa[kk][0], qa[kk][1], qa[kk][1], b[2], b[3]);
+        }
+        // this lane's four logits: keys 2 (lane mod 4), + 1 of either half (rows + 8 are copies)
+        float x[4] = {s[0][0] * scale_log2, s[0][1] * scale_log2, s[1][0] * scale_log2, s[1][1] * scale_log2};
+        if (base + kMmaRows > row1) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (base + (i >> 1) * 8 + (lane & 3) * 2 + (i & 1) >= row1) x[i] = -INFINITY;
+        }
+        float mx = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        if (__any_sync(0xffffffffu, mx > m + kMmaSlack)) {       // also the first step (m = -inf)
+            const float to = fmaxf(m, mx);
+            const float alpha = dec_ex2(m - to);                 // 0 when m was -inf (mx is finite: row 0 of a step is valid)
+            m = to;
+            l *= alpha;
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) o[j][c] *= alpha;
+        }
+        float pr[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { pr[i] = dec_ex2(x[i] - m); l += pr[i]; }
+        const uint32_t a0 = bf16_term(pr[0], pr[1], part_lo), a1 = bf16_term(pr[0], pr[1], part_hi);
+        const uint32_t a2 = bf16_term(pr[2], pr[3], part_lo), a3 = bf16_term(pr[2], pr[3], part_hi);
+        const uint32_t c0 = GP == 8 ? bf16_term(pr[0], pr[1], 2) : 0u, c2 = GP == 8 ? bf16_term(pr[2], pr[3], 2) : 0u;
+#pragma unroll
+        for (int j = 0; j < 16; j += 2) {
+            uint32_t b[4];
+            ldmatrix_x4_trans(b, vbuf + v_row * kDecRowBytes + (((j + v_chunk) ^ (v_row & 7)) << 4));
+            mma_bf16(o[j], a0, a1, a2, a3, b[0], b[1]);
+            mma_bf16(o[j + 1], a0, a1, a2, a3, b[2], b[3]);
+            if (GP == 8) {
+                mma_bf16(o[j], c0, 0u, c2, 0u, b[0], b[1]);
+                mma_bf16(o[j + 1], c0, 0u, c2, 0u, b[2], b[3]);
+            }
+        }
+        __syncwarp();                                // the buffer may be refilled
+    }
+
+    // ---- combine: the terms of a head in registers, then the warps in warp order -----------------
+    l += __shfl_xor_sync(0xffffffffu, l, 1);
+    l += __shfl_xor_sync(0xffffffffu, l, 2);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        float y0 = o[j][0] + o[j][2], y1 = o[j][1] + o[j][3];
+#pragma unroll
+        for (int ofs = 16; ofs >= 4 * GP; ofs >>= 1) {           // rows lane / 4 of the same head
+            y0 += __shfl_xor_sync(0xffffffffu, y0, ofs);
+            y1 += __shfl_xor_sync(0xffffffffu, y1, ofs);
+        }
+        if ((lane >> 2) < GP) {
+            sh.o[warp][head][8 * j + 2 * (lane & 3)] = y0;
+            sh.o[warp][head][8 * j + 2 * (lane & 3) + 1] = y1;
+        }
+    }
+    if ((lane >> 2) < GP && (lane & 3) == 0) { sh.m[warp][head] = m; sh.l[warp][head] = l; }
+    __syncthreads();
+    // thread t owns feature t of every query head of the pass; references leave the kernel in units
+    // of the raw product, as the scalar kernel's do
+    const int n_splits = rq.n_splits;
+    const long long part_stride = kHeadDim + 2;                  // m, l, o[128]
+    float* my_parts = parts + ((long long)rq.part_begin + ((long long)(h * n_pass + pass) * n_splits + split) * gt) * part_stride;
+    const int t = threadIdx.x;
+    for (int g = 0; g < gt; ++g) {
+        float mx = -INFINITY;
+#pragma unroll
+        for (int w = 0; w < kMmaWarps; ++w) mx = fmaxf(mx, sh.m[w][g]);
+        float lsum = 0.f, osum = 0.f;
+#pragma unroll
+        for (int w = 0; w < kMmaWarps; ++w) {
+            const float a = dec_ex2(sh.m[w][g] - mx);            // 0 for an idle warp
+            lsum = fmaf(sh.l[w][g], a, lsum);
+            osum = fmaf(sh.o[w][g][t], a, osum);
+        }
+        if (n_splits == 1) {
+            out[((long long)rq.index * n_q_heads + qh0 + g) * kHeadDim + t] = osum / lsum;
+        } else {
+            float* rec = my_parts + g * part_stride;
+            if (t == 0) { rec[0] = mx / scale_log2; rec[1] = lsum; }
+            rec[2 + t] = osum;
+        }
+    }
+}
+
 // Several splits: adds the partial results of one (request, KV head, pass, query head) in split
 // order.  One CTA of 128 threads per such unit, thread t owns feature t; the splits' reference
 // values are fetched in one round trip and the records of sixteen splits are requested together
@@ -331,32 +583,42 @@ decode_combine_kernel(const __grid_constant__ DecodeBatch batch, int gt, int n_p
 
 }  // namespace
 
-// The ring needs more dynamic shared memory than the default limit: raised once per device.
-static cudaError_t configure_decode() {
+namespace {
+
+// gt query heads per pass: one head alone stays on the scalar kernel (8192 rows x 32 heads: 24.2 us,
+// 0.85 of the copy bandwidth with the launches), several go to the tensor cores (scalar -> mma, us:
+// 32768 rows, 8 KV heads x 4: 40.5 -> 27.1; 16 requests of 400-3300 rows, 8 x 4: 51.5 -> 27.0;
+// 20000 rows, 16 x 2: 33.7 -> 31.5; 9000 rows, 4 x 16: 24.9 -> 13.5).
+typedef void (*MmaKernel)(DecodeBatch, const __nv_bfloat16*, const __nv_bfloat16*, const __nv_bfloat16*, __nv_bfloat16*,
+                          __nv_bfloat16*, long long, long long, int, int, int, int, int, float, float*, float*);
+MmaKernel mma_kernel(int gt) { return gt > 4 ? decode_mma_kernel<8> : gt > 2 ? decode_mma_kernel<4> : decode_mma_kernel<2>; }
+
+// The rings need more dynamic shared memory than the default limit: raised once per device.
+cudaError_t configure_decode() {
     static unsigned long long configured = 0;
     return once_per_device(configured, []() {
         cudaError_t e = cudaFuncSetAttribute(decode_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
+        for (int gt : {2, 4, 8})
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(mma_kernel(gt), cudaFuncAttributeMaxDynamicSharedMemorySize, kMmaRingBytes);
         return e;
     });
 }
 
-// CTAs of decode_kernel<gt> that one SM holds at a time on the current device (looked up once per
-// device); 0 if the query fails.  The planner sizes the grid to one such wave.
+}  // namespace
+
+// CTAs that one SM holds at a time of the kernel that handles gt query heads per pass, on the current
+// device (looked up once per device); 0 if the query fails.  The planner sizes the grid to one wave.
 int decode_ctas_per_sm(int gt) {
     static int cache[64][4] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    const int idx = gt == 8 ? 3 : gt == 4 ? 2 : gt == 2 ? 1 : 0;
+    const int idx = gt > 4 ? 3 : gt > 2 ? 2 : gt > 1 ? 1 : 0;
     int v = __atomic_load_n(&cache[dev][idx], __ATOMIC_ACQUIRE);
     if (v > 0) return v;
     if (configure_decode() != cudaSuccess) { cudaGetLastError(); return 0; }
     cudaError_t err;
-    if (idx == 3) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, decode_kernel<8>, kDecThreads, kDecRingBytes);
-    else if (idx == 2) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, decode_kernel<4>, kDecThreads, kDecRingBytes);
-    else if (idx == 1) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, decode_kernel<2>, kDecThreads, kDecRingBytes);
+    if (gt > 1) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, mma_kernel(gt), kMmaThreads, kMmaRingBytes);
     else err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, decode_kernel<1>, kDecThreads, kDecRingBytes);
     if (err != cudaSuccess || v <= 0) { cudaGetLastError(); return 0; }
     __atomic_store_n(&cache[dev][idx], v, __ATOMIC_RELEASE);
@@ -372,19 +634,15 @@ cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, cons
     const int group = n_q_heads / n_kv_heads;
     cudaError_t err = configure_decode();
     if (err != cudaSuccess) return err;
-#define LOOKM_LAUNCH_DECODE(GT)                                                                     \
-    err = launch_chained(decode_kernel<GT>, dim3((unsigned)total_ctas), dim3(kDecThreads),          \
-                         (size_t)kDecRingBytes, stream,                                             \
-                         batch, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_new,               \
-                         (const __nv_bfloat16*)v_new, (__nv_bfloat16*)cache_k, (__nv_bfloat16*)cache_v, \
-                         stride_row, stride_head, n_q_heads, n_kv_heads, group, rows_per_split,     \
-                         scale_log2, parts, out);
-    if (gt == 8) { LOOKM_LAUNCH_DECODE(8) }
-    else if (gt == 4) { LOOKM_LAUNCH_DECODE(4) }
-    else if (gt == 2) { LOOKM_LAUNCH_DECODE(2) }
-    else { LOOKM_LAUNCH_DECODE(1) }
-#undef LOOKM_LAUNCH_DECODE
-    return err;
+    if (gt > 1)
+        return launch_chained(mma_kernel(gt), dim3((unsigned)total_ctas), dim3(kMmaThreads), (size_t)kMmaRingBytes, stream,
+                              batch, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new,
+                              (__nv_bfloat16*)cache_k, (__nv_bfloat16*)cache_v, stride_row, stride_head, n_q_heads,
+                              n_kv_heads, group, gt, rows_per_split, scale_log2, parts, out);
+    return launch_chained(decode_kernel<1>, dim3((unsigned)total_ctas), dim3(kDecThreads), (size_t)kDecRingBytes, stream,
+                          batch, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new,
+                          (__nv_bfloat16*)cache_k, (__nv_bfloat16*)cache_v, stride_row, stride_head, n_q_heads, n_kv_heads,
+                          group, rows_per_split, scale_log2, parts, out);
 }
 
 cudaError_t launch_decode_combine(const DecodeBatch& batch, int gt, int n_q_heads, int n_kv_heads,

@@ -164,7 +164,7 @@ constexpr int kDecodeThreads = LOOKM_DEC_THREADS;             // threads per CTA
 constexpr int kDecodeMaxCtasPerSm = 2048 / kDecodeThreads;    // what an SM's thread limit allows
 int decode_ctas_per_sm(int gt);          // resident CTAs per SM of the kernel for this gt (0: unknown)
 
-// gt: query heads handled per pass over the rows (1, 2, 4 or 8; divides the group size)
+// gt: query heads handled per pass over the rows (1 .. 8; divides the group size)
 cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, const void* q,
                           const void* k_new, const void* v_new, void* cache_k, void* cache_v,
                           long long stride_row, long long stride_head, int n_q_heads, int n_kv_heads,

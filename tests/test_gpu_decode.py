@@ -74,6 +74,15 @@ def test_one_step_small_caches(B, Hq, Hkv, n, packed):
     run_step(B, Hq, Hkv, n, n + 3, packed, seed=600 + n)
 
 
+@pytest.mark.parametrize("Hq,Hkv,n,packed", [(2, 1, 15, False), (3, 1, 16, True), (10, 2, 31, False), (6, 1, 14, True),
+                                             (7, 1, 63, False), (16, 2, 128, True), (12, 1, 500, False), (22, 2, 40, False),
+                                             (64, 4, 2047, True), (8, 2, 9001, False)])
+def test_grouped_queries_at_the_edges_of_sixteen_row_steps(B, Hq, Hkv, n, packed):
+    """Groups of 2 to 16 heads (padded to 2, 4 or 8, cut into passes; 11 is prime: one head per pass),
+    with the appended row first, last and in the middle of a step, and splits with idle warps."""
+    run_step(B, Hq, Hkv, n, n + 2, packed, seed=760 + n, q_scale=1.0 + (n % 3))
+
+
 def test_long_cache_is_cut_into_many_splits(B):
     # 2 KV heads x 20001 rows: about 150 splits per head, combined by the last CTA to arrive
     run_step(B, 8, 2, 20000, 20001, False, seed=701)
