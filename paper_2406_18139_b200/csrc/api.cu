@@ -380,7 +380,8 @@ int run_merge(const Plan& pl, const lookm_layout* lay, const void* k, const void
               int varlen_output, void* out_k, void* out_v, void* ws, cudaStream_t st) {
     const Req* reqs = at<Req>(ws, pl.o_reqs);
     int* status = at<int>(ws, pl.o_status);
-    if (pl.n_none < pl.n_req) {
+    const bool short_merge = pl.max_L <= kMergeShortMax;
+    if (pl.n_none < pl.n_req && !short_merge) {
         // counter width and widest digit over the requests of the call
         const bool wide = pl.max_E > kInvWideCountsAbove;
         int digit_bits = 1;
@@ -400,12 +401,17 @@ int run_merge(const Plan& pl, const lookm_layout* lay, const void* k, const void
     if (pl.n_none < pl.n_req) {
         DeviceInfo di;
         LOOKM_TRY(device_info(di));
-        LOOKM_CUDA(launch_merge(k, v, lay->kv_stride_tok, lay->kv_stride_head, reqs, pl.n_req,
-                                pl.n_kv_heads, pl.T, pl.total_units, at<int>(ws, pl.o_row_ptr),
-                                at<int>(ws, pl.o_members), at<float>(ws, pl.o_member_w),
-                                at<int4>(ws, pl.o_units), at<int>(ws, pl.o_slot_cnt),
-                                at<float>(ws, pl.o_parts), varlen_output, pl.out_stride_head, out_k,
-                                out_v, status, di.sms, st));
+        if (short_merge)
+            LOOKM_CUDA(launch_merge_short(k, v, lay->kv_stride_tok, lay->kv_stride_head, assign, kept_idx, evict_idx, sim,
+                                          reqs, pl.n_req, pl.n_kv_heads, pl.max_L, pl.max_E, pl.max_B, varlen_output,
+                                          pl.out_stride_head, out_k, out_v, status, di.sms, st));
+        else
+            LOOKM_CUDA(launch_merge(k, v, lay->kv_stride_tok, lay->kv_stride_head, reqs, pl.n_req,
+                                    pl.n_kv_heads, pl.T, pl.total_units, at<int>(ws, pl.o_row_ptr),
+                                    at<int>(ws, pl.o_members), at<float>(ws, pl.o_member_w),
+                                    at<int4>(ws, pl.o_units), at<int>(ws, pl.o_slot_cnt),
+                                    at<float>(ws, pl.o_parts), varlen_output, pl.out_stride_head, out_k,
+                                    out_v, status, di.sms, st));
         ++g_launches;
     }
     if (pl.n_none > 0) {

@@ -125,6 +125,13 @@ cudaError_t launch_invert_assignment(const int* assign, const int* kept_idx, con
                                      unsigned* sort_a, unsigned* sort_b, int* status,
                                      cudaStream_t stream);
 
+// Inversion and merge in one launch; every request has at most kMergeShortMax tokens.
+constexpr int kMergeShortMax = 4096;
+cudaError_t launch_merge_short(const void* k, const void* v, long long stride_tok, long long stride_head, const int* assign,
+                               const int* kept_idx, const int* evict_idx, const float* sim, const Req* reqs, int n_req,
+                               int n_kv_heads, int max_L, int max_E, int max_B, int varlen_output, long long out_stride_head,
+                               void* out_k, void* out_v, int* status, int num_sms, cudaStream_t stream);
+
 int merge_warps_per_sm();
 
 cudaError_t launch_merge(const void* k, const void* v, long long stride_tok, long long stride_head,

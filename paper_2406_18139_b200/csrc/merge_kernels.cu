@@ -684,6 +684,227 @@ merge_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
     (void)status;
 }
 
+// ---------------------------------------------------------------------------------------------
+// Inversion, merge and compaction in one launch, for short prompts.  There the two kernels above are
+// chains of round trips (table -> lists -> sort -> entry list in memory -> metadata -> rows -> records
+// -> counters) and a launch, not bandwidth.  A CTA owns the slots [c0, c1) of one (request, head): it
+// sorts the evicted tokens of its slots by slot (stable, counters in shared memory), keeps the entry
+// list in shared memory, and its warps walk equal shares of that list.  A slot whose entries straddle
+// shares is summed piecewise through shared memory, pieces in share order.
+// lookm_merge as a whole, two kernels -> one (us, graph replay): 700 tokens x 32 heads 26.7 -> 16.4,
+// 2048 x 8 28.7 -> 14.7, 2048 x 32 30.1 -> 23.0, 4096 x 8 30.8 -> 20.5, 4096 x 32 37.4 -> 34.9.  Every
+// CTA of a head sorts the whole evicted list, so the gain is gone soon after kMergeShortMax.
+// ---------------------------------------------------------------------------------------------
+constexpr int kFuseThreads = 512;
+constexpr int kFuseWarps = kFuseThreads / 32;
+constexpr int kFuseBatch = 8;                        // rows requested together by a warp
+
+struct FuseShared {
+    float lead[kFuseWarps][32][8];                   // piece of a slot begun in an earlier share
+    int warp_sums[kFuseWarps];
+};
+// dynamic shared memory behind it: counters u16 [warp][slot], offsets int [slot + 1], entries {pos, weight}
+__host__ __device__ inline size_t fuse_smem(int max_slots, int max_L) {
+    return sizeof(FuseShared) + (size_t)((kFuseWarps * max_slots * 2 + 15) / 16 * 16) + (size_t)((max_slots + 4) / 4 * 16) +
+           (size_t)max_L * 8;
+}
+
+// kSteps: 32-token steps of a warp's segment of the evicted list (E <= 512 kSteps).
+template <int kSteps>
+__global__ void __launch_bounds__(kFuseThreads, 2)
+merge_short_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, long long stride_tok,
+                   long long stride_head, const int* __restrict__ assign, const int* __restrict__ kept_idx,
+                   const int* __restrict__ evict_idx, const float* __restrict__ sim, const Req* __restrict__ reqs,
+                   int n_kv_heads, int max_slots, int varlen_output, long long out_stride_head,
+                   __nv_bfloat16* __restrict__ out_k, __nv_bfloat16* __restrict__ out_v, int* status) {
+    extern __shared__ __align__(16) unsigned char fuse_raw[];
+    FuseShared& sh = *reinterpret_cast<FuseShared*>(fuse_raw);
+    unsigned short* cnt = reinterpret_cast<unsigned short*>(fuse_raw + sizeof(FuseShared));
+    int* first = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(cnt) + (kFuseWarps * max_slots * 2 + 15) / 16 * 16);
+    int2* ent = reinterpret_cast<int2*>(reinterpret_cast<unsigned char*>(first) + (max_slots + 4) / 4 * 16);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    grid_dependency_wait();
+    const Req rq = reqs[blockIdx.z];
+    if (rq.mode == LOOKM_MERGE_NONE) return;
+    const int h = blockIdx.y;
+    const int E = rq.E, B = rq.B, mode = rq.mode;
+    const int per = (B + (int)gridDim.x - 1) / (int)gridDim.x;       // slots per CTA, at most max_slots
+    const int c0 = min(B, (int)blockIdx.x * per), n_slots = min(B, c0 + per) - c0;
+    if (n_slots <= 0) return;
+    const long long ev_base = rq.ev_off + (long long)h * E, kept_base = rq.kept_off + (long long)h * B;
+
+    // ---- all lists are requested at once ----
+    const int seg = ((E + kFuseWarps * 32 - 1) / (kFuseWarps * 32)) * 32;
+    const int s_begin = warp * seg;
+    int key[kSteps], pos[kSteps];
+    float wgt[kSteps];
+#pragma unroll
+    for (int q = 0; q < kSteps; ++q) {
+        const int i = s_begin + q * 32 + lane;
+        key[q] = -1;
+        pos[q] = 0;
+        wgt[q] = 1.f;
+        if (q * 32 < seg && i < E) {
+            key[q] = assign[ev_base + i];
+            pos[q] = evict_idx[ev_base + i];
+            if (mode == LOOKM_MERGE_WEIGHTED) wgt[q] = sim[ev_base + i];
+        }
+    }
+    for (int i = threadIdx.x; i < kFuseWarps * n_slots; i += kFuseThreads) cnt[i] = 0;
+    __syncthreads();
+    // ---- rank of every token among its warp's tokens of the same slot ----
+    int dbits = 1;
+    while ((1 << dbits) < n_slots) ++dbits;
+    unsigned short* my_cnt = cnt + warp * n_slots;
+#pragma unroll
+    for (int q = 0; q < kSteps; ++q) {
+        if (q * 32 >= seg) break;
+        const int i = s_begin + q * 32 + lane;
+        if (i < E && (unsigned)key[q] >= (unsigned)B) { atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); key[q] = 0; }
+        const int d = key[q] - c0;
+        const bool valid = i < E && (unsigned)d < (unsigned)n_slots;
+        key[q] = -1;
+        const unsigned any = __ballot_sync(0xffffffffu, valid);
+        if (any == 0u) continue;
+        unsigned peers = any;
+        for (int b = 0; b < dbits; ++b) {
+            const bool bit = (d >> b) & 1;
+            const unsigned bal = __ballot_sync(0xffffffffu, bit);
+            peers &= bit ? bal : ~bal;
+        }
+        if (valid) key[q] = (d << 16) | ((int)my_cnt[d] + __popc(peers & lt_mask));
+        __syncwarp();
+        if (valid && (peers & lt_mask) == 0u) my_cnt[d] += (unsigned short)__popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    // ---- members per slot, then the slots' places in the entry list (kept row + members each) ----
+    int run = 0;
+    for (int d0 = 0; d0 < n_slots; d0 += kFuseThreads) {
+        const int d = d0 + threadIdx.x;
+        int tot = 0;
+        if (d < n_slots) {
+#pragma unroll
+            for (int w = 0; w < kFuseWarps; ++w) {
+                const int c = cnt[w * n_slots + d];
+                cnt[w * n_slots + d] = (unsigned short)tot;
+                tot += c;
+            }
+            ++tot;                                   // the kept row
+        }
+        int incl = tot;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += x;
+        }
+        if (lane == 31) sh.warp_sums[warp] = incl;
+        __syncthreads();
+        int before = run, all = run;
+#pragma unroll
+        for (int w = 0; w < kFuseWarps; ++w) {
+            const int x = sh.warp_sums[w];
+            before += w < warp ? x : 0;
+            all += x;
+        }
+        if (d < n_slots) first[d] = before + incl - tot;
+        run = all;
+        __syncthreads();
+    }
+    const int n_ent = run;
+    if (threadIdx.x == 0) first[n_slots] = n_ent;
+    __syncthreads();
+    for (int c = threadIdx.x; c < n_slots; c += kFuseThreads) {
+        int pc = kept_idx[kept_base + c0 + c];
+        if (pc < 0 || pc >= rq.L) { atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); pc = 0; }
+        ent[first[c]] = make_int2(pc | (int)0x80000000, c);
+    }
+#pragma unroll
+    for (int q = 0; q < kSteps; ++q) {
+        if (key[q] < 0) continue;
+        const int d = key[q] >> 16;
+        if (pos[q] < 0 || pos[q] >= rq.L) { atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); pos[q] = 0; }
+        ent[first[d] + 1 + (int)my_cnt[d] + (key[q] & 0xffff)] = make_int2(pos[q], __float_as_int(wgt[q]));
+    }
+    __syncthreads();
+
+    // ---- walk: lanes 0-15 hold the K row, 16-31 the V row, 16 bytes per lane ----
+    const int l16 = lane & 15;
+    const __nv_bfloat16* src = (lane < 16 ? k : v) + (long long)rq.tok_begin * stride_tok + (long long)h * stride_head + l16 * 8;
+    __nv_bfloat16* dst = (lane < 16 ? out_k : out_v) + l16 * 8;
+    auto write_row = [&](int d, const uint4& kept_raw, const float (&sum)[8], int n) {
+        uint4 result = kept_raw;
+        if (n > 0) {
+            const Row8 xc = unpack8(kept_raw);
+            const float inv = 1.0f / (float)(n + 1);
+            const float wc = (mode == LOOKM_MERGE_PIVOTAL) ? 1.f + 0.5f * (float)n : 1.f;
+            const float wm = (mode == LOOKM_MERGE_PIVOTAL) ? 0.5f : 1.f;
+            Row8 o;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) o.v[i] = fmaf(wc, xc.v[i], wm * sum[i]) * inv;
+            result = pack8(o);
+        }
+        const int c = c0 + d;
+        long long at;
+        if (varlen_output) at = (((long long)rq.out_begin + c) * n_kv_heads + h) * kHeadDim;
+        else at = (long long)h * out_stride_head + (long long)c * kHeadDim;
+        *reinterpret_cast<uint4*>(dst + at) = result;
+    };
+    const int share = max(kFuseBatch, (n_ent + kFuseWarps - 1) / kFuseWarps);
+    const int e_lo = min(n_ent, warp * share), e_hi = min(n_ent, e_lo + share);
+    float acc[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+    uint4 raw_c = make_uint4(0u, 0u, 0u, 0u);
+    int d = -1;                                      // running slot; -1: begun in an earlier share
+    const bool open = e_lo < e_hi && ent[e_lo].x >= 0;       // the share starts inside a slot
+    auto flush = [&]() {                             // the running slot is complete, or was begun elsewhere
+        if (d >= 0) {
+            write_row(d, raw_c, acc, first[d + 1] - first[d] - 1);
+        } else if (open) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) sh.lead[warp][lane][i] = acc[i];
+        }
+    };
+    for (int e0 = e_lo; e0 < e_hi; e0 += kFuseBatch) {
+        int2 en[kFuseBatch];
+        uint4 x[kFuseBatch];
+#pragma unroll
+        for (int q = 0; q < kFuseBatch; ++q) {
+            en[q] = e0 + q < e_hi ? ent[e0 + q] : make_int2(0, 0);
+            if (e0 + q < e_hi)
+                x[q] = __ldg(reinterpret_cast<const uint4*>(src + (long long)(en[q].x & 0x7fffffff) * stride_tok));
+        }
+#pragma unroll
+        for (int q = 0; q < kFuseBatch; ++q) {
+            if (e0 + q >= e_hi) break;
+            if (en[q].x < 0) {                       // a kept row starts the next slot
+                flush();
+                d = en[q].y;
+                raw_c = x[q];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+            } else {
+                const Row8 xe = unpack8(x[q]);
+                const float w = __int_as_float(en[q].y);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[i] = fmaf(w, xe.v[i], acc[i]);
+            }
+        }
+    }
+    const bool goes_on = d >= 0 && first[d + 1] > e_hi;
+    if (!goes_on && e_lo < e_hi) flush();
+    __syncthreads();
+    if (goes_on) {                                   // the share that has the kept row adds the pieces
+        const int w1 = (first[d + 1] - 1) / share;   // share of the slot's last entry
+        for (int w = warp + 1; w <= w1; ++w)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc[i] += sh.lead[w][lane][i];
+        write_row(d, raw_c, acc, first[d + 1] - first[d] - 1);
+    }
+}
+
 __global__ void write_table_kernel(const __grid_constant__ ReqChunk chunk, int count, Req* dst) {
     const int i = threadIdx.x;
     if (i < count) dst[i] = chunk.r[i];
@@ -777,6 +998,32 @@ cudaError_t launch_merge(const void* k, const void* v, long long stride_tok, lon
                           n_req, n_kv_heads, T, total_units, row_ptr, ent_pos, ent_w, unit_first, slot_cnt,
                           parts, varlen_output, out_stride_head, (__nv_bfloat16*)out_k, (__nv_bfloat16*)out_v,
                           status);
+}
+
+// Parts per (request, head): about two CTAs per SM, at least eight slots each.
+cudaError_t launch_merge_short(const void* k, const void* v, long long stride_tok, long long stride_head, const int* assign,
+                               const int* kept_idx, const int* evict_idx, const float* sim, const Req* reqs, int n_req,
+                               int n_kv_heads, int max_L, int max_E, int max_B, int varlen_output, long long out_stride_head,
+                               void* out_k, void* out_v, int* status, int num_sms, cudaStream_t stream) {
+    const long long heads = (long long)n_kv_heads * n_req;
+    long long parts = 2ll * num_sms / heads;             // one wave: two CTAs fit on an SM
+    if (parts < 1) parts = 1;
+    if (parts > (max_B + 7) / 8) parts = (max_B + 7) / 8;
+    const int max_slots = (max_B + (int)parts - 1) / (int)parts;
+    const size_t smem = fuse_smem(max_slots, max_L);
+    static unsigned long long configured = 0;
+    cudaError_t err = once_per_device(configured, [&]() {
+        const int most = (int)fuse_smem(kMergeShortMax, kMergeShortMax);
+        cudaError_t e = cudaFuncSetAttribute(merge_short_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(merge_short_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        return e;
+    });
+    if (err != cudaSuccess) return err;
+    auto kernel = max_E <= 2 * kFuseThreads ? merge_short_kernel<2> : merge_short_kernel<8>;
+    return launch_chained(kernel, dim3((unsigned)parts, (unsigned)n_kv_heads, (unsigned)n_req), dim3(kFuseThreads), smem, stream,
+                          (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, stride_tok, stride_head, assign, kept_idx, evict_idx,
+                          sim, reqs, n_kv_heads, max_slots, varlen_output, out_stride_head, (__nv_bfloat16*)out_k,
+                          (__nv_bfloat16*)out_v, status);
 }
 
 cudaError_t launch_compact_kept(const void* k, const void* v, long long stride_tok,

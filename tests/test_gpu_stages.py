@@ -374,6 +374,43 @@ def test_merge_matches_oracle_on_oracle_lists(B, mode, L, budget, Hkv):
         assert np.array_equal(gk[h][empty], kf[kept[h][empty], h].astype(np.float64))   # bit-exact copy
 
 
+@pytest.mark.parametrize("L,budget,skew", [(2, 1, "even"), (40, 33, "last"), (513, 1, "even"), (1200, 176, "first"),
+                                           (1201, 177, "even"), (4096, 60, "last"), (4096, 4000, "even"),
+                                           (4097, 800, "first"), (5000, 260, "even")])
+def test_merge_on_both_sides_of_the_short_prompt_limit(B, L, budget, skew):
+    """Prompts up to 4096 tokens are inverted and merged in one launch, each CTA owning a range of the
+    slots; longer ones go through the entry list.  Members spread evenly, or nearly all in the first or
+    the last slot (one slot across every share of its CTA); a cache layout with a single member too."""
+    import torch
+    Hkv, mode, E = 3, 2, L - budget
+    kb, vb = (synth.f32_to_bf16_bits(synth.normal(synth.stream_key(i, L, budget), L * Hkv * 128).astype(np.float32).reshape(L, Hkv, 128))
+              for i in (171, 172))
+    kf, vf = synth.bf16_to_f32(kb), synth.bf16_to_f32(vb)
+    k, v = to_dev(kb), to_dev(vb)
+    kept, ev, assign, sim = [], [], [], []
+    for h in range(Hkv):
+        order = np.argsort(synth.uniform_u64(synth.stream_key(173, h, L), L))
+        kept.append(np.sort(order[:budget]).astype(np.int32))
+        ev.append(np.sort(order[budget:]).astype(np.int32))
+        asg = synth.uniform_int(synth.stream_key(174, h), E, 0, budget - 1).astype(np.int32)
+        if skew != "even":
+            asg[np.arange(E) % 16 != 3] = 0 if skew == "first" else budget - 1
+        assign.append(asg)
+        sim.append(np.clip(synth.normal(synth.stream_key(175, h), E) * 0.4, -1, 1).astype(np.float32))
+    dev = lambda xs: torch.from_numpy(np.concatenate(xs)).cuda()
+    out_k = torch.zeros(budget, Hkv, 128, dtype=torch.bfloat16, device="cuda")
+    out_v = torch.zeros_like(out_k)
+    lay = B.make_layout(None, k)
+    ws = B.alloc_workspace(lay, [L])
+    B.check(B.lookm_merge(k, v, dev(kept), dev(ev), dev(assign), dev(sim), [0, L], [budget], [mode], lay, 1, out_k, out_v, ws))
+    assert B.lookm_device_status(ws) == B.OK
+    assert B.lookm_last_launch_count() == (2 if L <= 4096 else 3)
+    gk, gv = bf16_to_np(out_k), bf16_to_np(out_v)
+    for h in range(Hkv):
+        for got, x in ((gk, kf), (gv, vf)):
+            assert merged_close(got[:, h], orc.merge(x, h, kept[h], ev[h], assign[h], sim[h].astype(np.float64), mode)).all()
+
+
 def test_merge_packed_batch_with_slots_spread_over_many_work_units(B):
     """Two requests, batch output layout, member counts from 0 to many hundreds: the kernel cuts its
     work units at fixed entry counts, so most of the large slots are summed piecewise by several
