@@ -487,7 +487,7 @@ int compress_common(const void* q, const void* k, const void* v, const uint8_t* 
     // the selection launch also computes the key norms that the matching needs
     const bool need_match = pl.n_items[kMatch] > 0;
     LOOKM_CUDA(launch_select(scores, text_prior ? mask : nullptr, at<Req>(ws, pl.o_reqs), pl.n_req,
-                             pl.n_kv_heads, pl.T, kept, evict, rank, need_match ? k : nullptr,
+                             pl.n_kv_heads, pl.T, pl.max_L, kept, evict, rank, need_match ? k : nullptr,
                              lay->kv_stride_tok, lay->kv_stride_head, at<float>(ws, pl.o_rnorm_all),
                              di.sms, st));
     ++g_launches;
@@ -610,7 +610,7 @@ int lookm_select(const float* scores, const uint8_t* modality_mask, const int* c
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     LOOKM_TRY(begin_call(pl, workspace, st));
     LOOKM_CUDA(launch_select(scores, modality_mask, at<Req>(workspace, pl.o_reqs), pl.n_req,
-                             pl.n_kv_heads, pl.T, kept_idx, evict_idx, rank, nullptr, 0, 0, nullptr, 0, st));
+                             pl.n_kv_heads, pl.T, pl.max_L, kept_idx, evict_idx, rank, nullptr, 0, 0, nullptr, 0, st));
     ++g_launches;
     return LOOKM_OK;
 }

@@ -96,7 +96,7 @@ cudaError_t launch_lse_split(const float* lse, int n_q_heads, long long T, float
 cudaError_t launch_wait_probe(unsigned long long limit_ns, int* status, cudaStream_t stream);
 
 cudaError_t launch_select(const float* scores, const uint8_t* mask, const Req* reqs, int n_req,
-                          int n_kv_heads, long long T, int* kept_idx, int* evict_idx, int* rank,
+                          int n_kv_heads, long long T, int max_L, int* kept_idx, int* evict_idx, int* rank,
                           const void* k_for_norms, long long stride_tok, long long stride_head,
                           float* rnorm_all, int num_sms, cudaStream_t stream);
 
