@@ -118,14 +118,20 @@ def _ints(seq: Optional[Sequence[int]]):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> C.c_void_p:
+def _stream(stream) -> int:
+    """The raw handle of `stream`, or of PyTorch's current stream on the current device (asked for
+    directly: building a torch.cuda.Stream object takes longer than a small call)."""
     if stream is None:
         import torch
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
+
+
+def _nbytes(t) -> int:
+    return t.nbytes
 
 
 def lookm_strerror(status: int) -> str:
@@ -204,7 +210,7 @@ def lookm_compress_layer(q, k, v, modality_mask, seq_len, budget, recent_window,
     st = lib().lookm_compress_layer(_ptr(q), _ptr(k), _ptr(v), _ptr(modality_mask), int(seq_len),
                                     int(budget), int(recent_window), int(merge_mode), C.byref(layout),
                                     _ptr(out_k), _ptr(out_v), C.byref(out_len), _ptr(workspace),
-                                    workspace.numel() * workspace.element_size(), _stream(stream))
+                                    _nbytes(workspace), _stream(stream))
     return st, out_len.value
 
 
@@ -216,7 +222,7 @@ def lookm_compress_layer_opt(q, k, v, modality_mask, seq_len, budget, recent_win
                                         int(budget), int(recent_window), int(merge_mode), C.byref(layout),
                                         None if options is None else C.byref(options), _ptr(out_k),
                                         _ptr(out_v), C.byref(out_len), _ptr(workspace),
-                                        workspace.numel() * workspace.element_size(), _stream(stream))
+                                        _nbytes(workspace), _stream(stream))
     return st, out_len.value
 
 
@@ -228,7 +234,7 @@ def lookm_compress_varlen(q, k, v, modality_mask, cu_seqlens, budgets, windows, 
     st = lib().lookm_compress_varlen(_ptr(q), _ptr(k), _ptr(v), _ptr(modality_mask), _ints(cu_seqlens),
                                      n, _ints(budgets), _ints(windows), _ints(merge_modes),
                                      C.byref(layout), _ptr(out_k), _ptr(out_v), out_cu, _ptr(workspace),
-                                     workspace.numel() * workspace.element_size(), _stream(stream))
+                                     _nbytes(workspace), _stream(stream))
     return st, list(out_cu)
 
 
@@ -241,14 +247,14 @@ def lookm_compress_varlen_opt(q, k, v, modality_mask, cu_seqlens, budgets, windo
                                          n, _ints(budgets), _ints(windows), _ints(merge_modes),
                                          C.byref(layout), None if options is None else C.byref(options),
                                          _ptr(out_k), _ptr(out_v), out_cu, _ptr(workspace),
-                                         workspace.numel() * workspace.element_size(), _stream(stream))
+                                         _nbytes(workspace), _stream(stream))
     return st, list(out_cu)
 
 
 def lookm_score(q, k, cu_seqlens, layout, scores, lse, lse_is_input, workspace, stream=None):
     return lib().lookm_score(_ptr(q), _ptr(k), _ints(cu_seqlens), len(cu_seqlens) - 1, C.byref(layout),
                              _ptr(scores), _ptr(lse), int(bool(lse_is_input)), _ptr(workspace),
-                             workspace.numel() * workspace.element_size(), _stream(stream))
+                             _nbytes(workspace), _stream(stream))
 
 
 def lookm_select(scores, modality_mask, cu_seqlens, budgets, windows, n_kv_heads, kept_idx, evict_idx,
@@ -256,20 +262,20 @@ def lookm_select(scores, modality_mask, cu_seqlens, budgets, windows, n_kv_heads
     return lib().lookm_select(_ptr(scores), _ptr(modality_mask), _ints(cu_seqlens), len(cu_seqlens) - 1,
                               _ints(budgets), _ints(windows), int(n_kv_heads), _ptr(kept_idx),
                               _ptr(evict_idx), _ptr(rank), _ptr(workspace),
-                              workspace.numel() * workspace.element_size(), _stream(stream))
+                              _nbytes(workspace), _stream(stream))
 
 
 def lookm_match(k, kept_idx, evict_idx, cu_seqlens, budgets, layout, assign, sim, workspace, stream=None):
     return lib().lookm_match(_ptr(k), _ptr(kept_idx), _ptr(evict_idx), _ints(cu_seqlens),
                              len(cu_seqlens) - 1, _ints(budgets), C.byref(layout), _ptr(assign),
-                             _ptr(sim), _ptr(workspace), workspace.numel() * workspace.element_size(),
+                             _ptr(sim), _ptr(workspace), _nbytes(workspace),
                              _stream(stream))
 
 
 def lookm_match_from_sim(sim_matrix, cu_seqlens, budgets, n_kv_heads, assign, sim, workspace, stream=None):
     return lib().lookm_match_from_sim(_ptr(sim_matrix), _ints(cu_seqlens), len(cu_seqlens) - 1,
                                       _ints(budgets), int(n_kv_heads), _ptr(assign), _ptr(sim),
-                                      _ptr(workspace), workspace.numel() * workspace.element_size(),
+                                      _ptr(workspace), _nbytes(workspace),
                                       _stream(stream))
 
 
@@ -278,7 +284,7 @@ def lookm_merge(k, v, kept_idx, evict_idx, assign, sim, cu_seqlens, budgets, mer
     return lib().lookm_merge(_ptr(k), _ptr(v), _ptr(kept_idx), _ptr(evict_idx), _ptr(assign), _ptr(sim),
                              _ints(cu_seqlens), len(cu_seqlens) - 1, _ints(budgets), _ints(merge_modes),
                              C.byref(layout), int(bool(varlen_output)), _ptr(out_k), _ptr(out_v),
-                             _ptr(workspace), workspace.numel() * workspace.element_size(),
+                             _ptr(workspace), _nbytes(workspace),
                              _stream(stream))
 
 
@@ -312,7 +318,7 @@ def lookm_decode_step(q, k_new, v_new, cache_k, cache_v, cache_len, layout: Cach
                       stream=None):
     return lib().lookm_decode_step(_ptr(q), _ptr(k_new), _ptr(v_new), _ptr(cache_k), _ptr(cache_v),
                                    int(cache_len), C.byref(layout), _ptr(out), _ptr(workspace),
-                                   workspace.numel() * workspace.element_size(), _stream(stream))
+                                   _nbytes(workspace), _stream(stream))
 
 
 def lookm_decode_step_varlen(q, k_new, v_new, cache_k, cache_v, cache_begin, cache_lens, layout: CacheLayout,
@@ -321,7 +327,7 @@ def lookm_decode_step_varlen(q, k_new, v_new, cache_k, cache_v, cache_begin, cac
     return lib().lookm_decode_step_varlen(_ptr(q), _ptr(k_new), _ptr(v_new), _ptr(cache_k), _ptr(cache_v),
                                           begins, _ints(cache_lens), len(cache_lens), C.byref(layout),
                                           _ptr(out), _ptr(workspace),
-                                          workspace.numel() * workspace.element_size(), _stream(stream))
+                                          _nbytes(workspace), _stream(stream))
 
 
 _stage_event_array = None
@@ -341,7 +347,7 @@ def lookm_set_stage_events(events) -> int:
 
 def lookm_selftest_wait_expiry(limit_us: int, workspace, stream=None) -> int:
     return lib().lookm_selftest_wait_expiry(int(limit_us), _ptr(workspace),
-                                            workspace.numel() * workspace.element_size(), _stream(stream))
+                                            _nbytes(workspace), _stream(stream))
 
 
 def lookm_device_status(workspace, stream=None) -> int:
