@@ -809,8 +809,11 @@ extern "C" int lookm_noalloc_status(void* cuda_stream) {
 // ------------------------------------------------------------------------------------------------
 namespace {
 
+constexpr int kDecodeClusterRows = 256;
+
 struct DecodePlan {
     int n_req = 0, gt = 1, n_pass = 1, rows_per_split = 64;
+    int cluster = 1;                        // > 1: so many splits everywhere, added up inside the launch
     std::vector<DecodeReq> reqs;            // caller order
     size_t o_parts = 0, total = 0;
 };
@@ -869,6 +872,24 @@ int build_decode_plan(DecodePlan& dp, const lookm_cache_layout* lay, int n_req, 
             s = lo;
         }
     }
+    if (lens) {
+        // 2, 4 or 8 splits per (KV head, pass) that one cluster adds up, instead of a second launch: as
+        // many as leave every CTA an SM of its own (clusters of 8 fill about two thirds of the SMs
+        // before two share one, smaller ones seven eighths: 16 heads x 8 took 5.7 us where 12 x 8 took
+        // 3.1).  Worth it while a split is short, or at any length if the CTAs cover nearly all SMs;
+        // us per step, two launches -> one: 32 heads x 4 splits 409 rows 4.6 -> 3.8, 8192 rows
+        // 24.4 -> 23.2; 12 x 8 1638 rows 5.3 -> 4.9, 8192 rows 12.6 -> 13.0; 16 x 4 800 rows 4.6 -> 4.7
+        // (5.8 instead of 8.0 with the launches issued one by one), 3000 rows 7.0 -> 9.1.
+        int longest = 0;
+        for (int r = 0; r < n_req; ++r) longest = std::max(longest, lens[r] + 1);
+        int c = kDecodeMaxCluster;
+        while (c > 1 && n_req * units * c > (c == 8 ? sms * 2 / 3 : sms * 7 / 8)) c /= 2;
+        const long long rows = (longest + c - 1) / c;
+        if (c > 1 && s < longest && (rows <= kDecodeClusterRows || (n_req == 1 && units * c >= sms * 4 / 5))) {
+            dp.cluster = c;
+            s = rows;
+        }
+    }
     if (s >= (1ll << 31)) return LOOKM_ERR_UNSUPPORTED;
     dp.rows_per_split = (int)s;
     // at most one wave of the fullest kernel, or one (short) split per (request, KV head, pass)
@@ -883,7 +904,7 @@ int build_decode_plan(DecodePlan& dp, const lookm_cache_layout* lay, int n_req, 
             q.begin = begins ? begins[r] : 0;
             q.len = lens[r];
             q.index = r;
-            q.n_splits = (int)(((long long)lens[r] + 1 + s - 1) / s);
+            q.n_splits = dp.cluster > 1 ? dp.cluster : (int)(((long long)lens[r] + 1 + s - 1) / s);
             q.cta_begin = 0;
             q.part_begin = (int)parts;
             q.pad = 0;
@@ -924,10 +945,10 @@ int decode_common(const void* q, const void* k_new, const void* v_new, void* cac
             batch.r[i] = dp.reqs[base + i];
             batch.r[i].cta_begin = (int)ctas;
             ctas += (long long)batch.r[i].n_splits * units;
-            split = split || batch.r[i].n_splits > 1;
+            split = split || (batch.r[i].n_splits > 1 && dp.cluster == 1);
         }
         if (ctas >= (1ll << 31)) return LOOKM_ERR_UNSUPPORTED;
-        LOOKM_CUDA(launch_decode(batch, (int)ctas, dp.gt, q, k_new, v_new, cache_k, cache_v,
+        LOOKM_CUDA(launch_decode(batch, (int)ctas, dp.gt, dp.cluster, q, k_new, v_new, cache_k, cache_v,
                                  lay->cache_stride_row, lay->cache_stride_head, lay->n_q_heads,
                                  lay->n_kv_heads, dp.rows_per_split, scale * 1.4426950408889634f,
                                  at<float>(ws, dp.o_parts), out, st));

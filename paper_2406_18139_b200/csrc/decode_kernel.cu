@@ -56,6 +56,66 @@ __device__ __forceinline__ float dec_ex2(float x) {
     return y;
 }
 
+// Clusters: for short caches all splits of a (request, KV head, pass) are the CTAs of one thread-block
+// cluster, which add their results through distributed shared memory, so that no second kernel and no
+// partial results in memory are needed.
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// a float of this CTA's shared memory, in CTA `rank` of the cluster
+__device__ __forceinline__ float ld_cluster(const float* p, uint32_t rank) {
+    uint32_t at;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(at) : "memory");
+    return v;
+}
+// What a CTA leaves for the cluster: per query head of the pass reference, sum and weighted V sum.
+template <int GP>
+struct ClusterShared {
+    float m[GP], l[GP];
+    float o[GP][kHeadDim];
+};
+// Adds the n splits of the cluster in split order; every CTA writes its share of the features of gt
+// heads.  `unit`: factor that turns references into log2.
+template <int GP>
+__device__ __forceinline__ void cluster_combine(const ClusterShared<GP>& cs, int n, int gt, float unit, float* out) {
+    cluster_sync();
+    const int share = kHeadDim / n;
+    for (int i = threadIdx.x; i < gt * share; i += blockDim.x) {
+        const int g = i / share, t = (int)cluster_rank() * share + i % share;
+        float m[kDecodeMaxCluster], l[kDecodeMaxCluster], o[kDecodeMaxCluster];
+        float mx = -INFINITY;
+#pragma unroll
+        for (int c = 0; c < kDecodeMaxCluster; ++c) {
+            m[c] = -INFINITY;
+            l[c] = o[c] = 0.f;
+            if (c < n) {
+                m[c] = ld_cluster(&cs.m[g], c);
+                l[c] = ld_cluster(&cs.l[g], c);
+                o[c] = ld_cluster(&cs.o[g][t], c);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < kDecodeMaxCluster; ++c) mx = fmaxf(mx, m[c]);
+        float lsum = 0.f, osum = 0.f;
+#pragma unroll
+        for (int c = 0; c < kDecodeMaxCluster; ++c) {
+            const float a = m[c] == -INFINITY ? 0.f : dec_ex2((m[c] - mx) * unit);       // a split may be empty
+            lsum = fmaf(l[c], a, lsum);
+            osum = fmaf(o[c], a, osum);
+        }
+        out[(long long)g * kHeadDim + t] = osum / lsum;
+    }
+    cluster_sync();                                  // nobody leaves while its shared memory is read
+}
+
 template <int GT>
 struct DecShared {
     float m[kDecWarps][GT];                          // [warp][query head of the pass]
@@ -64,7 +124,7 @@ struct DecShared {
 };
 
 // GT query heads of the group are handled per pass over the rows; only GT = 1 is instantiated.
-template <int GT>
+template <int GT, bool kClustered>
 __global__ void __launch_bounds__(kDecThreads)
 decode_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __restrict__ q,
               const __nv_bfloat16* __restrict__ k_new, const __nv_bfloat16* __restrict__ v_new,
@@ -72,6 +132,7 @@ decode_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __
               long long stride_row, long long stride_head, int n_q_heads, int n_kv_heads, int group,
               int rows_per_split, float scale_log2, float* __restrict__ parts, float* __restrict__ out) {
     __shared__ DecShared<GT> sh;
+    __shared__ ClusterShared<GT> cs;
     extern __shared__ __align__(128) uint8_t dec_ring[];         // [warp][ring step][half][row][K|V][256 B]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int hw = threadIdx.x >> 4, l16 = lane & 15;
@@ -264,11 +325,14 @@ decode_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __
             float lsum = 0.f, osum = 0.f;
 #pragma unroll
             for (int w = 0; w < kDecWarps; ++w) {
-                const float a = dec_ex2((sh.m[w][g] - mx) * scale_log2);   // 0 for an idle warp
+                const float a = mx == -INFINITY ? 0.f : dec_ex2((sh.m[w][g] - mx) * scale_log2);   // 0 for an idle warp
                 lsum = fmaf(sh.l[w][g], a, lsum);
                 osum = fmaf(sh.o[w][g][t], a, osum);
             }
-            if (n_splits == 1) {
+            if (kClustered) {
+                if (t == 0) { cs.m[g] = mx; cs.l[g] = lsum; }
+                cs.o[g][t] = osum;
+            } else if (n_splits == 1) {
                 out[((long long)rq.index * n_q_heads + qh0 + g) * kHeadDim + t] = osum / lsum;
             } else {
                 float* rec = my_parts + g * part_stride;
@@ -277,6 +341,8 @@ decode_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __
             }
         }
     }
+    if (kClustered)
+        cluster_combine(cs, n_splits, GT, scale_log2, out + ((long long)rq.index * n_q_heads + qh0) * kHeadDim);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -332,7 +398,7 @@ struct MmaShared {
 };
 
 // gt <= GP query heads of the group are handled per pass over the rows.
-template <int GP>
+template <int GP, bool kClustered>
 __global__ void __launch_bounds__(kMmaThreads)
 decode_mma_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __restrict__ q,
                   const __nv_bfloat16* __restrict__ k_new, const __nv_bfloat16* __restrict__ v_new,
@@ -340,6 +406,7 @@ decode_mma_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16
                   long long stride_row, long long stride_head, int n_q_heads, int n_kv_heads, int group, int gt,
                   int rows_per_split, float scale_log2, float* __restrict__ parts, float* __restrict__ out) {
     __shared__ MmaShared<GP> sh;
+    __shared__ ClusterShared<GP> cs;
     extern __shared__ __align__(128) uint8_t dec_ring[];         // [warp][ring step][K|V][row][256 B, swizzled]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int r = 0;
@@ -515,11 +582,14 @@ decode_mma_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16
         float lsum = 0.f, osum = 0.f;
 #pragma unroll
         for (int w = 0; w < kMmaWarps; ++w) {
-            const float a = dec_ex2(sh.m[w][g] - mx);            // 0 for an idle warp
+            const float a = mx == -INFINITY ? 0.f : dec_ex2(sh.m[w][g] - mx);    // 0 for an idle warp
             lsum = fmaf(sh.l[w][g], a, lsum);
             osum = fmaf(sh.o[w][g][t], a, osum);
         }
-        if (n_splits == 1) {
+        if (kClustered) {
+            if (t == 0) { cs.m[g] = mx; cs.l[g] = lsum; }
+            cs.o[g][t] = osum;
+        } else if (n_splits == 1) {
             out[((long long)rq.index * n_q_heads + qh0 + g) * kHeadDim + t] = osum / lsum;
         } else {
             float* rec = my_parts + g * part_stride;
@@ -527,6 +597,7 @@ decode_mma_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16
             rec[2 + t] = osum;
         }
     }
+    if (kClustered) cluster_combine(cs, n_splits, gt, 1.f, out + ((long long)rq.index * n_q_heads + qh0) * kHeadDim);
 }
 
 // Several splits: adds the partial results of one (request, KV head, pass, query head) in split
@@ -591,16 +662,23 @@ namespace {
 // 20000 rows, 16 x 2: 33.7 -> 31.5; 9000 rows, 4 x 16: 24.9 -> 13.5).
 typedef void (*MmaKernel)(DecodeBatch, const __nv_bfloat16*, const __nv_bfloat16*, const __nv_bfloat16*, __nv_bfloat16*,
                           __nv_bfloat16*, long long, long long, int, int, int, int, int, float, float*, float*);
-MmaKernel mma_kernel(int gt) { return gt > 4 ? decode_mma_kernel<8> : gt > 2 ? decode_mma_kernel<4> : decode_mma_kernel<2>; }
+MmaKernel mma_kernel(int gt, bool clustered) {
+    if (clustered)
+        return gt > 4 ? decode_mma_kernel<8, true> : gt > 2 ? decode_mma_kernel<4, true> : decode_mma_kernel<2, true>;
+    return gt > 4 ? decode_mma_kernel<8, false> : gt > 2 ? decode_mma_kernel<4, false> : decode_mma_kernel<2, false>;
+}
 
 // The rings need more dynamic shared memory than the default limit: raised once per device.
 cudaError_t configure_decode() {
     static unsigned long long configured = 0;
     return once_per_device(configured, []() {
-        cudaError_t e = cudaFuncSetAttribute(decode_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
+        cudaError_t e = cudaFuncSetAttribute(decode_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(decode_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
         for (int gt : {2, 4, 8})
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(mma_kernel(gt), cudaFuncAttributeMaxDynamicSharedMemorySize, kMmaRingBytes);
+            for (bool clustered : {false, true})
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute(mma_kernel(gt, clustered), cudaFuncAttributeMaxDynamicSharedMemorySize, kMmaRingBytes);
         return e;
     });
 }
@@ -618,14 +696,14 @@ int decode_ctas_per_sm(int gt) {
     if (v > 0) return v;
     if (configure_decode() != cudaSuccess) { cudaGetLastError(); return 0; }
     cudaError_t err;
-    if (gt > 1) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, mma_kernel(gt), kMmaThreads, kMmaRingBytes);
-    else err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, decode_kernel<1>, kDecThreads, kDecRingBytes);
+    if (gt > 1) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, mma_kernel(gt, false), kMmaThreads, kMmaRingBytes);
+    else err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, decode_kernel<1, false>, kDecThreads, kDecRingBytes);
     if (err != cudaSuccess || v <= 0) { cudaGetLastError(); return 0; }
     __atomic_store_n(&cache[dev][idx], v, __ATOMIC_RELEASE);
     return v;
 }
 
-cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, const void* q,
+cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, int cluster, const void* q,
                           const void* k_new, const void* v_new, void* cache_k, void* cache_v,
                           long long stride_row, long long stride_head, int n_q_heads, int n_kv_heads,
                           int rows_per_split, float scale_log2, float* parts, float* out,
@@ -634,15 +712,17 @@ cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, cons
     const int group = n_q_heads / n_kv_heads;
     cudaError_t err = configure_decode();
     if (err != cudaSuccess) return err;
+    const bool clustered = cluster > 1;
     if (gt > 1)
-        return launch_chained(mma_kernel(gt), dim3((unsigned)total_ctas), dim3(kMmaThreads), (size_t)kMmaRingBytes, stream,
-                              batch, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new,
-                              (__nv_bfloat16*)cache_k, (__nv_bfloat16*)cache_v, stride_row, stride_head, n_q_heads,
-                              n_kv_heads, group, gt, rows_per_split, scale_log2, parts, out);
-    return launch_chained(decode_kernel<1>, dim3((unsigned)total_ctas), dim3(kDecThreads), (size_t)kDecRingBytes, stream,
-                          batch, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new,
-                          (__nv_bfloat16*)cache_k, (__nv_bfloat16*)cache_v, stride_row, stride_head, n_q_heads, n_kv_heads,
-                          group, rows_per_split, scale_log2, parts, out);
+        return launch_chained_clusters(mma_kernel(gt, clustered), dim3((unsigned)total_ctas), dim3(kMmaThreads), (unsigned)cluster,
+                                       (size_t)kMmaRingBytes, stream, batch, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_new,
+                                       (const __nv_bfloat16*)v_new, (__nv_bfloat16*)cache_k, (__nv_bfloat16*)cache_v, stride_row,
+                                       stride_head, n_q_heads, n_kv_heads, group, gt, rows_per_split, scale_log2, parts, out);
+    return launch_chained_clusters(clustered ? decode_kernel<1, true> : decode_kernel<1, false>, dim3((unsigned)total_ctas),
+                                   dim3(kDecThreads), (unsigned)cluster, (size_t)kDecRingBytes, stream, batch, (const __nv_bfloat16*)q,
+                                   (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, (__nv_bfloat16*)cache_k,
+                                   (__nv_bfloat16*)cache_v, stride_row, stride_head, n_q_heads, n_kv_heads, group,
+                                   rows_per_split, scale_log2, parts, out);
 }
 
 cudaError_t launch_decode_combine(const DecodeBatch& batch, int gt, int n_q_heads, int n_kv_heads,

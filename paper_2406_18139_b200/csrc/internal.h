@@ -169,10 +169,12 @@ struct DecodeBatch { int n_req; int pad; DecodeReq r[kDecodeChunk]; };
 #endif
 constexpr int kDecodeThreads = LOOKM_DEC_THREADS;             // threads per CTA of the decode kernel
 constexpr int kDecodeMaxCtasPerSm = 2048 / kDecodeThreads;    // what an SM's thread limit allows
+constexpr int kDecodeMaxCluster = 8;     // splits of a (KV head, pass) that one thread-block cluster adds up
 int decode_ctas_per_sm(int gt);          // resident CTAs per SM of the kernel for this gt (0: unknown)
 
 // gt: query heads handled per pass over the rows (1 .. 8; divides the group size)
-cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, const void* q,
+// cluster > 1: every request has that many splits, which add up inside the launch
+cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, int cluster, const void* q,
                           const void* k_new, const void* v_new, void* cache_k, void* cache_v,
                           long long stride_row, long long stride_head, int n_q_heads, int n_kv_heads,
                           int rows_per_split, float scale_log2, float* parts, float* out,
@@ -203,19 +205,28 @@ inline cudaError_t once_per_device(unsigned long long& mask, F configure) {
 // returns once that kernel has completed and its writes are visible (a no-op for plain launches).
 #ifdef __CUDACC__
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                  cudaStream_t stream, Args... args) {
+inline cudaError_t launch_chained_clusters(void (*kernel)(KArgs...), dim3 grid, dim3 block, unsigned cluster, size_t smem,
+                                           cudaStream_t stream, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                  cudaStream_t stream, Args... args) {
+    return launch_chained_clusters(kernel, grid, block, 1u, smem, stream, args...);
 }
 __device__ __forceinline__ void grid_dependency_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

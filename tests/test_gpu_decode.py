@@ -83,6 +83,15 @@ def test_grouped_queries_at_the_edges_of_sixteen_row_steps(B, Hq, Hkv, n, packed
     run_step(B, Hq, Hkv, n, n + 2, packed, seed=760 + n, q_scale=1.0 + (n % 3))
 
 
+@pytest.mark.parametrize("Hq,Hkv,n", [(1, 1, 17), (8, 8, 16), (12, 12, 409), (13, 13, 700), (32, 32, 18), (32, 32, 4095),
+                                      (48, 48, 401), (64, 16, 100), (24, 3, 50), (40, 40, 520)])
+def test_splits_added_up_by_a_cluster(B, Hq, Hkv, n):
+    """Clusters of 2, 4 and 8 CTAs, scalar and grouped queries, with splits that get no row at all
+    (17 rows over 8 splits of 3); one launch."""
+    run_step(B, Hq, Hkv, n, n + 1, n % 2 == 0, seed=790 + n + Hq)
+    assert B.lookm_last_launch_count() == (1 if n != 520 else 2)
+
+
 def test_long_cache_is_cut_into_many_splits(B):
     # 2 KV heads x 20001 rows: about 150 splits per head, combined by the last CTA to arrive
     run_step(B, 8, 2, 20000, 20001, False, seed=701)
