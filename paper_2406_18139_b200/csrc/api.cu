@@ -37,6 +37,10 @@ struct Plan {
     std::vector<Req> reqs;                  // table order (longest first)
     std::vector<int> out_len;               // caller order
     // workspace offsets (bytes)
+    int splits[2] = {1, 1};                 // ranges of a sweep 1 / sweep 2 item's streamed tiles
+    size_t n_arrived[2] = {0, 0};           // their arrival counters
+    size_t clear_words = 64;                // status word and arrival counters
+    size_t o_parts1 = 0, o_parts2 = 0;
     size_t o_status, o_reqs, o_lse, o_lse_split, o_scores, o_rank, o_rnorm_all, o_kept, o_evict, o_kept_keys,
         o_rnorm_kept, o_assign, o_sim, o_row_ptr, o_members, o_member_w, o_units, o_slot_cnt, o_parts, o_sort_a, o_sort_b,
         total;
@@ -44,6 +48,24 @@ struct Plan {
 
 struct DeviceInfo { int sms = 0; int cc_major = 0; bool ok = false; };
 int device_info(DeviceInfo& out);
+
+// Splits of the sweep items: as many as bring the longest item down to what an SM has on average, if it
+// is more than one and a half times that and ten tiles longer.  Both sweeps together, us: 5000 tokens
+// with 2 heads 63.5 -> 38, 12000 with 2 query on 1 KV head 188 -> 110, 2048 with 32 on 8 78 -> 63, 700
+// with 32 on 8 35 -> 25; below ten tiles the partial results cost more than they save (2048 tokens with
+// 8 heads, 16 tiles against 7: 33 -> 37).
+void plan_splits(Plan& pl) {
+    DeviceInfo di;
+    const long long sms = (device_info(di) == LOOKM_OK && di.sms > 0) ? di.sms : 148;
+    long long tiles = 0;
+    for (const Req& q : pl.reqs) tiles += (long long)q.nblk * (q.nblk + 1) / 2;
+    const long long mean = std::max<long long>(1, tiles * pl.n_q_heads / sms);
+    for (int s = 0; s < 2; ++s) {
+        const long long longest = (long long)pl.reqs[0].nblk * (s ? pl.group : 1);
+        if (2 * longest > 3 * mean && longest >= mean + 10)
+            pl.splits[s] = (int)std::min<long long>(kMaxSplits, (longest + mean - 1) / mean);
+    }
+}
 
 // Returns LOOKM_OK or the status describing the first bad argument.
 int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqlens,
@@ -101,7 +123,8 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
         return LOOKM_ERR_UNSUPPORTED;
     // table order: longest request first
     std::stable_sort(pl.reqs.begin(), pl.reqs.end(), [](const Req& a, const Req& b) { return a.L > b.L; });
-    long long it0 = 0, it1 = 0, it2 = 0, slots = 0, units = 0;
+    plan_splits(pl);
+    long long it0 = 0, it1 = 0, it2 = 0, slots = 0, units = 0, tiles = 0;
     // Merge work units (the kernel reads n_kv_heads * T rows): every warp gets the same number of
     // units, one if that keeps a unit within kMaxUnitEntries rows.  The units of a request are laid
     // out heads fastest, so a wave of warps reads one token window of all heads; with very long
@@ -125,11 +148,13 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
         q.slot_begin = (int)slots;
         q.unit_begin = (int)units;
         q.unit_entries = unit_entries;
+        q.tile_begin = (int)tiles;
+        tiles += q.nblk;
         const bool merges = q.mode != LOOKM_MERGE_NONE;
         const long long n_units = merges ? (q.L + unit_entries - 1) / unit_entries : 0;
         units += (long long)pl.n_kv_heads * n_units;
-        it0 += (long long)q.nblk * pl.n_q_heads;
-        it1 += (long long)q.nblk * pl.n_kv_heads;
+        it0 += (long long)q.nblk * pl.n_q_heads * pl.splits[0];
+        it1 += (long long)q.nblk * pl.n_kv_heads * pl.splits[1];
         // match items: blocks of 128 entries of every head's evicted list
         it2 += (q.E > 0 && merges) ? (long long)((q.E + kTile - 1) / kTile) * pl.n_kv_heads : 0;
         slots += (long long)q.B * pl.n_kv_heads;
@@ -144,7 +169,10 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
     const size_t Hq = pl.n_q_heads, Hkv = pl.n_kv_heads, T = (size_t)pl.T;
     // Every list is sized for the worst case over budgets (at most T kept and T evicted rows per
     // head), so the carving depends only on the prompt lengths and head counts.
-    pl.o_status = carve(256);
+    for (int s = 0; s < 2; ++s)
+        if (pl.splits[s] > 1) pl.n_arrived[s] = 4 * (size_t)tiles * (s ? Hkv : Hq);
+    pl.clear_words += pl.n_arrived[0] + pl.n_arrived[1];
+    pl.o_status = carve(4 * pl.clear_words);
     pl.o_reqs = carve(sizeof(Req) * n_req);
     pl.o_lse = carve(4 * Hq * T);
     pl.o_lse_split = carve(32 * Hq * T);
@@ -165,6 +193,8 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
     pl.o_parts = carve((size_t)kMergePartBytes * (size_t)pl.total_units);
     pl.o_sort_a = carve(8 * Hkv * T);
     pl.o_sort_b = carve(8 * Hkv * T);
+    pl.o_parts1 = carve(pl.splits[0] > 1 ? 8 * Hq * T * pl.splits[0] : 0);
+    pl.o_parts2 = carve(pl.splits[1] > 1 ? 4 * Hkv * T * pl.splits[1] : 0);
     pl.total = o;
     return LOOKM_OK;
 }
@@ -276,16 +306,16 @@ int make_map_2d(CUtensorMap* map, const void* base, long long rows) {
 template <class T>
 T* at(void* ws, size_t off) { return reinterpret_cast<T*>(static_cast<char*>(ws) + off); }
 
-// Clears the status word and writes the request table into the workspace.
+// Clears the status word and the arrival counters and writes the request table into the workspace.
 int begin_call(const Plan& pl, void* ws, cudaStream_t st) {
     g_launches = 0;
-    LOOKM_CUDA(cudaMemsetAsync(at<int>(ws, pl.o_status), 0, 256, st));
     for (int base = 0; base < pl.n_req; base += kReqChunk) {
         ReqChunk chunk;
         const int cnt = std::min(kReqChunk, pl.n_req - base);
         std::memset(&chunk, 0, sizeof(chunk));
         std::memcpy(chunk.r, pl.reqs.data() + base, sizeof(Req) * cnt);
-        LOOKM_CUDA(launch_write_table(chunk, cnt, at<Req>(ws, pl.o_reqs) + base, st));
+        LOOKM_CUDA(launch_write_table(chunk, cnt, at<Req>(ws, pl.o_reqs) + base, at<int>(ws, pl.o_status),
+                                      base == 0 ? pl.clear_words : 0, st));
         ++g_launches;
     }
     return LOOKM_OK;
@@ -324,6 +354,9 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     p.scores = scores;
     if (!lse_is_input) {
         p.n_items = pl.n_items[kSweep1];
+        p.splits = pl.splits[0];
+        p.parts1 = at<float2>(ws, pl.o_parts1);
+        p.arrived = p.status + 64;
         LOOKM_CUDA(launch_tile_kernel(kSweep1, map_q, map_k, nullptr, p, di.sms, st));
         ++g_launches;
     } else {
@@ -332,6 +365,9 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     }
     mark_stage(1, st);
     p.n_items = pl.n_items[kSweep2];
+    p.splits = pl.splits[1];
+    p.parts2 = at<float>(ws, pl.o_parts2);
+    p.arrived = p.status + 64 + pl.n_arrived[0];
     LOOKM_CUDA(launch_tile_kernel(kSweep2, map_k, map_q, &map_x, p, di.sms, st));
     ++g_launches;
     mark_stage(2, st);
@@ -776,6 +812,7 @@ extern "C" int lookm_merge_noalloc(const void* k, const void* v, const int* kept
     const size_t units = (size_t)pl.n_kv_heads * (size_t)pl.T;
     size_t o = 0;
     auto carve = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
+    pl.clear_words = 64;
     pl.o_status = carve(256);
     pl.o_reqs = carve(sizeof(Req) * (size_t)n_requests);
     pl.o_row_ptr = carve(4 * (units + (size_t)pl.n_kv_heads * (size_t)n_requests));

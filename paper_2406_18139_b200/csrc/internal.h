@@ -56,10 +56,12 @@ struct Req {
                           // of the merge kernel gets about one unit
     int unit_begin;       // first merge work unit of this request (table order); n_kv_heads *
                           // ceil(L / unit_entries) units per request, heads varying fastest
+    int tile_begin;       // 128-row blocks of the requests before this one (table order)
 };
 
 enum TileKind { kSweep1 = 0, kSweep2 = 1, kMatch = 2 };
 
+constexpr int kMaxSplits = 4;
 struct TileParams {
     const Req* reqs;
     int n_req;
@@ -71,6 +73,10 @@ struct TileParams {
     unsigned short* lse_split;   // [T, n_q_heads, 16] bf16: -lse / scale as three bf16 terms and 13
                                  // zeros per query row (sweep 1 writes, sweep 2 loads it by TMA)
     float* scores;               // [n_kv_heads, T]
+    int splits;                  // ranges that the streamed tiles of a sweep item are cut into
+    float2* parts1;              // [splits][n_q_heads, T]  reference and sum of a range (sweep 1)
+    float* parts2;               // [splits][n_kv_heads, T] column sums of a range (sweep 2)
+    int* arrived;                // [block][heads][4] finished ranges per 32 rows (zeroed)
     const int* evict_idx;        // evicted-list layout  (match: rows of the stationary tiles)
     const void* k_rows;          // K [tokens, heads, 128] bf16 with the strides below (match)
     long long k_stride_tok, k_stride_head;
@@ -116,7 +122,8 @@ cudaError_t launch_argmax_rows(const float* sim_matrix, const Req* reqs, int n_r
 // this keeps the host free of any synchronising copy.
 constexpr int kReqChunk = 40;
 struct ReqChunk { Req r[kReqChunk]; };
-cudaError_t launch_write_table(const ReqChunk& chunk, int count, Req* dst, cudaStream_t stream);
+// The launch also zeroes n_clear words from `clear` on (the status word and the counters).
+cudaError_t launch_write_table(const ReqChunk& chunk, int count, Req* dst, int* clear, size_t n_clear, cudaStream_t stream);
 
 cudaError_t launch_invert_assignment(const int* assign, const int* kept_idx, const int* evict_idx,
                                      const float* sim, const Req* reqs, int n_req, int n_kv_heads,

@@ -905,16 +905,20 @@ merge_short_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __r
     }
 }
 
-__global__ void write_table_kernel(const __grid_constant__ ReqChunk chunk, int count, Req* dst) {
+__global__ void __launch_bounds__(256)
+write_table_kernel(const __grid_constant__ ReqChunk chunk, int count, Req* dst, int* clear, size_t n_clear) {
+    grid_dependency_wait();
     const int i = threadIdx.x;
-    if (i < count) dst[i] = chunk.r[i];
+    if (blockIdx.x == 0 && i < count) dst[i] = chunk.r[i];
+    for (size_t j = (size_t)blockIdx.x * blockDim.x + i; j < n_clear; j += (size_t)gridDim.x * blockDim.x) clear[j] = 0;
 }
 
 }  // namespace
 
-cudaError_t launch_write_table(const ReqChunk& chunk, int count, Req* dst, cudaStream_t stream) {
-    write_table_kernel<<<1, 64, 0, stream>>>(chunk, count, dst);
-    return cudaGetLastError();
+cudaError_t launch_write_table(const ReqChunk& chunk, int count, Req* dst, int* clear, size_t n_clear, cudaStream_t stream) {
+    const size_t blocks = n_clear / 2048 + 1;            // eight words per thread
+    return launch_chained(write_table_kernel, dim3((unsigned)(blocks < 148 ? blocks : 148)), dim3(256), 0, stream, chunk, count,
+                          dst, clear, n_clear);
 }
 
 cudaError_t launch_key_norms(const void* k, long long stride_tok, long long stride_head,

@@ -27,6 +27,11 @@
 //            expects; B = tiles of the compacted kept keys.  Thread keeps the largest
 //            s_ij / |k_j| and its slot.
 //
+// A small problem has fewer or more uneven sweep items than the CTAs can share.  Then the streamed tiles of an item are cut into
+// p.splits ranges, items of their own that leave partial results in memory; the one that arrives last
+// (a counter per 32 rows) adds them in range order.  Large problems run a kernel without that code (with
+// it 8192 tokens x 32 heads took 1.5 % longer).
+//
 // Work items are laid out heaviest first and dealt to the CTAs in serpentine order; every role
 // walks the same item sequence on its own, so no scheduling state is shared.
 #include <cuda_bf16.h>
@@ -138,11 +143,14 @@ __global__ void lse_split_kernel(const float* __restrict__ lse, int n_q_heads, l
 
 struct Item {
     int tok_begin, L, B, E, blk, head, nt;
+    int t0;                   // first streamed tile of the item (the sweeps' splits)
+    int split, n_splits;      // which range of the block's tiles, of how many
+    int tile;                 // index of the block over the whole batch
     long long kept_row0;      // match: first row of this (request, head) in the kept-key matrix
     long long ev0;            // match: start of its evicted list
 };
 
-template <int KIND>
+template <int KIND, bool kSplits>
 __device__ __forceinline__ Item decode_item(const TileParams& p, const Req* tbl, int item) {
     int lo = 0, hi = p.n_req - 1;
     while (lo < hi) {
@@ -156,16 +164,30 @@ __device__ __forceinline__ Item decode_item(const TileParams& p, const Req* tbl,
     it.L = rq.L;
     it.B = rq.B;
     it.E = rq.E;
+    it.t0 = 0;
+    it.split = 0;
+    it.n_splits = 1;
     it.kept_row0 = 0;
     it.ev0 = 0;
-    if (KIND == kSweep1) {                       // heaviest first: last query block first
-        it.blk = rq.nblk - 1 - u / p.n_q_heads;
-        it.head = u % p.n_q_heads;
-        it.nt = it.blk + 1;
-    } else if (KIND == kSweep2) {                // heaviest first: first key block first
-        it.blk = u / p.n_kv_heads;
-        it.head = u % p.n_kv_heads;
-        it.nt = (rq.nblk - it.blk) * p.group;
+    if (KIND != kMatch) {                        // heaviest first: last query block, first key block
+        const int heads = (KIND == kSweep1 ? p.n_q_heads : p.n_kv_heads) * (kSplits ? p.splits : 1);
+        const int b = u / heads, v = u % heads;
+        it.blk = KIND == kSweep1 ? rq.nblk - 1 - b : b;
+        it.nt = KIND == kSweep1 ? it.blk + 1 : (rq.nblk - it.blk) * p.group;
+        it.head = v;
+        if (kSplits) {
+            it.head = v / p.splits;
+            it.split = v % p.splits;
+            it.n_splits = min(p.splits, it.nt);
+            it.tile = rq.tile_begin + it.blk;
+            const int all = it.nt;
+            if (it.split < it.n_splits) {
+                it.t0 = all * it.split / it.n_splits;
+                it.nt = all * (it.split + 1) / it.n_splits - it.t0;
+            } else {
+                it.nt = 0;                       // no tile: every role passes over the item
+            }
+        }
     } else {                                     // blk: block of 128 entries of the evicted list
         it.blk = u / p.n_kv_heads;
         it.head = u % p.n_kv_heads;
@@ -176,13 +198,20 @@ __device__ __forceinline__ Item decode_item(const TileParams& p, const Req* tbl,
     return it;
 }
 
+// Log-sum-exp of a query row (reference m in units of the accumulator, sum l) and its companion row.
+__device__ __forceinline__ void store_lse(const TileParams& p, const Item& it, int pos, float m, float l) {
+    const float lse = (m * p.scale_log2 + ptx::lg2(l)) * kLn2;       // natural log, of the scaled logits
+    p.lse[(long long)it.head * p.T + it.tok_begin + pos] = lse;
+    store_lse_split(p.lse_split + ((long long)(it.tok_begin + pos) * p.n_q_heads + it.head) * 16, lse, p.scale_log2);
+}
+
 // Serpentine deal of the item list: round k hands items k*G .. k*G+G-1 to the CTAs in forward
 // order when k is even and in reverse order when k is odd.
 __device__ __forceinline__ int item_of_round(int round, int cta, int n_cta) {
     return round * n_cta + ((round & 1) ? (n_cta - 1 - cta) : cta);
 }
 
-template <int KIND>
+template <int KIND, bool kSplits>
 __global__ void __launch_bounds__(threads_of(KIND), 1)
 tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
             const __grid_constant__ CUtensorMap map_x, const TileParams p) {
@@ -254,7 +283,8 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             for (int round = 0; !stop; ++round, ++n) {
                 const int item = item_of_round(round, blockIdx.x, n_cta);
                 if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; --n; continue; }
-                const Item it = decode_item<KIND>(p, tbl, item);
+                const Item it = decode_item<KIND, kSplits>(p, tbl, item);
+                if (kSplits && it.nt == 0) { --n; continue; }
                 const int ab = n % kABuf;
                 if (KIND != kMatch) {                    // the match's stationary tiles come from the gather warp
                     if (!ptx::mbar_wait(ptx::smem_u32(&sh.a_empty[ab]), ((n / kABuf) & 1) ^ 1, abort_flag)) break;
@@ -276,13 +306,13 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                     ptx::mbar_arrive_expect_tx(bbar, KIND == kSweep2 ? kTileBytes + kSplitBytes : kTileBytes);
                     const uint32_t bdst = ptx::smem_u32(&sh.b[s][0]);
                     if (KIND == kSweep1) {
-                        const int row = it.tok_begin + t * kTile;
+                        const int row = it.tok_begin + (it.t0 + t) * kTile;
                         const int h = it.head / p.group;
                         ptx::tma_load_3d(bdst, &map_b, 0, h, row, bbar);
                         ptx::tma_load_3d(bdst + kHalfBytes, &map_b, 64, h, row, bbar);
                     } else if (KIND == kSweep2) {
-                        const int row = it.tok_begin + (it.blk + t / p.group) * kTile;
-                        const int h = it.head * p.group + t % p.group;
+                        const int row = it.tok_begin + (it.blk + (it.t0 + t) / p.group) * kTile;
+                        const int h = it.head * p.group + (it.t0 + t) % p.group;
                         ptx::tma_load_3d(bdst, &map_b, 0, h, row, bbar);
                         ptx::tma_load_3d(bdst + kHalfBytes, &map_b, 64, h, row, bbar);
                         ptx::tma_load_3d(ptx::smem_u32(&sh.bx[s % Shared<KIND>::kXStages][0]), &map_x, 0, h, row, bbar);
@@ -324,7 +354,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         for (int round = 0;; ++round, ++n) {
             const int item = item_of_round(round, blockIdx.x, n_cta);
             if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; --n; continue; }
-            const Item it = decode_item<KIND>(p, tbl, item);
+            const Item it = decode_item<KIND, kSplits>(p, tbl, item);
             const int ab = n % kABuf;
             int free_now = 1;                            // one lane waits, the warp follows its verdict
             if (lane == 0)
@@ -367,7 +397,8 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             for (int round = 0; !stop; ++round, ++n) {
                 const int item = item_of_round(round, blockIdx.x, n_cta);
                 if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; --n; continue; }
-                const Item it = decode_item<KIND>(p, tbl, item);
+                const Item it = decode_item<KIND, kSplits>(p, tbl, item);
+                if (kSplits && it.nt == 0) { --n; continue; }
                 const int ab = n % kABuf;
                 if (!ptx::mbar_wait(ptx::smem_u32(&sh.a_full[ab]), (n / kABuf) & 1, abort_flag)) break;
                 const uint32_t a_addr = ptx::smem_u32(&sh.a[ab][0]);
@@ -428,7 +459,8 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         for (int round = 0;; ++round, ++n) {
             const int item = item_of_round(round, blockIdx.x, n_cta);
             if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; --n; continue; }
-            const Item it = decode_item<KIND>(p, tbl, item);
+            const Item it = decode_item<KIND, kSplits>(p, tbl, item);
+            if (kSplits && it.nt == 0) { --n; continue; }
             const int pos = it.blk * kTile + row;            // position of this thread's row (match: its
                                                              // index in the evicted list)
             float m_run = -INFINITY, l_run = 0.f;            // sweep 1
@@ -460,9 +492,9 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 int col_limit = kTile;                       // valid columns of the tile (match, sweep 2)
                 int diag_from = 0;                           // sweep 2: first column this row may use
                 if (KIND == kSweep1) {
-                    diag = (t == it.blk);
+                    diag = (it.t0 + t == it.blk);
                 } else if (KIND == kSweep2) {
-                    const int ib = it.blk + t / p.group;
+                    const int ib = it.blk + (it.t0 + t) / p.group;
                     // columns to mask: below the diagonal in the item's first query block, and past
                     // the end of the request in its last one (rows of the next request or zeros)
                     col_limit = min(kTile, it.L - ib * kTile);
@@ -669,17 +701,19 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         float l = lg[0] * ptx::ex2((mg[0] - m) * c2);
 #pragma unroll
                         for (int g = 1; g < kParts; ++g) l += lg[g] * ptx::ex2((mg[g] - m) * c2);
-                        // natural-log log-sum-exp of the scaled logits
-                        const float lse = (m * c2 + ptx::lg2(l)) * kLn2;
-                        p.lse[(long long)it.head * p.T + it.tok_begin + pos] = lse;
-                        store_lse_split(p.lse_split + ((long long)(it.tok_begin + pos) * p.n_q_heads + it.head) * 16,
-                                        lse, c2);
+                        if (kSplits && it.n_splits > 1)
+                            __stcg(p.parts1 + ((long long)it.split * p.n_q_heads + it.head) * p.T + it.tok_begin + pos, make_float2(m, l));
+                        else
+                            store_lse(p, it, pos, m, l);
                     } else if (KIND == kSweep2) {
                         const float own = (acc0 + acc1) + (acc2 + acc3);
                         float a = (part == 0) ? own : cb[0][0][row];
 #pragma unroll
                         for (int g = 1; g < kParts; ++g) a += (g == part) ? own : cb[g][0][row];
-                        p.scores[(long long)it.head * p.T + it.tok_begin + pos] = a;
+                        if (kSplits && it.n_splits > 1)
+                            __stcg(p.parts2 + ((long long)it.split * p.n_kv_heads + it.head) * p.T + it.tok_begin + pos, a);
+                        else
+                            p.scores[(long long)it.head * p.T + it.tok_begin + pos] = a;
                     } else {
                         if (!rnorm_asked) ask_rnorm();           // a part without a tile in this item
                         const int e = pos;
@@ -699,6 +733,34 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 }
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.comb_free[cslot]));
+                if (kSplits && it.n_splits > 1) {
+                    const int heads = KIND == kSweep1 ? p.n_q_heads : p.n_kv_heads;
+                    __threadfence();
+                    __syncwarp();
+                    int last = 0;
+                    if (lane == 0)
+                        last = atomicAdd(p.arrived + ((long long)it.tile * heads + it.head) * 4 + quarter, 1) == it.n_splits - 1;
+                    if (__shfl_sync(0xffffffffu, last, 0) && pos < it.L && !*abort_flag) {
+                        __threadfence();
+                        const long long at = (long long)it.head * p.T + it.tok_begin + pos, step = (long long)heads * p.T;
+                        if (KIND == kSweep1) {
+                            float2 ml[kMaxSplits];
+                            float m = -INFINITY, l = 0.f;
+#pragma unroll
+                            for (int i = 0; i < kMaxSplits; ++i) {
+                                ml[i] = i < it.n_splits ? __ldcg(p.parts1 + at + i * step) : make_float2(-INFINITY, 0.f);
+                                m = fmaxf(m, ml[i].x);
+                            }
+#pragma unroll
+                            for (int i = 0; i < kMaxSplits; ++i) l += ml[i].y * ptx::ex2((ml[i].x - m) * c2);
+                            store_lse(p, it, pos, m, l);
+                        } else {
+                            float a = __ldcg(p.parts2 + at);
+                            for (int i = 1; i < it.n_splits; ++i) a += __ldcg(p.parts2 + at + i * step);
+                            p.scores[at] = a;
+                        }
+                    }
+                }
             }
         }
     }
@@ -743,25 +805,24 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
                                const CUtensorMap* map_x, const TileParams& p, int num_sms,
                                cudaStream_t stream) {
     if (p.n_items <= 0) return cudaSuccess;
-    const int smem_of[3] = {(int)sizeof(Shared<kSweep1>) + 1024, (int)sizeof(Shared<kSweep2>) + 1024,
-                            (int)sizeof(Shared<kMatch>) + 1024};
+    typedef void (*Kernel)(CUtensorMap, CUtensorMap, CUtensorMap, TileParams);
+    static const Kernel kernels[3][2] = {{tile_kernel<kSweep1, false>, tile_kernel<kSweep1, true>},
+                                         {tile_kernel<kSweep2, false>, tile_kernel<kSweep2, true>},
+                                         {tile_kernel<kMatch, false>, tile_kernel<kMatch, false>}};
+    const size_t smem_of[3] = {sizeof(Shared<kSweep1>) + 1024, sizeof(Shared<kSweep2>) + 1024, sizeof(Shared<kMatch>) + 1024};
     const int grid = p.n_items < num_sms ? p.n_items : num_sms;
     const CUtensorMap& mx = map_x ? *map_x : map_b;      // only sweep 2 uses it
     static unsigned long long configured = 0;
     cudaError_t err = once_per_device(configured, [&]() {
-        cudaError_t e = cudaFuncSetAttribute(tile_kernel<kSweep1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_of[kSweep1]);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(tile_kernel<kSweep2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_of[kSweep2]);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(tile_kernel<kMatch>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_of[kMatch]);
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < 3; ++i)
+            for (int j = 0; j < 2; ++j)
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute(kernels[i][j], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of[i]);
         return e;
     });
     if (err != cudaSuccess) return err;
-    if (kind == kSweep1)
-        return launch_chained(tile_kernel<kSweep1>, dim3(grid), dim3(threads_of(kSweep1)), (size_t)smem_of[kSweep1], stream, map_a, map_b, mx, p);
-    if (kind == kSweep2)
-        return launch_chained(tile_kernel<kSweep2>, dim3(grid), dim3(threads_of(kSweep2)), (size_t)smem_of[kSweep2], stream, map_a, map_b, mx, p);
-    return launch_chained(tile_kernel<kMatch>, dim3(grid), dim3(threads_of(kMatch)), (size_t)smem_of[kMatch], stream, map_a, map_b, mx, p);
+    return launch_chained(kernels[kind][p.splits > 1], dim3(grid), dim3(threads_of(kind)), smem_of[kind], stream, map_a, map_b, mx, p);
 }
 
 cudaError_t launch_lse_split(const float* lse, int n_q_heads, long long T, float scale_log2,

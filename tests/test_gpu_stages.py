@@ -101,6 +101,37 @@ def test_scores_logits_that_grow_along_the_prompt(B):
     assert np.allclose(got.sum(axis=1), L, rtol=1e-5)
 
 
+@pytest.mark.parametrize("lens,Hq,Hkv", [([1900, 1, 130, 640], 4, 1), ([1409], 1, 1), ([2100, 2100], 2, 2)])
+def test_scores_of_items_cut_into_ranges(B, lens, Hq, Hkv):
+    """Few heads: both sweeps cut their items into up to four ranges (fewer where an item has fewer
+    tiles); logits rise along the prompts, so the ranges of a row have references far apart."""
+    import torch
+    T = sum(lens)
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    qn = synth.normal(synth.stream_key(145, T), T * Hq * 128).reshape(T, Hq, 128).astype(np.float32) * 0.5
+    kn = synth.normal(synth.stream_key(146, T), T * Hkv * 128).reshape(T, Hkv, 128).astype(np.float32) * 0.5
+    qn[:, :, 0] = 4.0
+    for a, n in zip(cu, lens):
+        kn[a:a + n, :, 0] = (4.0 * np.arange(n) / n)[:, None]
+    qb, kb = synth.f32_to_bf16_bits(qn), synth.f32_to_bf16_bits(kn)
+    q, k = to_dev(qb), to_dev(kb)
+    lay = B.make_layout(q, k, softmax_scale=1.0)
+    ws = B.alloc_workspace(lay, lens)
+    ws.fill_(0x7f)
+    scores = torch.zeros(Hkv, T, dtype=torch.float32, device="cuda")
+    lse = torch.zeros(Hq, T, dtype=torch.float32, device="cuda")
+    again = torch.zeros_like(scores)
+    B.check(B.lookm_score(q, k, cu, lay, scores, lse, False, ws))
+    assert B.lookm_device_status(ws) == B.OK
+    B.check(B.lookm_score(q, k, cu, lay, again, lse, True, ws))
+    assert torch.equal(scores, again)
+    for a, n in zip(cu, lens):
+        A, lse_o = orc.scores(synth.bf16_to_f32(qb[a:a + n]), synth.bf16_to_f32(kb[a:a + n]), scale=1.0, threads=8, want_lse=True)
+        got = scores[:, a:a + n].cpu().numpy().astype(np.float64)
+        assert np.all(np.abs(got - A) <= 5e-5 * A)              # exponent arguments reach 40
+        assert np.allclose(lse[:, a:a + n].cpu().numpy().reshape(Hkv, Hq // Hkv, n), lse_o, rtol=1e-6, atol=2e-5)
+
+
 def test_scores_packed_batch_equals_separate_requests(B):
     import torch
     lens = [200, 131, 1, 400]
