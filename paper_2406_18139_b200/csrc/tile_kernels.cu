@@ -115,6 +115,70 @@ __device__ __forceinline__ float exp2_mixed(int column, float x) {
     return (column % kPolyEvery == kPolyEvery - 1) ? ptx::ex2_fma(x) : ptx::ex2(x);
 }
 
+// ---- epilogue of the sweeps on 32 accumulator columns, one row per thread ------------------------
+// Sweep 1: softmax statistics of a query row; l is the sum of exp2(x - m c2), where m is a REFERENCE,
+// not necessarily the maximum so far.  Diagonal tile (the last of the item; columns from c0 on, usable
+// up to `row`): exact running maximum.
+__device__ __forceinline__ void sweep1_diagonal(const uint32_t (&raw)[32], int c0, int row, float c2, float& m, float& l) {
+    float mx = m;
+#pragma unroll
+    for (int c = 0; c < 32; ++c)
+        if (c0 + c <= row) mx = fmaxf(mx, __uint_as_float(raw[c]));
+    if (mx != -INFINITY) {                               // false only above the diagonal
+        const float mc = mx * c2;
+        float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+        for (int c = 0; c < 32; c += 2) {
+            const float e0 = exp2_mixed(c, fmaf(__uint_as_float(raw[c]), c2, -mc));
+            const float e1 = exp2_mixed(c + 1, fmaf(__uint_as_float(raw[c + 1]), c2, -mc));
+            s0 += (c0 + c <= row) ? e0 : 0.f;
+            s1 += (c0 + c + 1 <= row) ? e1 : 0.f;
+        }
+        l = l * ptx::ex2(m * c2 - mc) + (s0 + s1);
+        m = mx;
+    }
+}
+// Full tiles: no maximum is taken.  The reference is the maximum of the row's first 32 columns; later
+// logits may exceed it as long as the chunk's sum stays below 2^60 (fp32 has the range, and the relative
+// precision does not depend on the reference).  When it does not, or overflows, the chunk is redone
+// against its true maximum.
+__device__ __forceinline__ void sweep1_columns(const uint32_t (&raw)[32], float c2, float& m, float& l) {
+    float ref = m;                                       // -inf at the row's first chunk: the sum
+    float sum;                                           // overflows and the second round sets it
+#pragma unroll 1
+    for (int round2 = 0;; ++round2) {
+        const float mc = ref * c2;
+        float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+        for (int c = 0; c < 32; c += 2) {
+            s0 += exp2_mixed(c, fmaf(__uint_as_float(raw[c]), c2, -mc));
+            s1 += exp2_mixed(c + 1, fmaf(__uint_as_float(raw[c + 1]), c2, -mc));
+        }
+        sum = s0 + s1;
+        if (sum < kReferenceSlack || round2) break;
+        float mx = ref;
+#pragma unroll
+        for (int c = 0; c < 32; c += 2) mx = ptx::fmax3(mx, __uint_as_float(raw[c]), __uint_as_float(raw[c + 1]));
+        l *= ptx::ex2(ref * c2 - mx * c2);
+        ref = mx;
+    }
+    l += sum;
+    m = ref;
+}
+// Sweep 2: probabilities of a key under 32 query columns (the accumulator holds s_ij - lse_i / scale);
+// columns [from, limit) count.
+__device__ __forceinline__ void sweep2_diagonal(const uint32_t (&raw)[32], int c0, int from, int limit, float c2, float (&acc)[4]) {
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+        const float e = exp2_mixed(c, __uint_as_float(raw[c]) * c2);
+        acc[c & 3] += (c0 + c >= from && c0 + c < limit) ? e : 0.f;
+    }
+}
+__device__ __forceinline__ void sweep2_columns(const uint32_t (&raw)[32], float c2, float (&acc)[4]) {
+#pragma unroll
+    for (int c = 0; c < 32; ++c) acc[c & 3] += exp2_mixed(c, __uint_as_float(raw[c]) * c2);
+}
+
 // -lse / scale of one query row as three bf16 terms (their sum carries 24 bits) and 13 zeros:
 // the row of the 16-column companion tensor that sweep 2 multiplies with ones.
 __device__ __forceinline__ void store_lse_split(unsigned short* row16, float lse, float scale_log2) {
@@ -139,6 +203,16 @@ __global__ void lse_split_kernel(const float* __restrict__ lse, int n_q_heads, l
     if (i >= T * n_q_heads) return;
     const long long h = i / T, tok = i % T;
     store_lse_split(lse_split + (tok * n_q_heads + h) * 16, lse[i], scale_log2);
+}
+
+// Row r of the ones tile: (1, 1, 1, 0, ... 0) in bf16; with the 32-byte swizzle the two 16-byte halves
+// of a row trade places in rows 4-7 of every group of eight.
+__device__ __forceinline__ void write_ones_row(uint8_t* ax, int r) {
+    const int first = (r >> 2) & 1;
+    uint4* row = reinterpret_cast<uint4*>(ax + r * 32);
+    row[first] = make_uint4(0x3F803F80u, 0x00003F80u, 0u, 0u);
+    row[first ^ 1] = make_uint4(0u, 0u, 0u, 0u);
+    ptx::fence_proxy_async_shared();             // the tensor core reads it through the async proxy
 }
 
 struct Item {
@@ -199,10 +273,10 @@ __device__ __forceinline__ Item decode_item(const TileParams& p, const Req* tbl,
 }
 
 // Log-sum-exp of a query row (reference m in units of the accumulator, sum l) and its companion row.
-__device__ __forceinline__ void store_lse(const TileParams& p, const Item& it, int pos, float m, float l) {
+__device__ __forceinline__ void store_lse(const TileParams& p, int head, int tok, float m, float l) {
     const float lse = (m * p.scale_log2 + ptx::lg2(l)) * kLn2;       // natural log, of the scaled logits
-    p.lse[(long long)it.head * p.T + it.tok_begin + pos] = lse;
-    store_lse_split(p.lse_split + ((long long)(it.tok_begin + pos) * p.n_q_heads + it.head) * 16, lse, p.scale_log2);
+    p.lse[(long long)head * p.T + tok] = lse;
+    store_lse_split(p.lse_split + ((long long)tok * p.n_q_heads + head) * 16, lse, p.scale_log2);
 }
 
 // Serpentine deal of the item list: round k hands items k*G .. k*G+G-1 to the CTAs in forward
@@ -243,14 +317,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         ptx::fence_mbar_init();
     }
     if (KIND == kSweep2 && threadIdx.x < kTile) {
-        // ones tile: row r = (1, 1, 1, 0, ... 0) in bf16; with the 32-byte swizzle the two 16-byte
-        // halves of a row trade places in rows 4-7 of every group of eight
-        const int r = threadIdx.x;
-        const int first = (r >> 2) & 1;
-        uint4* row = reinterpret_cast<uint4*>(sh.ax + r * 32);
-        row[first] = make_uint4(0x3F803F80u, 0x00003F80u, 0u, 0u);
-        row[first ^ 1] = make_uint4(0u, 0u, 0u, 0u);
-        ptx::fence_proxy_async_shared();         // the tensor core reads it through the async proxy
+        write_ones_row(sh.ax, threadIdx.x);
     }
     // everything above touches only this CTA's shared memory; from here on global memory written
     // by the kernel before this one is read
@@ -464,7 +531,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             const int pos = it.blk * kTile + row;            // position of this thread's row (match: its
                                                              // index in the evicted list)
             float m_run = -INFINITY, l_run = 0.f;            // sweep 1
-            float acc0 = 0.f, acc1 = 0.f, acc2 = 0.f, acc3 = 0.f;   // sweep 2
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};             // sweep 2
             float best = -INFINITY;                          // match
             int best_slot = 0x7fffffff;
             // match: 1 / |k| of this thread's evicted row takes two dependent loads (its position, then
@@ -572,82 +639,11 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 // work on 32 columns of the accumulator, c0 = first column of the chunk
                 auto process = [&](const uint32_t (&raw)[32], int c0) {
                     if (KIND == kSweep1) {
-                        // softmax statistics of row `pos` over key columns c0..c0+31: l_run is the
-                        // sum of exp2(x - m_run), where m_run is a REFERENCE, not necessarily the
-                        // maximum so far
-                        if (diag) {
-                            // diagonal tile (the last of the item): exact running maximum
-                            float mx = m_run;
-#pragma unroll
-                            for (int c = 0; c < 32; ++c)
-                                if (c0 + c <= row) mx = fmaxf(mx, __uint_as_float(raw[c]));
-                            if (mx != -INFINITY) {           // false only above the diagonal
-                                const float mc = mx * c2;
-                                float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-                                for (int c = 0; c < 32; c += 2) {
-                                    const float e0 = exp2_mixed(c, fmaf(__uint_as_float(raw[c]), c2, -mc));
-                                    const float e1 = exp2_mixed(c + 1, fmaf(__uint_as_float(raw[c + 1]), c2, -mc));
-                                    s0 += (c0 + c <= row) ? e0 : 0.f;
-                                    s1 += (c0 + c + 1 <= row) ? e1 : 0.f;
-                                }
-                                l_run = l_run * ptx::ex2(m_run * c2 - mc) + (s0 + s1);
-                                m_run = mx;
-                            }
-                        } else {
-                            // Full tiles: no maximum is taken.  The reference is the maximum of the
-                            // row's first 32 columns; later logits may exceed it as long as the
-                            // chunk's sum stays below 2^60 (fp32 has the range, and the relative
-                            // precision does not depend on the reference).  When it does not, or
-                            // overflows, the chunk is redone against its true maximum.
-                            float ref = m_run;           // -inf at the row's first chunk: the sum
-                            float sum;                   // overflows and the second round sets it
-#pragma unroll 1
-                            for (int round2 = 0;; ++round2) {
-                                const float mc = ref * c2;
-                                float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-                                for (int c = 0; c < 32; c += 2) {
-                                    s0 += exp2_mixed(c, fmaf(__uint_as_float(raw[c]), c2, -mc));
-                                    s1 += exp2_mixed(c + 1, fmaf(__uint_as_float(raw[c + 1]), c2, -mc));
-                                }
-                                sum = s0 + s1;
-                                if (sum < kReferenceSlack || round2) break;
-                                float mx = ref;
-#pragma unroll
-                                for (int c = 0; c < 32; c += 2)
-                                    mx = ptx::fmax3(mx, __uint_as_float(raw[c]), __uint_as_float(raw[c + 1]));
-                                l_run *= ptx::ex2(ref * c2 - mx * c2);
-                                ref = mx;
-                            }
-                            l_run += sum;
-                            m_run = ref;
-                        }
+                        if (diag) sweep1_diagonal(raw, c0, row, c2, m_run, l_run);
+                        else sweep1_columns(raw, c2, m_run, l_run);
                     } else if (KIND == kSweep2) {
-                        // probabilities of key `pos` under query columns c0..c0+31: the accumulator
-                        // holds s_ij - lse_i / scale
-                        if (diag) {
-#pragma unroll
-                            for (int c4 = 0; c4 < 8; ++c4) {
-                                const int c = c0 + c4 * 4;
-                                const float e0 = exp2_mixed(c4 * 4 + 0, __uint_as_float(raw[c4 * 4 + 0]) * c2);
-                                const float e1 = exp2_mixed(c4 * 4 + 1, __uint_as_float(raw[c4 * 4 + 1]) * c2);
-                                const float e2 = exp2_mixed(c4 * 4 + 2, __uint_as_float(raw[c4 * 4 + 2]) * c2);
-                                const float e3 = exp2_mixed(c4 * 4 + 3, __uint_as_float(raw[c4 * 4 + 3]) * c2);
-                                acc0 += (c + 0 >= diag_from && c + 0 < col_limit) ? e0 : 0.f;
-                                acc1 += (c + 1 >= diag_from && c + 1 < col_limit) ? e1 : 0.f;
-                                acc2 += (c + 2 >= diag_from && c + 2 < col_limit) ? e2 : 0.f;
-                                acc3 += (c + 3 >= diag_from && c + 3 < col_limit) ? e3 : 0.f;
-                            }
-                        } else {
-#pragma unroll
-                            for (int c4 = 0; c4 < 8; ++c4) {
-                                acc0 += exp2_mixed(c4 * 4 + 0, __uint_as_float(raw[c4 * 4 + 0]) * c2);
-                                acc1 += exp2_mixed(c4 * 4 + 1, __uint_as_float(raw[c4 * 4 + 1]) * c2);
-                                acc2 += exp2_mixed(c4 * 4 + 2, __uint_as_float(raw[c4 * 4 + 2]) * c2);
-                                acc3 += exp2_mixed(c4 * 4 + 3, __uint_as_float(raw[c4 * 4 + 3]) * c2);
-                            }
-                        }
+                        if (diag) sweep2_diagonal(raw, c0, diag_from, col_limit, c2, acc);
+                        else sweep2_columns(raw, c2, acc);
                     }
                 };
                 // the last columns are in registers: hand the accumulator back, so that the next
@@ -681,7 +677,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 // the buffer's previous contents (two items ago) have been read
                 ptx::mbar_wait(ptx::smem_u32(&sh.comb_free[cslot]), (cuse & 1u) ^ 1u, abort_flag);
                 if (KIND == kSweep1) { cb[part][0][row] = m_run; cb[part][kP1][row] = l_run; }
-                else if (KIND == kSweep2) { cb[part][0][row] = (acc0 + acc1) + (acc2 + acc3); }
+                else if (KIND == kSweep2) { cb[part][0][row] = (acc[0] + acc[1]) + (acc[2] + acc[3]); }
                 else { cb[part][0][row] = best; cb[part][kP1][row] = __int_as_float(best_slot); }
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.comb_full[cslot]));
@@ -704,9 +700,9 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         if (kSplits && it.n_splits > 1)
                             __stcg(p.parts1 + ((long long)it.split * p.n_q_heads + it.head) * p.T + it.tok_begin + pos, make_float2(m, l));
                         else
-                            store_lse(p, it, pos, m, l);
+                            store_lse(p, it.head, it.tok_begin + pos, m, l);
                     } else if (KIND == kSweep2) {
-                        const float own = (acc0 + acc1) + (acc2 + acc3);
+                        const float own = (acc[0] + acc[1]) + (acc[2] + acc[3]);
                         float a = (part == 0) ? own : cb[0][0][row];
 #pragma unroll
                         for (int g = 1; g < kParts; ++g) a += (g == part) ? own : cb[g][0][row];
@@ -753,7 +749,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                             }
 #pragma unroll
                             for (int i = 0; i < kMaxSplits; ++i) l += ml[i].y * ptx::ex2((ml[i].x - m) * c2);
-                            store_lse(p, it, pos, m, l);
+                            store_lse(p, it.head, it.tok_begin + pos, m, l);
                         } else {
                             float a = __ldcg(p.parts2 + at);
                             for (int i = 1; i < it.n_splits; ++i) a += __ldcg(p.parts2 + at + i * step);
@@ -761,6 +757,326 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         }
                     }
                 }
+            }
+        }
+    }
+
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    if (warp == 0) {
+        ptx::tc_fence_after_sync();
+        ptx::tmem_dealloc(tmem_base, 512);
+    }
+    if (threadIdx.x == 0 && sh.abort_flag) atomicExch(p.status, (int)LOOKM_ERR_DEVICE_TIMEOUT);
+}
+
+// ------------------------------------------------------------------------------------------------
+// The sweeps of large problems: an item owns TWO adjacent stationary blocks (halves 0 and 1) and every
+// streamed tile is multiplied with both, so a tile is brought into shared memory once per two products.
+// The sweeps of large prompts run at the board's power limit, where time is energy, and a tenth of
+// that goes into moving tiles from L2 (a build without the loads ran 9-11 % faster).
+// Whole layers in a row, one block per item -> two: 16384 tokens x 40 heads 4.45 -> 4.10 ms, 32768 x 32
+// query heads on 8 11.2 -> 10.6 ms, 16 ragged prompts x 32 heads 24.2 -> 23.2 ms, 8192 x 32 0.918 -> 0.886.
+// Streamed tile g of the CTA goes to accumulators 2 (g mod 2) + half, and each accumulator has one
+// issuing thread (g mod 2) and one epilogue group: group w works on half w mod 2 and on the tiles of
+// parity w / 2, so its running results belong to one block.  The two groups of a half are combined at
+// the item's end like the four of tile_kernel.  Across the diagonal a half may have no product with a
+// tile (sweep 1: the last tile and half 0; sweep 2: the first query block and half 1).
+// ------------------------------------------------------------------------------------------------
+template <int KIND>
+struct __align__(1024) PairShared {
+    static constexpr int kXStages = (KIND == kSweep2) ? kStages : 1;
+    static constexpr int kPlanes = (KIND == kSweep2) ? 1 : 2;
+    uint8_t a[2][kTileBytes];                    // stationary blocks
+    uint8_t b[kStages][kTileBytes];              // streamed tiles
+    uint8_t bx[kXStages][kSplitBytes];           // sweep 2: their 16-column companions
+    uint8_t ax[kSplitBytes];                     // sweep 2: constant ones tile that multiplies bx
+    float comb[2][2][kPlanes][kTile];            // partial results, [buffer][half]
+    Req reqs[kReqCache];
+    unsigned long long a_full[2], a_empty[2];
+    unsigned long long b_full[kStages], b_empty[kStages];
+    unsigned long long t_full[kAccum], t_empty[kAccum];
+    unsigned long long comb_full[2][2], comb_free[2][2];     // [half][buffer]
+    unsigned long long mma_done;
+    uint32_t tmem_base;
+    int abort_flag;
+};
+static_assert(sizeof(PairShared<kSweep1>) + 1024 <= 232448 && sizeof(PairShared<kSweep2>) + 1024 <= 232448,
+              "shared memory of the paired sweeps exceeds 227 KB");
+static_assert(kAccum == 4 && kGroups == 4 && kHalves == 1 && kIssuers == 2, "the paired sweeps assume this layout");
+
+struct PairItem {
+    int tok_begin, L, blk, head, nt;
+    bool both;                                   // half 1 exists
+    // is streamed tile t multiplied with the half?  group: query heads that take turns (sweep 2)
+    template <int KIND>
+    __device__ __forceinline__ bool active(int half, int t, int group) const {
+        if (half == 0) return KIND == kSweep2 || t <= blk;
+        return both && (KIND == kSweep1 || t >= group);
+    }
+};
+
+template <int KIND>
+__device__ __forceinline__ PairItem decode_pair(const TileParams& p, const Req* tbl, int item) {
+    int lo = 0, hi = p.n_req - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (tbl[mid].item_begin[KIND] <= item) lo = mid; else hi = mid - 1;
+    }
+    const Req& rq = tbl[lo];
+    const int u = item - rq.item_begin[KIND];
+    const int heads = KIND == kSweep1 ? p.n_q_heads : p.n_kv_heads;
+    const int n_pairs = (rq.nblk + 1) >> 1;
+    PairItem it;
+    it.tok_begin = rq.tok_begin;
+    it.L = rq.L;
+    it.blk = 2 * (KIND == kSweep1 ? n_pairs - 1 - u / heads : u / heads);        // heaviest first
+    it.head = u % heads;
+    it.both = it.blk + 1 < rq.nblk;
+    it.nt = KIND == kSweep1 ? it.blk + (it.both ? 2 : 1) : (rq.nblk - it.blk) * p.group;
+    return it;
+}
+
+template <int KIND>
+__global__ void __launch_bounds__(threads_of(kSweep1), 1)
+pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+            const __grid_constant__ CUtensorMap map_x, const TileParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    PairShared<KIND>& sh = *reinterpret_cast<PairShared<KIND>*>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    volatile int* abort_flag = &sh.abort_flag;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 2; ++i) {
+            ptx::mbar_init(ptx::smem_u32(&sh.a_full[i]), 1);
+            ptx::mbar_init(ptx::smem_u32(&sh.a_empty[i]), kIssuers);
+            for (int j = 0; j < 2; ++j) {
+                ptx::mbar_init(ptx::smem_u32(&sh.comb_full[i][j]), 4);
+                ptx::mbar_init(ptx::smem_u32(&sh.comb_free[i][j]), 4);
+            }
+        }
+        for (int i = 0; i < kStages; ++i) {
+            ptx::mbar_init(ptx::smem_u32(&sh.b_full[i]), 1);
+            ptx::mbar_init(ptx::smem_u32(&sh.b_empty[i]), 1);
+        }
+        for (int i = 0; i < kAccum; ++i) {
+            ptx::mbar_init(ptx::smem_u32(&sh.t_full[i]), 1);
+            ptx::mbar_init(ptx::smem_u32(&sh.t_empty[i]), 4);
+        }
+        ptx::mbar_init(ptx::smem_u32(&sh.mma_done), kIssuers);
+        sh.abort_flag = 0;
+        ptx::fence_mbar_init();
+    }
+    if (KIND == kSweep2 && threadIdx.x < kTile) write_ones_row(sh.ax, threadIdx.x);
+    grid_dependency_wait();
+    const Req* tbl = p.reqs;
+    if (p.n_req <= kReqCache) {
+        for (int i = threadIdx.x; i < p.n_req * (int)(sizeof(Req) / 4); i += threads_of(kSweep1))
+            reinterpret_cast<int*>(sh.reqs)[i] = reinterpret_cast<const int*>(p.reqs)[i];
+        tbl = sh.reqs;
+    }
+    if (warp == 0) {
+        ptx::tmem_alloc(ptx::smem_u32(&sh.tmem_base), 512);
+        ptx::tmem_relinquish();
+    }
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    ptx::tc_fence_after_sync();
+    const uint32_t tmem_base = sh.tmem_base;
+    const int n_cta = gridDim.x;
+
+    if (warp == 0) {
+        // ------------------------------------------------------------ TMA producer ----------
+        if (lane == 0) {
+            ptx::prefetch_tensormap(&map_a);
+            ptx::prefetch_tensormap(&map_b);
+            if (KIND == kSweep2) ptx::prefetch_tensormap(&map_x);
+            uint32_t gb = 0;                         // streamed tiles armed so far
+            uint32_t na[2] = {0, 0};                 // stationary blocks armed so far, per half
+            bool stop = false;                       // a wait gave up: arm nothing more
+            for (int round = 0; !stop; ++round) {
+                const int item = item_of_round(round, blockIdx.x, n_cta);
+                if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; continue; }
+                const PairItem it = decode_pair<KIND>(p, tbl, item);
+                for (int half = 0; half < (it.both ? 2 : 1); ++half) {
+                    if (!ptx::mbar_wait(ptx::smem_u32(&sh.a_empty[half]), (na[half] & 1) ^ 1, abort_flag)) { stop = true; break; }
+                    const uint32_t bar = ptx::smem_u32(&sh.a_full[half]), dst = ptx::smem_u32(&sh.a[half][0]);
+                    const int row = it.tok_begin + (it.blk + half) * kTile;
+                    ptx::mbar_arrive_expect_tx(bar, kTileBytes);
+                    ptx::tma_load_3d(dst, &map_a, 0, it.head, row, bar);
+                    ptx::tma_load_3d(dst + kHalfBytes, &map_a, 64, it.head, row, bar);
+                    ++na[half];
+                }
+                int ib = it.blk, qs = 0;             // sweep 2: query block and query head of the group
+                for (int t = 0; t < it.nt && !stop; ++t, ++gb) {
+                    const int s = gb % kStages;
+                    if (!ptx::mbar_wait(ptx::smem_u32(&sh.b_empty[s]), ((gb / kStages) & 1) ^ 1, abort_flag)) { stop = true; break; }
+                    const uint32_t bar = ptx::smem_u32(&sh.b_full[s]), dst = ptx::smem_u32(&sh.b[s][0]);
+                    ptx::mbar_arrive_expect_tx(bar, KIND == kSweep2 ? kTileBytes + kSplitBytes : kTileBytes);
+                    const int row = it.tok_begin + (KIND == kSweep1 ? t : ib) * kTile;
+                    const int h = KIND == kSweep1 ? it.head / p.group : it.head * p.group + qs;
+                    ptx::tma_load_3d(dst, &map_b, 0, h, row, bar);
+                    ptx::tma_load_3d(dst + kHalfBytes, &map_b, 64, h, row, bar);
+                    if (KIND == kSweep2) {
+                        ptx::tma_load_3d(ptx::smem_u32(&sh.bx[s % PairShared<KIND>::kXStages][0]), &map_x, 0, h, row, bar);
+                        if (++qs == p.group) { qs = 0; ++ib; }
+                    }
+                }
+            }
+            // after an abort: wait for the copies that may not have been consumed (see tile_kernel)
+            if (*abort_flag) {
+                int ignore = 0;
+                for (uint32_t g = (gb > (uint32_t)kStages ? gb - kStages : 0); g < gb; ++g)
+                    ptx::mbar_wait(ptx::smem_u32(&sh.b_full[g % kStages]), (g / kStages) & 1, &ignore, 200000000ull);
+                for (int half = 0; half < 2; ++half)
+                    if (na[half]) ptx::mbar_wait(ptx::smem_u32(&sh.a_full[half]), (na[half] - 1) & 1, &ignore, 200000000ull);
+            }
+        }
+    } else if (warp == 1 || warp == kEpiWarp0 + 16) {
+        // ------------------------------------------------------------ MMA issuers -----------
+        if (lane == 0) {
+            const uint32_t me = (warp == 1) ? 0u : 1u;       // takes the streamed tiles of this parity
+            constexpr uint32_t idesc = ptx::umma_idesc_bf16(kTile, kTile);
+            uint32_t gb = 0, na[2] = {0, 0}, used[2] = {0, 0};
+            bool stop = false;
+            for (int round = 0; !stop; ++round) {
+                const int item = item_of_round(round, blockIdx.x, n_cta);
+                if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; continue; }
+                const PairItem it = decode_pair<KIND>(p, tbl, item);
+                bool have[2] = {false, false};       // the item's stationary block has been waited for
+                for (int t = 0; t < it.nt && !stop; ++t, ++gb) {
+                    if ((gb & 1u) != me) continue;
+                    const int s = gb % kStages;
+                    if (!ptx::mbar_wait(ptx::smem_u32(&sh.b_full[s]), (gb / kStages) & 1, abort_flag)) { stop = true; break; }
+                    const uint32_t b_addr = ptx::smem_u32(&sh.b[s][0]);
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        if (!it.template active<KIND>(half, t, p.group)) continue;
+                        const int acc = 2 * (int)me + half;
+                        if ((!have[half] && !ptx::mbar_wait(ptx::smem_u32(&sh.a_full[half]), na[half] & 1, abort_flag)) ||
+                            !ptx::mbar_wait(ptx::smem_u32(&sh.t_empty[acc]), (used[half] & 1) ^ 1, abort_flag)) {
+                            stop = true;
+                            break;
+                        }
+                        have[half] = true;
+                        ++used[half];
+                        ptx::tc_fence_after_sync();
+                        const uint32_t a_addr = ptx::smem_u32(&sh.a[half][0]), d_tmem = tmem_base + acc * kTile;
+#pragma unroll
+                        for (int kk = 0; kk < 8; ++kk) {
+                            const uint32_t off = (kk >> 2) * kHalfBytes + (kk & 3) * 32;
+                            ptx::umma_bf16(d_tmem, ptx::umma_desc_sw128(a_addr + off), ptx::umma_desc_sw128(b_addr + off), idesc, kk > 0);
+                        }
+                        if (KIND == kSweep2)             // accumulator += ones x (-lse / scale)^T
+                            ptx::umma_bf16(d_tmem, ptx::umma_desc_sw32(ptx::smem_u32(&sh.ax[0])),
+                                           ptx::umma_desc_sw32(ptx::smem_u32(&sh.bx[s % PairShared<KIND>::kXStages][0])), idesc, 1u);
+                        ptx::umma_commit(ptx::smem_u32(&sh.t_full[acc]));
+                    }
+                    if (stop) break;
+                    ptx::umma_commit(ptx::smem_u32(&sh.b_empty[s]));
+                }
+                if (stop) break;
+                // A stationary block is free when both issuers are through with the item.  An issuer that
+                // had no tile for it waits for its arrival all the same: otherwise its arrivals for two
+                // items could complete one phase.
+                for (int half = 0; half < (it.both ? 2 : 1) && !stop; ++half) {
+                    if (have[half]) ptx::umma_commit(ptx::smem_u32(&sh.a_empty[half]));
+                    else if (ptx::mbar_wait(ptx::smem_u32(&sh.a_full[half]), na[half] & 1, abort_flag))
+                        ptx::mbar_arrive(ptx::smem_u32(&sh.a_empty[half]));
+                    else stop = true;
+                    ++na[half];
+                }
+            }
+            int ignore = 0;                          // no MMA may be running when TMEM is released
+            ptx::umma_commit(ptx::smem_u32(&sh.mma_done));
+            ptx::mbar_wait(ptx::smem_u32(&sh.mma_done), 0, &ignore, 1000000000ull);
+        }
+    } else {
+        // ------------------------------------------------------------ epilogue --------------
+        const int grp = (warp - kEpiWarp0) >> 2;             // = its accumulator
+        const int half = grp & 1, parity = grp >> 1;
+        const int quarter = warp & 3;
+        const int row = quarter * 32 + lane;
+        const uint32_t tacc = tmem_base + grp * kTile + (static_cast<uint32_t>(quarter * 32) << 16);
+        const float c2 = p.scale_log2;
+        uint32_t gb = 0, used = 0, nh = 0;                   // streamed tiles, own tiles, items with this half
+        for (int round = 0;; ++round) {
+            const int item = item_of_round(round, blockIdx.x, n_cta);
+            if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; continue; }
+            const PairItem it = decode_pair<KIND>(p, tbl, item);
+            const uint32_t gb0 = gb;
+            gb += it.nt;
+            if (half == 1 && !it.both) continue;
+            const int blk = it.blk + half;
+            const int pos = blk * kTile + row;
+            const int t_first = (KIND == kSweep2 && half == 1) ? p.group : 0;            // active tiles [t_first, t_end)
+            const int t_end = (KIND == kSweep1 && half == 0) ? it.blk + 1 : it.nt;
+            float m_run = -INFINITY, l_run = 0.f;            // sweep 1
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};             // sweep 2
+            // tiles of this group: the first one of its parity, then every other one
+            int t = t_first + (int)(((gb0 + t_first) ^ parity) & 1u);
+            int ib = 0, qs = 0;                              // sweep 2: query block, head in the group
+            if (KIND == kSweep2) { ib = it.blk + t / p.group; qs = t % p.group; }
+            for (; t < t_end; t += 2, ++used) {
+                ptx::mbar_wait(ptx::smem_u32(&sh.t_full[grp]), used & 1, abort_flag);
+                ptx::tc_fence_after_sync();
+                bool diag = KIND == kSweep1 && t == blk;
+                int col_limit = kTile, diag_from = 0;
+                if (KIND == kSweep2) {
+                    // columns to mask: below the diagonal, and past the end of the request
+                    col_limit = min(kTile, it.L - ib * kTile);
+                    diag = ib == blk || col_limit < kTile;
+                    diag_from = ib == blk ? row : 0;
+                    qs += 2;
+                    while (qs >= p.group) { qs -= p.group; ++ib; }
+                }
+#pragma unroll 1
+                for (int ch = 0; ch < kTile / 32; ++ch) {
+                    uint32_t raw[32];
+                    ptx::tmem_ld_32x32(tacc + ch * 32, raw);
+                    ptx::tmem_ld_wait();
+                    if (ch == kTile / 32 - 1) {              // everything is in registers
+                        ptx::tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.t_empty[grp]));
+                    }
+                    if (KIND == kSweep1) {
+                        if (diag) sweep1_diagonal(raw, ch * 32, row, c2, m_run, l_run);
+                        else sweep1_columns(raw, c2, m_run, l_run);
+                    } else {
+                        if (diag) sweep2_diagonal(raw, ch * 32, diag_from, col_limit, c2, acc);
+                        else sweep2_columns(raw, c2, acc);
+                    }
+                }
+            }
+            // ---- combine the half's two groups: the one with its last tile finishes last ----
+            const int buf = nh & 1;
+            const uint32_t use = nh >> 1;
+            ++nh;
+            float (*cb)[kTile] = sh.comb[buf][half];
+            constexpr int kP1 = PairShared<KIND>::kPlanes - 1;
+            if ((int)((gb0 + t_end - 1) & 1u) != parity) {
+                ptx::mbar_wait(ptx::smem_u32(&sh.comb_free[half][buf]), (use & 1u) ^ 1u, abort_flag);
+                if (KIND == kSweep1) { cb[0][row] = m_run; cb[kP1][row] = l_run; }
+                else cb[0][row] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.comb_full[half][buf]));
+            } else {
+                ptx::mbar_wait(ptx::smem_u32(&sh.comb_full[half][buf]), use & 1u, abort_flag);
+                if (pos < it.L && !*abort_flag) {
+                    if (KIND == kSweep1) {
+                        const float m1 = cb[0][row], l1 = cb[kP1][row];
+                        const float m = fmaxf(m_run, m1);
+                        const float l = l_run * ptx::ex2((m_run - m) * c2) + l1 * ptx::ex2((m1 - m) * c2);
+                        store_lse(p, it.head, it.tok_begin + pos, m, l);
+                    } else {
+                        p.scores[(long long)it.head * p.T + it.tok_begin + pos] = ((acc[0] + acc[1]) + (acc[2] + acc[3])) + cb[0][row];
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.comb_free[half][buf]));
             }
         }
     }
@@ -812,9 +1128,12 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
     const size_t smem_of[3] = {sizeof(Shared<kSweep1>) + 1024, sizeof(Shared<kSweep2>) + 1024, sizeof(Shared<kMatch>) + 1024};
     const int grid = p.n_items < num_sms ? p.n_items : num_sms;
     const CUtensorMap& mx = map_x ? *map_x : map_b;      // only sweep 2 uses it
+    const size_t pair_smem[2] = {sizeof(PairShared<kSweep1>) + 1024, sizeof(PairShared<kSweep2>) + 1024};
     static unsigned long long configured = 0;
     cudaError_t err = once_per_device(configured, [&]() {
-        cudaError_t e = cudaSuccess;
+        cudaError_t e = cudaFuncSetAttribute(pair_kernel<kSweep1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_smem[0]);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(pair_kernel<kSweep2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_smem[1]);
         for (int i = 0; i < 3; ++i)
             for (int j = 0; j < 2; ++j)
                 if (e == cudaSuccess)
@@ -822,6 +1141,9 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
         return e;
     });
     if (err != cudaSuccess) return err;
+    if (p.pairs)
+        return launch_chained(kind == kSweep1 ? pair_kernel<kSweep1> : pair_kernel<kSweep2>, dim3(grid), dim3(threads_of(kSweep1)),
+                              pair_smem[kind], stream, map_a, map_b, mx, p);
     return launch_chained(kernels[kind][p.splits > 1], dim3(grid), dim3(threads_of(kind)), smem_of[kind], stream, map_a, map_b, mx, p);
 }
 

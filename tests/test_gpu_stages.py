@@ -132,6 +132,40 @@ def test_scores_of_items_cut_into_ranges(B, lens, Hq, Hkv):
         assert np.allclose(lse[:, a:a + n].cpu().numpy().reshape(Hkv, Hq // Hkv, n), lse_o, rtol=1e-6, atol=2e-5)
 
 
+@pytest.mark.parametrize("lens,Hq,Hkv", [([1665], 64, 64), ([1664], 64, 64), ([1500, 129, 1, 800, 128], 72, 24), ([200] * 16, 32, 16)])
+def test_scores_of_items_of_two_blocks(B, lens, Hq, Hkv):
+    """Enough heads for items of two blocks (in sweep 1 alone with 24 KV heads): odd and even numbers of
+    blocks, requests of one block, a last block of one row; logits rise along the prompts."""
+    import torch
+    T = sum(lens)
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    qn = synth.normal(synth.stream_key(147, T), T * Hq * 128).reshape(T, Hq, 128).astype(np.float32) * 0.5
+    kn = synth.normal(synth.stream_key(148, T), T * Hkv * 128).reshape(T, Hkv, 128).astype(np.float32) * 0.5
+    qn[:, :, 0] = 4.0
+    for a, n in zip(cu, lens):
+        kn[a:a + n, :, 0] = (4.0 * np.arange(n) / n)[:, None]
+    qb, kb = synth.f32_to_bf16_bits(qn), synth.f32_to_bf16_bits(kn)
+    q, k = to_dev(qb), to_dev(kb)
+    lay = B.make_layout(q, k, softmax_scale=1.0)
+    ws = B.alloc_workspace(lay, lens)
+    ws.fill_(0x7f)
+    scores = torch.zeros(Hkv, T, dtype=torch.float32, device="cuda")
+    lse = torch.zeros(Hq, T, dtype=torch.float32, device="cuda")
+    again = torch.zeros_like(scores)
+    B.check(B.lookm_score(q, k, cu, lay, scores, lse, False, ws))
+    assert B.lookm_device_status(ws) == B.OK
+    B.check(B.lookm_score(q, k, cu, lay, again, lse, True, ws))
+    assert torch.equal(scores, again)
+    g, heads = Hq // Hkv, [0, Hkv // 2, Hkv - 1]
+    qs = [h * g + i for h in heads for i in range(g)]
+    qf, kf = synth.bf16_to_f32(qb[:, qs]), synth.bf16_to_f32(kb[:, heads])
+    for a, n in zip(cu, lens):
+        A, lse_o = orc.scores(qf[a:a + n], kf[a:a + n], scale=1.0, threads=8, want_lse=True)
+        got = scores[heads, a:a + n].cpu().numpy().astype(np.float64)
+        assert np.all(np.abs(got - A) <= 5e-5 * A)              # exponent arguments reach 40
+        assert np.allclose(lse[qs, a:a + n].cpu().numpy().reshape(len(heads), g, n), lse_o, rtol=1e-6, atol=2e-5)
+
+
 def test_scores_packed_batch_equals_separate_requests(B):
     import torch
     lens = [200, 131, 1, 400]
