@@ -38,7 +38,7 @@ struct Plan {
     std::vector<int> out_len;               // caller order
     // workspace offsets (bytes)
     int splits[2] = {1, 1};                 // ranges of a sweep 1 / sweep 2 item's streamed tiles
-    bool pairs[2] = {false, false};         // sweep items of two blocks
+    int blocks[2] = {1, 1};                 // blocks per sweep item
     size_t n_arrived[2] = {0, 0};           // their arrival counters
     size_t clear_words = 64;                // status word and arrival counters
     size_t o_parts1 = 0, o_parts2 = 0;
@@ -50,9 +50,11 @@ struct Plan {
 struct DeviceInfo { int sms = 0; int cc_major = 0; bool ok = false; };
 int device_info(DeviceInfo& out);
 
-// Items of two blocks need three per SM to be shared evenly (2048 tokens x 8 heads, 64 of them: 66 us a
-// layer with single blocks, 85 with pairs; 7777 x 8 KV heads, 248 for sweep 2: 390 against 393).
+// Items of two blocks need three per SM to be shared evenly, items of four six (two: 2048 tokens x 8
+// heads, 64 items: 66 us a layer with single blocks, 85 with pairs; 7777 x 8 KV heads, 248 for sweep 2:
+// 390 against 393; four: 8192 x 32 heads, 512 items: 807-833 us with pairs, 844-885 with four).
 constexpr long long kPairItemsPerSm = 3;
+constexpr long long kQuadItemsPerSm = 6;
 // Splits of the sweep items: as many as bring the longest item down to what an SM has on average, if it
 // is more than one and a half times that and ten tiles longer.  Both sweeps together, us: 5000 tokens
 // with 2 heads 63.5 -> 38, 12000 with 2 query on 1 KV head 188 -> 110, 2048 with 32 on 8 78 -> 63, 700
@@ -66,10 +68,12 @@ void plan_splits(Plan& pl) {
     const long long mean = std::max<long long>(1, tiles * pl.n_q_heads / sms);
     for (int s = 0; s < 2; ++s) {
         const long long longest = (long long)pl.reqs[0].nblk * (s ? pl.group : 1);
-        long long pair_items = 0;
-        for (const Req& q : pl.reqs) pair_items += (long long)((q.nblk + 1) / 2) * (s ? pl.n_kv_heads : pl.n_q_heads);
-        pl.pairs[s] = pair_items >= kPairItemsPerSm * sms;
-        if (!pl.pairs[s] && 2 * longest > 3 * mean && longest >= mean + 10)
+        for (int b : {2, 4}) {
+            long long items = 0;
+            for (const Req& q : pl.reqs) items += (long long)((q.nblk + b - 1) / b) * (s ? pl.n_kv_heads : pl.n_q_heads);
+            if (items >= (b == 2 ? kPairItemsPerSm : kQuadItemsPerSm) * sms) pl.blocks[s] = b;
+        }
+        if (pl.blocks[s] == 1 && 2 * longest > 3 * mean && longest >= mean + 10)
             pl.splits[s] = (int)std::min<long long>(kMaxSplits, (longest + mean - 1) / mean);
     }
 }
@@ -160,8 +164,8 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
         const bool merges = q.mode != LOOKM_MERGE_NONE;
         const long long n_units = merges ? (q.L + unit_entries - 1) / unit_entries : 0;
         units += (long long)pl.n_kv_heads * n_units;
-        it0 += (long long)(pl.pairs[0] ? (q.nblk + 1) / 2 : q.nblk) * pl.n_q_heads * pl.splits[0];
-        it1 += (long long)(pl.pairs[1] ? (q.nblk + 1) / 2 : q.nblk) * pl.n_kv_heads * pl.splits[1];
+        it0 += (long long)((q.nblk + pl.blocks[0] - 1) / pl.blocks[0]) * pl.n_q_heads * pl.splits[0];
+        it1 += (long long)((q.nblk + pl.blocks[1] - 1) / pl.blocks[1]) * pl.n_kv_heads * pl.splits[1];
         // match items: blocks of 128 entries of every head's evicted list
         it2 += (q.E > 0 && merges) ? (long long)((q.E + kTile - 1) / kTile) * pl.n_kv_heads : 0;
         slots += (long long)q.B * pl.n_kv_heads;
@@ -361,7 +365,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     p.scores = scores;
     if (!lse_is_input) {
         p.n_items = pl.n_items[kSweep1];
-        p.pairs = pl.pairs[0];
+        p.blocks = pl.blocks[0];
         p.splits = pl.splits[0];
         p.parts1 = at<float2>(ws, pl.o_parts1);
         p.arrived = p.status + 64;
@@ -373,7 +377,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     }
     mark_stage(1, st);
     p.n_items = pl.n_items[kSweep2];
-    p.pairs = pl.pairs[1];
+    p.blocks = pl.blocks[1];
     p.splits = pl.splits[1];
     p.parts2 = at<float>(ws, pl.o_parts2);
     p.arrived = p.status + 64 + pl.n_arrived[0];

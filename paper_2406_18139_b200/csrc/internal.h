@@ -73,7 +73,7 @@ struct TileParams {
     unsigned short* lse_split;   // [T, n_q_heads, 16] bf16: -lse / scale as three bf16 terms and 13
                                  // zeros per query row (sweep 1 writes, sweep 2 loads it by TMA)
     float* scores;               // [n_kv_heads, T]
-    int pairs;                   // sweep items of two blocks (pair_kernel); no splits then
+    int blocks;                  // blocks per sweep item: 1, or 2 or 4 (multi_kernel; no splits then)
     int splits;                  // ranges that the streamed tiles of a sweep item are cut into
     float2* parts1;              // [splits][n_q_heads, T]  reference and sum of a range (sweep 1)
     float* parts2;               // [splits][n_kv_heads, T] column sums of a range (sweep 2)

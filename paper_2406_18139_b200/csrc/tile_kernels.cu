@@ -771,53 +771,55 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 }
 
 // ------------------------------------------------------------------------------------------------
-// The sweeps of large problems: an item owns TWO adjacent stationary blocks (halves 0 and 1) and every
-// streamed tile is multiplied with both, so a tile is brought into shared memory once per two products.
-// The sweeps of large prompts run at the board's power limit, where time is energy, and a tenth of
-// that goes into moving tiles from L2 (a build without the loads ran 9-11 % faster).
-// Whole layers in a row, one block per item -> two: 16384 tokens x 40 heads 4.45 -> 4.10 ms, 32768 x 32
-// query heads on 8 11.2 -> 10.6 ms, 16 ragged prompts x 32 heads 24.2 -> 23.2 ms, 8192 x 32 0.918 -> 0.886.
-// Streamed tile g of the CTA goes to accumulators 2 (g mod 2) + half, and each accumulator has one
-// issuing thread (g mod 2) and one epilogue group: group w works on half w mod 2 and on the tiles of
-// parity w / 2, so its running results belong to one block.  The two groups of a half are combined at
-// the item's end like the four of tile_kernel.  Across the diagonal a half may have no product with a
-// tile (sweep 1: the last tile and half 0; sweep 2: the first query block and half 1).
+// The sweeps of large problems: an item owns kBlocks = 2 or 4 adjacent stationary blocks and every
+// streamed tile is multiplied with all of them, so a tile is brought into shared memory once per two or
+// four products.  These sweeps run at the board's power limit, where time is energy, and a tenth of that
+// goes into moving tiles from L2 (a build without the loads ran 9-11 % faster).  Whole layers in a row,
+// one block per item -> two -> four: 16384 tokens x 40 heads 4.45 -> 4.10 -> 3.92 ms, 32768 x 32 query
+// heads on 8 11.2 -> 10.6 -> 10.4 ms, 16 ragged prompts x 32 heads 24.4 -> 23.4 -> 22.5 ms, 8192 x 32
+// 0.918 -> 0.886 (four blocks, 3.5 items per SM: 0.93).
+// Two blocks: streamed tile g of the CTA goes to accumulators 2 (g mod 2) + block, and each accumulator
+// has one issuing thread (g mod 2) and one epilogue group, which works on one block and on the tiles of
+// one parity; the two groups of a block are combined at the item's end like the four of tile_kernel.
+// Four blocks: one accumulator and one epilogue group each, nothing to combine.  Across the diagonal a
+// tile skips the blocks it lies above (sweep 1) or below (sweep 2).
 // ------------------------------------------------------------------------------------------------
-template <int KIND>
-struct __align__(1024) PairShared {
-    static constexpr int kXStages = (KIND == kSweep2) ? kStages : 1;
+template <int KIND, int kBlocks>
+struct __align__(1024) MultiShared {
+    static constexpr int kRing = kBlocks == 2 ? 4 : 2;   // streamed tiles
+    static constexpr int kXStages = (KIND == kSweep2) ? kRing : 1;
     static constexpr int kPlanes = (KIND == kSweep2) ? 1 : 2;
-    uint8_t a[2][kTileBytes];                    // stationary blocks
-    uint8_t b[kStages][kTileBytes];              // streamed tiles
+    uint8_t a[kBlocks][kTileBytes];              // stationary blocks
+    uint8_t b[kRing][kTileBytes];                // streamed tiles
     uint8_t bx[kXStages][kSplitBytes];           // sweep 2: their 16-column companions
     uint8_t ax[kSplitBytes];                     // sweep 2: constant ones tile that multiplies bx
     float comb[2][2][kPlanes][kTile];            // partial results, [buffer][half]
     Req reqs[kReqCache];
-    unsigned long long a_full[2], a_empty[2];
-    unsigned long long b_full[kStages], b_empty[kStages];
+    unsigned long long a_full[kBlocks], a_empty[kBlocks];
+    unsigned long long b_full[kRing], b_empty[kRing];
     unsigned long long t_full[kAccum], t_empty[kAccum];
     unsigned long long comb_full[2][2], comb_free[2][2];     // [half][buffer]
     unsigned long long mma_done;
     uint32_t tmem_base;
     int abort_flag;
 };
-static_assert(sizeof(PairShared<kSweep1>) + 1024 <= 232448 && sizeof(PairShared<kSweep2>) + 1024 <= 232448,
-              "shared memory of the paired sweeps exceeds 227 KB");
+static_assert(sizeof(MultiShared<kSweep1, 2>) + 1024 <= 232448 && sizeof(MultiShared<kSweep2, 2>) + 1024 <= 232448 &&
+              sizeof(MultiShared<kSweep1, 4>) + 1024 <= 232448 && sizeof(MultiShared<kSweep2, 4>) + 1024 <= 232448,
+              "shared memory of the multi-block sweeps exceeds 227 KB");
 static_assert(kAccum == 4 && kGroups == 4 && kHalves == 1 && kIssuers == 2, "the paired sweeps assume this layout");
 
-struct PairItem {
+struct MultiItem {
     int tok_begin, L, blk, head, nt;
-    bool both;                                   // half 1 exists
-    // is streamed tile t multiplied with the half?  group: query heads that take turns (sweep 2)
+    int n;                                       // blocks of the item that exist
+    // is streamed tile t multiplied with block b?  group: query heads that take turns (sweep 2)
     template <int KIND>
-    __device__ __forceinline__ bool active(int half, int t, int group) const {
-        if (half == 0) return KIND == kSweep2 || t <= blk;
-        return both && (KIND == kSweep1 || t >= group);
+    __device__ __forceinline__ bool active(int b, int t, int group) const {
+        return b < n && (KIND == kSweep1 ? t <= blk + b : t >= b * group);
     }
 };
 
-template <int KIND>
-__device__ __forceinline__ PairItem decode_pair(const TileParams& p, const Req* tbl, int item) {
+template <int KIND, int kBlocks>
+__device__ __forceinline__ MultiItem decode_multi(const TileParams& p, const Req* tbl, int item) {
     int lo = 0, hi = p.n_req - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -826,40 +828,44 @@ __device__ __forceinline__ PairItem decode_pair(const TileParams& p, const Req* 
     const Req& rq = tbl[lo];
     const int u = item - rq.item_begin[KIND];
     const int heads = KIND == kSweep1 ? p.n_q_heads : p.n_kv_heads;
-    const int n_pairs = (rq.nblk + 1) >> 1;
-    PairItem it;
+    const int n_sets = (rq.nblk + kBlocks - 1) / kBlocks;
+    MultiItem it;
     it.tok_begin = rq.tok_begin;
     it.L = rq.L;
-    it.blk = 2 * (KIND == kSweep1 ? n_pairs - 1 - u / heads : u / heads);        // heaviest first
+    it.blk = kBlocks * (KIND == kSweep1 ? n_sets - 1 - u / heads : u / heads);   // heaviest first
     it.head = u % heads;
-    it.both = it.blk + 1 < rq.nblk;
-    it.nt = KIND == kSweep1 ? it.blk + (it.both ? 2 : 1) : (rq.nblk - it.blk) * p.group;
+    it.n = min(kBlocks, rq.nblk - it.blk);
+    it.nt = KIND == kSweep1 ? it.blk + it.n : (rq.nblk - it.blk) * p.group;
     return it;
 }
 
-template <int KIND>
+template <int KIND, int kBlocks>
 __global__ void __launch_bounds__(threads_of(kSweep1), 1)
-pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
             const __grid_constant__ CUtensorMap map_x, const TileParams p) {
     extern __shared__ uint8_t smem_raw[];
-    PairShared<KIND>& sh = *reinterpret_cast<PairShared<KIND>*>(
+    typedef MultiShared<KIND, kBlocks> Sh;
+    constexpr int kRing = Sh::kRing;
+    Sh& sh = *reinterpret_cast<Sh*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     volatile int* abort_flag = &sh.abort_flag;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < kBlocks; ++i) {
             ptx::mbar_init(ptx::smem_u32(&sh.a_full[i]), 1);
-            ptx::mbar_init(ptx::smem_u32(&sh.a_empty[i]), kIssuers);
+            ptx::mbar_init(ptx::smem_u32(&sh.a_empty[i]), kBlocks == 2 ? kIssuers : 1);      // issuers that use it
+        }
+        for (int i = 0; i < 2; ++i) {
             for (int j = 0; j < 2; ++j) {
                 ptx::mbar_init(ptx::smem_u32(&sh.comb_full[i][j]), 4);
                 ptx::mbar_init(ptx::smem_u32(&sh.comb_free[i][j]), 4);
             }
         }
-        for (int i = 0; i < kStages; ++i) {
+        for (int i = 0; i < kRing; ++i) {
             ptx::mbar_init(ptx::smem_u32(&sh.b_full[i]), 1);
-            ptx::mbar_init(ptx::smem_u32(&sh.b_empty[i]), 1);
+            ptx::mbar_init(ptx::smem_u32(&sh.b_empty[i]), kBlocks == 2 ? 1 : kIssuers);
         }
         for (int i = 0; i < kAccum; ++i) {
             ptx::mbar_init(ptx::smem_u32(&sh.t_full[i]), 1);
@@ -894,13 +900,15 @@ pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             ptx::prefetch_tensormap(&map_b);
             if (KIND == kSweep2) ptx::prefetch_tensormap(&map_x);
             uint32_t gb = 0;                         // streamed tiles armed so far
-            uint32_t na[2] = {0, 0};                 // stationary blocks armed so far, per half
+            uint32_t na[kBlocks] = {};               // stationary blocks armed so far, per place
             bool stop = false;                       // a wait gave up: arm nothing more
             for (int round = 0; !stop; ++round) {
                 const int item = item_of_round(round, blockIdx.x, n_cta);
                 if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; continue; }
-                const PairItem it = decode_pair<KIND>(p, tbl, item);
-                for (int half = 0; half < (it.both ? 2 : 1); ++half) {
+                const MultiItem it = decode_multi<KIND, kBlocks>(p, tbl, item);
+#pragma unroll
+                for (int half = 0; half < kBlocks; ++half) {
+                    if (half >= it.n) break;
                     if (!ptx::mbar_wait(ptx::smem_u32(&sh.a_empty[half]), (na[half] & 1) ^ 1, abort_flag)) { stop = true; break; }
                     const uint32_t bar = ptx::smem_u32(&sh.a_full[half]), dst = ptx::smem_u32(&sh.a[half][0]);
                     const int row = it.tok_begin + (it.blk + half) * kTile;
@@ -911,8 +919,8 @@ pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 }
                 int ib = it.blk, qs = 0;             // sweep 2: query block and query head of the group
                 for (int t = 0; t < it.nt && !stop; ++t, ++gb) {
-                    const int s = gb % kStages;
-                    if (!ptx::mbar_wait(ptx::smem_u32(&sh.b_empty[s]), ((gb / kStages) & 1) ^ 1, abort_flag)) { stop = true; break; }
+                    const int s = gb % kRing;
+                    if (!ptx::mbar_wait(ptx::smem_u32(&sh.b_empty[s]), ((gb / kRing) & 1) ^ 1, abort_flag)) { stop = true; break; }
                     const uint32_t bar = ptx::smem_u32(&sh.b_full[s]), dst = ptx::smem_u32(&sh.b[s][0]);
                     ptx::mbar_arrive_expect_tx(bar, KIND == kSweep2 ? kTileBytes + kSplitBytes : kTileBytes);
                     const int row = it.tok_begin + (KIND == kSweep1 ? t : ib) * kTile;
@@ -920,7 +928,7 @@ pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                     ptx::tma_load_3d(dst, &map_b, 0, h, row, bar);
                     ptx::tma_load_3d(dst + kHalfBytes, &map_b, 64, h, row, bar);
                     if (KIND == kSweep2) {
-                        ptx::tma_load_3d(ptx::smem_u32(&sh.bx[s % PairShared<KIND>::kXStages][0]), &map_x, 0, h, row, bar);
+                        ptx::tma_load_3d(ptx::smem_u32(&sh.bx[s % Sh::kXStages][0]), &map_x, 0, h, row, bar);
                         if (++qs == p.group) { qs = 0; ++ib; }
                     }
                 }
@@ -928,34 +936,38 @@ pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             // after an abort: wait for the copies that may not have been consumed (see tile_kernel)
             if (*abort_flag) {
                 int ignore = 0;
-                for (uint32_t g = (gb > (uint32_t)kStages ? gb - kStages : 0); g < gb; ++g)
-                    ptx::mbar_wait(ptx::smem_u32(&sh.b_full[g % kStages]), (g / kStages) & 1, &ignore, 200000000ull);
-                for (int half = 0; half < 2; ++half)
+                for (uint32_t g = (gb > (uint32_t)kRing ? gb - kRing : 0); g < gb; ++g)
+                    ptx::mbar_wait(ptx::smem_u32(&sh.b_full[g % kRing]), (g / kRing) & 1, &ignore, 200000000ull);
+#pragma unroll
+                for (int half = 0; half < kBlocks; ++half)
                     if (na[half]) ptx::mbar_wait(ptx::smem_u32(&sh.a_full[half]), (na[half] - 1) & 1, &ignore, 200000000ull);
             }
         }
     } else if (warp == 1 || warp == kEpiWarp0 + 16) {
         // ------------------------------------------------------------ MMA issuers -----------
         if (lane == 0) {
-            const uint32_t me = (warp == 1) ? 0u : 1u;       // takes the streamed tiles of this parity
+            // of two blocks an issuer takes both for the streamed tiles of its parity, of four it takes
+            // two for every tile; either way it owns two accumulators
+            const uint32_t me = (warp == 1) ? 0u : 1u;
+            const int b0 = kBlocks == 2 ? 0 : 2 * (int)me;
             constexpr uint32_t idesc = ptx::umma_idesc_bf16(kTile, kTile);
             uint32_t gb = 0, na[2] = {0, 0}, used[2] = {0, 0};
             bool stop = false;
             for (int round = 0; !stop; ++round) {
                 const int item = item_of_round(round, blockIdx.x, n_cta);
                 if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; continue; }
-                const PairItem it = decode_pair<KIND>(p, tbl, item);
+                const MultiItem it = decode_multi<KIND, kBlocks>(p, tbl, item);
                 bool have[2] = {false, false};       // the item's stationary block has been waited for
                 for (int t = 0; t < it.nt && !stop; ++t, ++gb) {
-                    if ((gb & 1u) != me) continue;
-                    const int s = gb % kStages;
-                    if (!ptx::mbar_wait(ptx::smem_u32(&sh.b_full[s]), (gb / kStages) & 1, abort_flag)) { stop = true; break; }
+                    if (kBlocks == 2 && (gb & 1u) != me) continue;
+                    const int s = gb % kRing;
+                    if (!ptx::mbar_wait(ptx::smem_u32(&sh.b_full[s]), (gb / kRing) & 1, abort_flag)) { stop = true; break; }
                     const uint32_t b_addr = ptx::smem_u32(&sh.b[s][0]);
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
-                        if (!it.template active<KIND>(half, t, p.group)) continue;
+                        if (!it.template active<KIND>(b0 + half, t, p.group)) continue;
                         const int acc = 2 * (int)me + half;
-                        if ((!have[half] && !ptx::mbar_wait(ptx::smem_u32(&sh.a_full[half]), na[half] & 1, abort_flag)) ||
+                        if ((!have[half] && !ptx::mbar_wait(ptx::smem_u32(&sh.a_full[b0 + half]), na[half] & 1, abort_flag)) ||
                             !ptx::mbar_wait(ptx::smem_u32(&sh.t_empty[acc]), (used[half] & 1) ^ 1, abort_flag)) {
                             stop = true;
                             break;
@@ -963,7 +975,7 @@ pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         have[half] = true;
                         ++used[half];
                         ptx::tc_fence_after_sync();
-                        const uint32_t a_addr = ptx::smem_u32(&sh.a[half][0]), d_tmem = tmem_base + acc * kTile;
+                        const uint32_t a_addr = ptx::smem_u32(&sh.a[b0 + half][0]), d_tmem = tmem_base + acc * kTile;
 #pragma unroll
                         for (int kk = 0; kk < 8; ++kk) {
                             const uint32_t off = (kk >> 2) * kHalfBytes + (kk & 3) * 32;
@@ -971,20 +983,22 @@ pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         }
                         if (KIND == kSweep2)             // accumulator += ones x (-lse / scale)^T
                             ptx::umma_bf16(d_tmem, ptx::umma_desc_sw32(ptx::smem_u32(&sh.ax[0])),
-                                           ptx::umma_desc_sw32(ptx::smem_u32(&sh.bx[s % PairShared<KIND>::kXStages][0])), idesc, 1u);
+                                           ptx::umma_desc_sw32(ptx::smem_u32(&sh.bx[s % Sh::kXStages][0])), idesc, 1u);
                         ptx::umma_commit(ptx::smem_u32(&sh.t_full[acc]));
                     }
                     if (stop) break;
                     ptx::umma_commit(ptx::smem_u32(&sh.b_empty[s]));
                 }
                 if (stop) break;
-                // A stationary block is free when both issuers are through with the item.  An issuer that
+                // A stationary block is free when its issuers are through with the item.  An issuer that
                 // had no tile for it waits for its arrival all the same: otherwise its arrivals for two
                 // items could complete one phase.
-                for (int half = 0; half < (it.both ? 2 : 1) && !stop; ++half) {
-                    if (have[half]) ptx::umma_commit(ptx::smem_u32(&sh.a_empty[half]));
-                    else if (ptx::mbar_wait(ptx::smem_u32(&sh.a_full[half]), na[half] & 1, abort_flag))
-                        ptx::mbar_arrive(ptx::smem_u32(&sh.a_empty[half]));
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    if (b0 + half >= it.n || stop) continue;
+                    if (have[half]) ptx::umma_commit(ptx::smem_u32(&sh.a_empty[b0 + half]));
+                    else if (ptx::mbar_wait(ptx::smem_u32(&sh.a_full[b0 + half]), na[half] & 1, abort_flag))
+                        ptx::mbar_arrive(ptx::smem_u32(&sh.a_empty[b0 + half]));
                     else stop = true;
                     ++na[half];
                 }
@@ -996,7 +1010,8 @@ pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     } else {
         // ------------------------------------------------------------ epilogue --------------
         const int grp = (warp - kEpiWarp0) >> 2;             // = its accumulator
-        const int half = grp & 1, parity = grp >> 1;
+        const int half = kBlocks == 2 ? grp & 1 : grp;       // its block of the item
+        const int parity = grp >> 1;                         // two blocks: of the streamed tiles it works on
         const int quarter = warp & 3;
         const int row = quarter * 32 + lane;
         const uint32_t tacc = tmem_base + grp * kTile + (static_cast<uint32_t>(quarter * 32) << 16);
@@ -1005,21 +1020,23 @@ pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         for (int round = 0;; ++round) {
             const int item = item_of_round(round, blockIdx.x, n_cta);
             if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; continue; }
-            const PairItem it = decode_pair<KIND>(p, tbl, item);
+            const MultiItem it = decode_multi<KIND, kBlocks>(p, tbl, item);
             const uint32_t gb0 = gb;
             gb += it.nt;
-            if (half == 1 && !it.both) continue;
+            if (half >= it.n) continue;
             const int blk = it.blk + half;
             const int pos = blk * kTile + row;
-            const int t_first = (KIND == kSweep2 && half == 1) ? p.group : 0;            // active tiles [t_first, t_end)
-            const int t_end = (KIND == kSweep1 && half == 0) ? it.blk + 1 : it.nt;
+            const int t_first = KIND == kSweep2 ? half * p.group : 0;        // active tiles [t_first, t_end)
+            const int t_end = KIND == kSweep1 ? blk + 1 : it.nt;
             float m_run = -INFINITY, l_run = 0.f;            // sweep 1
-            float acc[4] = {0.f, 0.f, 0.f, 0.f};             // sweep 2
-            // tiles of this group: the first one of its parity, then every other one
-            int t = t_first + (int)(((gb0 + t_first) ^ parity) & 1u);
+            float total = 0.f;                               // sweep 2: sums of whole tiles (short chains of
+                                                             // additions, whatever the prompt's length)
+            // tiles of this group: all of them, or the first one of its parity and every other one
+            constexpr int kStep = kBlocks == 2 ? 2 : 1;
+            int t = t_first + (kBlocks == 2 ? (int)(((gb0 + t_first) ^ parity) & 1u) : 0);
             int ib = 0, qs = 0;                              // sweep 2: query block, head in the group
             if (KIND == kSweep2) { ib = it.blk + t / p.group; qs = t % p.group; }
-            for (; t < t_end; t += 2, ++used) {
+            for (; t < t_end; t += kStep, ++used) {
                 ptx::mbar_wait(ptx::smem_u32(&sh.t_full[grp]), used & 1, abort_flag);
                 ptx::tc_fence_after_sync();
                 bool diag = KIND == kSweep1 && t == blk;
@@ -1029,9 +1046,10 @@ pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                     col_limit = min(kTile, it.L - ib * kTile);
                     diag = ib == blk || col_limit < kTile;
                     diag_from = ib == blk ? row : 0;
-                    qs += 2;
+                    qs += kStep;
                     while (qs >= p.group) { qs -= p.group; ++ib; }
                 }
+                float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
                 for (int ch = 0; ch < kTile / 32; ++ch) {
                     uint32_t raw[32];
@@ -1050,21 +1068,29 @@ pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         else sweep2_columns(raw, c2, acc);
                     }
                 }
+                if (KIND == kSweep2) total += (acc[0] + acc[1]) + (acc[2] + acc[3]);
             }
-            // ---- combine the half's two groups: the one with its last tile finishes last ----
+            if (kBlocks == 4) {                              // nobody else worked on the block
+                if (pos < it.L && !*abort_flag) {
+                    if (KIND == kSweep1) store_lse(p, it.head, it.tok_begin + pos, m_run, l_run);
+                    else p.scores[(long long)it.head * p.T + it.tok_begin + pos] = total;
+                }
+                continue;
+            }
+            // ---- combine the block's two groups: the one with its last tile finishes last ----
             const int buf = nh & 1;
             const uint32_t use = nh >> 1;
             ++nh;
-            float (*cb)[kTile] = sh.comb[buf][half];
-            constexpr int kP1 = PairShared<KIND>::kPlanes - 1;
+            float (*cb)[kTile] = sh.comb[buf][half & 1];
+            constexpr int kP1 = Sh::kPlanes - 1;
             if ((int)((gb0 + t_end - 1) & 1u) != parity) {
-                ptx::mbar_wait(ptx::smem_u32(&sh.comb_free[half][buf]), (use & 1u) ^ 1u, abort_flag);
+                ptx::mbar_wait(ptx::smem_u32(&sh.comb_free[half & 1][buf]), (use & 1u) ^ 1u, abort_flag);
                 if (KIND == kSweep1) { cb[0][row] = m_run; cb[kP1][row] = l_run; }
-                else cb[0][row] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+                else cb[0][row] = total;
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.comb_full[half][buf]));
+                if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.comb_full[half & 1][buf]));
             } else {
-                ptx::mbar_wait(ptx::smem_u32(&sh.comb_full[half][buf]), use & 1u, abort_flag);
+                ptx::mbar_wait(ptx::smem_u32(&sh.comb_full[half & 1][buf]), use & 1u, abort_flag);
                 if (pos < it.L && !*abort_flag) {
                     if (KIND == kSweep1) {
                         const float m1 = cb[0][row], l1 = cb[kP1][row];
@@ -1072,11 +1098,11 @@ pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         const float l = l_run * ptx::ex2((m_run - m) * c2) + l1 * ptx::ex2((m1 - m) * c2);
                         store_lse(p, it.head, it.tok_begin + pos, m, l);
                     } else {
-                        p.scores[(long long)it.head * p.T + it.tok_begin + pos] = ((acc[0] + acc[1]) + (acc[2] + acc[3])) + cb[0][row];
+                        p.scores[(long long)it.head * p.T + it.tok_begin + pos] = total + cb[0][row];
                     }
                 }
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.comb_free[half][buf]));
+                if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.comb_free[half & 1][buf]));
             }
         }
     }
@@ -1128,12 +1154,17 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
     const size_t smem_of[3] = {sizeof(Shared<kSweep1>) + 1024, sizeof(Shared<kSweep2>) + 1024, sizeof(Shared<kMatch>) + 1024};
     const int grid = p.n_items < num_sms ? p.n_items : num_sms;
     const CUtensorMap& mx = map_x ? *map_x : map_b;      // only sweep 2 uses it
-    const size_t pair_smem[2] = {sizeof(PairShared<kSweep1>) + 1024, sizeof(PairShared<kSweep2>) + 1024};
+    static const Kernel multi[2][2] = {{multi_kernel<kSweep1, 2>, multi_kernel<kSweep1, 4>},
+                                       {multi_kernel<kSweep2, 2>, multi_kernel<kSweep2, 4>}};
+    const size_t multi_smem[2][2] = {{sizeof(MultiShared<kSweep1, 2>) + 1024, sizeof(MultiShared<kSweep1, 4>) + 1024},
+                                     {sizeof(MultiShared<kSweep2, 2>) + 1024, sizeof(MultiShared<kSweep2, 4>) + 1024}};
     static unsigned long long configured = 0;
     cudaError_t err = once_per_device(configured, [&]() {
-        cudaError_t e = cudaFuncSetAttribute(pair_kernel<kSweep1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_smem[0]);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(pair_kernel<kSweep2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_smem[1]);
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < 2; ++i)
+            for (int j = 0; j < 2; ++j)
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute(multi[i][j], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)multi_smem[i][j]);
         for (int i = 0; i < 3; ++i)
             for (int j = 0; j < 2; ++j)
                 if (e == cudaSuccess)
@@ -1141,9 +1172,9 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
         return e;
     });
     if (err != cudaSuccess) return err;
-    if (p.pairs)
-        return launch_chained(kind == kSweep1 ? pair_kernel<kSweep1> : pair_kernel<kSweep2>, dim3(grid), dim3(threads_of(kSweep1)),
-                              pair_smem[kind], stream, map_a, map_b, mx, p);
+    if (p.blocks > 1)
+        return launch_chained(multi[kind][p.blocks == 4], dim3(grid), dim3(threads_of(kSweep1)), multi_smem[kind][p.blocks == 4],
+                              stream, map_a, map_b, mx, p);
     return launch_chained(kernels[kind][p.splits > 1], dim3(grid), dim3(threads_of(kind)), smem_of[kind], stream, map_a, map_b, mx, p);
 }
 
