@@ -51,8 +51,10 @@ struct DeviceInfo { int sms = 0; int cc_major = 0; bool ok = false; };
 int device_info(DeviceInfo& out);
 
 // Items of two blocks need three per SM to be shared evenly, items of four six (two: 2048 tokens x 8
-// heads, 64 items: 66 us a layer with single blocks, 85 with pairs; 7777 x 8 KV heads, 248 for sweep 2:
-// 390 against 393; four: 8192 x 32 heads, 512 items: 807-833 us with pairs, 844-885 with four).
+// heads, 64 items: 66 us a layer with single blocks, 85 with pairs; four: 8192 x 32 heads, 512 items:
+// 807-833 us with pairs, 844-885 with four).  Grouped query heads count one by one, in sweep 2 as well:
+// 7777 tokens x 32 query heads on 8, sweep 2 alone, 392 us a layer with single blocks for whole groups,
+// 378 with pairs for single query heads.
 constexpr long long kPairItemsPerSm = 3;
 constexpr long long kQuadItemsPerSm = 6;
 // Splits of the sweep items: as many as bring the longest item down to what an SM has on average, if it
@@ -70,7 +72,7 @@ void plan_splits(Plan& pl) {
         const long long longest = (long long)pl.reqs[0].nblk * (s ? pl.group : 1);
         for (int b : {2, 4}) {
             long long items = 0;
-            for (const Req& q : pl.reqs) items += (long long)((q.nblk + b - 1) / b) * (s ? pl.n_kv_heads : pl.n_q_heads);
+            for (const Req& q : pl.reqs) items += (long long)((q.nblk + b - 1) / b) * pl.n_q_heads;
             if (items >= (b == 2 ? kPairItemsPerSm : kQuadItemsPerSm) * sms) pl.blocks[s] = b;
         }
         if (pl.blocks[s] == 1 && 2 * longest > 3 * mean && longest >= mean + 10)
@@ -165,7 +167,8 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
         const long long n_units = merges ? (q.L + unit_entries - 1) / unit_entries : 0;
         units += (long long)pl.n_kv_heads * n_units;
         it0 += (long long)((q.nblk + pl.blocks[0] - 1) / pl.blocks[0]) * pl.n_q_heads * pl.splits[0];
-        it1 += (long long)((q.nblk + pl.blocks[1] - 1) / pl.blocks[1]) * pl.n_kv_heads * pl.splits[1];
+        // (several blocks per item: the query heads of a group are items of their own in sweep 2 too)
+        it1 += (long long)((q.nblk + pl.blocks[1] - 1) / pl.blocks[1]) * (pl.blocks[1] > 1 ? pl.n_q_heads : pl.n_kv_heads) * pl.splits[1];
         // match items: blocks of 128 entries of every head's evicted list
         it2 += (q.E > 0 && merges) ? (long long)((q.E + kTile - 1) / kTile) * pl.n_kv_heads : 0;
         slots += (long long)q.B * pl.n_kv_heads;
@@ -180,8 +183,9 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
     const size_t Hq = pl.n_q_heads, Hkv = pl.n_kv_heads, T = (size_t)pl.T;
     // Every list is sized for the worst case over budgets (at most T kept and T evicted rows per
     // head), so the carving depends only on the prompt lengths and head counts.
+    const size_t score_parts = pl.blocks[1] > 1 ? pl.group : pl.splits[1];       // partial column sums of sweep 2
     for (int s = 0; s < 2; ++s)
-        if (pl.splits[s] > 1) pl.n_arrived[s] = 4 * (size_t)tiles * (s ? Hkv : Hq);
+        if (pl.splits[s] > 1 || (s && score_parts > 1)) pl.n_arrived[s] = 4 * (size_t)tiles * (s ? Hkv : Hq);
     pl.clear_words += pl.n_arrived[0] + pl.n_arrived[1];
     pl.o_status = carve(4 * pl.clear_words);
     pl.o_reqs = carve(sizeof(Req) * n_req);
@@ -205,7 +209,7 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
     pl.o_sort_a = carve(8 * Hkv * T);
     pl.o_sort_b = carve(8 * Hkv * T);
     pl.o_parts1 = carve(pl.splits[0] > 1 ? 8 * Hq * T * pl.splits[0] : 0);
-    pl.o_parts2 = carve(pl.splits[1] > 1 ? 4 * Hkv * T * pl.splits[1] : 0);
+    pl.o_parts2 = carve(score_parts > 1 ? 4 * Hkv * T * score_parts : 0);
     pl.total = o;
     return LOOKM_OK;
 }

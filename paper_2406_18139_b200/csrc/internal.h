@@ -76,7 +76,8 @@ struct TileParams {
     int blocks;                  // blocks per sweep item: 1, or 2 or 4 (multi_kernel; no splits then)
     int splits;                  // ranges that the streamed tiles of a sweep item are cut into
     float2* parts1;              // [splits][n_q_heads, T]  reference and sum of a range (sweep 1)
-    float* parts2;               // [splits][n_kv_heads, T] column sums of a range (sweep 2)
+    float* parts2;               // [splits][n_kv_heads, T] column sums of a range, or of a query head of the
+                                 // group (sweep 2)
     int* arrived;                // [block][heads][4] finished ranges per 32 rows (zeroed)
     const int* evict_idx;        // evicted-list layout  (match: rows of the stationary tiles)
     const void* k_rows;          // K [tokens, heads, 128] bf16 with the strides below (match)

@@ -811,12 +811,36 @@ static_assert(kAccum == 4 && kGroups == 4 && kHalves == 1 && kIssuers == 2, "the
 struct MultiItem {
     int tok_begin, L, blk, head, nt;
     int n;                                       // blocks of the item that exist
-    // is streamed tile t multiplied with block b?  group: query heads that take turns (sweep 2)
+    int tile;                                    // index of the first block over the whole batch
+    // is streamed tile t multiplied with block b?
     template <int KIND>
-    __device__ __forceinline__ bool active(int b, int t, int group) const {
-        return b < n && (KIND == kSweep1 ? t <= blk + b : t >= b * group);
+    __device__ __forceinline__ bool active(int b, int t) const {
+        return b < n && (KIND == kSweep1 ? t <= blk + b : t >= b);
     }
 };
+
+// Column sums of one query head for this warp's 32 keys.  With grouped queries they go to memory, and
+// the query head of the group that arrives last adds the group in head order.
+__device__ __forceinline__ void store_scores(const TileParams& p, int head, int tile, int quarter, int tok, bool mine, float a) {
+    if (p.group == 1) {
+        if (mine) p.scores[(long long)head * p.T + tok] = a;
+        return;
+    }
+    const int kvh = head / p.group;
+    const long long step = (long long)p.n_kv_heads * p.T;
+    float* part = p.parts2 + (long long)kvh * p.T + tok;             // of the group's first head
+    if (mine) __stcg(part + (head - kvh * p.group) * step, a);
+    __threadfence();
+    __syncwarp();
+    int last = 0;
+    if ((threadIdx.x & 31) == 0)
+        last = atomicAdd(p.arrived + ((long long)tile * p.n_kv_heads + kvh) * 4 + quarter, 1) == p.group - 1;
+    if (!__shfl_sync(0xffffffffu, last, 0) || !mine) return;
+    __threadfence();
+    float sum = __ldcg(part);
+    for (int g = 1; g < p.group; ++g) sum += __ldcg(part + g * step);
+    p.scores[(long long)kvh * p.T + tok] = sum;
+}
 
 template <int KIND, int kBlocks>
 __device__ __forceinline__ MultiItem decode_multi(const TileParams& p, const Req* tbl, int item) {
@@ -827,7 +851,7 @@ __device__ __forceinline__ MultiItem decode_multi(const TileParams& p, const Req
     }
     const Req& rq = tbl[lo];
     const int u = item - rq.item_begin[KIND];
-    const int heads = KIND == kSweep1 ? p.n_q_heads : p.n_kv_heads;
+    const int heads = p.n_q_heads;
     const int n_sets = (rq.nblk + kBlocks - 1) / kBlocks;
     MultiItem it;
     it.tok_begin = rq.tok_begin;
@@ -835,7 +859,8 @@ __device__ __forceinline__ MultiItem decode_multi(const TileParams& p, const Req
     it.blk = kBlocks * (KIND == kSweep1 ? n_sets - 1 - u / heads : u / heads);   // heaviest first
     it.head = u % heads;
     it.n = min(kBlocks, rq.nblk - it.blk);
-    it.nt = KIND == kSweep1 ? it.blk + it.n : (rq.nblk - it.blk) * p.group;
+    it.tile = rq.tile_begin + it.blk;
+    it.nt = KIND == kSweep1 ? it.blk + it.n : rq.nblk - it.blk;
     return it;
 }
 
@@ -906,6 +931,8 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                 const int item = item_of_round(round, blockIdx.x, n_cta);
                 if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; continue; }
                 const MultiItem it = decode_multi<KIND, kBlocks>(p, tbl, item);
+                const int kv_head = it.head / p.group;
+                const int a_head = KIND == kSweep1 ? it.head : kv_head, b_head = KIND == kSweep1 ? kv_head : it.head;
 #pragma unroll
                 for (int half = 0; half < kBlocks; ++half) {
                     if (half >= it.n) break;
@@ -913,24 +940,20 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                     const uint32_t bar = ptx::smem_u32(&sh.a_full[half]), dst = ptx::smem_u32(&sh.a[half][0]);
                     const int row = it.tok_begin + (it.blk + half) * kTile;
                     ptx::mbar_arrive_expect_tx(bar, kTileBytes);
-                    ptx::tma_load_3d(dst, &map_a, 0, it.head, row, bar);
-                    ptx::tma_load_3d(dst + kHalfBytes, &map_a, 64, it.head, row, bar);
+                    ptx::tma_load_3d(dst, &map_a, 0, a_head, row, bar);
+                    ptx::tma_load_3d(dst + kHalfBytes, &map_a, 64, a_head, row, bar);
                     ++na[half];
                 }
-                int ib = it.blk, qs = 0;             // sweep 2: query block and query head of the group
                 for (int t = 0; t < it.nt && !stop; ++t, ++gb) {
                     const int s = gb % kRing;
                     if (!ptx::mbar_wait(ptx::smem_u32(&sh.b_empty[s]), ((gb / kRing) & 1) ^ 1, abort_flag)) { stop = true; break; }
                     const uint32_t bar = ptx::smem_u32(&sh.b_full[s]), dst = ptx::smem_u32(&sh.b[s][0]);
                     ptx::mbar_arrive_expect_tx(bar, KIND == kSweep2 ? kTileBytes + kSplitBytes : kTileBytes);
-                    const int row = it.tok_begin + (KIND == kSweep1 ? t : ib) * kTile;
-                    const int h = KIND == kSweep1 ? it.head / p.group : it.head * p.group + qs;
-                    ptx::tma_load_3d(dst, &map_b, 0, h, row, bar);
-                    ptx::tma_load_3d(dst + kHalfBytes, &map_b, 64, h, row, bar);
-                    if (KIND == kSweep2) {
-                        ptx::tma_load_3d(ptx::smem_u32(&sh.bx[s % Sh::kXStages][0]), &map_x, 0, h, row, bar);
-                        if (++qs == p.group) { qs = 0; ++ib; }
-                    }
+                    const int row = it.tok_begin + (KIND == kSweep1 ? t : it.blk + t) * kTile;
+                    ptx::tma_load_3d(dst, &map_b, 0, b_head, row, bar);
+                    ptx::tma_load_3d(dst + kHalfBytes, &map_b, 64, b_head, row, bar);
+                    if (KIND == kSweep2)
+                        ptx::tma_load_3d(ptx::smem_u32(&sh.bx[s % Sh::kXStages][0]), &map_x, 0, b_head, row, bar);
                 }
             }
             // after an abort: wait for the copies that may not have been consumed (see tile_kernel)
@@ -965,7 +988,7 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                     const uint32_t b_addr = ptx::smem_u32(&sh.b[s][0]);
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
-                        if (!it.template active<KIND>(b0 + half, t, p.group)) continue;
+                        if (!it.template active<KIND>(b0 + half, t)) continue;
                         const int acc = 2 * (int)me + half;
                         if ((!have[half] && !ptx::mbar_wait(ptx::smem_u32(&sh.a_full[b0 + half]), na[half] & 1, abort_flag)) ||
                             !ptx::mbar_wait(ptx::smem_u32(&sh.t_empty[acc]), (used[half] & 1) ^ 1, abort_flag)) {
@@ -1026,7 +1049,7 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             if (half >= it.n) continue;
             const int blk = it.blk + half;
             const int pos = blk * kTile + row;
-            const int t_first = KIND == kSweep2 ? half * p.group : 0;        // active tiles [t_first, t_end)
+            const int t_first = KIND == kSweep2 ? half : 0;        // active tiles [t_first, t_end)
             const int t_end = KIND == kSweep1 ? blk + 1 : it.nt;
             float m_run = -INFINITY, l_run = 0.f;            // sweep 1
             float total = 0.f;                               // sweep 2: sums of whole tiles (short chains of
@@ -1034,8 +1057,6 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             // tiles of this group: all of them, or the first one of its parity and every other one
             constexpr int kStep = kBlocks == 2 ? 2 : 1;
             int t = t_first + (kBlocks == 2 ? (int)(((gb0 + t_first) ^ parity) & 1u) : 0);
-            int ib = 0, qs = 0;                              // sweep 2: query block, head in the group
-            if (KIND == kSweep2) { ib = it.blk + t / p.group; qs = t % p.group; }
             for (; t < t_end; t += kStep, ++used) {
                 ptx::mbar_wait(ptx::smem_u32(&sh.t_full[grp]), used & 1, abort_flag);
                 ptx::tc_fence_after_sync();
@@ -1043,11 +1064,10 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                 int col_limit = kTile, diag_from = 0;
                 if (KIND == kSweep2) {
                     // columns to mask: below the diagonal, and past the end of the request
+                    const int ib = it.blk + t;
                     col_limit = min(kTile, it.L - ib * kTile);
                     diag = ib == blk || col_limit < kTile;
                     diag_from = ib == blk ? row : 0;
-                    qs += kStep;
-                    while (qs >= p.group) { qs -= p.group; ++ib; }
                 }
                 float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
@@ -1071,10 +1091,9 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                 if (KIND == kSweep2) total += (acc[0] + acc[1]) + (acc[2] + acc[3]);
             }
             if (kBlocks == 4) {                              // nobody else worked on the block
-                if (pos < it.L && !*abort_flag) {
-                    if (KIND == kSweep1) store_lse(p, it.head, it.tok_begin + pos, m_run, l_run);
-                    else p.scores[(long long)it.head * p.T + it.tok_begin + pos] = total;
-                }
+                const bool mine = pos < it.L && !*abort_flag;
+                if (KIND == kSweep2) store_scores(p, it.head, it.tile + half, quarter, it.tok_begin + pos, mine, total);
+                else if (mine) store_lse(p, it.head, it.tok_begin + pos, m_run, l_run);
                 continue;
             }
             // ---- combine the block's two groups: the one with its last tile finishes last ----
@@ -1091,18 +1110,17 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.comb_full[half & 1][buf]));
             } else {
                 ptx::mbar_wait(ptx::smem_u32(&sh.comb_full[half & 1][buf]), use & 1u, abort_flag);
-                if (pos < it.L && !*abort_flag) {
-                    if (KIND == kSweep1) {
-                        const float m1 = cb[0][row], l1 = cb[kP1][row];
-                        const float m = fmaxf(m_run, m1);
-                        const float l = l_run * ptx::ex2((m_run - m) * c2) + l1 * ptx::ex2((m1 - m) * c2);
-                        store_lse(p, it.head, it.tok_begin + pos, m, l);
-                    } else {
-                        p.scores[(long long)it.head * p.T + it.tok_begin + pos] = total + cb[0][row];
-                    }
+                const bool mine = pos < it.L && !*abort_flag;
+                const float other = KIND == kSweep2 ? cb[0][row] : 0.f;
+                if (KIND == kSweep1 && mine) {
+                    const float m1 = cb[0][row], l1 = cb[kP1][row];
+                    const float m = fmaxf(m_run, m1);
+                    const float l = l_run * ptx::ex2((m_run - m) * c2) + l1 * ptx::ex2((m1 - m) * c2);
+                    store_lse(p, it.head, it.tok_begin + pos, m, l);
                 }
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.comb_free[half & 1][buf]));
+                if (KIND == kSweep2) store_scores(p, it.head, it.tile + half, quarter, it.tok_begin + pos, mine, total + other);
             }
         }
     }
