@@ -370,6 +370,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     if (!lse_is_input) {
         p.n_items = pl.n_items[kSweep1];
         p.blocks = pl.blocks[0];
+        p.next_item = p.status + 16 + kSweep1;
         p.splits = pl.splits[0];
         p.parts1 = at<float2>(ws, pl.o_parts1);
         p.arrived = p.status + 64;
@@ -382,6 +383,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     mark_stage(1, st);
     p.n_items = pl.n_items[kSweep2];
     p.blocks = pl.blocks[1];
+    p.next_item = p.status + 16 + kSweep2;
     p.splits = pl.splits[1];
     p.parts2 = at<float>(ws, pl.o_parts2);
     p.arrived = p.status + 64 + pl.n_arrived[0];

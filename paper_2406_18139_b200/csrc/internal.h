@@ -78,6 +78,7 @@ struct TileParams {
     float2* parts1;              // [splits][n_q_heads, T]  reference and sum of a range (sweep 1)
     float* parts2;               // [splits][n_kv_heads, T] column sums of a range, or of a query head of the
                                  // group (sweep 2)
+    int* next_item;              // items taken beyond the CTAs' first ones (multi_kernel; zeroed)
     int* arrived;                // [block][heads][4] finished ranges per 32 rows (zeroed)
     const int* evict_idx;        // evicted-list layout  (match: rows of the stationary tiles)
     const void* k_rows;          // K [tokens, heads, 128] bf16 with the strides below (match)
