@@ -39,6 +39,8 @@ struct Plan {
     // workspace offsets (bytes)
     int splits[2] = {1, 1};                 // ranges of a sweep 1 / sweep 2 item's streamed tiles
     int blocks[2] = {1, 1};                 // blocks per sweep item
+    int tail_sets[2] = {0, 0};              // several blocks per item: shortest sets that every request keeps
+    int tail_begin[2] = {0, 0};             // for the end, and the first item of these
     size_t n_arrived[2] = {0, 0};           // their arrival counters
     size_t clear_words = 64;                // status word and arrival counters
     size_t o_parts1 = 0, o_parts2 = 0;
@@ -50,13 +52,22 @@ struct Plan {
 struct DeviceInfo { int sms = 0; int cc_major = 0; bool ok = false; };
 int device_info(DeviceInfo& out);
 
-// Items of two blocks need three per SM to be shared evenly, items of four six (two: 2048 tokens x 8
-// heads, 64 items: 66 us a layer with single blocks, 85 with pairs; four: 8192 x 32 heads, 512 items:
-// 807-833 us with pairs, 844-885 with four).  Grouped query heads count one by one, in sweep 2 as well:
-// 7777 tokens x 32 query heads on 8, sweep 2 alone, 392 us a layer with single blocks for whole groups,
-// 378 with pairs for single query heads.
-constexpr long long kPairItemsPerSm = 3;
-constexpr long long kQuadItemsPerSm = 6;
+// Items of two blocks need two and a half per SM to be shared evenly, items of four four, and six if the
+// prompts differ in length.  Scores in us, single blocks | pairs: 2600 tokens x 32 heads (2.3
+// pairs per SM) 93.5 | 96, 2850 x 32 query on 8 KV heads (2.49) 110 | 115, 3000 x 32 on 8 (2.6) 124 | 118,
+// a layer of 2048 x 8 (0.4) 66 | 85; pairs | fours: 9000 x 32 (3.8 fours per SM) 834 | 832, 10000 x 32
+// (4.3) 1017 | 1007, 9000 x 40 (4.8) 1046 | 1022, 8192 x 64 (6.9) 1415 | 1363; of several lengths: two
+// prompts of 10000 to 14000 x 16 (5.0) 1357 | 1376, four of 1000 to 12000 x 32 on 8 (8) 3350 | 3260.
+// Grouped query heads count one by one, in sweep 2 as well: 7777 tokens x 32 query heads on 8, a layer 392
+// us with single blocks for whole groups in sweep 2, 378 with pairs for single query heads.
+constexpr long long kPairBlocksPerSm = 5;
+constexpr long long kQuadItemsPerSm = 4, kRaggedQuadItemsPerSm = 6;
+// The kTailSets shortest items of all prompts come last: with each prompt's items in a row the last
+// prompt's longest ones would end the sweep.  Scores of eight prompts of 4000 to 6000 tokens x 16 heads
+// (8.6 items per SM) 1122 -> 1094 us, four of 1000 to 12000 x 8 603 -> 590, three of 2000 to 3000 x 32 291 ->
+// 285.  Neighbouring CTAs then share no tiles in L2, which costs more where there are many items: 16 prompts
+// of 1000 to 3000 x 32 (14 per SM) 937 -> 944.
+constexpr int kTailSets = 6, kTailItemsPerSm = 12;
 // Splits of the sweep items: as many as bring the longest item down to what an SM has on average, if it
 // is more than one and a half times that and ten tiles longer.  Both sweeps together, us: 5000 tokens
 // with 2 heads 63.5 -> 38, 12000 with 2 query on 1 KV head 188 -> 110, 2048 with 32 on 8 78 -> 63, 700
@@ -65,16 +76,19 @@ constexpr long long kQuadItemsPerSm = 6;
 void plan_splits(Plan& pl) {
     DeviceInfo di;
     const long long sms = (device_info(di) == LOOKM_OK && di.sms > 0) ? di.sms : 148;
-    long long tiles = 0;
-    for (const Req& q : pl.reqs) tiles += (long long)q.nblk * (q.nblk + 1) / 2;
+    long long tiles = 0, blocks = 0;
+    for (const Req& q : pl.reqs) {
+        tiles += (long long)q.nblk * (q.nblk + 1) / 2;
+        blocks += (long long)q.nblk * pl.n_q_heads;
+    }
     const long long mean = std::max<long long>(1, tiles * pl.n_q_heads / sms);
     for (int s = 0; s < 2; ++s) {
         const long long longest = (long long)pl.reqs[0].nblk * (s ? pl.group : 1);
-        for (int b : {2, 4}) {
-            long long items = 0;
-            for (const Req& q : pl.reqs) items += (long long)((q.nblk + b - 1) / b) * pl.n_q_heads;
-            if (items >= (b == 2 ? kPairItemsPerSm : kQuadItemsPerSm) * sms) pl.blocks[s] = b;
-        }
+        const long long quad = pl.reqs[0].nblk == pl.reqs.back().nblk ? kQuadItemsPerSm : kRaggedQuadItemsPerSm;
+        if (blocks >= kPairBlocksPerSm * sms) pl.blocks[s] = 2;
+        if (blocks >= 4 * quad * sms) pl.blocks[s] = 4;
+        if (pl.blocks[s] > 1 && blocks < kTailItemsPerSm * pl.blocks[s] * sms)
+            pl.tail_sets[s] = std::min(kTailSets, (pl.reqs.back().nblk + pl.blocks[s] - 1) / pl.blocks[s]);
         if (pl.blocks[s] == 1 && 2 * longest > 3 * mean && longest >= mean + 10)
             pl.splits[s] = (int)std::min<long long>(kMaxSplits, (longest + mean - 1) / mean);
     }
@@ -166,16 +180,19 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
         const bool merges = q.mode != LOOKM_MERGE_NONE;
         const long long n_units = merges ? (q.L + unit_entries - 1) / unit_entries : 0;
         units += (long long)pl.n_kv_heads * n_units;
-        it0 += (long long)((q.nblk + pl.blocks[0] - 1) / pl.blocks[0]) * pl.n_q_heads * pl.splits[0];
+        it0 += (long long)((q.nblk + pl.blocks[0] - 1) / pl.blocks[0] - pl.tail_sets[0]) * pl.n_q_heads * pl.splits[0];
         // (several blocks per item: the query heads of a group are items of their own in sweep 2 too)
-        it1 += (long long)((q.nblk + pl.blocks[1] - 1) / pl.blocks[1]) * (pl.blocks[1] > 1 ? pl.n_q_heads : pl.n_kv_heads) * pl.splits[1];
+        it1 += (long long)((q.nblk + pl.blocks[1] - 1) / pl.blocks[1] - pl.tail_sets[1]) *
+               (pl.blocks[1] > 1 ? pl.n_q_heads : pl.n_kv_heads) * pl.splits[1];
         // match items: blocks of 128 entries of every head's evicted list
         it2 += (q.E > 0 && merges) ? (long long)((q.E + kTile - 1) / kTile) * pl.n_kv_heads : 0;
         slots += (long long)q.B * pl.n_kv_heads;
     }
     pl.total_units = units;
-    pl.n_items[kSweep1] = (int)it0;
-    pl.n_items[kSweep2] = (int)it1;
+    pl.tail_begin[0] = (int)it0;
+    pl.tail_begin[1] = (int)it1;
+    pl.n_items[kSweep1] = (int)(it0 + (long long)pl.tail_sets[0] * n_req * pl.n_q_heads);
+    pl.n_items[kSweep2] = (int)(it1 + (long long)pl.tail_sets[1] * n_req * pl.n_q_heads);
     pl.n_items[kMatch] = (int)it2;
 
     size_t o = 0;
@@ -371,6 +388,8 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
         p.n_items = pl.n_items[kSweep1];
         p.blocks = pl.blocks[0];
         p.next_item = p.status + 16 + kSweep1;
+        p.tail_begin = pl.tail_begin[0];
+        p.tail_sets = pl.tail_sets[0];
         p.splits = pl.splits[0];
         p.parts1 = at<float2>(ws, pl.o_parts1);
         p.arrived = p.status + 64;
@@ -384,6 +403,8 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     p.n_items = pl.n_items[kSweep2];
     p.blocks = pl.blocks[1];
     p.next_item = p.status + 16 + kSweep2;
+    p.tail_begin = pl.tail_begin[1];
+    p.tail_sets = pl.tail_sets[1];
     p.splits = pl.splits[1];
     p.parts2 = at<float>(ws, pl.o_parts2);
     p.arrived = p.status + 64 + pl.n_arrived[0];

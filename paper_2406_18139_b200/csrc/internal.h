@@ -78,6 +78,7 @@ struct TileParams {
     float2* parts1;              // [splits][n_q_heads, T]  reference and sum of a range (sweep 1)
     float* parts2;               // [splits][n_kv_heads, T] column sums of a range, or of a query head of the
                                  // group (sweep 2)
+    int tail_begin, tail_sets;   // multi_kernel: the last items are the shortest tail_sets sets of all requests
     int* next_item;              // items taken beyond the CTAs' first ones (multi_kernel; zeroed)
     int* arrived;                // [block][heads][4] finished ranges per 32 rows (zeroed)
     const int* evict_idx;        // evicted-list layout  (match: rows of the stationary tiles)

@@ -778,7 +778,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 // goes into moving tiles from L2 (a build without the loads ran 9-11 % faster).  Whole layers in a row,
 // one block per item -> two -> four: 16384 tokens x 40 heads 4.45 -> 4.10 -> 3.92 ms, 32768 x 32 query
 // heads on 8 11.2 -> 10.6 -> 10.4 ms, 16 ragged prompts x 32 heads 24.4 -> 23.4 -> 22.5 ms, 8192 x 32
-// 0.918 -> 0.886 (four blocks, 3.5 items per SM: 0.93).
+// 0.918 -> 0.886 (four blocks: 0.93).
 // Two blocks: streamed tile g of the CTA goes to accumulators 2 (g mod 2) + block, and each accumulator
 // has one issuing thread (g mod 2) and one epilogue group, which works on one block and on the tiles of
 // one parity; the two groups of a block are combined at the item's end like the four of tile_kernel.
@@ -789,8 +789,8 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 // Prompts of different lengths come out uneven from a fixed deal (three prompts of 4655, 4945 and 1831
 // tokens x 32 heads: the fullest CTA 1.17 times the average): their scores took 597 us and take 567,
 // the batch of 16 prompts 22.7 -> 22.0 ms, 8192 x 32 901 -> 889 us.  Which CTA takes an item changes no
-// result: a block's tiles are added in their order,
-// two blocks per item in the two parities of the tile's index in the item.
+// result: a block's tiles are added in their order, two blocks per item in the two parities of the
+// tile's index in the item.
 // ------------------------------------------------------------------------------------------------
 template <int KIND, int kBlocks>
 struct __align__(1024) MultiShared {
@@ -854,20 +854,29 @@ __device__ __forceinline__ void store_scores(const TileParams& p, int head, int 
 
 template <int KIND, int kBlocks>
 __device__ __forceinline__ MultiItem decode_multi(const TileParams& p, const Req* tbl, int item) {
-    int lo = 0, hi = p.n_req - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (tbl[mid].item_begin[KIND] <= item) lo = mid; else hi = mid - 1;
-    }
-    const Req& rq = tbl[lo];
-    const int u = item - rq.item_begin[KIND];
+    // index of the set of kBlocks blocks among the request's, by length (0: the longest)
     const int heads = p.n_q_heads;
+    int r, set;
+    if (item < p.tail_begin) {
+        int lo = 0, hi = p.n_req - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (tbl[mid].item_begin[KIND] <= item) lo = mid; else hi = mid - 1;
+        }
+        r = lo;
+        set = (item - tbl[r].item_begin[KIND]) / heads;
+    } else {
+        const int v = (item - p.tail_begin) / heads;                          // [set][request]
+        r = v % p.n_req;
+        set = (tbl[r].nblk + kBlocks - 1) / kBlocks - p.tail_sets + v / p.n_req;
+    }
+    const Req& rq = tbl[r];
     const int n_sets = (rq.nblk + kBlocks - 1) / kBlocks;
     MultiItem it;
     it.tok_begin = rq.tok_begin;
     it.L = rq.L;
-    it.blk = kBlocks * (KIND == kSweep1 ? n_sets - 1 - u / heads : u / heads);   // heaviest first
-    it.head = u % heads;
+    it.blk = kBlocks * (KIND == kSweep1 ? n_sets - 1 - set : set);
+    it.head = item % heads;          // (the items of a request, and those of the tail, begin at a multiple of it)
     it.n = min(kBlocks, rq.nblk - it.blk);
     it.tile = rq.tile_begin + it.blk;
     it.nt = KIND == kSweep1 ? it.blk + it.n : rq.nblk - it.blk;

@@ -133,10 +133,11 @@ def test_scores_of_items_cut_into_ranges(B, lens, Hq, Hkv):
 
 
 @pytest.mark.parametrize("lens,Hq,Hkv", [([1665], 64, 64), ([1664], 64, 64), ([1500, 129, 1, 800, 128], 72, 24), ([200] * 16, 32, 16),
-                                         ([600, 513, 512, 640, 1, 129, 300, 900], 96, 96), ([1300, 1300, 770], 192, 48)])
+                                         ([600, 513, 512, 640, 1, 129, 300, 900], 96, 96), ([1300, 1300, 770], 192, 48), ([2000, 1700], 40, 8),
+                                         ([600, 513, 512, 640, 1, 129, 300, 900], 128, 128)])
 def test_scores_of_items_of_two_or_four_blocks(B, lens, Hq, Hkv):
-    """Enough heads for items of two blocks (in sweep 1 alone with 24 KV heads) or four (96 and 192 query
-    heads): one to four blocks in the last item of a prompt, requests of one block, a last block of one
+    """Enough heads for items of two blocks (in sweep 1 alone with 24 KV heads) or four (128 and 192
+    query heads): one to four blocks in the last item of a prompt, requests of one block, a last block of one
     row; logits rise along the prompts."""
     import torch
     T = sum(lens)
