@@ -451,6 +451,10 @@ int run_match(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     return LOOKM_OK;
 }
 
+// The inversion's CTAs (kInvMaxCluster at most per request and head) fill the SMs twice at most, and each
+// gets kInvMinShare evicted tokens at least.
+constexpr long long kInvCtasPerSm = 2;
+constexpr int kInvMinShare = 512;
 int run_merge(const Plan& pl, const lookm_layout* lay, const void* k, const void* v,
               const int* kept_idx, const int* evict_idx, const int* assign, const float* sim,
               int varlen_output, void* out_k, void* out_v, void* ws, cudaStream_t st) {
@@ -466,7 +470,13 @@ int run_merge(const Plan& pl, const lookm_layout* lay, const void* k, const void
             invert_digits(r.B, wide ? kInvDigitBits32 : kInvDigitBits16, n_pass, dbits);
             digit_bits = std::max(digit_bits, dbits);
         }
-        LOOKM_CUDA(launch_invert_assignment(assign, kept_idx, evict_idx, sim, reqs, pl.n_req, pl.n_kv_heads,
+        DeviceInfo di;
+        LOOKM_TRY(device_info(di));
+        int ctas = 1;                            // per (request, head)
+        while (ctas < kInvMaxCluster && 2ll * ctas * pl.n_kv_heads * pl.n_req <= kInvCtasPerSm * di.sms &&
+               pl.max_E >= 2 * ctas * kInvMinShare)
+            ctas *= 2;
+        LOOKM_CUDA(launch_invert_assignment(assign, kept_idx, evict_idx, sim, reqs, pl.n_req, pl.n_kv_heads, ctas,
                                             pl.T, wide, digit_bits, at<int>(ws, pl.o_row_ptr), at<int>(ws, pl.o_members),
                                             at<float>(ws, pl.o_member_w), at<int4>(ws, pl.o_units),
                                             at<int>(ws, pl.o_slot_cnt), at<unsigned>(ws, pl.o_sort_a),

@@ -22,6 +22,7 @@
 #include <math.h>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace lookm {
 namespace {
@@ -59,23 +60,7 @@ __device__ __forceinline__ float dec_ex2(float x) {
 // Clusters: for short caches all splits of a (request, KV head, pass) are the CTAs of one thread-block
 // cluster, which add their results through distributed shared memory, so that no second kernel and no
 // partial results in memory are needed.
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// a float of this CTA's shared memory, in CTA `rank` of the cluster
-__device__ __forceinline__ float ld_cluster(const float* p, uint32_t rank) {
-    uint32_t at;
-    float v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(at) : "memory");
-    return v;
-}
+
 // What a CTA leaves for the cluster: per query head of the pass reference, sum and weighted V sum.
 template <int GP>
 struct ClusterShared {
@@ -86,10 +71,10 @@ struct ClusterShared {
 // heads.  `unit`: factor that turns references into log2.
 template <int GP>
 __device__ __forceinline__ void cluster_combine(const ClusterShared<GP>& cs, int n, int gt, float unit, float* out) {
-    cluster_sync();
+    ptx::cluster_sync();
     const int share = kHeadDim / n;
     for (int i = threadIdx.x; i < gt * share; i += blockDim.x) {
-        const int g = i / share, t = (int)cluster_rank() * share + i % share;
+        const int g = i / share, t = (int)ptx::cluster_rank() * share + i % share;
         float m[kDecodeMaxCluster], l[kDecodeMaxCluster], o[kDecodeMaxCluster];
         float mx = -INFINITY;
 #pragma unroll
@@ -97,9 +82,9 @@ __device__ __forceinline__ void cluster_combine(const ClusterShared<GP>& cs, int
             m[c] = -INFINITY;
             l[c] = o[c] = 0.f;
             if (c < n) {
-                m[c] = ld_cluster(&cs.m[g], c);
-                l[c] = ld_cluster(&cs.l[g], c);
-                o[c] = ld_cluster(&cs.o[g][t], c);
+                m[c] = ptx::ld_cluster(&cs.m[g], c);
+                l[c] = ptx::ld_cluster(&cs.l[g], c);
+                o[c] = ptx::ld_cluster(&cs.o[g][t], c);
             }
         }
 #pragma unroll
@@ -113,7 +98,7 @@ __device__ __forceinline__ void cluster_combine(const ClusterShared<GP>& cs, int
         }
         out[(long long)g * kHeadDim + t] = osum / lsum;
     }
-    cluster_sync();                                  // nobody leaves while its shared memory is read
+    ptx::cluster_sync();                                  // nobody leaves while its shared memory is read
 }
 
 template <int GT>

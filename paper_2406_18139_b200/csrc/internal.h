@@ -21,6 +21,7 @@ constexpr int kMaxUnitEntries = LOOKM_MAX_UNIT_ENTRIES;   // most rows in one
 // is sorted in one pass).  16-bit counters allow 11-bit digits, 32-bit counters 10-bit ones.
 constexpr int kInvDigitBits16 = 11;
 constexpr int kInvDigitBits32 = 10;
+constexpr int kInvMaxCluster = 8;
 constexpr int kInvWideCountsAbove = 65535;   // evicted tokens per head beyond which counts need 32 bits
 #ifdef __CUDACC__
 __host__ __device__
@@ -130,7 +131,7 @@ struct ReqChunk { Req r[kReqChunk]; };
 cudaError_t launch_write_table(const ReqChunk& chunk, int count, Req* dst, int* clear, size_t n_clear, cudaStream_t stream);
 
 cudaError_t launch_invert_assignment(const int* assign, const int* kept_idx, const int* evict_idx,
-                                     const float* sim, const Req* reqs, int n_req, int n_kv_heads,
+                                     const float* sim, const Req* reqs, int n_req, int n_kv_heads, int ctas,
                                      long long T, bool wide_counts, int digit_bits, int* row_ptr,
                                      int* ent_pos, float* ent_w, int4* unit_first, int* slot_cnt,
                                      unsigned* sort_a, unsigned* sort_b, int* status,

@@ -7,6 +7,7 @@
 #include <cuda_bf16.h>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace lookm {
 namespace {
@@ -156,31 +157,39 @@ argmax_rows_kernel(const float* __restrict__ sim_matrix, const Req* __restrict__
 // ---------------------------------------------------------------------------------------------
 // Inversion of the assignment: for each (request, head) a stable sort of the evicted ranks by
 // their kept slot gives, per kept row, its members in ascending position, as CSR
-// (row_ptr [B + 1 per (request, head)], member positions and weights [E]).  One CTA per (request, head); stable LSD
-// radix sort with 8-bit digits: every warp owns a contiguous segment of the list, ranks equal
-// digits inside a 32-element step with match.any, and adds the counts of earlier steps and
-// earlier warps.  Keys are packed as (slot << 0) in one array and values in the other.
+// (row_ptr [B + 1 per (request, head)], member positions and weights [E]).  A cluster of CTAs per
+// (request, head); stable LSD radix sort: every warp of the cluster owns a contiguous segment of the
+// list, ranks equal digits inside a 32-element step with ballots, and adds the counts of earlier steps,
+// of earlier warps and, read from their shared memory, of earlier CTAs.
+// What bounds it is the chain of dependent steps, not the bytes: a list of 26214 evicted tokens is 100
+// KB.  One CTA of 32 warps per list -> up to eight of 16: 26214 evicted tokens x 8 heads into 6554 slots
+// 164 -> 43 us, 13107 x 40 into 3277 92 -> 46, 7388 x 8 into 389 22 -> 16.
 // ---------------------------------------------------------------------------------------------
-constexpr int kInvThreads = 1024;
+constexpr int kInvThreads = 512;
+constexpr int kInvWarps = kInvThreads / 32;
+constexpr int kInvBatch = 8;                         // loop steps whose loads are issued together
 
 // Second half of the entry list: the kept rows (flagged with the sign bit, weight = member count),
 // for every work unit (unit u of a head covers the entries [u * unit_entries, (u + 1) * unit_entries))
 // the slot its first entry belongs to, with that slot's first entry and member count, and a
-// cleared arrival counter per slot.
-__device__ __forceinline__ void write_kept_entries(const Req& rq, int h, int n_kv_heads, int B, const int* rp,
+// cleared arrival counter per slot.  row_begin(c): members of the slots before c.  For the slots
+// c0, c0 + step, ...
+template <typename RowBegin>
+__device__ __forceinline__ void write_kept_entries(const Req& rq, int h, int n_kv_heads, int c0, int step, RowBegin row_begin,
                                                    const int* kept_idx_head, int* ent, float* entw,
                                                    int4* unit_first, int* slot_cnt, int* status) {
     const int ue = rq.unit_entries;
-    for (int c = threadIdx.x; c < B; c += blockDim.x) {
+    for (int c = c0; c < rq.B; c += step) {
         int pc = kept_idx_head[c];
         if (pc < 0 || pc >= rq.L) { atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); pc = 0; }
-        const int s_c = c + rp[c];                       // entry of the kept row
-        const int s_next = c + 1 + rp[c + 1];            // entry of the next kept row (L after the last)
+        const int begin = row_begin(c), n = row_begin(c + 1) - begin;
+        const int s_c = c + begin;                       // entry of the kept row
+        const int s_next = s_c + n + 1;                  // entry of the next kept row (L after the last)
         ent[s_c] = pc | (int)0x80000000;
-        entw[s_c] = (float)(rp[c + 1] - rp[c]);
+        entw[s_c] = (float)n;
         slot_cnt[c] = 0;
         for (int u = (s_c + ue - 1) / ue; u * ue < s_next; ++u)
-            unit_first[(long long)u * n_kv_heads + h] = make_int4(c, s_c, rp[c + 1] - rp[c], 0);
+            unit_first[(long long)u * n_kv_heads + h] = make_int4(c, s_c, n, 0);
     }
 }
 
@@ -199,31 +208,32 @@ __device__ __forceinline__ unsigned same_digit_lanes(unsigned d, bool valid, int
     return peers;
 }
 
-constexpr int kInvBatch = 8;                         // loop steps whose loads are issued together
-
 // CountT / kMaxBits: 16-bit counters with digits of up to 11 bits when no request of the call evicts
 // more than 65535 tokens per head (every count and prefix then fits), else 32-bit counters with
-// digits of up to 10 bits; either way at most 136 KB of counters per CTA.
+// digits of up to 10 bits.
 template <typename CountT, int kMaxBits>
-__global__ void __launch_bounds__(kInvThreads)
+__global__ void __launch_bounds__(kInvThreads, 2)
 invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__ kept_idx,
                          const int* __restrict__ evict_idx,
                          const float* __restrict__ sim, const Req* __restrict__ reqs,
-                         int n_kv_heads, long long T, int* __restrict__ row_ptr,
+                         int n_kv_heads, int ctas, long long T, int* row_ptr,
                          int* __restrict__ ent_pos, float* __restrict__ ent_w,
                          int4* __restrict__ unit_first, int* __restrict__ slot_cnt,
-                         unsigned* __restrict__ sort_a, unsigned* __restrict__ sort_b, int* status) {
+                         unsigned* sort_a, unsigned* sort_b, int* status) {
+    static_assert((1 << kMaxBits) <= 4 * kInvThreads, "a thread scans four digits");
     extern __shared__ __align__(16) unsigned char inv_smem[];
-    __shared__ int warp_sums[32];
+    __shared__ int warp_sums[kInvWarps];
     grid_dependency_wait();
     const Req rq = reqs[blockIdx.y];
     if (rq.mode == LOOKM_MERGE_NONE) return;             // its kept rows are copied, nothing is merged
-    const int h = blockIdx.x;
+    const int h = blockIdx.x / ctas, cta = blockIdx.x % ctas;     // the cluster: the CTAs of one head
     const int E = rq.E, B = rq.B;
     const long long ev_base = rq.ev_off + (long long)h * E;
     int* rp = row_ptr + rq.rp_off + (long long)h * (B + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
+    const int thread = cta * kInvThreads + threadIdx.x, n_threads = ctas * kInvThreads;   // of the cluster
+    auto sync = [&]() { if (ctas > 1) ptx::cluster_sync(); else __syncthreads(); };
 
     // entry list of this (request, head): for every kept slot its kept row, then its members
     int* ent = ent_pos + (long long)h * T + rq.tok_begin;
@@ -233,87 +243,118 @@ invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__
     const int* kept_idx_head = kept_idx + rq.kept_off + (long long)h * B;
     const bool weighted = (rq.mode == LOOKM_MERGE_WEIGHTED);
     if (E == 0) {
-        for (int c = threadIdx.x; c <= B; c += kInvThreads) rp[c] = 0;
-        __syncthreads();
-        write_kept_entries(rq, h, n_kv_heads, B, rp, kept_idx_head, ent, entw, units, cnts, status);
+        for (int c = thread; c <= B; c += n_threads) rp[c] = 0;
+        write_kept_entries(rq, h, n_kv_heads, thread, n_threads, [](int) { return 0; }, kept_idx_head, ent, entw, units, cnts, status);
         return;
     }
     // segment of the list owned by each warp: a multiple of 32 elements
-    const int seg = ((E + 32 * 32 - 1) / (32 * 32)) * 32;
-    const int s_begin = min(E, warp * seg), s_end = min(E, s_begin + seg);
+    const int n_warps = ctas * kInvWarps;
+    const int seg = ((E + n_warps * 32 - 1) / (n_warps * 32)) * 32;
+    const int s_begin = (int)min((long long)E, (long long)(cta * kInvWarps + warp) * seg), s_end = min(E, s_begin + seg);
 
     int n_pass, dbits;
     invert_digits(B, kMaxBits, n_pass, dbits);
     const int nd = 1 << dbits;
     const unsigned dmask = (unsigned)nd - 1u;
+    const int padded = max(nd, 4);
     CountT* cnt = reinterpret_cast<CountT*>(inv_smem);                          // [warp][digit]
-    int* digit_tot = reinterpret_cast<int*>(inv_smem + (size_t)32 * nd * sizeof(CountT));
-    const bool single = (n_pass == 1);
-    // One pass over a segment of at most kInvBatch steps per warp: the count phase already knows
-    // every element's rank among the equal slots of its warp, so the scatter phase needs neither
-    // the ballots nor the running counts again.
-    const bool keep_ranks = single && seg <= 32 * kInvBatch;
+    int* digit_tot = reinterpret_cast<int*>(inv_smem + (size_t)kInvWarps * padded * sizeof(CountT));   // of this CTA
+    int* digit_begin = digit_tot + padded;               // elements with a smaller digit
+    int* digit_off = digit_begin + padded;               // ... and those with the digit in earlier CTAs
+    // A segment of at most kInvBatch steps stays in registers: the count phase then also knows every
+    // element's rank among the equal digits of its warp, so the scatter phase needs neither the
+    // ballots nor the running counts again.
+    const bool keep = seg <= 32 * kInvBatch;
+    unsigned key[kInvBatch], val[kInvBatch];
     int local_rank[kInvBatch];
-#pragma unroll
-    for (int q = 0; q < kInvBatch; ++q) local_rank[q] = 0;
 
-    // pass p reads (key, value) from src and writes to dst; pass 0 reads assign directly.  With a
-    // single pass the sorted position is final, and the entries are written straight away.
+    // pass p reads (key, value) from src and writes to dst; pass 0 reads assign directly.  The position
+    // in the last pass is final, and the member entries are written straight away.
     unsigned* key_buf[2] = {sort_a + 2 * ev_base, sort_b + 2 * ev_base};   // [E keys][E values] each
     for (int pass = 0; pass < n_pass; ++pass) {
         const int shift = pass * dbits;
+        const bool last = pass == n_pass - 1;
         const unsigned* src_k = pass ? key_buf[(pass - 1) & 1] : nullptr;
         const unsigned* src_v = pass ? key_buf[(pass - 1) & 1] + E : nullptr;
         unsigned* dst_k = key_buf[pass & 1];
         unsigned* dst_v = key_buf[pass & 1] + E;
-        for (int i = threadIdx.x; i < (int)(32 * sizeof(CountT) / 4) * nd; i += kInvThreads)
-            reinterpret_cast<unsigned*>(cnt)[i] = 0u;
-        __syncthreads();
-        // count (the loads of kInvBatch steps are issued together: the loop is bound by their latency)
-        for (int b0 = s_begin; b0 < s_end; b0 += 32 * kInvBatch) {
-            unsigned key[kInvBatch];
+        auto load = [&](int b0) {                        // loads of kInvBatch steps together
 #pragma unroll
             for (int q = 0; q < kInvBatch; ++q) {
                 const int i = b0 + q * 32 + lane;
                 key[q] = 0u;
-                if (i < s_end) key[q] = pass ? src_k[i] : (unsigned)assign[ev_base + i];
+                val[q] = (unsigned)i;
+                if (i < s_end) {
+                    if (pass) { key[q] = __ldcg(src_k + i); val[q] = __ldcg(src_v + i); }
+                    else key[q] = (unsigned)assign[ev_base + i];
+                }
             }
+            if (pass) return;
 #pragma unroll
             for (int q = 0; q < kInvBatch; ++q) {
-                const int i = b0 + q * 32 + lane;
-                const bool valid = i < s_end;
-                if (valid && !pass && key[q] >= (unsigned)B) {
-                    atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX);
-                    key[q] = 0u;
-                }
-                const unsigned d = (key[q] >> shift) & dmask;
-                const unsigned peers = same_digit_lanes(d, valid, dbits);
-                if (keep_ranks) {
-                    local_rank[q] = valid ? (int)cnt[warp * nd + d] + __popc(peers & lt_mask) : 0;
-                    __syncwarp();
-                }
-                if (valid && (peers & lt_mask) == 0u) cnt[warp * nd + d] += (CountT)__popc(peers);
-                __syncwarp();
+                if (key[q] < (unsigned)B) continue;
+                atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX);
+                key[q] = 0u;
             }
+        };
+        // rank among the elements of the warp's segment with the same digit, which it counts
+        auto rank_in_warp = [&](unsigned d, bool valid) {
+            const unsigned peers = same_digit_lanes(d, valid, dbits);
+            const int r = valid ? (int)cnt[warp * nd + d] + __popc(peers & lt_mask) : 0;
+            __syncwarp();
+            if (valid && (peers & lt_mask) == 0u) cnt[warp * nd + d] += (CountT)__popc(peers);
+            __syncwarp();
+            return r;
+        };
+        if (keep) load(s_begin);
+        for (int i = threadIdx.x; i < (int)(kInvWarps * sizeof(CountT)) * padded / 16; i += kInvThreads)
+            reinterpret_cast<uint4*>(cnt)[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        for (int b0 = s_begin; b0 < s_end; b0 += 32 * kInvBatch) {
+            if (!keep) load(b0);
+#pragma unroll
+            for (int q = 0; q < kInvBatch; ++q)
+                if (b0 + q * 32 < s_end) local_rank[q] = rank_in_warp((key[q] >> shift) & dmask, b0 + q * 32 + lane < s_end);
         }
         __syncthreads();
-        // exclusive scan over (digit major, warp minor): first over the warps of every digit ...
-        for (int d = threadIdx.x; d < nd; d += kInvThreads) {
-            int tot = 0;
-            for (int w = 0; w < 32; ++w) {
-                const int c = cnt[w * nd + d];
-                cnt[w * nd + d] = (CountT)tot;
-                tot += c;
-            }
-            digit_tot[d] = tot;
-        }
-        __syncthreads();
-        // ... then over the digit totals (two digits per thread; nd <= 2 * kInvThreads)
+        // exclusive scan over (digit major, warp minor): first over the warps, one 32-bit word of counts
+        // at a time (two 16-bit sums stay apart) ...
         {
-            const int d0 = 2 * threadIdx.x;
-            const int a = d0 < nd ? digit_tot[d0] : 0;
-            const int b = d0 + 1 < nd ? digit_tot[d0 + 1] : 0;
-            int incl = a + b;
+            constexpr int kPer = 4 / (int)sizeof(CountT);
+            const int words = nd / kPer;
+            unsigned* cw = reinterpret_cast<unsigned*>(cnt);
+            for (int i = threadIdx.x; i < words; i += kInvThreads) {
+                unsigned c[kInvWarps], tot = 0u;
+#pragma unroll
+                for (int w = 0; w < kInvWarps; ++w) c[w] = cw[w * words + i];
+#pragma unroll
+                for (int w = 0; w < kInvWarps; ++w) { cw[w * words + i] = tot; tot += c[w]; }
+                if (kPer == 2) {
+                    digit_tot[2 * i] = (int)(tot & 0xffffu);
+                    digit_tot[2 * i + 1] = (int)(tot >> 16);
+                } else {
+                    digit_tot[i] = (int)tot;
+                }
+            }
+            for (int i = nd + threadIdx.x; i < padded; i += kInvThreads) digit_tot[i] = 0;
+        }
+        sync();
+        // ... then over the digit totals of all CTAs, four digits per thread
+        {
+            const int d0 = 4 * threadIdx.x;
+            const bool mine = d0 < padded;
+            int4 all = make_int4(0, 0, 0, 0), before = make_int4(0, 0, 0, 0);
+            if (mine) {
+#pragma unroll
+                for (int c = 0; c < kInvMaxCluster; ++c) {
+                    if (c >= ctas) continue;
+                    const int4 x = ctas == 1 ? *reinterpret_cast<const int4*>(digit_tot + d0) : ptx::ld_cluster_int4(digit_tot + d0, c);
+                    all.x += x.x; all.y += x.y; all.z += x.z; all.w += x.w;
+                    if (c < cta) { before.x += x.x; before.y += x.y; before.z += x.z; before.w += x.w; }
+                }
+            }
+            const int sum = all.x + all.y + all.z + all.w;
+            int incl = sum;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int x = __shfl_up_sync(0xffffffffu, incl, o);
@@ -321,116 +362,76 @@ invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__
             }
             if (lane == 31) warp_sums[warp] = incl;
             __syncthreads();
-            if (warp == 0) {
-                int ws = warp_sums[lane];
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int x = __shfl_up_sync(0xffffffffu, ws, o);
-                    if (lane >= o) ws += x;
-                }
-                warp_sums[lane] = ws;
+            int base = incl - sum;
+            for (int w = 0; w < warp; ++w) base += warp_sums[w];
+            if (mine) {
+                const int4 b = make_int4(base, base + all.x, base + all.x + all.y, base + all.x + all.y + all.z);
+                *reinterpret_cast<int4*>(digit_begin + d0) = b;
+                *reinterpret_cast<int4*>(digit_off + d0) = make_int4(b.x + before.x, b.y + before.y, b.z + before.z, b.w + before.w);
             }
-            __syncthreads();
-            const int base = (warp ? warp_sums[warp - 1] : 0) + incl - (a + b);
-            if (d0 < nd) digit_tot[d0] = base;
-            if (d0 + 1 < nd) digit_tot[d0 + 1] = base + a;
         }
         __syncthreads();
-        if (single) {
-            // row boundaries: row_ptr[c] = first sorted index whose slot is >= c
-            for (int c = threadIdx.x; c <= B; c += kInvThreads) rp[c] = c < nd ? digit_tot[c] : E;
-        }
-        // scatter
+        // scatter; the running counts of a segment that was not kept in registers go on from the scan's
         for (int b0 = s_begin; b0 < s_end; b0 += 32 * kInvBatch) {
-            unsigned key[kInvBatch], val[kInvBatch];
+            if (!keep) load(b0);
             int pe[kInvBatch];
             float w[kInvBatch];
 #pragma unroll
             for (int q = 0; q < kInvBatch; ++q) {
-                const int i = b0 + q * 32 + lane;
-                key[q] = 0u;
-                val[q] = (unsigned)i;
                 pe[q] = 0;
                 w[q] = 1.0f;
-                if (i < s_end) {
-                    if (pass) { key[q] = src_k[i]; val[q] = src_v[i]; }
-                    else key[q] = (unsigned)assign[ev_base + i];
-                    if (single) {
-                        pe[q] = evict_idx[ev_base + i];
-                        if (weighted) w[q] = sim[ev_base + i];
-                    }
-                }
+                if (!last || b0 + q * 32 + lane >= s_end) continue;
+                pe[q] = evict_idx[ev_base + val[q]];
+                if (weighted) w[q] = sim[ev_base + val[q]];
             }
 #pragma unroll
             for (int q = 0; q < kInvBatch; ++q) {
-                const int i = b0 + q * 32 + lane;
-                const bool valid = i < s_end;
-                if (!pass && key[q] >= (unsigned)B) key[q] = 0u;
+                if (b0 + q * 32 >= s_end) continue;
+                const bool valid = b0 + q * 32 + lane < s_end;
                 const unsigned d = (key[q] >> shift) & dmask;
-                int off = 0;
-                if (keep_ranks) {
-                    if (valid) off = digit_tot[d] + (int)cnt[warp * nd + d] + local_rank[q];
+                const int off = digit_off[d] + (keep ? (int)cnt[warp * nd + d] + local_rank[q] : rank_in_warp(d, valid));
+                if (!valid) continue;
+                if (last) {
+                    if (pe[q] < 0 || pe[q] >= rq.L) { atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); pe[q] = 0; }
+                    ent[off + (int)key[q] + 1] = pe[q];      // sits after key + 1 kept rows
+                    entw[off + (int)key[q] + 1] = w[q];
+                    if (pass) __stcg(dst_k + off, key[q]);
                 } else {
-                    const unsigned peers = same_digit_lanes(d, valid, dbits);
-                    if (valid) off = digit_tot[d] + (int)cnt[warp * nd + d] + __popc(peers & lt_mask);
-                    __syncwarp();
-                    if (valid && (peers & lt_mask) == 0u) cnt[warp * nd + d] += (CountT)__popc(peers);
-                    __syncwarp();
-                }
-                if (valid) {
-                    if (single) {
-                        if (pe[q] < 0 || pe[q] >= rq.L) { atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); pe[q] = 0; }
-                        ent[off + (int)key[q] + 1] = pe[q];      // sits after key + 1 kept rows
-                        entw[off + (int)key[q] + 1] = w[q];
-                    } else {
-                        dst_k[off] = key[q];
-                        dst_v[off] = val[q];
-                    }
+                    __stcg(dst_k + off, key[q]);
+                    __stcg(dst_v + off, val[q]);
                 }
             }
         }
-        __syncthreads();
+        sync();
     }
-    if (!single) {
-        const unsigned* fin_k = key_buf[(n_pass - 1) & 1];
-        const unsigned* fin_v = fin_k + E;
-        // member entries and the row boundaries: row_ptr[c] = first sorted index whose slot is >= c
-        for (int i0 = threadIdx.x; i0 < E; i0 += kInvThreads * kInvBatch) {
-            int e[kInvBatch], cur[kInvBatch], prev[kInvBatch], pe[kInvBatch];
-            float w[kInvBatch];
+    if (n_pass == 1) {
+        // digit = slot: digit_begin[c] is the first sorted index whose slot is >= c
+        auto row_begin = [&](int c) { return c < nd ? digit_begin[c] : E; };
+        for (int c = thread; c <= B; c += n_threads) rp[c] = row_begin(c);
+        write_kept_entries(rq, h, n_kv_heads, thread, n_threads, row_begin, kept_idx_head, ent, entw, units, cnts, status);
+        return;
+    }
+    // row boundaries: row_ptr[c] = first sorted index whose slot is >= c
+    const unsigned* fin_k = key_buf[(n_pass - 1) & 1];
+    for (int i0 = thread; i0 < E; i0 += n_threads * kInvBatch) {
+        int cur[kInvBatch], prev[kInvBatch];
 #pragma unroll
-            for (int q = 0; q < kInvBatch; ++q) {
-                const int i = i0 + q * kInvThreads;
-                e[q] = 0; cur[q] = 0; prev[q] = -1;
-                if (i < E) {
-                    e[q] = (int)fin_v[i];
-                    cur[q] = (int)fin_k[i];
-                    if (i) prev[q] = (int)fin_k[i - 1];
-                }
-            }
+        for (int q = 0; q < kInvBatch; ++q) {
+            const int i = i0 + q * n_threads;
+            cur[q] = i < E ? (int)__ldcg(fin_k + i) : 0;
+            prev[q] = i < E && i ? (int)__ldcg(fin_k + i - 1) : -1;
+        }
 #pragma unroll
-            for (int q = 0; q < kInvBatch; ++q) {
-                const int i = i0 + q * kInvThreads;
-                pe[q] = 0; w[q] = 1.0f;
-                if (i < E) {
-                    pe[q] = evict_idx[ev_base + e[q]];
-                    if (weighted) w[q] = sim[ev_base + e[q]];
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < kInvBatch; ++q) {
-                const int i = i0 + q * kInvThreads;
-                if (i >= E) continue;
-                if (pe[q] < 0 || pe[q] >= rq.L) { atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); pe[q] = 0; }
-                ent[i + cur[q] + 1] = pe[q];             // i-th member sits after cur + 1 kept rows
-                entw[i + cur[q] + 1] = w[q];
-                for (int c = prev[q] + 1; c <= cur[q]; ++c) rp[c] = i;
-                if (i == E - 1) for (int c = cur[q] + 1; c <= B; ++c) rp[c] = E;
-            }
+        for (int q = 0; q < kInvBatch; ++q) {
+            const int i = i0 + q * n_threads;
+            if (i >= E) continue;
+            for (int c = prev[q] + 1; c <= cur[q]; ++c) __stcg(rp + c, i);
+            if (i == E - 1) for (int c = cur[q] + 1; c <= B; ++c) __stcg(rp + c, E);
         }
     }
-    __syncthreads();
-    write_kept_entries(rq, h, n_kv_heads, B, rp, kept_idx_head, ent, entw, units, cnts, status);
+    sync();
+    write_kept_entries(rq, h, n_kv_heads, thread, n_threads, [&](int c) { return __ldcg(rp + c); }, kept_idx_head, ent, entw, units,
+                       cnts, status);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -946,37 +947,25 @@ cudaError_t launch_gather_kept(const void* k, long long stride_tok, long long st
 }
 
 cudaError_t launch_invert_assignment(const int* assign, const int* kept_idx, const int* evict_idx,
-                                     const float* sim, const Req* reqs, int n_req, int n_kv_heads,
+                                     const float* sim, const Req* reqs, int n_req, int n_kv_heads, int ctas,
                                      long long T, bool wide_counts, int digit_bits, int* row_ptr,
                                      int* ent_pos, float* ent_w, int4* unit_first, int* slot_cnt,
                                      unsigned* sort_a, unsigned* sort_b, int* status,
                                      cudaStream_t stream) {
-    // counters of the widest digit any request of the call needs: 32 warps x 2^digit_bits counts
-    // and 2^digit_bits totals
-    const size_t smem = ((size_t)32 * (wide_counts ? sizeof(unsigned) : sizeof(unsigned short)) + sizeof(int))
-                        << digit_bits;
-    dim3 grid(n_kv_heads, n_req);
-    // the shared-memory limit is raised once per device to the most either instantiation can ask
-    // for (32 warps x 2^bits counters and 2^bits totals)
+    // counters of the widest digit any request of the call needs: per warp, and three totals
+    const auto bytes = [](int count, int bits) { return (size_t)(kInvWarps * count + 3 * (int)sizeof(int)) << (bits < 2 ? 2 : bits); };
+    auto* narrow = invert_assignment_kernel<unsigned short, kInvDigitBits16>;
+    auto* wide = invert_assignment_kernel<unsigned, kInvDigitBits32>;
+    // the shared-memory limit is raised once per device to the most either instantiation can ask for
     static unsigned long long configured = 0;
     cudaError_t err = once_per_device(configured, [&]() {
-        const int max16 = (int)(((size_t)32 * sizeof(unsigned short) + sizeof(int)) << kInvDigitBits16);
-        const int max32 = (int)(((size_t)32 * sizeof(unsigned) + sizeof(int)) << kInvDigitBits32);
-        cudaError_t e = cudaFuncSetAttribute(invert_assignment_kernel<unsigned short, kInvDigitBits16>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, max16);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(invert_assignment_kernel<unsigned, kInvDigitBits32>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, max32);
-        return e;
+        cudaError_t e = cudaFuncSetAttribute(narrow, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(2, kInvDigitBits16));
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(4, kInvDigitBits32));
     });
     if (err != cudaSuccess) return err;
-    if (wide_counts)
-        return launch_chained(invert_assignment_kernel<unsigned, kInvDigitBits32>, grid, dim3(kInvThreads), smem,
-                              stream, assign, kept_idx, evict_idx, sim, reqs, n_kv_heads, T, row_ptr, ent_pos,
-                              ent_w, unit_first, slot_cnt, sort_a, sort_b, status);
-    return launch_chained(invert_assignment_kernel<unsigned short, kInvDigitBits16>, grid, dim3(kInvThreads), smem,
-                          stream, assign, kept_idx, evict_idx, sim, reqs, n_kv_heads, T, row_ptr, ent_pos,
-                          ent_w, unit_first, slot_cnt, sort_a, sort_b, status);
+    return launch_chained_clusters(wide_counts ? wide : narrow, dim3((unsigned)(n_kv_heads * ctas), (unsigned)n_req), dim3(kInvThreads),
+                                   (unsigned)ctas, bytes(wide_counts ? 4 : 2, digit_bits), stream, assign, kept_idx, evict_idx, sim,
+                                   reqs, n_kv_heads, ctas, T, row_ptr, ent_pos, ent_w, unit_first, slot_cnt, sort_a, sort_b, status);
 }
 
 int merge_warps_per_sm() { return kMergeWarps; }

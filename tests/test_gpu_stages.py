@@ -494,6 +494,43 @@ def test_merge_on_both_sides_of_the_short_prompt_limit(B, L, budget, skew):
             assert merged_close(got[:, h], orc.merge(x, h, kept[h], ev[h], assign[h], sim[h].astype(np.float64), mode)).all()
 
 
+@pytest.mark.parametrize("L,budget,Hkv,skew", [(4097, 1, 3, "even"), (4097, 2, 1, "even"), (4097, 4096, 2, "even"), (5200, 2048, 3, "first"),
+                                               (5200, 2049, 3, "last"), (33000, 6600, 1, "first"), (9000, 300, 75, "even"),
+                                               (9500, 2100, 75, "last"), (4500, 90, 150, "even")])
+def test_merge_of_long_prompts_with_one_to_eight_inverting_ctas_per_head(B, L, budget, Hkv, skew):
+    """Slots of one digit or two, lists that stay in registers or not, one CTA per head (150 heads), two
+    (75) or eight; a single kept or evicted row; two calls agree bit for bit."""
+    import torch
+    E, mode, kv = L - budget, 2, []
+    gen = torch.Generator(device="cuda").manual_seed(L + budget)
+    for _ in range(2):
+        kv.append(torch.randn(L, Hkv, 128, generator=gen, device="cuda").bfloat16())
+    kept, ev, assign, sim = [], [], [], []
+    for h in range(Hkv):
+        order = np.argsort(synth.uniform_u64(synth.stream_key(183, h, L), L))
+        kept.append(np.sort(order[:budget]).astype(np.int32))
+        ev.append(np.sort(order[budget:]).astype(np.int32))
+        asg = synth.uniform_int(synth.stream_key(184, h), E, 0, budget - 1).astype(np.int32)
+        if skew != "even":
+            asg[np.arange(E) % 16 != 3] = 0 if skew == "first" else budget - 1
+        assign.append(asg)
+        sim.append(np.clip(synth.normal(synth.stream_key(185, h), E) * 0.4, -1, 1).astype(np.float32))
+    dev = lambda xs: torch.from_numpy(np.concatenate(xs)).cuda()
+    lay, got = B.make_layout(None, kv[0]), []
+    ws = B.alloc_workspace(lay, [L])
+    for _ in range(2):
+        out = [torch.zeros(Hkv, budget, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+        B.check(B.lookm_merge(kv[0], kv[1], dev(kept), dev(ev), dev(assign), dev(sim), [0, L], [budget], [mode], lay, 0, *out, ws))
+        assert B.lookm_device_status(ws) == B.OK
+        got.append(out)
+    for x, a, b in zip(kv, *got):
+        assert torch.equal(a, b)
+        for h in sorted({0, Hkv // 2, Hkv - 1}):
+            xf = x[:, h:h + 1].float().cpu().numpy()
+            ref = orc.merge(xf, 0, kept[h], ev[h], assign[h], sim[h].astype(np.float64), mode)
+            assert merged_close(bf16_to_np(a[h]), ref).all()
+
+
 def test_merge_packed_batch_with_slots_spread_over_many_work_units(B):
     """Two requests, batch output layout, member counts from 0 to many hundreds: the kernel cuts its
     work units at fixed entry counts, so most of the large slots are summed piecewise by several
