@@ -45,7 +45,7 @@ struct Plan {
     size_t clear_words = 64;                // status word and arrival counters
     size_t o_parts1 = 0, o_parts2 = 0;
     size_t o_status, o_reqs, o_lse, o_lse_split, o_scores, o_rank, o_rnorm_all, o_kept, o_evict, o_kept_keys,
-        o_rnorm_kept, o_assign, o_sim, o_row_ptr, o_members, o_member_w, o_units, o_slot_cnt, o_parts, o_sort_a, o_sort_b,
+        o_rnorm_kept, o_assign, o_sim, o_row_ptr, o_entries, o_units, o_slot_cnt, o_parts, o_sort_a, o_sort_b,
         total;
 };
 
@@ -218,8 +218,7 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
     pl.o_assign = carve(4 * Hkv * T);
     pl.o_sim = carve(4 * Hkv * T);
     pl.o_row_ptr = carve(4 * (Hkv * T + Hkv * (size_t)n_req));
-    pl.o_members = carve(4 * Hkv * T);
-    pl.o_member_w = carve(4 * Hkv * T);
+    pl.o_entries = carve(8 * Hkv * T);
     pl.o_units = carve(16 * (size_t)pl.total_units);
     pl.o_slot_cnt = carve(4 * Hkv * T);
     pl.o_parts = carve((size_t)kMergePartBytes * (size_t)pl.total_units);
@@ -451,42 +450,61 @@ int run_match(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     return LOOKM_OK;
 }
 
-// The inversion's CTAs (kInvMaxCluster at most per request and head) fill the SMs twice at most, and each
-// gets kInvMinShare evicted tokens at least.
-constexpr long long kInvCtasPerSm = 2;
+// The inversion's CTAs (kInvMaxCluster at most per request and head) run all at once, two per SM if their
+// shared memory allows, and each gets kInvMinShare evicted tokens at least.
+constexpr long long kInvCtasPerSm = 2, kInvSmemPerSm = 220 << 10;
 constexpr int kInvMinShare = 512;
+cudaError_t run_inversion(const Plan& pl, const DeviceInfo& di, const int* kept_idx, const int* evict_idx, const int* assign,
+                          const float* sim, void* ws, cudaStream_t st) {
+    const Req* reqs = at<Req>(ws, pl.o_reqs);
+    int *status = at<int>(ws, pl.o_status), *row_ptr = at<int>(ws, pl.o_row_ptr);
+    int2* entries = at<int2>(ws, pl.o_entries);
+    int4* units = at<int4>(ws, pl.o_units);
+    int* slot_cnt = at<int>(ws, pl.o_slot_cnt);
+    const auto ctas_per_head = [&](long long per_sm) {
+        int ctas = 1;
+        while (ctas < kInvMaxCluster && 2ll * ctas * pl.n_kv_heads * pl.n_req <= per_sm * di.sms &&
+               pl.max_E >= 2 * ctas * kInvMinShare)
+            ctas *= 2;
+        return ctas;
+    };
+    // counting, where it fits: a count per slot and warp in shared memory, a warp's rows in registers and
+    // their counts in bytes (42 us sorted, 25 counted for 26214 evicted rows x 8 heads and 6554 slots)
+    const long long slot_bytes = (long long)(pl.max_B + 4 * kInvMaxCluster) * kCountSlotBytes;
+    int ctas = ctas_per_head(std::min(kInvCtasPerSm, std::max(1ll, kInvSmemPerSm / slot_bytes)));
+    if (pl.max_B <= kCountMaxSlots && pl.max_E <= ctas * kCountWarps * kCountSeg) {
+        const int max_slots = ctas * (((pl.max_B + ctas - 1) / ctas + 3) / 4 * 4);
+        return launch_invert_counting(assign, kept_idx, evict_idx, sim, reqs, pl.n_req, pl.n_kv_heads, ctas, max_slots, pl.T, row_ptr,
+                                      entries, units, slot_cnt, status, st);
+    }
+    // counter width and widest digit over the requests of the call
+    ctas = ctas_per_head(kInvCtasPerSm);
+    const bool wide = pl.max_E > kInvWideCountsAbove;
+    int digit_bits = 1;
+    for (const Req& r : pl.reqs) {
+        int n_pass, dbits;
+        invert_digits(r.B, wide ? kInvDigitBits32 : kInvDigitBits16, n_pass, dbits);
+        digit_bits = std::max(digit_bits, dbits);
+    }
+    return launch_invert_assignment(assign, kept_idx, evict_idx, sim, reqs, pl.n_req, pl.n_kv_heads, ctas, pl.T, wide, digit_bits, row_ptr,
+                                    entries, units, slot_cnt, at<unsigned>(ws, pl.o_sort_a), at<unsigned>(ws, pl.o_sort_b),
+                                    status, st);
+}
+
 int run_merge(const Plan& pl, const lookm_layout* lay, const void* k, const void* v,
               const int* kept_idx, const int* evict_idx, const int* assign, const float* sim,
               int varlen_output, void* out_k, void* out_v, void* ws, cudaStream_t st) {
     const Req* reqs = at<Req>(ws, pl.o_reqs);
     int* status = at<int>(ws, pl.o_status);
     const bool short_merge = pl.max_L <= kMergeShortMax;
+    DeviceInfo di;
+    LOOKM_TRY(device_info(di));
     if (pl.n_none < pl.n_req && !short_merge) {
-        // counter width and widest digit over the requests of the call
-        const bool wide = pl.max_E > kInvWideCountsAbove;
-        int digit_bits = 1;
-        for (const Req& r : pl.reqs) {
-            int n_pass, dbits;
-            invert_digits(r.B, wide ? kInvDigitBits32 : kInvDigitBits16, n_pass, dbits);
-            digit_bits = std::max(digit_bits, dbits);
-        }
-        DeviceInfo di;
-        LOOKM_TRY(device_info(di));
-        int ctas = 1;                            // per (request, head)
-        while (ctas < kInvMaxCluster && 2ll * ctas * pl.n_kv_heads * pl.n_req <= kInvCtasPerSm * di.sms &&
-               pl.max_E >= 2 * ctas * kInvMinShare)
-            ctas *= 2;
-        LOOKM_CUDA(launch_invert_assignment(assign, kept_idx, evict_idx, sim, reqs, pl.n_req, pl.n_kv_heads, ctas,
-                                            pl.T, wide, digit_bits, at<int>(ws, pl.o_row_ptr), at<int>(ws, pl.o_members),
-                                            at<float>(ws, pl.o_member_w), at<int4>(ws, pl.o_units),
-                                            at<int>(ws, pl.o_slot_cnt), at<unsigned>(ws, pl.o_sort_a),
-                                            at<unsigned>(ws, pl.o_sort_b), status, st));
+        LOOKM_CUDA(run_inversion(pl, di, kept_idx, evict_idx, assign, sim, ws, st));
         ++g_launches;
     }
     mark_stage(6, st);
     if (pl.n_none < pl.n_req) {
-        DeviceInfo di;
-        LOOKM_TRY(device_info(di));
         if (short_merge)
             LOOKM_CUDA(launch_merge_short(k, v, lay->kv_stride_tok, lay->kv_stride_head, assign, kept_idx, evict_idx, sim,
                                           reqs, pl.n_req, pl.n_kv_heads, pl.max_L, pl.max_E, pl.max_B, varlen_output,
@@ -494,7 +512,7 @@ int run_merge(const Plan& pl, const lookm_layout* lay, const void* k, const void
         else
             LOOKM_CUDA(launch_merge(k, v, lay->kv_stride_tok, lay->kv_stride_head, reqs, pl.n_req,
                                     pl.n_kv_heads, pl.T, pl.total_units, at<int>(ws, pl.o_row_ptr),
-                                    at<int>(ws, pl.o_members), at<float>(ws, pl.o_member_w),
+                                    at<int2>(ws, pl.o_entries),
                                     at<int4>(ws, pl.o_units), at<int>(ws, pl.o_slot_cnt),
                                     at<float>(ws, pl.o_parts), varlen_output, pl.out_stride_head, out_k,
                                     out_v, status, di.sms, st));
@@ -866,8 +884,7 @@ extern "C" int lookm_merge_noalloc(const void* k, const void* v, const int* kept
     pl.o_status = carve(256);
     pl.o_reqs = carve(sizeof(Req) * (size_t)n_requests);
     pl.o_row_ptr = carve(4 * (units + (size_t)pl.n_kv_heads * (size_t)n_requests));
-    pl.o_members = carve(4 * units);
-    pl.o_member_w = carve(4 * units);
+    pl.o_entries = carve(8 * units);
     pl.o_units = carve(16 * (size_t)pl.total_units);
     pl.o_slot_cnt = carve(4 * (size_t)pl.total_slots);
     pl.o_parts = carve((size_t)kMergePartBytes * (size_t)pl.total_units);

@@ -22,6 +22,9 @@ constexpr int kMaxUnitEntries = LOOKM_MAX_UNIT_ENTRIES;   // most rows in one
 constexpr int kInvDigitBits16 = 11;
 constexpr int kInvDigitBits32 = 10;
 constexpr int kInvMaxCluster = 8;
+// The counting inversion: sixteen warps a CTA, at most kCountSeg evicted rows a warp and kCountMaxSlots
+// kept rows, which take kCountSlotBytes of shared memory each.
+constexpr int kCountWarps = 16, kCountSeg = 224, kCountMaxSlots = 8192, kCountSlotBytes = 22;
 constexpr int kInvWideCountsAbove = 65535;   // evicted tokens per head beyond which counts need 32 bits
 #ifdef __CUDACC__
 __host__ __device__
@@ -133,9 +136,13 @@ cudaError_t launch_write_table(const ReqChunk& chunk, int count, Req* dst, int* 
 cudaError_t launch_invert_assignment(const int* assign, const int* kept_idx, const int* evict_idx,
                                      const float* sim, const Req* reqs, int n_req, int n_kv_heads, int ctas,
                                      long long T, bool wide_counts, int digit_bits, int* row_ptr,
-                                     int* ent_pos, float* ent_w, int4* unit_first, int* slot_cnt,
+                                     int2* entries, int4* unit_first, int* slot_cnt,
                                      unsigned* sort_a, unsigned* sort_b, int* status,
                                      cudaStream_t stream);
+
+cudaError_t launch_invert_counting(const int* assign, const int* kept_idx, const int* evict_idx, const float* sim, const Req* reqs,
+                                   int n_req, int n_kv_heads, int ctas, int max_slots, long long T, int* row_ptr, int2* entries,
+                                   int4* unit_first, int* slot_cnt, int* status, cudaStream_t stream);
 
 // Inversion and merge in one launch; every request has at most kMergeShortMax tokens.
 constexpr int kMergeShortMax = 4096;
@@ -148,8 +155,8 @@ int merge_warps_per_sm();
 
 cudaError_t launch_merge(const void* k, const void* v, long long stride_tok, long long stride_head,
                          const Req* reqs, int n_req, int n_kv_heads, long long T,
-                         long long total_units, const int* row_ptr, const int* ent_pos,
-                         const float* ent_w, const int4* unit_first, int* slot_cnt, float* parts,
+                         long long total_units, const int* row_ptr, const int2* entries,
+                         const int4* unit_first, int* slot_cnt, float* parts,
                          int varlen_output, long long out_stride_head, void* out_k, void* out_v,
                          int* status, int num_sms, cudaStream_t stream);
 

@@ -172,33 +172,32 @@ constexpr int kInvBatch = 8;                         // loop steps whose loads a
 // Second half of the entry list: the kept rows (flagged with the sign bit, weight = member count),
 // for every work unit (unit u of a head covers the entries [u * unit_entries, (u + 1) * unit_entries))
 // the slot its first entry belongs to, with that slot's first entry and member count, and a
-// cleared arrival counter per slot.  row_begin(c): members of the slots before c.  For the slots
-// c0, c0 + step, ...
-template <typename RowBegin>
-__device__ __forceinline__ void write_kept_entries(const Req& rq, int h, int n_kv_heads, int c0, int step, RowBegin row_begin,
-                                                   const int* kept_idx_head, int* ent, float* entw,
-                                                   int4* unit_first, int* slot_cnt, int* status) {
-    const int ue = rq.unit_entries;
-    for (int c = c0; c < rq.B; c += step) {
-        int pc = kept_idx_head[c];
-        if (pc < 0 || pc >= rq.L) { atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); pc = 0; }
-        const int begin = row_begin(c), n = row_begin(c + 1) - begin;
+// cleared arrival counter per slot.  Slot c, whose kept row is at position pc, has n members, after
+// those of the slots before it.
+struct KeptEntries {
+    int2* ent;                                           // position and weight
+    int4* units;                                         // [unit of the head][head]
+    int* slot_cnt;
+    int* status;
+    int L, unit_entries, h, n_kv_heads;
+    __device__ __forceinline__ void write(int c, int pc, int begin, int n) const {
+        if (pc < 0 || pc >= L) { atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); pc = 0; }
         const int s_c = c + begin;                       // entry of the kept row
         const int s_next = s_c + n + 1;                  // entry of the next kept row (L after the last)
-        ent[s_c] = pc | (int)0x80000000;
-        entw[s_c] = (float)n;
+        ent[s_c] = make_int2(pc | (int)0x80000000, __float_as_int((float)n));
         slot_cnt[c] = 0;
-        for (int u = (s_c + ue - 1) / ue; u * ue < s_next; ++u)
-            unit_first[(long long)u * n_kv_heads + h] = make_int4(c, s_c, n, 0);
+        for (int u = (s_c + unit_entries - 1) / unit_entries; u * unit_entries < s_next; ++u)
+            units[(long long)u * n_kv_heads + h] = make_int4(c, s_c, n, 0);
     }
-}
+};
 
 // Lanes of the warp that hold a valid element with the same digit as the caller: one ballot per
 // digit bit (match.any takes a step per distinct value, i.e. up to 32 for well-mixed digits).
+template <int kMaxBits>
 __device__ __forceinline__ unsigned same_digit_lanes(unsigned d, bool valid, int dbits) {
     unsigned peers = __ballot_sync(0xffffffffu, valid);
 #pragma unroll
-    for (int b = 0; b < kInvDigitBits16; ++b) {
+    for (int b = 0; b < kMaxBits; ++b) {
         if (b < dbits) {
             const bool bit = (d >> b) & 1u;
             const unsigned bal = __ballot_sync(0xffffffffu, bit);
@@ -217,7 +216,7 @@ invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__
                          const int* __restrict__ evict_idx,
                          const float* __restrict__ sim, const Req* __restrict__ reqs,
                          int n_kv_heads, int ctas, long long T, int* row_ptr,
-                         int* __restrict__ ent_pos, float* __restrict__ ent_w,
+                         int2* __restrict__ entries,
                          int4* __restrict__ unit_first, int* __restrict__ slot_cnt,
                          unsigned* sort_a, unsigned* sort_b, int* status) {
     static_assert((1 << kMaxBits) <= 4 * kInvThreads, "a thread scans four digits");
@@ -236,15 +235,14 @@ invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__
     auto sync = [&]() { if (ctas > 1) ptx::cluster_sync(); else __syncthreads(); };
 
     // entry list of this (request, head): for every kept slot its kept row, then its members
-    int* ent = ent_pos + (long long)h * T + rq.tok_begin;
-    float* entw = ent_w + (long long)h * T + rq.tok_begin;
-    int4* units = unit_first + rq.unit_begin;            // [unit of the head][head]
-    int* cnts = slot_cnt + rq.kept_off + (long long)h * B;
+    int2* ent = entries + (long long)h * T + rq.tok_begin;
+    const KeptEntries kept = {ent, unit_first + rq.unit_begin, slot_cnt + rq.kept_off + (long long)h * B, status,
+                              rq.L, rq.unit_entries, h, n_kv_heads};
     const int* kept_idx_head = kept_idx + rq.kept_off + (long long)h * B;
     const bool weighted = (rq.mode == LOOKM_MERGE_WEIGHTED);
     if (E == 0) {
         for (int c = thread; c <= B; c += n_threads) rp[c] = 0;
-        write_kept_entries(rq, h, n_kv_heads, thread, n_threads, [](int) { return 0; }, kept_idx_head, ent, entw, units, cnts, status);
+        for (int c = thread; c < B; c += n_threads) kept.write(c, kept_idx_head[c], 0, 0);
         return;
     }
     // segment of the list owned by each warp: a multiple of 32 elements
@@ -299,7 +297,7 @@ invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__
         };
         // rank among the elements of the warp's segment with the same digit, which it counts
         auto rank_in_warp = [&](unsigned d, bool valid) {
-            const unsigned peers = same_digit_lanes(d, valid, dbits);
+            const unsigned peers = same_digit_lanes<kMaxBits>(d, valid, dbits);
             const int r = valid ? (int)cnt[warp * nd + d] + __popc(peers & lt_mask) : 0;
             __syncwarp();
             if (valid && (peers & lt_mask) == 0u) cnt[warp * nd + d] += (CountT)__popc(peers);
@@ -393,8 +391,7 @@ invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__
                 if (!valid) continue;
                 if (last) {
                     if (pe[q] < 0 || pe[q] >= rq.L) { atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); pe[q] = 0; }
-                    ent[off + (int)key[q] + 1] = pe[q];      // sits after key + 1 kept rows
-                    entw[off + (int)key[q] + 1] = w[q];
+                    ent[off + (int)key[q] + 1] = make_int2(pe[q], __float_as_int(w[q]));   // sits after key + 1 kept rows
                     if (pass) __stcg(dst_k + off, key[q]);
                 } else {
                     __stcg(dst_k + off, key[q]);
@@ -408,7 +405,7 @@ invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__
         // digit = slot: digit_begin[c] is the first sorted index whose slot is >= c
         auto row_begin = [&](int c) { return c < nd ? digit_begin[c] : E; };
         for (int c = thread; c <= B; c += n_threads) rp[c] = row_begin(c);
-        write_kept_entries(rq, h, n_kv_heads, thread, n_threads, row_begin, kept_idx_head, ent, entw, units, cnts, status);
+        for (int c = thread; c < B; c += n_threads) kept.write(c, kept_idx_head[c], row_begin(c), row_begin(c + 1) - row_begin(c));
         return;
     }
     // row boundaries: row_ptr[c] = first sorted index whose slot is >= c
@@ -430,8 +427,190 @@ invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__
         }
     }
     sync();
-    write_kept_entries(rq, h, n_kv_heads, thread, n_threads, [&](int c) { return __ldcg(rp + c); }, kept_idx_head, ent, entw, units,
-                       cnts, status);
+    for (int c = thread; c < B; c += n_threads) {
+        const int begin = __ldcg(rp + c);
+        kept.write(c, kept_idx_head[c], begin, __ldcg(rp + c + 1) - begin);
+    }
+}
+
+// The same result in one pass, a digit being a whole slot: every warp has a count per slot, in a byte, so
+// that the sixteen counts of a slot are one 16-byte word and the sum over the warps before one's own four
+// byte-wise dot products.  A warp's segment is at most kCountSeg elements and stays in registers.
+// Every CTA of the cluster owns a share of the slots: it adds up the CTAs' totals of these, leaves each
+// CTA the position of its first member per slot, and writes the kept rows' entries.  26214 evicted tokens
+// x 8 heads into 6554 slots 42 us with two sorting passes, 25 counted; 13107 x 40 into 3277 46 and 32; 6554
+// x 32 into 1638 (one sorting pass) 23.5 and 21.4; 7388 x 8 into 389 16.4 both.
+constexpr int kCountSteps = kCountSeg / 32;
+static_assert(kCountSeg % 32 == 0 && kCountSeg < 256 && kCountWarps == kInvWarps && kInvWarps == 16, "byte counts of sixteen warps");
+constexpr int kCountBits = 13;
+static_assert((1 << kCountBits) == kCountMaxSlots, "ballots per slot");
+__device__ __forceinline__ int bytes_sum(const uint4& v, const uint4& m) {
+    return (int)__dp4a(v.x, m.x, __dp4a(v.y, m.y, __dp4a(v.z, m.z, __dp4a(v.w, m.w, 0u))));
+}
+
+__global__ void __launch_bounds__(kInvThreads, 2)
+invert_counting_kernel(const int* __restrict__ assign, const int* __restrict__ kept_idx, const int* __restrict__ evict_idx,
+                       const float* __restrict__ sim, const Req* __restrict__ reqs, int n_kv_heads, int ctas, int max_slots,
+                       long long T, int* __restrict__ row_ptr, int2* __restrict__ entries,
+                       int4* __restrict__ unit_first, int* __restrict__ slot_cnt, int* status) {
+    extern __shared__ __align__(16) unsigned char inv_smem[];
+    __shared__ int warp_sums[kInvWarps];
+    __shared__ int owner_tot[kInvMaxCluster];            // of this CTA's elements, those in each CTA's slots
+    __shared__ int slots_begin;                          // elements in the slots of earlier CTAs
+    uint4* cnt = reinterpret_cast<uint4*>(inv_smem);                                  // [slot] 16 warps
+    int* off = reinterpret_cast<int*>(inv_smem + (size_t)max_slots * 16);             // [slot]
+    unsigned short* tot = reinterpret_cast<unsigned short*>(off + max_slots);         // [slot]
+    grid_dependency_wait();
+    const Req rq = reqs[blockIdx.y];
+    if (rq.mode == LOOKM_MERGE_NONE) return;             // its kept rows are copied, nothing is merged
+    const int h = blockIdx.x / ctas, cta = blockIdx.x % ctas;     // the cluster: the CTAs of one head
+    const int E = rq.E, B = rq.B;
+    const long long ev_base = rq.ev_off + (long long)h * E;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    auto sync = [&]() { if (ctas > 1) ptx::cluster_sync(); else __syncthreads(); };
+    int2* ent = entries + (long long)h * T + rq.tok_begin;
+    const KeptEntries kept = {ent, unit_first + rq.unit_begin, slot_cnt + rq.kept_off + (long long)h * B, status,
+                              rq.L, rq.unit_entries, h, n_kv_heads};
+    const int* kept_idx_head = kept_idx + rq.kept_off + (long long)h * B;
+    int* rp = row_ptr + rq.rp_off + (long long)h * (B + 1);
+
+    // the warp's elements
+    const int seg = (E + ctas * kInvThreads - 1) / (ctas * kInvThreads) * 32;
+    const int s_begin = min(E, (cta * kInvWarps + warp) * seg), s_end = min(E, s_begin + seg);
+    unsigned key[kCountSteps];
+    int pos[kCountSteps], local_rank[kCountSteps];
+    float w[kCountSteps];
+#pragma unroll
+    for (int q = 0; q < kCountSteps; ++q) {
+        const int i = s_begin + q * 32 + lane;
+        key[q] = 0u;
+        pos[q] = 0;
+        w[q] = 1.0f;
+        if (i >= s_end) continue;
+        key[q] = (unsigned)assign[ev_base + i];
+        pos[q] = evict_idx[ev_base + i];
+        if (rq.mode == LOOKM_MERGE_WEIGHTED) w[q] = sim[ev_base + i];
+    }
+    for (int c = threadIdx.x; c < B; c += kInvThreads) cnt[c] = make_uint4(0u, 0u, 0u, 0u);
+    if (threadIdx.x < kInvMaxCluster) owner_tot[threadIdx.x] = 0;
+    if (threadIdx.x == 0) slots_begin = 0;
+    int bits = 0;
+    while ((1 << bits) < B) ++bits;
+#pragma unroll
+    for (int q = 0; q < kCountSteps; ++q) {
+        if (key[q] >= (unsigned)B || pos[q] < 0 || pos[q] >= rq.L) {
+            atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX);
+            if (key[q] >= (unsigned)B) key[q] = 0u;
+            if (pos[q] < 0 || pos[q] >= rq.L) pos[q] = 0;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kCountSteps; ++q) {
+        if (s_begin + q * 32 >= s_end) continue;
+        const bool valid = s_begin + q * 32 + lane < s_end;
+        const unsigned peers = same_digit_lanes<kCountBits>(key[q], valid, bits);
+        unsigned char* n = reinterpret_cast<unsigned char*>(cnt + key[q]) + warp;
+        local_rank[q] = valid ? (int)*n + __popc(peers & lt_mask) : 0;
+        __syncwarp();
+        if (valid && (peers & lt_mask) == 0u) *n = (unsigned char)(*n + __popc(peers));
+        __syncwarp();
+    }
+    __syncthreads();
+
+    // this CTA's total of every slot, and of every CTA's share of the slots
+    const int share = ((B + ctas - 1) / ctas + 3) / 4 * 4;         // (ctas * share <= max_slots)
+    const uint4 ones = make_uint4(0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u);
+#pragma unroll
+    for (int o = 0; o < kInvMaxCluster; ++o) {
+        if (o >= ctas) continue;
+        int sum = 0;
+        for (int c = o * share + threadIdx.x; c < (o + 1) * share; c += kInvThreads) {
+            const int t = c < B ? bytes_sum(cnt[c], ones) : 0;
+            tot[c] = (unsigned short)t;
+            sum += t;
+        }
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == 0 && sum) atomicAdd(&owner_tot[o], sum);
+    }
+    sync();
+    if (threadIdx.x < kInvMaxCluster * kInvMaxCluster) {
+        const int c = threadIdx.x / kInvMaxCluster, o = threadIdx.x % kInvMaxCluster;
+        if (c < ctas && o < cta) atomicAdd(&slots_begin, ptx::ld_cluster_int(&owner_tot[o], c));
+    }
+    // own slots, four per thread: members before each, and where every CTA's first one goes
+    for (int t0 = 0, run = 0; t0 < share; t0 += 4 * kInvThreads) {
+        const int d0 = cta * share + t0 + 4 * threadIdx.x;
+        const bool mine = t0 + 4 * threadIdx.x < share;
+        uint2 x[kInvMaxCluster];
+        int pc[4] = {0, 0, 0, 0}, all[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int c = 0; c < kInvMaxCluster; ++c) {
+            x[c] = make_uint2(0u, 0u);
+            if (mine && c < ctas)
+                x[c] = ctas > 1 ? ptx::ld_cluster_uint2(tot + d0, c) : *reinterpret_cast<const uint2*>(tot + d0);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (mine && d0 + j < B) pc[j] = kept_idx_head[d0 + j];
+#pragma unroll
+        for (int c = 0; c < kInvMaxCluster; ++c) {
+            all[0] += x[c].x & 0xffffu;
+            all[1] += x[c].x >> 16;
+            all[2] += x[c].y & 0xffffu;
+            all[3] += x[c].y >> 16;
+        }
+        const int sum = all[0] + all[1] + all[2] + all[3];
+        int incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        __syncthreads();                                 // slots_begin; the last turn's warp_sums have been read
+        if (lane == 31) warp_sums[warp] = incl;
+        __syncthreads();
+        int begin = slots_begin + run + incl - sum;
+        for (int v = 0; v < kInvWarps; ++v) {
+            if (v < warp) begin += warp_sums[v];
+            run += warp_sums[v];
+        }
+        if (!mine) continue;
+        int4 at = make_int4(begin, begin + all[0], begin + all[0] + all[1], begin + all[0] + all[1] + all[2]);
+        const int first[4] = {at.x, at.y, at.z, at.w};
+#pragma unroll
+        for (int c = 0; c < kInvMaxCluster; ++c) {
+            if (c >= ctas) continue;
+            if (ctas > 1) ptx::st_cluster_int4(off + d0, c, at);
+            else *reinterpret_cast<int4*>(off + d0) = at;
+            at.x += x[c].x & 0xffffu;
+            at.y += x[c].x >> 16;
+            at.z += x[c].y & 0xffffu;
+            at.w += x[c].y >> 16;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (d0 + j >= B) continue;
+            rp[d0 + j] = first[j];
+            kept.write(d0 + j, pc[j], first[j], all[j]);
+        }
+    }
+    if (cta == 0 && threadIdx.x == 0) rp[B] = E;
+    sync();
+
+    const auto before = [&](int v) {                     // ones in the bytes of word v that belong to earlier warps
+        const int n = min(max(warp - 4 * v, 0), 4);
+        return n == 4 ? 0x01010101u : 0x01010101u & ((1u << (8 * n)) - 1u);
+    };
+    const uint4 earlier = make_uint4(before(0), before(1), before(2), before(3));
+#pragma unroll
+    for (int q = 0; q < kCountSteps; ++q) {
+        if (s_begin + q * 32 + lane >= s_end) continue;
+        // sits after key + 1 kept rows
+        const int at = off[key[q]] + bytes_sum(cnt[key[q]], earlier) + local_rank[q] + (int)key[q] + 1;
+        ent[at] = make_int2(pos[q], __float_as_int(w[q]));
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -483,7 +662,7 @@ __global__ void __launch_bounds__(kMergeWarps * 32)
 merge_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
              long long stride_tok, long long stride_head, const Req* __restrict__ reqs, int n_req,
              int n_kv_heads, long long T, long long total_units, const int* __restrict__ row_ptr,
-             const int* __restrict__ ent_pos, const float* __restrict__ ent_w,
+             const int2* __restrict__ entries,
              const int4* __restrict__ unit_first, int* __restrict__ slot_cnt, float* __restrict__ parts,
              int varlen_output, long long out_stride_head, __nv_bfloat16* __restrict__ out_k,
              __nv_bfloat16* __restrict__ out_v, int* status) {
@@ -511,8 +690,7 @@ merge_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
         int4 first = make_int4(0, 0, 0, 0);           // slot of the first entry; its first entry, member count
         if (lane == 0) first = __ldg(unit_first + g); // needed at the first kept row at the earliest
         int* cnt = slot_cnt + rq.kept_off + (long long)h * B;
-        const int* ent = ent_pos + (long long)h * T + rq.tok_begin;
-        const float* entw = ent_w + (long long)h * T + rq.tok_begin;
+        const int2* ent = entries + (long long)h * T + rq.tok_begin;
         const char* src = reinterpret_cast<const char*>(tensor + (long long)rq.tok_begin * stride_tok +
                                                         (long long)h * stride_head + l16 * 8);
         const int n_chunks = (e_hi - e_lo + kChunk - 1) / kChunk;
@@ -522,7 +700,7 @@ merge_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
             pos = 0;
             w = 0.f;
             const int e = e_lo + kc * kChunk + lane;
-            if (lane < kChunk && kc < n_chunks && e < e_hi) { pos = ent[e]; w = entw[e]; }
+            if (lane < kChunk && kc < n_chunks && e < e_hi) { const int2 x = ent[e]; pos = x.x; w = __int_as_float(x.y); }
         };
         // start the row copies of chunk kc: for every entry, lanes 0-15 copy its K row and lanes
         // 16-31 its V row, 16 bytes each; one commit group per chunk
@@ -949,7 +1127,7 @@ cudaError_t launch_gather_kept(const void* k, long long stride_tok, long long st
 cudaError_t launch_invert_assignment(const int* assign, const int* kept_idx, const int* evict_idx,
                                      const float* sim, const Req* reqs, int n_req, int n_kv_heads, int ctas,
                                      long long T, bool wide_counts, int digit_bits, int* row_ptr,
-                                     int* ent_pos, float* ent_w, int4* unit_first, int* slot_cnt,
+                                     int2* entries, int4* unit_first, int* slot_cnt,
                                      unsigned* sort_a, unsigned* sort_b, int* status,
                                      cudaStream_t stream) {
     // counters of the widest digit any request of the call needs: per warp, and three totals
@@ -965,15 +1143,29 @@ cudaError_t launch_invert_assignment(const int* assign, const int* kept_idx, con
     if (err != cudaSuccess) return err;
     return launch_chained_clusters(wide_counts ? wide : narrow, dim3((unsigned)(n_kv_heads * ctas), (unsigned)n_req), dim3(kInvThreads),
                                    (unsigned)ctas, bytes(wide_counts ? 4 : 2, digit_bits), stream, assign, kept_idx, evict_idx, sim,
-                                   reqs, n_kv_heads, ctas, T, row_ptr, ent_pos, ent_w, unit_first, slot_cnt, sort_a, sort_b, status);
+                                   reqs, n_kv_heads, ctas, T, row_ptr, entries, unit_first, slot_cnt, sort_a, sort_b, status);
+}
+
+cudaError_t launch_invert_counting(const int* assign, const int* kept_idx, const int* evict_idx, const float* sim, const Req* reqs,
+                                   int n_req, int n_kv_heads, int ctas, int max_slots, long long T, int* row_ptr, int2* entries,
+                                   int4* unit_first, int* slot_cnt, int* status, cudaStream_t stream) {
+    static unsigned long long configured = 0;
+    cudaError_t err = once_per_device(configured, [&]() {
+        return cudaFuncSetAttribute(invert_counting_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (kCountMaxSlots + 4 * kInvMaxCluster) * kCountSlotBytes);
+    });
+    if (err != cudaSuccess) return err;
+    return launch_chained_clusters(invert_counting_kernel, dim3((unsigned)(n_kv_heads * ctas), (unsigned)n_req), dim3(kInvThreads),
+                                   (unsigned)ctas, (size_t)max_slots * kCountSlotBytes, stream, assign, kept_idx, evict_idx, sim,
+                                   reqs, n_kv_heads, ctas, max_slots, T, row_ptr, entries, unit_first, slot_cnt, status);
 }
 
 int merge_warps_per_sm() { return kMergeWarps; }
 
 cudaError_t launch_merge(const void* k, const void* v, long long stride_tok, long long stride_head,
                          const Req* reqs, int n_req, int n_kv_heads, long long T,
-                         long long total_units, const int* row_ptr, const int* ent_pos,
-                         const float* ent_w, const int4* unit_first, int* slot_cnt, float* parts,
+                         long long total_units, const int* row_ptr, const int2* entries,
+                         const int4* unit_first, int* slot_cnt, float* parts,
                          int varlen_output, long long out_stride_head, void* out_k, void* out_v,
                          int* status, int num_sms, cudaStream_t stream) {
     if (total_units <= 0) return cudaSuccess;
@@ -988,7 +1180,7 @@ cudaError_t launch_merge(const void* k, const void* v, long long stride_tok, lon
     if (blocks > num_sms) blocks = num_sms;              // persistent: one CTA per SM
     return launch_chained(merge_kernel, dim3((unsigned)blocks), dim3(kMergeWarps * 32), (size_t)smem, stream,
                           (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, stride_tok, stride_head, reqs,
-                          n_req, n_kv_heads, T, total_units, row_ptr, ent_pos, ent_w, unit_first, slot_cnt,
+                          n_req, n_kv_heads, T, total_units, row_ptr, entries, unit_first, slot_cnt,
                           parts, varlen_output, out_stride_head, (__nv_bfloat16*)out_k, (__nv_bfloat16*)out_v,
                           status);
 }

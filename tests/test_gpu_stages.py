@@ -496,10 +496,13 @@ def test_merge_on_both_sides_of_the_short_prompt_limit(B, L, budget, skew):
 
 @pytest.mark.parametrize("L,budget,Hkv,skew", [(4097, 1, 3, "even"), (4097, 2, 1, "even"), (4097, 4096, 2, "even"), (5200, 2048, 3, "first"),
                                                (5200, 2049, 3, "last"), (33000, 6600, 1, "first"), (9000, 300, 75, "even"),
-                                               (9500, 2100, 75, "last"), (4500, 90, 150, "even")])
+                                               (9500, 2100, 75, "last"), (4500, 90, 150, "even"),
+                                               (36864, 8192, 1, "even"), (36865, 8192, 1, "first"), (40000, 9000, 2, "even"),
+                                               (4674, 1090, 150, "last"), (4675, 1090, 150, "even"), (7005, 1001, 1, "even")])
 def test_merge_of_long_prompts_with_one_to_eight_inverting_ctas_per_head(B, L, budget, Hkv, skew):
-    """Slots of one digit or two, lists that stay in registers or not, one CTA per head (150 heads), two
-    (75) or eight; a single kept or evicted row; two calls agree bit for bit."""
+    """Counted or sorted (beyond 8192 kept rows or 3584 evicted ones per CTA); slots of one digit or two,
+    lists that stay in registers or not, one CTA per head (150 heads), two (75) or eight; a single kept
+    or evicted row; two calls agree bit for bit."""
     import torch
     E, mode, kv = L - budget, 2, []
     gen = torch.Generator(device="cuda").manual_seed(L + budget)
