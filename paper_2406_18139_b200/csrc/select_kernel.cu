@@ -11,8 +11,8 @@
 // largest key (order-preserving 32-bit image of the score) is found by bisection between the smallest
 // and the largest one: a step counts the keys at or above the middle, with the keys in registers and
 // one block barrier.  Ties at the threshold go to the lowest positions.  An ordered pass over the same
-// registers (eight consecutive tokens per thread, one block scan per pass) writes the kept and evicted
-// lists in ascending position.
+// registers writes the kept and evicted lists in ascending position: ballots number a warp's tokens, one
+// block scan the warps.
 //
 // The kernel is bound by the latency of one CTA's barriers and round trips.  A four-pass radix select
 // over a shared-memory histogram (its first digits nearly equal for all scores, so that the atomics
@@ -32,35 +32,25 @@
 namespace lookm {
 namespace {
 
-constexpr int kPerThread = 8;                        // consecutive tokens of a thread per pass
-
 __device__ __forceinline__ unsigned order_key(float s) {
     unsigned b = __float_as_uint(s);
     if (b == 0x80000000u) b = 0u;                        // -0 and +0 compare equal
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);   // larger float <=> larger key
 }
 
-// Exclusive block scan of two ints per thread; returns the block totals through ta / tb.
+// Sums of two ints per warp over the warps before the caller's, and over all (ta, tb).
 template <int kThreads>
-__device__ __forceinline__ void block_scan2(int a, int b, int& ea, int& eb, int& ta, int& tb, int (*warp_tot)[2]) {
+__device__ __forceinline__ void warp_scan2(int a, int b, int& ea, int& eb, int& ta, int& tb, int (*warp_tot)[2]) {
     constexpr int kWarps = kThreads / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int ia = a, ib = b;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int xa = __shfl_up_sync(0xffffffffu, ia, o);
-        const int xb = __shfl_up_sync(0xffffffffu, ib, o);
-        if (lane >= o) { ia += xa; ib += xb; }
-    }
     __syncthreads();                                     // protects warp_tot from the previous use
-    if (lane == 31) { warp_tot[warp][0] = ia; warp_tot[warp][1] = ib; }
+    if (lane == 0) { warp_tot[warp][0] = a; warp_tot[warp][1] = b; }
     __syncthreads();
-    // every warp adds the totals of the warps before it
     const int wa = lane < kWarps ? warp_tot[lane][0] : 0, wb = lane < kWarps ? warp_tot[lane][1] : 0;
     ta = __reduce_add_sync(0xffffffffu, wa);
     tb = __reduce_add_sync(0xffffffffu, wb);
-    ea = __reduce_add_sync(0xffffffffu, lane < warp ? wa : 0) + ia - a;
-    eb = __reduce_add_sync(0xffffffffu, lane < warp ? wb : 0) + ib - b;
+    ea = __reduce_add_sync(0xffffffffu, lane < warp ? wa : 0);
+    eb = __reduce_add_sync(0xffffffffu, lane < warp ? wb : 0);
 }
 
 // |row|^2 of the row whose sixteen 16-byte pieces the half-warp holds.
@@ -122,16 +112,18 @@ __device__ __forceinline__ void key_norms(const __nv_bfloat16* __restrict__ k, l
     }
 }
 
-// kThreads * 8 tokens per pass; the keys of the first kPasses passes stay in registers, those of later
-// ones are read again.
-template <int kThreads, int kPasses>
+// The first kThreads * kSteps tokens are shared out evenly: a warp has steps * 32 consecutive ones, a step
+// is one per lane, and their keys stay in registers.  Tokens beyond are read again in every step of the
+// bisection, and once more for the lists.
+template <int kThreads, int kSteps>
 __global__ void __launch_bounds__(kThreads)
 select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask,
               const Req* __restrict__ reqs, int n_select_blocks, int n_kv_heads, long long T,
               int* __restrict__ kept_idx, int* __restrict__ evict_idx, int* __restrict__ rank,
               const __nv_bfloat16* __restrict__ keys, long long stride_tok, long long stride_head,
               float* __restrict__ rnorm_all) {
-    constexpr int kWarps = kThreads / 32, kPass = kThreads * kPerThread;
+    constexpr int kWarps = kThreads / 32, kChunk = kThreads * kSteps;
+    static_assert(kSteps % 8 == 0 && kSteps <= 32, "steps are skipped by eights; a bit per step");
     __shared__ int warp_tot[kWarps][2];
     __shared__ int counts[2][32];
     __shared__ unsigned extremes[2][32];
@@ -161,25 +153,25 @@ select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask
     };
 
     // ---- keys and classes of this thread's tokens --------------------------------------------------
-    unsigned key[kPasses][kPerThread];
-    unsigned img[kPasses];                               // bit q: candidate q of the pass is an image token
-    int cnt = 0;                                         // text candidates
+    const int steps = min(kSteps, (L + kThreads - 1) / kThreads);
+    const int first = warp * steps * 32 + lane;          // token of step q: first + 32 q
+    unsigned key[kSteps];
+    unsigned img = 0u;                                   // bit q: candidate of step q is an image token
+    auto load = [&](int j0) {
 #pragma unroll
-    for (int p = 0; p < kPasses; ++p) {
-        img[p] = 0u;
-#pragma unroll
-        for (int q = 0; q < kPerThread; ++q) {
-            const int j = p * kPass + threadIdx.x * kPerThread + q;
-            key[p][q] = 0u;
-            if (j < nc) {
-                key[p][q] = order_key(s[j]);
-                const bool im = is_image(j);
-                img[p] |= (im ? 1u : 0u) << q;
-                cnt += !im;
+        for (int q = 0; q < kSteps; ++q) {
+            const int j = j0 + q * 32;
+            key[q] = 0u;
+            if (q < steps && j < nc) {
+                key[q] = order_key(s[j]);
+                img |= (is_image(j) ? 1u : 0u) << q;
             }
         }
-    }
-    for (int j = kPasses * kPass + threadIdx.x; j < nc; j += kThreads) cnt += !is_image(j);
+    };
+    load(first);
+    // text candidates: candidates less image tokens among them
+    int cnt = min(steps, max(0, (nc - first + 31) / 32)) - __popc(img);
+    for (int j = kChunk + threadIdx.x; j < nc; j += kThreads) cnt += !is_image(j);
     const int n_text = block_sum(cnt);
     // class whose members are ranked (1 = image); the other class is kept entirely or not at all
     const int sel_cls = (n_text <= N) ? 1 : 0;
@@ -195,14 +187,12 @@ select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask
         // members keep their key, everything else gets 0 (no finite score maps to it)
         unsigned lo = 0xffffffffu, hi = 0u;
 #pragma unroll
-        for (int p = 0; p < kPasses; ++p)
-#pragma unroll
-            for (int q = 0; q < kPerThread; ++q) {
-                const bool member = p * kPass + (int)threadIdx.x * kPerThread + q < nc && ((img[p] >> q) & 1u) == (unsigned)sel_cls;
-                if (!member) key[p][q] = 0u;
-                if (member) { lo = min(lo, key[p][q]); hi = max(hi, key[p][q]); }
-            }
-        for (int j = kPasses * kPass + threadIdx.x; j < nc; j += kThreads)
+        for (int q = 0; q < kSteps; ++q) {
+            const bool member = q < steps && first + q * 32 < nc && ((img >> q) & 1u) == (unsigned)sel_cls;
+            if (!member) key[q] = 0u;
+            if (member) { lo = min(lo, key[q]); hi = max(hi, key[q]); }
+        }
+        for (int j = kChunk + threadIdx.x; j < nc; j += kThreads)
             if (is_image(j) == (sel_cls != 0)) { const unsigned x = order_key(s[j]); lo = min(lo, x); hi = max(hi, x); }
         lo = __reduce_min_sync(0xffffffffu, lo);
         hi = __reduce_max_sync(0xffffffffu, hi);
@@ -216,10 +206,11 @@ select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask
             const unsigned mid = lo + (hi - lo) / 2u + 1u;
             int c = 0;
 #pragma unroll
-            for (int p = 0; p < kPasses; ++p)
+            for (int g = 0; g < kSteps; g += 8)
+                if (g < steps)
 #pragma unroll
-                for (int q = 0; q < kPerThread; ++q) c += key[p][q] >= mid;
-            for (int j = kPasses * kPass + threadIdx.x; j < nc; j += kThreads)
+                    for (int q = g; q < g + 8; ++q) c += key[q] >= mid;
+            for (int j = kChunk + threadIdx.x; j < nc; j += kThreads)
                 c += is_image(j) == (sel_cls != 0) && order_key(s[j]) >= mid;
             c = block_sum(c);
             if (c == k) { thr = mid - 1u; exact = true; }
@@ -233,52 +224,41 @@ select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask
     const long long kept_base = rq.kept_off + (long long)h * B;
     const long long ev_base = rq.ev_off + (long long)h * rq.E;
     int* rk = rank ? rank + (long long)h * T + rq.tok_begin : nullptr;
+    const unsigned lt_mask = (1u << lane) - 1u;
     int kept_run = 0, tie_run = 0;
-    for (int p = 0; p * kPass < L; ++p) {
-        unsigned key_p[kPerThread], img_p = 0u;
-        const int j0 = p * kPass + threadIdx.x * kPerThread;
-        bool cached = false;
+    for (int c0 = 0; c0 < L; c0 += kChunk) {             // (steps == kSteps if there is more than one turn)
+        const int j0 = c0 + first;
+        if (c0) { img = 0u; load(j0); }
+        unsigned keep = 0u, tie = 0u;                    // bit q: token of step q
 #pragma unroll
-        for (int pp = 0; pp < kPasses; ++pp)
-            if (pp == p) {
-                cached = true;
-                img_p = img[pp];
-#pragma unroll
-                for (int q = 0; q < kPerThread; ++q) key_p[q] = key[pp][q];
-            }
-        if (!cached) {
-#pragma unroll
-            for (int q = 0; q < kPerThread; ++q) {
-                key_p[q] = 0u;
-                if (j0 + q < nc) { key_p[q] = order_key(s[j0 + q]); img_p |= (is_image(j0 + q) ? 1u : 0u) << q; }
-            }
-        }
-        unsigned keep = 0u, tie = 0u;                    // bit q: token j0 + q
-#pragma unroll
-        for (int q = 0; q < kPerThread; ++q) {
-            const int j = j0 + q;
-            if (j >= L) continue;
+        for (int q = 0; q < kSteps; ++q) {
+            const int j = j0 + q * 32;
+            if (q >= steps || j >= L) continue;
             if (j >= nc) keep |= 1u << q;
-            else if (((img_p >> q) & 1u) != (unsigned)sel_cls) keep |= (other_kept ? 1u : 0u) << q;
+            else if (((img >> q) & 1u) != (unsigned)sel_cls) keep |= (other_kept ? 1u : 0u) << q;
             else if (take_all) keep |= 1u << q;
             else if (!take_none) {
-                if (key_p[q] > thr) keep |= 1u << q;
-                else if (key_p[q] == thr) tie |= 1u << q;
+                if (key[q] > thr) keep |= 1u << q;
+                else if (key[q] == thr) tie |= 1u << q;
             }
         }
         // a tie is kept while fewer than need_ties equal keys precede it, so the kept ones before a
         // token are the sure ones before it and min(need_ties, ties before it)
-        int e_keep, e_tie, t_keep, t_tie;
-        block_scan2<kThreads>(__popc(keep), __popc(tie), e_keep, e_tie, t_keep, t_tie, warp_tot);
-        int sure = kept_run + e_keep, ties = tie_run + e_tie;
+        int sure, ties, t_keep, t_tie;
+        warp_scan2<kThreads>(__reduce_add_sync(0xffffffffu, __popc(keep)), __reduce_add_sync(0xffffffffu, __popc(tie)), sure, ties,
+                             t_keep, t_tie, warp_tot);
+        sure += kept_run;
+        ties += tie_run;
 #pragma unroll
-        for (int q = 0; q < kPerThread; ++q) {
-            const int j = j0 + q;
-            const int slot = sure + min(need_ties, ties);
-            const bool is_tie = (tie >> q) & 1u;
-            const bool kept = ((keep >> q) & 1u) || (is_tie && ties < need_ties);
+        for (int q = 0; q < kSteps; ++q) {
+            if (q >= steps) continue;
+            const int j = j0 + q * 32;
+            const bool is_keep = (keep >> q) & 1u, is_tie = (tie >> q) & 1u;
+            const unsigned keeps = __ballot_sync(0xffffffffu, is_keep), tied = __ballot_sync(0xffffffffu, is_tie);
+            const int before = ties + __popc(tied & lt_mask);
+            const int slot = sure + __popc(keeps & lt_mask) + min(need_ties, before);
             if (j < L) {
-                if (kept) {
+                if (is_keep || (is_tie && before < need_ties)) {
                     kept_idx[kept_base + slot] = j;
                     if (rk) rk[j] = -1 - slot;
                 } else {
@@ -287,8 +267,8 @@ select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask
                     if (rk) rk[j] = e;
                 }
             }
-            sure += (keep >> q) & 1u;
-            ties += is_tie;
+            sure += __popc(keeps);
+            ties += __popc(tied);
         }
         kept_run += t_keep;
         tie_run += t_tie;
@@ -302,8 +282,8 @@ cudaError_t launch_select(const float* scores, const uint8_t* mask, const Req* r
                           const void* k_for_norms, long long stride_tok, long long stride_head,
                           float* rnorm_all, int num_sms, cudaStream_t stream) {
     const int n_select = n_kv_heads * n_req;
-    // one pass of eight tokens per thread as long as 1024 threads can hold the prompt, with fewer
-    // threads (cheaper barriers) for short ones; up to 32768 tokens stay in registers
+    // eight tokens per thread as long as 1024 threads can hold the prompt, with fewer threads (cheaper
+    // barriers) for short ones; up to 32768 tokens stay in registers
     const int threads = max_L <= 2048 ? 256 : 1024;
     int n_norm = 0;
     if (k_for_norms) {
@@ -315,7 +295,7 @@ cudaError_t launch_select(const float* scores, const uint8_t* mask, const Req* r
         // norms: then a full wave of norm CTAs follows the selection CTAs instead)
         n_norm = (int)std::min<long long>(want, (long long)per_sm * (n_select < num_sms / 2 ? num_sms - n_select : num_sms));
     }
-    auto kernel = max_L <= 2048 ? select_kernel<256, 1> : max_L <= 8192 ? select_kernel<1024, 1> : select_kernel<1024, 4>;
+    auto kernel = max_L <= 2048 ? select_kernel<256, 8> : max_L <= 8192 ? select_kernel<1024, 8> : select_kernel<1024, 32>;
     return launch_chained(kernel, dim3(n_select + n_norm), dim3(threads), 0, stream,
                           scores, mask, reqs, n_select, n_kv_heads, T, kept_idx, evict_idx, rank,
                           (const __nv_bfloat16*)k_for_norms, stride_tok, stride_head, rnorm_all);
