@@ -17,8 +17,8 @@
 // The kernel is bound by the latency of one CTA's barriers and round trips.  A four-pass radix select
 // over a shared-memory histogram (its first digits nearly equal for all scores, so that the atomics
 // collide), two block scans and a second reading of the scores for the lists took, lookm_select with
-// 32 heads and in us, 14.4 at 700 tokens, 18.5 at 4096 and 22.6 at 8192; this takes 9.3, 14.4 and 22.6
-// (32768 tokens x 8 heads: 80 -> 69).
+// 32 heads and in us, 14.4 at 700 tokens, 18.5 at 4096 and 22.6 at 8192; this takes 9.3, 12.3 and 14.4 (32768
+// tokens x 8 heads with the norms: 80 -> 50).
 //
 // The selection occupies only n_requests * n_kv_heads CTAs, so the same launch carries, in further
 // CTAs, work that does not depend on it and is needed next: 1 / |k| of every key row (the cosine
@@ -53,8 +53,8 @@ __device__ __forceinline__ void warp_scan2(int a, int b, int& ea, int& eb, int& 
     eb = __reduce_add_sync(0xffffffffu, lane < warp ? wb : 0);
 }
 
-// |row|^2 of the row whose sixteen 16-byte pieces the half-warp holds.
-__device__ __forceinline__ float row_square(const uint4& u) {
+// A lane's share of |row|^2: the squares of its eight elements.
+__device__ __forceinline__ float sum_squares(const uint4& u) {
     const unsigned w[4] = {u.x, u.y, u.z, u.w};
     float ss = 0.f;
 #pragma unroll
@@ -63,52 +63,62 @@ __device__ __forceinline__ float row_square(const uint4& u) {
         ss = fmaf(lo, lo, ss);
         ss = fmaf(hi, hi, ss);
     }
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o, 16);
     return ss;
 }
 
 // 1 / |k| of every key row (0 for a zero row): half a warp per row, 16 bytes per lane, four rows
 // in flight per half-warp (the loop is bound by memory latency otherwise).  Row r is token
-// r / n_kv_heads of head r % n_kv_heads; the quotient and remainder are carried along instead of
-// divided out every time.
+// r / n_kv_heads of head r % n_kv_heads; quotient, remainder and address are carried along instead of
+// computed every time.  The four rows are added up together, each ending in a quarter of the half-warp,
+// so that one root and one division serve all of them (with four sums over the half-warp and four of
+// these the loop was bound by instructions; the launch takes, before and after, 28.6 and 20.5 us with 8192
+// tokens x 32 heads, 66.6 and 49.6 with 16384 x 40, 437 and 317 with 16 prompts, 153000 tokens x 32).
 template <int kThreads>
 __device__ __forceinline__ void key_norms(const __nv_bfloat16* __restrict__ k, long long stride_tok,
                                           long long stride_head, int n_kv_heads, long long T,
                                           float* __restrict__ rnorm_all, int block, int n_blocks) {
     constexpr int kRowsPerBlock = kThreads / 16;
-    constexpr int kFlight = 4;
     const int half = threadIdx.x >> 4, l16 = threadIdx.x & 15;
     const long long n_rows = T * n_kv_heads;
     const long long step = (long long)n_blocks * kRowsPerBlock;      // rows between two of my rows
     const long long step_tok = step / n_kv_heads;
     const int step_h = (int)(step % n_kv_heads);
+    const long long step_at = step_tok * stride_tok + step_h * stride_head, wrap_at = stride_tok - n_kv_heads * stride_head;
+    const long long step_out = step_h * T + step_tok, wrap_out = 1 - n_kv_heads * T;
     long long r = (long long)block * kRowsPerBlock + half;
-    long long tok = r / n_kv_heads;
+    const long long tok = r / n_kv_heads;
     int h = (int)(r % n_kv_heads);
+    const __nv_bfloat16* at = k + tok * stride_tok + h * stride_head + l16 * 8;
+    long long out = h * T + tok;
+    const bool bit8 = l16 & 8, bit4 = l16 & 4;
     // the loop bound is the warp's first row, so that both half-warps always reach the shuffles
-    for (long long rw = r - (half & 1); rw < n_rows; rw += kFlight * step) {
-        uint4 u[kFlight];
-        long long tok_i[kFlight];
-        int h_i[kFlight];
-        bool valid[kFlight];
+    for (long long rw = r - (half & 1); rw < n_rows; rw += 4 * step) {
+        uint4 u[4];
+        long long mine = -1;                             // where this lane's quarter's row goes
 #pragma unroll
-        for (int i = 0; i < kFlight; ++i) {
-            valid[i] = r < n_rows;
-            tok_i[i] = tok;
-            h_i[i] = h;
+        for (int i = 0; i < 4; ++i) {
             u[i] = make_uint4(0u, 0u, 0u, 0u);
-            if (valid[i]) u[i] = *reinterpret_cast<const uint4*>(k + tok * stride_tok + h * stride_head + l16 * 8);
+            if (r < n_rows) {
+                u[i] = *reinterpret_cast<const uint4*>(at);
+                if (l16 == i * 4) mine = out;
+            }
             r += step;
-            tok += step_tok;
+            at += step_at;
+            out += step_out;
             h += step_h;
-            if (h >= n_kv_heads) { h -= n_kv_heads; ++tok; }
+            if (h >= n_kv_heads) { h -= n_kv_heads; at += wrap_at; out += wrap_out; }
         }
+        float x[4];
 #pragma unroll
-        for (int i = 0; i < kFlight; ++i) {
-            const float ss = row_square(u[i]);
-            if (l16 == 0 && valid[i]) rnorm_all[(long long)h_i[i] * T + tok_i[i]] = ss > 0.f ? 1.0f / sqrtf(ss) : 0.f;
-        }
+        for (int i = 0; i < 4; ++i) x[i] = sum_squares(u[i]);
+        // lanes with bit 8 take rows 2 and 3, of these lanes with bit 4 rows 1 and 3
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            x[i] = (bit8 ? x[i + 2] : x[i]) + __shfl_xor_sync(0xffffffffu, bit8 ? x[i] : x[i + 2], 8, 16);
+        float ss = (bit4 ? x[1] : x[0]) + __shfl_xor_sync(0xffffffffu, bit4 ? x[0] : x[1], 4, 16);
+        ss += __shfl_xor_sync(0xffffffffu, ss, 2, 16);
+        ss += __shfl_xor_sync(0xffffffffu, ss, 1, 16);
+        if (mine >= 0) rnorm_all[mine] = ss > 0.f ? 1.0f / sqrtf(ss) : 0.f;
     }
 }
 
