@@ -72,7 +72,7 @@ __device__ __forceinline__ float sum_squares(const uint4& u) {
 // computed every time.  The four rows are added up together, each ending in a quarter of the half-warp,
 // so that one root and one division serve all of them (with four sums over the half-warp and four of
 // these the loop was bound by instructions; the launch takes, before and after, 28.6 and 20.5 us with 8192
-// tokens x 32 heads, 66.6 and 49.6 with 16384 x 40, 437 and 317 with 16 prompts, 153000 tokens x 32).
+// tokens x 32 heads, 66.6 and 49.6 with 16384 x 40, 437 and 317 with 16 prompts, 158314 tokens x 32).
 template <int kThreads>
 __device__ __forceinline__ void key_norms(const __nv_bfloat16* __restrict__ k, long long stride_tok,
                                           long long stride_head, int n_kv_heads, long long T,
@@ -292,9 +292,10 @@ cudaError_t launch_select(const float* scores, const uint8_t* mask, const Req* r
                           const void* k_for_norms, long long stride_tok, long long stride_head,
                           float* rnorm_all, int num_sms, cudaStream_t stream) {
     const int n_select = n_kv_heads * n_req;
-    // eight tokens per thread as long as 1024 threads can hold the prompt, with fewer threads (cheaper
-    // barriers) for short ones; up to 32768 tokens stay in registers
-    const int threads = max_L <= 2048 ? 256 : 1024;
+    // cheaper barriers with fewer threads, a shorter chain of steps with more: a layer of 2048 tokens x 8
+    // heads takes 67.0 us with 256 threads, 64.9 with 512 and 65.8 with 1024, 2048 x 32 123, 119.5 and
+    // 119.5, 3000 x 8 85.1 with 512 and 84.2 with 1024; up to 32768 tokens stay in registers
+    const int threads = max_L <= 2048 ? 512 : 1024;
     int n_norm = 0;
     if (k_for_norms) {
         // the norm CTAs take the SMs that the selection leaves free, so that all of them run at once
@@ -305,7 +306,7 @@ cudaError_t launch_select(const float* scores, const uint8_t* mask, const Req* r
         // norms: then a full wave of norm CTAs follows the selection CTAs instead)
         n_norm = (int)std::min<long long>(want, (long long)per_sm * (n_select < num_sms / 2 ? num_sms - n_select : num_sms));
     }
-    auto kernel = max_L <= 2048 ? select_kernel<256, 8> : max_L <= 8192 ? select_kernel<1024, 8> : select_kernel<1024, 32>;
+    auto kernel = max_L <= 2048 ? select_kernel<512, 8> : max_L <= 8192 ? select_kernel<1024, 8> : select_kernel<1024, 32>;
     return launch_chained(kernel, dim3(n_select + n_norm), dim3(threads), 0, stream,
                           scores, mask, reqs, n_select, n_kv_heads, T, kept_idx, evict_idx, rank,
                           (const __nv_bfloat16*)k_for_norms, stride_tok, stride_head, rnorm_all);
