@@ -74,6 +74,12 @@ constexpr int kFullRing = 2 * kAccum;
 constexpr int kIssuers = 2;                      // MMA-issuing threads (tiles alternate between them)
 constexpr int kEpiWarp0 = 2;                     // first epilogue warp
 constexpr int kGatherWarp = kEpiWarp0 + kParts * 4 + 1;    // match: gathers the evicted rows of the A tiles
+// Match: items of at most so many tiles wait for their stationary rows, so the gather warp sends all its
+// copies at once; with longer items, one ahead of the MMAs, it reads positions and sends copies in eights,
+// which leaves the streamed tiles more room.  Match in us, in eights and at once: 2 tiles an item (700
+// tokens x 32 heads) 16.4 and 14.3, 4 tiles (7777 x 8 at 5 %) 32.7 and 26.6, (2048 x 32) 24.6 and 20.5, 7
+// tiles (4096 x 32) 47 and 57, 13 tiles (8192 x 32) 126 and 155.
+constexpr int kBurstTiles = 4;
 // producer warp, MMA warp, kParts x 4 epilogue warps, second MMA warp (+ the gather warp of the match)
 __host__ __device__ constexpr int threads_of(int kind) { return 64 + kParts * 128 + 32 + (kind == kMatch ? 32 : 0); }
 constexpr int kHalfBytes = kTile * 64 * 2;       // one TMA box: 128 rows x 64 bf16 (128 B rows)
@@ -433,16 +439,36 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             const int n_rows = min(kTile, it.E - it.blk * kTile);
             const char* src0 = reinterpret_cast<const char*>(p.k_rows) +
                                2 * ((long long)it.tok_begin * p.k_stride_tok + (long long)it.head * p.k_stride_head) + l16 * 16;
-#pragma unroll 8
-            for (int st = 0; st < kTile / 2; ++st) {
+            const auto copy_rows = [&](int st, int pos) {            // rows 2 st and 2 st + 1
                 const int r = 2 * st + (lane >> 4);
-                const bool valid = r < n_rows;
-                int pos = valid ? __ldg(ev + r) : 0;
-                if (pos < 0 || pos >= it.L) { atomicExch(p.status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); pos = 0; }
                 const char* src = src0 + 2 * (long long)pos * p.k_stride_tok;
                 const uint32_t dst = adst + r * 128 + ((c8 ^ (r & 7)) << 4);
-                const int nbytes = valid ? 16 : 0;
+                const int nbytes = r < n_rows ? 16 : 0;
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(nbytes) : "memory");
+            };
+            const auto checked = [&](int pos) {
+                if (pos >= 0 && pos < it.L) return pos;
+                atomicExch(p.status, (int)LOOKM_ERR_DEVICE_BAD_INDEX);
+                return 0;
+            };
+            if (it.nt <= kBurstTiles) {
+                // all positions first, four per lane, so that all the copies go out together
+                int at[kTile / 32];
+#pragma unroll
+                for (int j = 0; j < kTile / 32; ++j) at[j] = j * 32 + lane < n_rows ? __ldg(ev + j * 32 + lane) : 0;
+#pragma unroll
+                for (int j = 0; j < kTile / 32; ++j) {
+                    const int mine = checked(at[j]);
+#pragma unroll
+                    for (int st = 16 * j; st < 16 * j + 16; ++st)
+                        copy_rows(st, __shfl_sync(0xffffffffu, mine, (2 * st + (lane >> 4)) & 31));
+                }
+            } else {
+#pragma unroll 8
+                for (int st = 0; st < kTile / 2; ++st) {
+                    const int r = 2 * st + (lane >> 4);
+                    copy_rows(st, checked(r < n_rows ? __ldg(ev + r) : 0));
+                }
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
             asm volatile("cp.async.wait_group 0;" ::: "memory");
