@@ -700,9 +700,12 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             const int combiner = static_cast<int>((gb - 1u) % kGroups) * kHalves + (kHalves - 1);
             float (*cb)[Shared<KIND>::kPlanes][kTile] = sh.comb[cslot];
             constexpr int kP1 = Shared<KIND>::kPlanes - 1;       // second value of a row (not in sweep 2)
+            // The buffer's previous contents (two items ago) have been read.  The combining part waits for
+            // this too: the parity of comb_full tells one use from the next only once the use before is
+            // over, and a warp may come here ahead of others that have yet to arrive for that one (groups
+            // without a tile in short items hold nobody back).
+            ptx::mbar_wait(ptx::smem_u32(&sh.comb_free[cslot]), (cuse & 1u) ^ 1u, abort_flag);
             if (part != combiner) {
-                // the buffer's previous contents (two items ago) have been read
-                ptx::mbar_wait(ptx::smem_u32(&sh.comb_free[cslot]), (cuse & 1u) ^ 1u, abort_flag);
                 if (KIND == kSweep1) { cb[part][0][row] = m_run; cb[part][kP1][row] = l_run; }
                 else if (KIND == kSweep2) { cb[part][0][row] = (acc[0] + acc[1]) + (acc[2] + acc[3]); }
                 else { cb[part][0][row] = best; cb[part][kP1][row] = __int_as_float(best_slot); }
@@ -1163,8 +1166,9 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             ++nh;
             float (*cb)[kTile] = sh.comb[buf][half & 1];
             constexpr int kP1 = Sh::kPlanes - 1;
+            // (both groups wait until the buffer's use before this one is over: see tile_kernel)
+            ptx::mbar_wait(ptx::smem_u32(&sh.comb_free[half & 1][buf]), (use & 1u) ^ 1u, abort_flag);
             if ((int)((gb0 + t_end - 1) & 1u) != parity) {
-                ptx::mbar_wait(ptx::smem_u32(&sh.comb_free[half & 1][buf]), (use & 1u) ^ 1u, abort_flag);
                 if (KIND == kSweep1) { cb[0][row] = m_run; cb[kP1][row] = l_run; }
                 else cb[0][row] = total;
                 __syncwarp();

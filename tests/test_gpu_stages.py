@@ -169,6 +169,32 @@ def test_scores_of_items_of_two_or_four_blocks(B, lens, Hq, Hkv):
         assert np.allclose(lse[qs, a:a + n].cpu().numpy().reshape(len(heads), g, n), lse_o, rtol=1e-6, atol=2e-5)
 
 
+@pytest.mark.parametrize("Hq,Hkv", [(4, 2), (16, 16), (40, 8), (64, 32)])
+def test_scores_of_many_short_prompts_of_one_to_three_blocks(B, Hq, Hkv):
+    """Items in which some epilogue groups have no tile, one after another: which group adds up a block
+    changes from item to item and nothing but the barriers of the combination orders them.  More requests
+    than the kernels cache in shared memory; every repetition must give the same bits."""
+    import torch
+    lens = [256, 128, 256, 130, 129, 256, 1, 384] * 5
+    T, cu = sum(lens), np.concatenate([[0], np.cumsum(lens)]).tolist()
+    qb = synth.f32_to_bf16_bits(synth.normal(synth.stream_key(153, Hq), T * Hq * 128).reshape(T, Hq, 128).astype(np.float32))
+    kb = synth.f32_to_bf16_bits(synth.normal(synth.stream_key(154, Hq), T * Hkv * 128).reshape(T, Hkv, 128).astype(np.float32))
+    q, k = to_dev(qb), to_dev(kb)
+    lay = B.make_layout(q, k)
+    ws = B.alloc_workspace(lay, lens)
+    scores, lse = torch.zeros(Hkv, T, device="cuda"), torch.zeros(Hq, T, device="cuda")
+    B.check(B.lookm_score(q, k, cu, lay, scores, lse, False, ws))
+    for _ in range(20):
+        again, lse2 = torch.zeros_like(scores), torch.zeros_like(lse)
+        B.check(B.lookm_score(q, k, cu, lay, again, lse2, False, ws))
+        assert torch.equal(scores, again) and torch.equal(lse, lse2)
+    assert B.lookm_device_status(ws) == B.OK
+    for a, n in zip(cu, lens):
+        A, lse_o = orc.scores(synth.bf16_to_f32(qb[a:a + n]), synth.bf16_to_f32(kb[a:a + n]), threads=8, want_lse=True)
+        assert np.all(np.abs(scores[:, a:a + n].cpu().numpy().astype(np.float64) - A) <= 2e-5 * A)
+        assert np.allclose(lse[:, a:a + n].cpu().numpy().reshape(Hkv, Hq // Hkv, n), lse_o, atol=2e-5, rtol=0)
+
+
 def test_scores_packed_batch_equals_separate_requests(B):
     import torch
     lens = [200, 131, 1, 400]
