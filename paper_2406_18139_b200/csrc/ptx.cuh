@@ -52,8 +52,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 // `*abort_flag` (shared memory); on giving up it raises the flag itself and returns false.  The
 // callers then carry on through the rest of their protocol without waiting, so that every role
 // still reaches the end of the kernel, where TMEM is released and the status word is written.
+constexpr uint64_t kWaitLimitNs = 2000000000ull;
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                          uint64_t limit_ns = 2000000000ull) {
+                                          uint64_t limit_ns = kWaitLimitNs) {
     if (mbar_try_wait(bar, parity)) return true;
     if (*abort_flag) return false;
     const uint64_t t0 = globaltimer_ns();

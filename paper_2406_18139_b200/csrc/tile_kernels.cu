@@ -821,6 +821,24 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 // result: a block's tiles are added in their order, two blocks per item in the two parities of the
 // tile's index in the item.
 // ------------------------------------------------------------------------------------------------
+// Items announced to the roles of a CTA, -1: no more.
+struct ItemRing {
+    unsigned long long full[kItemRing], empty[kItemRing];
+    int items[kItemRing];
+};
+// The n-th announced item; -1 at the end, and after the wait has given up.  For one thread ...
+__device__ __forceinline__ int wait_item(ItemRing& ring, int n, volatile int* abort_flag, uint64_t limit_ns = ptx::kWaitLimitNs) {
+    if (!ptx::mbar_wait(ptx::smem_u32(&ring.full[n % kItemRing]), (n / kItemRing) & 1, abort_flag, limit_ns)) return -1;
+    return *reinterpret_cast<volatile int*>(&ring.items[n % kItemRing]);
+}
+// ... and for a warp: lane 0 waits and the others follow its verdict (lanes that gave up one by one
+// could leave the rest behind in the next warp-wide instruction).
+__device__ __forceinline__ int warp_wait_item(ItemRing& ring, int n, volatile int* abort_flag, uint64_t limit_ns = ptx::kWaitLimitNs) {
+    int item = 0;
+    if ((threadIdx.x & 31) == 0) item = wait_item(ring, n, abort_flag, limit_ns);
+    return __shfl_sync(0xffffffffu, item, 0);
+}
+
 template <int KIND, int kBlocks>
 struct __align__(1024) MultiShared {
     static constexpr int kRing = kBlocks == 2 ? 4 : 2;   // streamed tiles
@@ -837,8 +855,7 @@ struct __align__(1024) MultiShared {
     unsigned long long t_full[kAccum], t_empty[kAccum];
     unsigned long long comb_full[2][2], comb_free[2][2];     // [half][buffer]
     unsigned long long mma_done;
-    unsigned long long item_full[kItemRing], item_empty[kItemRing];
-    int items[kItemRing];                        // announced items, -1: no more
+    ItemRing ring;
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -946,8 +963,8 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         }
         ptx::mbar_init(ptx::smem_u32(&sh.mma_done), kIssuers);
         for (int i = 0; i < kItemRing; ++i) {
-            ptx::mbar_init(ptx::smem_u32(&sh.item_full[i]), 1);
-            ptx::mbar_init(ptx::smem_u32(&sh.item_empty[i]), kIssuers + 16);         // MMA threads, epilogue warps
+            ptx::mbar_init(ptx::smem_u32(&sh.ring.full[i]), 1);
+            ptx::mbar_init(ptx::smem_u32(&sh.ring.empty[i]), kIssuers + 16);         // MMA threads, epilogue warps
         }
         sh.abort_flag = 0;
         ptx::fence_mbar_init();
@@ -968,12 +985,7 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = sh.tmem_base;
-    // the n-th announced item for a role; -1 at the end, and after a wait has given up
-    auto wait_item = [&](int n) {
-        if (!ptx::mbar_wait(ptx::smem_u32(&sh.item_full[n % kItemRing]), (n / kItemRing) & 1, abort_flag)) return -1;
-        return *reinterpret_cast<volatile int*>(&sh.items[n % kItemRing]);
-    };
-    auto release_item = [&](int n) { ptx::mbar_arrive(ptx::smem_u32(&sh.item_empty[n % kItemRing])); };
+    auto release_item = [&](int n) { ptx::mbar_arrive(ptx::smem_u32(&sh.ring.empty[n % kItemRing])); };
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer ----------
@@ -986,9 +998,9 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             bool stop = false;                       // a wait gave up: arm nothing more
             int item = blockIdx.x;                   // the grid has at most n_items CTAs
             for (int n = 0; !stop; ++n) {
-                if (!ptx::mbar_wait(ptx::smem_u32(&sh.item_empty[n % kItemRing]), ((n / kItemRing) & 1) ^ 1, abort_flag)) break;
-                sh.items[n % kItemRing] = item < p.n_items ? item : -1;
-                ptx::mbar_arrive(ptx::smem_u32(&sh.item_full[n % kItemRing]));
+                if (!ptx::mbar_wait(ptx::smem_u32(&sh.ring.empty[n % kItemRing]), ((n / kItemRing) & 1) ^ 1, abort_flag)) break;
+                sh.ring.items[n % kItemRing] = item < p.n_items ? item : -1;
+                ptx::mbar_arrive(ptx::smem_u32(&sh.ring.full[n % kItemRing]));
                 if (item >= p.n_items) break;
                 const MultiItem it = decode_multi<KIND, kBlocks>(p, tbl, item);
                 item = (int)gridDim.x + atomicAdd(p.next_item, 1);   // wanted after this item's loads
@@ -1038,7 +1050,7 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             uint32_t gb = 0, na[2] = {0, 0}, used[2] = {0, 0};
             bool stop = false;
             for (int n = 0; !stop; ++n) {
-                const int item = wait_item(n);
+                const int item = wait_item(sh.ring, n, abort_flag);
                 if (item < 0) break;
                 release_item(n);
                 const MultiItem it = decode_multi<KIND, kBlocks>(p, tbl, item);
@@ -1103,9 +1115,8 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         const float c2 = p.scale_log2;
         uint32_t gb = 0, used = 0, nh = 0;                   // streamed tiles, own tiles, items with this half
         for (int n = 0;; ++n) {
-            const int item = wait_item(n);
+            const int item = warp_wait_item(sh.ring, n, abort_flag);
             if (item < 0) break;
-            __syncwarp();
             if (lane == 0) release_item(n);
             const MultiItem it = decode_multi<KIND, kBlocks>(p, tbl, item);
             const uint32_t gb0 = gb;
@@ -1201,23 +1212,28 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
 }
 
 // The failure path of the bounded waits, exercised without starving a production kernel: thread 0
-// waits with ptx::mbar_wait on an mbarrier that nobody arrives at, the other threads on the same
-// barrier see either the limit or the abort flag, and the CTA reports the expiry exactly as
+// waits with ptx::mbar_wait on an mbarrier that nobody arrives at, warp 0's other threads on the same
+// barrier see either the limit or the abort flag, the other warps wait like multi_kernel's epilogue for an
+// item that nobody announces and must leave together, and the CTA reports the expiry exactly as
 // tile_kernel does (shared abort flag -> status word).
 __global__ void __launch_bounds__(128)
 wait_probe_kernel(unsigned long long limit_ns, int* status) {
     __shared__ unsigned long long bar;
+    __shared__ ItemRing ring;
     __shared__ int abort_flag;
     if (threadIdx.x == 0) {
         ptx::mbar_init(ptx::smem_u32(&bar), 1);
+        for (int i = 0; i < kItemRing; ++i) ptx::mbar_init(ptx::smem_u32(&ring.full[i]), 1);
         abort_flag = 0;
         ptx::fence_mbar_init();
     }
     __syncthreads();
     volatile int* flag = &abort_flag;
-    const bool arrived = ptx::mbar_wait(ptx::smem_u32(&bar), 0, flag, limit_ns);
-    __syncthreads();
-    if (threadIdx.x == 0 && (abort_flag || !arrived)) atomicExch(status, (int)LOOKM_ERR_DEVICE_TIMEOUT);
+    bool arrived;
+    if (threadIdx.x < 32) arrived = ptx::mbar_wait(ptx::smem_u32(&bar), 0, flag, limit_ns);
+    else arrived = __any_sync(0xffffffffu, warp_wait_item(ring, 0, flag, limit_ns) >= 0);
+    if (__syncthreads_or(arrived)) return;                   // (nobody arrives: the status word then says that nothing expired)
+    if (threadIdx.x == 0) atomicExch(status, (int)LOOKM_ERR_DEVICE_TIMEOUT);
 }
 
 }  // namespace
