@@ -43,7 +43,6 @@ struct Plan {
     int tail_begin[2] = {0, 0};             // for the end, and the first item of these
     size_t n_arrived[2] = {0, 0};           // their arrival counters
     size_t clear_words = 64;                // status word and arrival counters
-    size_t o_parts1 = 0, o_parts2 = 0;
     size_t o_status, o_reqs, o_lse, o_lse_split, o_scores, o_rank, o_rnorm_all, o_kept, o_evict, o_kept_keys,
         o_rnorm_kept, o_assign, o_sim, o_row_ptr, o_entries, o_units, o_slot_cnt, o_parts, o_sort_a, o_sort_b,
         total;
@@ -92,6 +91,8 @@ void plan_splits(Plan& pl) {
         if (pl.blocks[s] == 1 && 2 * longest > 3 * mean && longest >= mean + 10)
             pl.splits[s] = (int)std::min<long long>(kMaxSplits, (longest + mean - 1) / mean);
     }
+    // (sweep 1's partial results, 8 bytes per range, query head and token, have room where the kept keys go)
+    pl.splits[0] = std::min(pl.splits[0], std::max(1, 2 * kHeadDim / (8 * pl.group)));
 }
 
 // Returns LOOKM_OK or the status describing the first bad argument.
@@ -199,12 +200,14 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
     auto carve = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
     const size_t Hq = pl.n_q_heads, Hkv = pl.n_kv_heads, T = (size_t)pl.T;
     // Every list is sized for the worst case over budgets (at most T kept and T evicted rows per
-    // head), so the carving depends only on the prompt lengths and head counts.
+    // head) and over how the sweeps are cut, so the carving depends only on the prompt lengths and head
+    // counts and never shrinks with more query heads: a size computed for a layout also serves the entry
+    // points that know its KV heads alone.
     const size_t score_parts = pl.blocks[1] > 1 ? pl.group : pl.splits[1];       // partial column sums of sweep 2
     for (int s = 0; s < 2; ++s)
         if (pl.splits[s] > 1 || (s && score_parts > 1)) pl.n_arrived[s] = 4 * (size_t)tiles * (s ? Hkv : Hq);
     pl.clear_words += pl.n_arrived[0] + pl.n_arrived[1];
-    pl.o_status = carve(4 * pl.clear_words);
+    pl.o_status = carve(4 * (64 + 4 * (size_t)tiles * (Hq + Hkv)));
     pl.o_reqs = carve(sizeof(Req) * n_req);
     pl.o_lse = carve(4 * Hq * T);
     pl.o_lse_split = carve(32 * Hq * T);
@@ -213,7 +216,9 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
     pl.o_rnorm_all = carve(4 * Hkv * T);
     pl.o_kept = carve(4 * Hkv * T);
     pl.o_evict = carve(4 * Hkv * T);
-    pl.o_kept_keys = carve(2 * (size_t)kHeadDim * Hkv * T);
+    // The kept keys are gathered after both sweeps are done; until then their place holds the sweeps'
+    // partial results: sweep 1's ranges (see plan_splits), sweep 2's ranges or query heads of a group.
+    pl.o_kept_keys = carve(std::max(2 * (size_t)kHeadDim * Hkv * T, 4 * Hq * T));
     pl.o_rnorm_kept = carve(4 * Hkv * T);
     pl.o_assign = carve(4 * Hkv * T);
     pl.o_sim = carve(4 * Hkv * T);
@@ -224,8 +229,6 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
     pl.o_parts = carve((size_t)kMergePartBytes * (size_t)pl.total_units);
     pl.o_sort_a = carve(8 * Hkv * T);
     pl.o_sort_b = carve(8 * Hkv * T);
-    pl.o_parts1 = carve(pl.splits[0] > 1 ? 8 * Hq * T * pl.splits[0] : 0);
-    pl.o_parts2 = carve(score_parts > 1 ? 4 * Hkv * T * score_parts : 0);
     pl.total = o;
     return LOOKM_OK;
 }
@@ -390,7 +393,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
         p.tail_begin = pl.tail_begin[0];
         p.tail_sets = pl.tail_sets[0];
         p.splits = pl.splits[0];
-        p.parts1 = at<float2>(ws, pl.o_parts1);
+        p.parts1 = at<float2>(ws, pl.o_kept_keys);
         p.arrived = p.status + 64;
         LOOKM_CUDA(launch_tile_kernel(kSweep1, map_q, map_k, nullptr, p, di.sms, st));
         ++g_launches;
@@ -405,7 +408,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     p.tail_begin = pl.tail_begin[1];
     p.tail_sets = pl.tail_sets[1];
     p.splits = pl.splits[1];
-    p.parts2 = at<float>(ws, pl.o_parts2);
+    p.parts2 = at<float>(ws, pl.o_kept_keys);
     p.arrived = p.status + 64 + pl.n_arrived[0];
     LOOKM_CUDA(launch_tile_kernel(kSweep2, map_k, map_q, &map_x, p, di.sms, st));
     ++g_launches;

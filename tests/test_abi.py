@@ -38,6 +38,18 @@ def test_strerror_and_workspace_size():
     assert B.lookm_workspace_size(_layout(), [100], [0]) == 0
 
 
+def test_a_workspace_for_grouped_queries_serves_the_entry_points_that_know_the_kv_heads_alone():
+    # lookm_select and lookm_match_from_sim are given n_kv_heads, not a layout: they plan as if each KV
+    # head had one query head, which may cut the sweeps in other ways
+    batches = [[6168], [6180], [3097], [1950], [1881, 4252, 8457, 3525], [556, 2389, 1813], [33], [16384], [200] * 40]
+    batches += [[n] for n in range(1000, 9000, 211)]
+    for lens in batches:
+        for hkv in (1, 2, 3, 4, 6, 8, 32):
+            stage = B.lookm_workspace_size(_layout(hkv, hkv), lens)
+            for group in (2, 3, 4, 8, 16, 128):
+                assert B.lookm_workspace_size(_layout(hkv * group, hkv), lens) >= stage, (lens, hkv, group)
+
+
 def test_host_side_argument_errors_need_no_device():
     lib = B.lib()
     lay = _layout()

@@ -297,6 +297,24 @@ def test_select_ties_and_duplicates_and_batches(B):
 
 # ------------------------------------------------------------------------------ matching -----
 
+def test_selection_and_argmax_on_a_workspace_sized_for_grouped_queries(B):
+    """With 4 query heads on 2 KV heads and 6168 tokens the two plan for more ranges than the layout has."""
+    import torch
+    torch.manual_seed(5)
+    L, Hq, Hkv, budget = 6168, 4, 2, 8
+    lay = B.Layout(Hq, Hkv, 128, Hq * 128, 128, Hkv * 128, 128, 0.0)
+    ws = B.alloc_workspace(lay, [L])
+    scores = torch.rand(Hkv, L, device="cuda")
+    kept, ev = (torch.empty(Hkv * n, dtype=torch.int32, device="cuda") for n in (budget, L - budget))
+    B.check(B.lookm_select(scores, None, [0, L], [budget], [0], Hkv, kept, ev, None, ws))
+    assert torch.equal(kept.view(Hkv, budget).long(), scores.topk(budget, dim=1).indices.sort(dim=1).values)
+    sim = torch.rand(Hkv, L - budget, budget, device="cuda")
+    assign, best = torch.empty_like(ev), torch.empty(Hkv * (L - budget), device="cuda")
+    B.check(B.lookm_match_from_sim(sim, [0, L], [budget], Hkv, assign, best, ws))
+    assert torch.equal(best, sim.amax(dim=2).flatten())
+    assert B.lookm_device_status(ws) == B.OK
+
+
 def test_match_from_sim_is_bit_exact(B):
     import torch
     Hkv, lens, budgets = 2, [90, 400], [20, 130]
