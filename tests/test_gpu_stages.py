@@ -422,6 +422,35 @@ def test_match_whole_blocks_single_rows_and_strided_keys(B, L, budget):
             assert S[e, a_ref[e]] - S[e, a_got[h, e]] <= 1e-4
 
 
+def test_match_of_many_short_prompts_one_kept_tile_each(B):
+    """Items of a single tile: three of the four epilogue groups have no tile in an item and may run ahead
+    of the one that has; every repetition must give the same bits, and no wait may run out."""
+    import torch
+    n_req, L, budget, Hkv = 40, 200, 40, 16
+    lens, cu = [L] * n_req, list(range(0, n_req * L + 1, L))
+    kb = synth.f32_to_bf16_bits(synth.normal(synth.stream_key(97), n_req * L * Hkv * 128).reshape(n_req * L, Hkv, 128).astype(np.float32))
+    k, kf = to_dev(kb), synth.bf16_to_f32(kb)
+    kept1, ev1 = np.arange(0, L, 5, dtype=np.int32), np.array([j for j in range(L) if j % 5], dtype=np.int32)
+    kept, ev = (torch.from_numpy(np.tile(x, n_req * Hkv)).cuda() for x in (kept1, ev1))
+    lay = B.make_layout(None, k)
+    ws = B.alloc_workspace(lay, lens)
+    first = None
+    for _ in range(20):
+        assign, sim = torch.full_like(ev, -7), torch.full((ev.numel(),), -7.0, device="cuda")
+        B.check(B.lookm_match(k, kept, ev, cu, [budget] * n_req, lay, assign, sim, ws))
+        first = first or (assign, sim)
+        assert torch.equal(assign, first[0]) and torch.equal(sim, first[1])
+    assert B.lookm_device_status(ws) == B.OK
+    a_got = first[0].cpu().numpy().reshape(n_req, Hkv, L - budget)
+    s_got = first[1].cpu().numpy().reshape(n_req, Hkv, L - budget).astype(np.float64)
+    for r in range(n_req):
+        for h in range(Hkv):
+            a_ref, s_ref, S = orc.match(kf[cu[r]:cu[r + 1]], h, kept1, ev1, want_matrix=True)
+            assert np.allclose(s_got[r, h], s_ref, atol=2e-6, rtol=0)
+            for e in np.where(a_got[r, h] != a_ref)[0]:
+                assert S[e, a_ref[e]] - S[e, a_got[r, h, e]] <= 1e-4
+
+
 def test_match_packed_batch_and_out_of_range_evicted_position(B):
     import torch
     Hkv = 2
