@@ -19,6 +19,7 @@
 //
 // Query heads that share a KV head go to decode_mma_kernel below, which has the same structure.
 #include <cuda_bf16.h>
+#include <float.h>
 #include <math.h>
 
 #include "internal.h"
@@ -476,8 +477,8 @@ decode_mma_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16
 #pragma unroll
         for (int c = 0; c < 4; ++c) o[j][c] = 0.f;
     // Reference (in units of the raw product, like the scalar kernel's) and sum (over this lane's keys) of the
-    // head.
-    float m = -INFINITY, l = 0.f;
+    // head.  The reference starts finite, so that logits of -inf met before any other count nothing.
+    float m = -FLT_MAX, l = 0.f;
     // ldmatrix: matrix i of an x4 is addressed by lanes 8i .. 8i + 7
     const int mi = lane >> 3, mr = lane & 7;
     const int k_row = (mi >> 1) * 8 + mr, k_chunk = mi & 1;      // K: (rows 0-7, 8-15) x (chunk, next chunk)
@@ -539,9 +540,12 @@ decode_mma_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16
             float t0[4] = {0.f, 0.f, 0.f, 0.f}, t1[4] = {0.f, 0.f, 0.f, 0.f};
             mma_bf16(t0, a0, a1, a2, a3, b[0], b[1]);
             mma_bf16(t1, a0, a1, a2, a3, b[2], b[3]);
-            if (GP == 8) {
-                mma_bf16(t0, 0u, c0, 0u, c2, b[0], b[1]);
-                mma_bf16(t1, 0u, c0, 0u, c2, b[2], b[3]);
+            if (GP == 8) {                           // (rows 0-7 of this product are zeros: only rows 8-15 are taken)
+                float u0[4] = {0.f, 0.f, 0.f, 0.f}, u1[4] = {0.f, 0.f, 0.f, 0.f};
+                mma_bf16(u0, 0u, c0, 0u, c2, b[0], b[1]);
+                mma_bf16(u1, 0u, c0, 0u, c2, b[2], b[3]);
+                t0[2] += u0[2], t0[3] += u0[3];
+                t1[2] += u1[2], t1[3] += u1[3];
             }
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
@@ -555,20 +559,24 @@ decode_mma_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16
     // ---- combine: the terms of a head in registers, then the warps in warp order -----------------
     l += __shfl_xor_sync(0xffffffffu, l, 1);
     l += __shfl_xor_sync(0xffffffffu, l, 2);
+    // The first term of a probability takes part on its own, the sum of the others is a correction: with
+    // an infinite value the first term's sum is the result (the others may be zero times infinity).
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
-        float y0 = o[j][0] + o[j][2], y1 = o[j][1] + o[j][3];
+        float y[2];
 #pragma unroll
-        for (int ofs = 16; ofs >= 4 * GP; ofs >>= 1) {           // rows lane / 4 of the same head
-            y0 += __shfl_xor_sync(0xffffffffu, y0, ofs);
-            y1 += __shfl_xor_sync(0xffffffffu, y1, ofs);
+        for (int c = 0; c < 2; ++c) {
+            float low = (part_lo > 0 && part_lo < 3 ? o[j][c] : 0.f) + (part_hi < 3 ? o[j][c + 2] : 0.f);
+#pragma unroll
+            for (int ofs = 16; ofs >= 4 * GP; ofs >>= 1) low += __shfl_xor_sync(0xffffffffu, low, ofs);      // rows lane / 4 of the same head
+            y[c] = isinf(o[j][c]) ? o[j][c] : o[j][c] + low;
         }
-        if ((lane >> 2) < GP) {
-            sh.o[warp][head][8 * j + 2 * (lane & 3)] = y0;
-            sh.o[warp][head][8 * j + 2 * (lane & 3) + 1] = y1;
+        if (part_lo == 0) {
+            sh.o[warp][head][8 * j + 2 * (lane & 3)] = y[0];
+            sh.o[warp][head][8 * j + 2 * (lane & 3) + 1] = y[1];
         }
     }
-    if ((lane >> 2) < GP && (lane & 3) == 0) { sh.m[warp][head] = m; sh.l[warp][head] = l; }
+    if (part_lo == 0 && (lane & 3) == 0) { sh.m[warp][head] = m; sh.l[warp][head] = l; }
     __syncthreads();
     // thread t owns feature t of every query head of the pass
     const int n_splits = rq.n_splits;
@@ -582,7 +590,7 @@ decode_mma_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16
         float lsum = 0.f, osum = 0.f;
 #pragma unroll
         for (int w = 0; w < kMmaWarps; ++w) {
-            const float a = mx == -INFINITY ? 0.f : dec_ex2((sh.m[w][g] - mx) * scale_log2);     // 0 for an idle warp
+            const float a = dec_ex2((sh.m[w][g] - mx) * scale_log2);             // (an idle warp's sums are 0)
             lsum = fmaf(sh.l[w][g], a, lsum);
             osum = fmaf(sh.o[w][g][t], a, osum);
         }

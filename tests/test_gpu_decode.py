@@ -107,6 +107,31 @@ def test_grouped_queries_are_as_precise_as_single_ones(B, Hq, Hkv, n, q_scale):
     assert err[0] <= 1.5 * err[1], err / 4
 
 
+@pytest.mark.parametrize("Hq,Hkv,n", [(2, 2, 300), (2, 1, 300), (4, 1, 300), (8, 1, 300), (12, 2, 3000), (4, 2, 9000), (16, 4, 40)])
+def test_logits_of_minus_infinity_and_infinite_values(B, Hq, Hkv, n):
+    """Rows whose logits overflow to -inf count nothing, also where a warp meets them first; an infinite
+    value makes its feature infinite and leaves the others alone.  One query head or several per row."""
+    import torch
+    k, v = (synth.bf16_to_f32(_bits((Hkv, n, 128), (870 + n, i))) for i in (1, 2))
+    q = np.abs(synth.bf16_to_f32(_bits((Hq, 128), (870 + n, 3)))) + 1.0
+    k[:, :n // 2] = -3e38                                 # q . k = -inf in fp32, a weight of zero either way
+    k[:, n // 2 + 5, :] = -3e38
+    v[:, n // 2 + 1, 7], v[:, n // 2 + 2, 9] = np.inf, -np.inf
+    kn, vn = (synth.bf16_to_f32(_bits((Hkv, 128), (870 + n, i))) for i in (4, 5))
+    bits = [synth.f32_to_bf16_bits(np.ascontiguousarray(x)) for x in (q, kn, vn, np.pad(k, ((0, 0), (0, 1), (0, 0))), np.pad(v, ((0, 0), (0, 1), (0, 0))))]
+    dq, dkn, dvn, dk, dv = (to_dev(b) for b in bits)
+    lay = B.CacheLayout(Hq, Hkv, 128, 128, (n + 1) * 128, 0.05)
+    out = torch.zeros(Hq, 128, device="cuda")
+    B.check(B.lookm_decode_step(dq, dkn, dvn, dk, dv, n, lay, out, B.alloc_decode_workspace(lay)))
+    f = [synth.bf16_to_f32(b) for b in bits]
+    ref, _, _ = orc.decode_step(f[0], f[1], f[2], f[3][:, :n], f[4][:, :n], scale=0.05)
+    got = out.cpu().numpy().astype(np.float64)
+    assert np.all(got[:, 7] == np.inf) and np.all(got[:, 9] == -np.inf)
+    rest = np.ones(128, dtype=bool)
+    rest[[7, 9]] = False
+    assert close(got[:, rest], ref[:, rest]).all()
+
+
 @pytest.mark.parametrize("Hq,Hkv,n", [(1, 1, 17), (8, 8, 16), (12, 12, 409), (13, 13, 700), (32, 32, 18), (32, 32, 4095),
                                       (48, 48, 401), (64, 16, 100), (24, 3, 50), (40, 40, 520)])
 def test_splits_added_up_by_a_cluster(B, Hq, Hkv, n):
