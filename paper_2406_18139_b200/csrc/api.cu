@@ -917,10 +917,19 @@ extern "C" int lookm_noalloc_status(void* cuda_stream) {
 namespace {
 
 constexpr int kDecodeClusterRows = 256;
+constexpr int kDecodeStepRows = 64;         // rows a CTA of any decode kernel takes at a time
 
-struct DecodePlan {
-    int n_req = 0, gt = 1, n_pass = 1, rows_per_split = 64;
+// One way to take the step: which kernel, and how the caches are cut.
+struct DecodeWay {
+    int gt = 1, n_pass = 1;                 // query heads per pass over the rows, passes per group
+    bool mma = false;
+    long long rows_per_split = 64;
     int cluster = 1;                        // > 1: so many splits everywhere, added up inside the launch
+    double us = 0.;                         // estimated time
+};
+struct DecodePlan {
+    int n_req = 0;
+    DecodeWay way;
     std::vector<DecodeReq> reqs;            // caller order
     size_t o_parts = 0, total = 0;
 };
@@ -928,6 +937,74 @@ struct DecodePlan {
 int decode_sms() {
     DeviceInfo di;
     return (device_info(di) == LOOKM_OK && di.sms > 0) ? di.sms : 148;
+}
+
+// Time of a step in us: a launch, the CTAs' steps of 64 rows in every wave of CTAs, a start per further
+// wave, and where the splits take a second launch that and its chain over the splits.  Fitted to 400 steps
+// (groups of 2 to 16 heads, 1 to 32 KV heads, 1 to 32768 rows, 1 to 100 requests); the way it picks takes 0.5 %
+// longer than the fastest of the three on average and 10 % at most.
+struct DecodeCost { double launch, step, wave, combine, splits16; };
+constexpr DecodeCost kCostOneHead = {0.9, 0.59, 1.0, 2.4, 0.7}, kCostTwoHeads = {1.25, 0.78, 1.4, 2.6, 0.7},
+                     kCostMma = {1.9, 1.33, 1.35, 2.7, 0.85};
+constexpr double kMmaStepAlone = 1.9;       // of a CTA that has its SM to itself and waits for each of its steps
+
+DecodeWay decode_way(const lookm_cache_layout* lay, int n_req, const int* lens, int gt, bool mma, int sms) {
+    DecodeWay w;
+    w.gt = gt;
+    w.mma = mma;
+    w.n_pass = lay->n_q_heads / lay->n_kv_heads / gt;
+    const long long units = (long long)lay->n_kv_heads * w.n_pass;       // (KV head, pass) per request
+    // The grid is one wave: as many CTAs as the GPU holds at a time (a second, partly filled wave
+    // would cost as much as the first).  Rows per split: the smallest count with which the splits
+    // of all requests fit into that wave; on the tensor cores, where a short step takes as long as a
+    // full one, two steps at least.
+    const int per_sm = decode_ctas_per_sm(gt, mma);
+    const long long wave = (long long)sms * (per_sm > 0 ? per_sm : 2);
+    long long total_rows = 0;
+    int longest = 0;
+    for (int r = 0; r < n_req; ++r) {
+        total_rows += ((long long)lens[r] + 1) * units;
+        longest = std::max(longest, lens[r] + 1);
+    }
+    auto ctas_with = [&](long long rows) {
+        long long c = 0;
+        for (int r = 0; r < n_req; ++r) c += (((long long)lens[r] + rows) / rows) * units;
+        return c;
+    };
+    long long s = std::max<long long>(mma ? 2 * kDecodeStepRows : 16, (total_rows + wave - 1) / wave);
+    if (ctas_with(s) > wave) {
+        // smallest count in (s, longest cache + 1] that fits (the CTA count never grows with
+        // it); with the upper end every request is a single split, the least there can be
+        long long lo = s, hi = std::max<long long>(s, longest);
+        while (lo < hi) {
+            const long long mid = lo + (hi - lo) / 2;
+            if (ctas_with(mid) > wave) lo = mid + 1; else hi = mid;
+        }
+        s = lo;
+    }
+    // 2, 4 or 8 splits per (KV head, pass) that one cluster adds up, instead of a second launch: as
+    // many as leave every CTA an SM of its own (clusters of 8 fill about two thirds of the SMs
+    // before two share one, smaller ones seven eighths: 16 heads x 8 took 5.7 us where 12 x 8 took
+    // 3.1).  Worth it while a split is short, or at any length if the CTAs cover nearly all SMs (one
+    // request of 32 heads x 4 or 64 x 2: 119 to 129 CTAs);
+    // us per step, two launches -> one: 32 heads x 4 splits 409 rows 4.6 -> 3.8, 8192 rows
+    // 24.4 -> 23.2; 12 x 8 1638 rows 5.3 -> 4.9, 8192 rows 12.6 -> 13.0; 16 x 4 800 rows 4.6 -> 4.7
+    // (5.8 instead of 8.0 with the launches issued one by one), 3000 rows 7.0 -> 9.1.
+    int c = kDecodeMaxCluster;
+    while (c > 1 && n_req * units * c > (c == 8 ? sms * 2 / 3 : sms * 7 / 8)) c /= 2;
+    const long long rows = (longest + c - 1) / c;
+    if (c > 1 && s < longest && (rows <= kDecodeClusterRows || (n_req == 1 && units * c >= sms * 4 / 5))) {
+        w.cluster = c;
+        s = rows;
+    }
+    w.rows_per_split = s;
+    const long long ctas = w.cluster > 1 ? n_req * units * w.cluster : ctas_with(s), splits = (longest + s - 1) / s;
+    const double waves = (double)std::max<long long>(1, (ctas + wave - 1) / wave);
+    const double steps = (double)((std::min<long long>(s, longest) + kDecodeStepRows - 1) / kDecodeStepRows);
+    const DecodeCost& cost = mma ? kCostMma : gt == 2 ? kCostTwoHeads : kCostOneHead;
+    w.us = cost.launch + waves * steps * (mma && ctas <= sms ? kMmaStepAlone : cost.step) + (waves - 1.) * cost.wave;
+    if (w.cluster == 1 && splits > 1) w.us += cost.combine + cost.splits16 * std::max<long long>(0, splits - 16) / 16.;
+    return w;
 }
 
 // lens may be NULL (sizing only).  The workspace is sized for the largest number of splits any
@@ -945,82 +1022,49 @@ int build_decode_plan(DecodePlan& dp, const lookm_cache_layout* lay, int n_req, 
     if (!(lay->softmax_scale >= 0.f) || !std::isfinite(lay->softmax_scale)) return LOOKM_ERR_INVALID_ARG;
     const int group = lay->n_q_heads / lay->n_kv_heads;
     dp.n_req = n_req;
-    for (dp.gt = std::min(group, 8); group % dp.gt; --dp.gt) {}    // largest divisor of the group up to 8
-    dp.n_pass = group / dp.gt;
-    const long long units = (long long)lay->n_kv_heads * dp.n_pass;      // (KV head, pass) per request
+    int widest = std::min(group, 8);        // largest divisor of the group up to 8
+    while (group % widest) --widest;
     const int sms = decode_sms();
-    // The grid is one wave: as many CTAs as the GPU holds at a time (a second, partly filled wave
-    // would cost as much as the first).  Rows per split: the smallest count with which the splits
-    // of all requests fit into that wave.
-    long long s = 16;
     if (lens) {
-        const int per_sm = decode_ctas_per_sm(dp.gt);
-        const long long wave = (long long)sms * (per_sm > 0 ? per_sm : 2);
-        long long total_rows = 0;
-        for (int r = 0; r < n_req; ++r) {
+        for (int r = 0; r < n_req; ++r)
             if (lens[r] < 0 || lens[r] >= (1 << 30) || (begins && begins[r] < 0)) return LOOKM_ERR_INVALID_ARG;
-            total_rows += ((long long)lens[r] + 1) * units;
+        // Query heads of a group one by one, two by two, or all of them on the tensor cores.  Which is the
+        // fastest depends on the rows, the heads and the requests together, us: 32 heads on 16 with 409 rows
+        // 3.7, 4.0 and 5.5, with 3276 9.7, 8.8 and 9.4, with 32768 74, 50 and 45; 64 requests of 30 rows, 16 heads
+        // on 1, 13.4, 9.5 and 4.4; 32 heads on 8 with 409 rows 3.7, 4.0 and 4.3, with 8192 20.6, 16.0 and 11.4.
+        dp.way = decode_way(lay, n_req, lens, 1, false, sms);
+        if (group > 1) {
+            const auto better = [&](const DecodeWay& w) { if (w.us < dp.way.us) dp.way = w; };
+            if (group % 2 == 0) better(decode_way(lay, n_req, lens, 2, false, sms));
+            if (widest > 1) better(decode_way(lay, n_req, lens, widest, true, sms));
         }
-        auto ctas_with = [&](long long rows) {
-            long long c = 0;
-            for (int r = 0; r < n_req; ++r) c += (((long long)lens[r] + rows) / rows) * units;
-            return c;
-        };
-        s = std::max<long long>(16, (total_rows + wave - 1) / wave);
-        if (ctas_with(s) > wave) {
-            // smallest count in (s, longest cache + 1] that fits (the CTA count never grows with
-            // it); with the upper end every request is a single split, the least there can be
-            long long lo = s, hi = s;
-            for (int r = 0; r < n_req; ++r) hi = std::max<long long>(hi, (long long)lens[r] + 1);
-            while (lo < hi) {
-                const long long mid = lo + (hi - lo) / 2;
-                if (ctas_with(mid) > wave) lo = mid + 1; else hi = mid;
-            }
-            s = lo;
-        }
+        if (dp.way.rows_per_split >= (1ll << 31)) return LOOKM_ERR_UNSUPPORTED;
     }
-    if (lens) {
-        // 2, 4 or 8 splits per (KV head, pass) that one cluster adds up, instead of a second launch: as
-        // many as leave every CTA an SM of its own (clusters of 8 fill about two thirds of the SMs
-        // before two share one, smaller ones seven eighths: 16 heads x 8 took 5.7 us where 12 x 8 took
-        // 3.1).  Worth it while a split is short, or at any length if the CTAs cover nearly all SMs;
-        // us per step, two launches -> one: 32 heads x 4 splits 409 rows 4.6 -> 3.8, 8192 rows
-        // 24.4 -> 23.2; 12 x 8 1638 rows 5.3 -> 4.9, 8192 rows 12.6 -> 13.0; 16 x 4 800 rows 4.6 -> 4.7
-        // (5.8 instead of 8.0 with the launches issued one by one), 3000 rows 7.0 -> 9.1.
-        int longest = 0;
-        for (int r = 0; r < n_req; ++r) longest = std::max(longest, lens[r] + 1);
-        int c = kDecodeMaxCluster;
-        while (c > 1 && n_req * units * c > (c == 8 ? sms * 2 / 3 : sms * 7 / 8)) c /= 2;
-        const long long rows = (longest + c - 1) / c;
-        if (c > 1 && s < longest && (rows <= kDecodeClusterRows || (n_req == 1 && units * c >= sms * 4 / 5))) {
-            dp.cluster = c;
-            s = rows;
-        }
-    }
-    if (s >= (1ll << 31)) return LOOKM_ERR_UNSUPPORTED;
-    dp.rows_per_split = (int)s;
     // at most one wave of the fullest kernel, or one (short) split per (request, KV head, pass)
-    // when the batch alone has more units than a wave holds
+    // when the batch alone has more units than a wave holds; with the most heads per pass these
+    // records need the most room
+    const long long units = (long long)lay->n_kv_heads * (group / widest);
     const long long max_splits = (long long)kDecodeMaxCtasPerSm * sms + (long long)n_req * units;
-    if (max_splits * dp.gt >= (1ll << 31)) return LOOKM_ERR_UNSUPPORTED;
+    if (max_splits * widest >= (1ll << 31)) return LOOKM_ERR_UNSUPPORTED;
     if (lens) {
         dp.reqs.resize(n_req);
         long long parts = 0;
+        const long long s = dp.way.rows_per_split;
         for (int r = 0; r < n_req; ++r) {
             DecodeReq& q = dp.reqs[r];
             q.begin = begins ? begins[r] : 0;
             q.len = lens[r];
             q.index = r;
-            q.n_splits = dp.cluster > 1 ? dp.cluster : (int)(((long long)lens[r] + 1 + s - 1) / s);
+            q.n_splits = dp.way.cluster > 1 ? dp.way.cluster : (int)(((long long)lens[r] + 1 + s - 1) / s);
             q.cta_begin = 0;
             q.part_begin = (int)parts;
             q.pad = 0;
-            parts += (long long)q.n_splits * units * dp.gt;
+            parts += (long long)q.n_splits * lay->n_kv_heads * dp.way.n_pass * dp.way.gt;
         }
     }
     size_t o = 0;
     auto carve = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
-    dp.o_parts = carve(4 * (size_t)(kHeadDim + 2) * (size_t)max_splits * (size_t)dp.gt);
+    dp.o_parts = carve(4 * (size_t)(kHeadDim + 2) * (size_t)max_splits * (size_t)widest);
     dp.total = o;
     return LOOKM_OK;
 }
@@ -1041,7 +1085,7 @@ int decode_common(const void* q, const void* k_new, const void* v_new, void* cac
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     g_launches = 0;
     const float scale = lay->softmax_scale > 0.f ? lay->softmax_scale : 1.0f / std::sqrt((float)lay->head_dim);
-    const long long units = (long long)lay->n_kv_heads * dp.n_pass;
+    const long long units = (long long)lay->n_kv_heads * dp.way.n_pass;
     for (int base = 0; base < n_req; base += kDecodeChunk) {
         DecodeBatch batch;
         std::memset(&batch, 0, sizeof(batch));
@@ -1052,16 +1096,16 @@ int decode_common(const void* q, const void* k_new, const void* v_new, void* cac
             batch.r[i] = dp.reqs[base + i];
             batch.r[i].cta_begin = (int)ctas;
             ctas += (long long)batch.r[i].n_splits * units;
-            split = split || (batch.r[i].n_splits > 1 && dp.cluster == 1);
+            split = split || (batch.r[i].n_splits > 1 && dp.way.cluster == 1);
         }
         if (ctas >= (1ll << 31)) return LOOKM_ERR_UNSUPPORTED;
-        LOOKM_CUDA(launch_decode(batch, (int)ctas, dp.gt, dp.cluster, q, k_new, v_new, cache_k, cache_v,
+        LOOKM_CUDA(launch_decode(batch, (int)ctas, dp.way.gt, dp.way.mma, dp.way.cluster, q, k_new, v_new, cache_k, cache_v,
                                  lay->cache_stride_row, lay->cache_stride_head, lay->n_q_heads,
-                                 lay->n_kv_heads, dp.rows_per_split, scale * 1.4426950408889634f,
+                                 lay->n_kv_heads, (int)dp.way.rows_per_split, scale * 1.4426950408889634f,
                                  at<float>(ws, dp.o_parts), out, st));
         ++g_launches;
         if (split) {
-            LOOKM_CUDA(launch_decode_combine(batch, dp.gt, lay->n_q_heads, lay->n_kv_heads,
+            LOOKM_CUDA(launch_decode_combine(batch, dp.way.gt, lay->n_q_heads, lay->n_kv_heads,
                                              scale * 1.4426950408889634f, at<float>(ws, dp.o_parts), out, st));
             ++g_launches;
         }

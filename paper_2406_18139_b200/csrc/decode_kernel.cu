@@ -17,7 +17,8 @@
 // behind the first, adds the splits in split order.  No CTA waits for another and the order of
 // additions never depends on timing, so results are reproducible bit for bit.
 //
-// Query heads that share a KV head go to decode_mma_kernel below, which has the same structure.
+// Several query heads that share a KV head can go to decode_mma_kernel below, which has the same structure;
+// the planner compares (decode_way in api.cu).
 #include <cuda_bf16.h>
 #include <float.h>
 #include <math.h>
@@ -109,7 +110,7 @@ struct DecShared {
     float o[kDecWarps][GT][kHeadDim];
 };
 
-// GT query heads of the group are handled per pass over the rows; only GT = 1 is instantiated.
+// GT = 1 or 2 query heads of the group are handled per pass over the rows.
 template <int GT, bool kClustered>
 __global__ void __launch_bounds__(kDecThreads)
 decode_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __restrict__ q,
@@ -664,10 +665,6 @@ decode_combine_kernel(const __grid_constant__ DecodeBatch batch, int gt, int n_p
 
 namespace {
 
-// gt query heads per pass: one head alone stays on the scalar kernel (8192 rows x 32 heads: 24.2 us,
-// 0.85 of the copy bandwidth with the launches), several go to the tensor cores (scalar -> mma, us:
-// 32768 rows, 8 KV heads x 4: 40.5 -> 27.1; 16 requests of 400-3300 rows, 8 x 4: 51.5 -> 27.0;
-// 20000 rows, 16 x 2: 33.7 -> 31.5; 9000 rows, 4 x 16: 24.9 -> 13.5).
 typedef void (*MmaKernel)(DecodeBatch, const __nv_bfloat16*, const __nv_bfloat16*, const __nv_bfloat16*, __nv_bfloat16*,
                           __nv_bfloat16*, long long, long long, int, int, int, int, int, float, float*, float*);
 MmaKernel mma_kernel(int gt, bool clustered) {
@@ -683,6 +680,10 @@ cudaError_t configure_decode() {
         cudaError_t e = cudaFuncSetAttribute(decode_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(decode_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(decode_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(decode_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
         for (int gt : {2, 4, 8})
             for (bool clustered : {false, true})
                 if (e == cudaSuccess)
@@ -695,23 +696,24 @@ cudaError_t configure_decode() {
 
 // CTAs that one SM holds at a time of the kernel that handles gt query heads per pass, on the current
 // device (looked up once per device); 0 if the query fails.  The planner sizes the grid to one wave.
-int decode_ctas_per_sm(int gt) {
-    static int cache[64][4] = {};
+int decode_ctas_per_sm(int gt, bool mma) {
+    static int cache[64][5] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    const int idx = gt > 4 ? 3 : gt > 2 ? 2 : gt > 1 ? 1 : 0;
+    const int idx = !mma ? gt - 1 : gt > 4 ? 4 : gt > 2 ? 3 : 2;
     int v = __atomic_load_n(&cache[dev][idx], __ATOMIC_ACQUIRE);
     if (v > 0) return v;
     if (configure_decode() != cudaSuccess) { cudaGetLastError(); return 0; }
     cudaError_t err;
-    if (gt > 1) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, mma_kernel(gt, false), kMmaThreads, kMmaRingBytes);
+    if (mma) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, mma_kernel(gt, false), kMmaThreads, kMmaRingBytes);
+    else if (gt == 2) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, decode_kernel<2, false>, kDecThreads, kDecRingBytes);
     else err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, decode_kernel<1, false>, kDecThreads, kDecRingBytes);
     if (err != cudaSuccess || v <= 0) { cudaGetLastError(); return 0; }
     __atomic_store_n(&cache[dev][idx], v, __ATOMIC_RELEASE);
     return v;
 }
 
-cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, int cluster, const void* q,
+cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, bool mma, int cluster, const void* q,
                           const void* k_new, const void* v_new, void* cache_k, void* cache_v,
                           long long stride_row, long long stride_head, int n_q_heads, int n_kv_heads,
                           int rows_per_split, float scale_log2, float* parts, float* out,
@@ -721,12 +723,14 @@ cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, int 
     cudaError_t err = configure_decode();
     if (err != cudaSuccess) return err;
     const bool clustered = cluster > 1;
-    if (gt > 1)
+    if (mma)
         return launch_chained_clusters(mma_kernel(gt, clustered), dim3((unsigned)total_ctas), dim3(kMmaThreads), (unsigned)cluster,
                                        (size_t)kMmaRingBytes, stream, batch, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_new,
                                        (const __nv_bfloat16*)v_new, (__nv_bfloat16*)cache_k, (__nv_bfloat16*)cache_v, stride_row,
                                        stride_head, n_q_heads, n_kv_heads, group, gt, rows_per_split, scale_log2, parts, out);
-    return launch_chained_clusters(clustered ? decode_kernel<1, true> : decode_kernel<1, false>, dim3((unsigned)total_ctas),
+    const auto scalar = gt == 2 ? (clustered ? decode_kernel<2, true> : decode_kernel<2, false>)
+                                : (clustered ? decode_kernel<1, true> : decode_kernel<1, false>);
+    return launch_chained_clusters(scalar, dim3((unsigned)total_ctas),
                                    dim3(kDecThreads), (unsigned)cluster, (size_t)kDecRingBytes, stream, batch, (const __nv_bfloat16*)q,
                                    (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, (__nv_bfloat16*)cache_k,
                                    (__nv_bfloat16*)cache_v, stride_row, stride_head, n_q_heads, n_kv_heads, group,

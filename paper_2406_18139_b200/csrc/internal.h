@@ -189,11 +189,11 @@ struct DecodeBatch { int n_req; int pad; DecodeReq r[kDecodeChunk]; };
 constexpr int kDecodeThreads = LOOKM_DEC_THREADS;             // threads per CTA of the decode kernel
 constexpr int kDecodeMaxCtasPerSm = 2048 / kDecodeThreads;    // what an SM's thread limit allows
 constexpr int kDecodeMaxCluster = 8;     // splits of a (KV head, pass) that one thread-block cluster adds up
-int decode_ctas_per_sm(int gt);          // resident CTAs per SM of the kernel for this gt (0: unknown)
+int decode_ctas_per_sm(int gt, bool mma);    // resident CTAs per SM of the kernel (0: unknown)
 
-// gt: query heads handled per pass over the rows (1 .. 8; divides the group size)
+// gt: query heads handled per pass over the rows (divides the group size): 1 or 2, up to 8 on the tensor cores (mma)
 // cluster > 1: every request has that many splits, which add up inside the launch
-cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, int cluster, const void* q,
+cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, bool mma, int cluster, const void* q,
                           const void* k_new, const void* v_new, void* cache_k, void* cache_v,
                           long long stride_row, long long stride_head, int n_q_heads, int n_kv_heads,
                           int rows_per_split, float scale_log2, float* parts, float* out,

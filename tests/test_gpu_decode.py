@@ -141,6 +141,35 @@ def test_splits_added_up_by_a_cluster(B, Hq, Hkv, n):
     assert B.lookm_last_launch_count() == (1 if n != 520 else 2)
 
 
+@pytest.mark.parametrize("Hq,Hkv,n", [(32, 16, 3276), (64, 32, 409), (8, 4, 9000), (48, 8, 60), (64, 32, 5000), (16, 1, 700)])
+def test_grouped_queries_one_or_two_heads_at_a_time(B, Hq, Hkv, n):
+    """Groups whose heads are cheaper taken one by one or two by two: clusters and split records."""
+    run_step(B, Hq, Hkv, n, n + 1, n % 2 == 0, seed=830 + n)
+
+
+@pytest.mark.parametrize("group", [2, 3, 4, 5, 6, 7, 8, 12, 16])
+def test_batches_of_grouped_queries_at_the_edges_of_sixteen_row_steps(B, group):
+    """Enough requests for the tensor-core kernel whatever the rows: caches that end just before, at and after
+    the sixteen rows of a warp's step and the sixty-four of a CTA's, the appended row in any of them."""
+    import torch
+    Hkv, f = 8, synth.bf16_to_f32
+    lens = [0, 1, 7, 14, 15, 16, 17, 30, 31, 32, 47, 62, 63, 64, 65, 79, 80, 126, 127, 128, 129, 200, 255, 256, 257] * 3
+    begins = np.concatenate([[0], np.cumsum([n + 1 for n in lens])]).tolist()
+    ck_b, cv_b = _bits((begins[-1], Hkv, 128), (840, group)), _bits((begins[-1], Hkv, 128), (841, group))
+    q_b, kn_b, vn_b = (_bits((len(lens), h, 128), (842 + i, group)) for i, h in enumerate((Hkv * group, Hkv, Hkv)))
+    dk, dv, q, kn, vn = (to_dev(t) for t in (ck_b, cv_b, q_b, kn_b, vn_b))
+    lay = B.CacheLayout(Hkv * group, Hkv, 128, Hkv * 128, 128, 0.2)
+    out = torch.full((len(lens), Hkv * group, 128), np.nan, device="cuda")
+    B.check(B.lookm_decode_step_varlen(q, kn, vn, dk, dv, begins[:-1], lens, lay, out, B.alloc_decode_workspace(lay, len(lens))))
+    got = out.cpu().numpy().astype(np.float64)
+    for r, n in enumerate(lens):
+        a = begins[r]
+        ref, _, _ = orc.decode_step(f(q_b[r]), f(kn_b[r]), f(vn_b[r]), f(ck_b[a:a + n]).transpose(1, 0, 2),
+                                    f(cv_b[a:a + n]).transpose(1, 0, 2), scale=0.2)
+        assert close(got[r], ref).all(), (r, n)
+        assert torch.equal(dk[a + n], kn[r]) and torch.equal(dv[a + n], vn[r])
+
+
 def test_long_cache_is_cut_into_many_splits(B):
     # 2 KV heads x 20001 rows: about 150 splits per head, combined by the last CTA to arrive
     run_step(B, 8, 2, 20000, 20001, False, seed=701)
