@@ -123,9 +123,11 @@ __device__ __forceinline__ void key_norms(const __nv_bfloat16* __restrict__ k, l
 }
 
 // The first kThreads * kSteps tokens are shared out evenly: a warp has steps * 32 consecutive ones, a step
-// is one per lane, and their keys stay in registers.  Tokens beyond are read again in every step of the
-// bisection, and once more for the lists.
-template <int kThreads, int kSteps>
+// is one per lane, and their keys stay in registers.  kLong: there may be tokens beyond, which every pass has
+// to read again.  Then a pass counts 2048 parts of the range between the smallest and the largest key, and
+// goes on in the one that holds the k-th largest: three passes where the bisection takes some 27.
+constexpr int kParts = 2048;
+template <int kThreads, int kSteps, bool kLong>
 __global__ void __launch_bounds__(kThreads)
 select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask,
               const Req* __restrict__ reqs, int n_select_blocks, int n_kv_heads, long long T,
@@ -179,9 +181,26 @@ select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask
         }
     };
     load(first);
+    // the candidates beyond, with the loads of eight in flight together
+    constexpr int kBatch = 8;
+    auto beyond = [&](auto visit) {
+        for (int j0 = kChunk + threadIdx.x; kLong && j0 < nc; j0 += kBatch * kThreads) {
+            float v[kBatch];
+            bool image[kBatch];
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q) {
+                const int j = j0 + q * kThreads;
+                v[q] = j < nc ? s[j] : 0.f;
+                image[q] = j < nc && is_image(j);
+            }
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q)
+                if (j0 + q * kThreads < nc) visit(order_key(v[q]), image[q]);
+        }
+    };
     // text candidates: candidates less image tokens among them
     int cnt = min(steps, max(0, (nc - first + 31) / 32)) - __popc(img);
-    for (int j = kChunk + threadIdx.x; j < nc; j += kThreads) cnt += !is_image(j);
+    beyond([&](unsigned, bool image) { cnt += !image; });
     const int n_text = block_sum(cnt);
     // class whose members are ranked (1 = image); the other class is kept entirely or not at all
     const int sel_cls = (n_text <= N) ? 1 : 0;
@@ -202,32 +221,71 @@ select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask
             if (!member) key[q] = 0u;
             if (member) { lo = min(lo, key[q]); hi = max(hi, key[q]); }
         }
-        for (int j = kChunk + threadIdx.x; j < nc; j += kThreads)
-            if (is_image(j) == (sel_cls != 0)) { const unsigned x = order_key(s[j]); lo = min(lo, x); hi = max(hi, x); }
+        beyond([&](unsigned x, bool image) { if (image == (sel_cls != 0)) { lo = min(lo, x); hi = max(hi, x); } });
         lo = __reduce_min_sync(0xffffffffu, lo);
         hi = __reduce_max_sync(0xffffffffu, hi);
         if (lane == 0) { extremes[0][warp] = lo; extremes[1][warp] = hi; }
         __syncthreads();
         lo = __reduce_min_sync(0xffffffffu, lane < kWarps ? extremes[0][lane] : 0xffffffffu);
         hi = __reduce_max_sync(0xffffffffu, lane < kWarps ? extremes[1][lane] : 0u);
-        int above = 0;                                   // members above hi
-        bool exact = false;
-        while (lo < hi && !exact) {                      // at least k members >= lo, fewer than k above hi
-            const unsigned mid = lo + (hi - lo) / 2u + 1u;
-            int c = 0;
+        if (kLong) {
+            __shared__ int parts[kParts], found[2];
+            need_ties = k;                               // of those left in [lo, hi]
+            while (lo < hi) {
+                const int shift = max(0, 32 - __clz(hi - lo) - 11);
+                for (int i = threadIdx.x; i < kParts; i += kThreads) parts[i] = 0;
+                __syncthreads();
+                auto count = [&](unsigned x) { if (x >= lo && x <= hi) atomicAdd(&parts[(x - lo) >> shift], 1); };
 #pragma unroll
-            for (int g = 0; g < kSteps; g += 8)
-                if (g < steps)
+                for (int q = 0; q < kSteps; ++q)
+                    if (q < steps && first + q * 32 < nc && ((img >> q) & 1u) == (unsigned)sel_cls) count(key[q]);
+                beyond([&](unsigned x, bool image) { if (image == (sel_cls != 0)) count(x); });
+                __syncthreads();
+                // parts from the top, kOwn per thread: the one in which the count reaches need_ties
+                constexpr int kOwn = kParts / kThreads;
+                int c[kOwn], mine = 0, before, other, all, none;
 #pragma unroll
-                    for (int q = g; q < g + 8; ++q) c += key[q] >= mid;
-            for (int j = kChunk + threadIdx.x; j < nc; j += kThreads)
-                c += is_image(j) == (sel_cls != 0) && order_key(s[j]) >= mid;
-            c = block_sum(c);
-            if (c == k) { thr = mid - 1u; exact = true; }
-            else if (c > k) lo = mid;
-            else { hi = mid - 1u; above = c; }
+                for (int q = 0; q < kOwn; ++q) mine += c[q] = parts[kParts - 1 - (int)threadIdx.x * kOwn - q];
+                int incl = mine;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int x = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += x;
+                }
+                warp_scan2<kThreads>(__shfl_sync(0xffffffffu, incl, 31), 0, before, other, all, none, warp_tot);
+                before += incl - mine;
+#pragma unroll
+                for (int q = 0; q < kOwn; ++q) {
+                    if (before < need_ties && before + c[q] >= need_ties) {
+                        found[0] = kParts - 1 - (int)threadIdx.x * kOwn - q;
+                        found[1] = need_ties - before;
+                    }
+                    before += c[q];
+                }
+                __syncthreads();
+                lo += (unsigned)found[0] << shift;
+                if (hi - lo > (1u << shift) - 1u) hi = lo + ((1u << shift) - 1u);
+                need_ties = found[1];
+            }
+            thr = lo;
+        } else {
+            int above = 0;                               // members above hi
+            bool exact = false;
+            while (lo < hi && !exact) {                  // at least k members >= lo, fewer than k above hi
+                const unsigned mid = lo + (hi - lo) / 2u + 1u;
+                int c = 0;
+#pragma unroll
+                for (int g = 0; g < kSteps; g += 8)
+                    if (g < steps)
+#pragma unroll
+                        for (int q = g; q < g + 8; ++q) c += key[q] >= mid;
+                c = block_sum(c);
+                if (c == k) { thr = mid - 1u; exact = true; }
+                else if (c > k) lo = mid;
+                else { hi = mid - 1u; above = c; }
+            }
+            if (!exact) { thr = lo; need_ties = k - above; }
         }
-        if (!exact) { thr = lo; need_ties = k - above; }
     }
 
     // ---- ordered emission -----------------------------------------------------------------------
@@ -236,9 +294,9 @@ select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask
     int* rk = rank ? rank + (long long)h * T + rq.tok_begin : nullptr;
     const unsigned lt_mask = (1u << lane) - 1u;
     int kept_run = 0, tie_run = 0;
-    for (int c0 = 0; c0 < L; c0 += kChunk) {             // (steps == kSteps if there is more than one turn)
+    for (int c0 = 0; c0 < (kLong ? L : 1); c0 += kChunk) {       // (steps == kSteps if there is more than one turn)
         const int j0 = c0 + first;
-        if (c0) { img = 0u; load(j0); }
+        if (kLong && c0) { img = 0u; load(j0); }
         unsigned keep = 0u, tie = 0u;                    // bit q: token of step q
 #pragma unroll
         for (int q = 0; q < kSteps; ++q) {
@@ -292,10 +350,20 @@ cudaError_t launch_select(const float* scores, const uint8_t* mask, const Req* r
                           const void* k_for_norms, long long stride_tok, long long stride_head,
                           float* rnorm_all, int num_sms, cudaStream_t stream) {
     const int n_select = n_kv_heads * n_req;
-    // cheaper barriers with fewer threads, a shorter chain of steps with more: a layer of 2048 tokens x 8
+    // Cheaper barriers with fewer threads, a shorter chain of steps with more: a layer of 2048 tokens x 8
     // heads takes 67.0 us with 256 threads, 64.9 with 512 and 65.8 with 1024, 2048 x 32 123, 119.5 and
-    // 119.5, 3000 x 8 85.1 with 512 and 84.2 with 1024; up to 32768 tokens stay in registers
-    const int threads = max_L <= 2048 ? 512 : 1024;
+    // 119.5, 3000 x 8 85.1 with 512 and 84.2 with 1024.  Registers hold up to 32768 tokens, in variants of 8, 16 and
+    // 32 per thread (the last spills: 16384 tokens x 8 heads 32.8 us with 32, 21.3 with 16); beyond, sixteen are
+    // held and the rest is read again (65536 tokens x 8 heads 88 us; bisected with 32 held 179).
+    typedef void (*Kernel)(const float*, const uint8_t*, const Req*, int, int, long long, int*, int*, int*, const __nv_bfloat16*,
+                           long long, long long, float*);
+    struct Variant { int threads, most; Kernel kernel; };
+    static const Variant variants[] = {{512, 512 * 4, select_kernel<512, 8, false>}, {1024, 1024 * 8, select_kernel<1024, 8, false>},
+                                       {1024, 1024 * 16, select_kernel<1024, 16, false>}, {1024, 1024 * 32, select_kernel<1024, 32, false>},
+                                       {1024, 0x7fffffff, select_kernel<1024, 16, true>}};
+    const Variant* use = variants;
+    while (max_L > use->most) ++use;
+    const int threads = use->threads;
     int n_norm = 0;
     if (k_for_norms) {
         // the norm CTAs take the SMs that the selection leaves free, so that all of them run at once
@@ -306,8 +374,7 @@ cudaError_t launch_select(const float* scores, const uint8_t* mask, const Req* r
         // norms: then a full wave of norm CTAs follows the selection CTAs instead)
         n_norm = (int)std::min<long long>(want, (long long)per_sm * (n_select < num_sms / 2 ? num_sms - n_select : num_sms));
     }
-    auto kernel = max_L <= 2048 ? select_kernel<512, 8> : max_L <= 8192 ? select_kernel<1024, 8> : select_kernel<1024, 32>;
-    return launch_chained(kernel, dim3(n_select + n_norm), dim3(threads), 0, stream,
+    return launch_chained(use->kernel, dim3(n_select + n_norm), dim3(threads), 0, stream,
                           scores, mask, reqs, n_select, n_kv_heads, T, kept_idx, evict_idx, rank,
                           (const __nv_bfloat16*)k_for_norms, stride_tok, stride_head, rnorm_all);
 }

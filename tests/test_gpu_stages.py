@@ -280,6 +280,24 @@ def test_select_at_the_edges_of_what_stays_in_registers(B, L, budget, window, n_
     _run_select(B, s32, mask, [0, L], [budget], [window], Hkv)
 
 
+@pytest.mark.parametrize("lens,budgets,windows,n_text,values", [
+    ([16384], [4000], [32], 2000, 0), ([16385], [300], [0], 16385, 0), ([32768], [3000], [0], 100, 3), ([32769], [1], [0], 0, 0),
+    ([40000, 700, 1, 16385], [3000, 100, 1, 2000], [64, 64, 0, 5], 2000, 0), ([70001], [1500], [3], 70000, 0),
+    ([50000], [2000], [100], 1500, 2), ([50000], [7], [0], 0, 1), ([131075], [900], [64], 500, 1000)])
+def test_select_of_long_prompts(B, lens, budgets, windows, n_text, values):
+    """Keys of sixteen and of 32 tokens per thread, and prompts that are read again in three counting passes:
+    all scores different over 40 orders of magnitude and both signs, or so few values that most are equal."""
+    Hkv, T = 2, sum(lens)
+    x = synth.normal(synth.stream_key(79, T), Hkv * T).reshape(Hkv, T)
+    s32 = (np.exp(15 * x) * np.where(x > 1.5, -1, 1)).astype(np.float32)
+    if values:
+        s32 = (np.floor(np.abs(x) * values).clip(0, values - 1) + 0.5).astype(np.float32)
+    mask = np.ones(T, dtype=np.uint8)
+    if n_text:
+        mask[synth.uniform_int(synth.stream_key(80, T), n_text, 0, T - 1).astype(int)] = 0
+    _run_select(B, s32, mask, np.concatenate([[0], np.cumsum(lens)]).tolist(), budgets, windows, Hkv)
+
+
 def test_select_ties_and_duplicates_and_batches(B):
     L, Hkv = 3000, 2
     # heavy duplication: only 7 distinct score values, so every threshold is a tie
