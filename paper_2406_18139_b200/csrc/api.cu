@@ -51,16 +51,38 @@ struct Plan {
 struct DeviceInfo { int sms = 0; int cc_major = 0; bool ok = false; };
 int device_info(DeviceInfo& out);
 
-// Items of two blocks need two and a half per SM to be shared evenly, items of four four, and six if the
-// prompts differ in length.  Scores in us, single blocks | pairs: 2600 tokens x 32 heads (2.3
-// pairs per SM) 93.5 | 96, 2850 x 32 query on 8 KV heads (2.49) 110 | 115, 3000 x 32 on 8 (2.6) 124 | 118,
-// a layer of 2048 x 8 (0.4) 66 | 85; pairs | fours: 9000 x 32 (3.8 fours per SM) 834 | 832, 10000 x 32
-// (4.3) 1017 | 1007, 9000 x 40 (4.8) 1046 | 1022, 8192 x 64 (6.9) 1415 | 1363; of several lengths: two
-// prompts of 10000 to 14000 x 16 (5.0) 1357 | 1376, four of 1000 to 12000 x 32 on 8 (8) 3350 | 3260.
-// Grouped query heads count one by one, in sweep 2 as well: 7777 tokens x 32 query heads on 8, a layer 392
-// us with single blocks for whole groups in sweep 2, 378 with pairs for single query heads.
-constexpr long long kPairBlocksPerSm = 5;
-constexpr long long kQuadItemsPerSm = 4, kRaggedQuadItemsPerSm = 6;
+// Blocks per sweep item, from the scores of some 370 problems with one, two and four blocks per item (us).
+// Several blocks pay where there are enough items and the items are full.
+//   Two blocks, one or two prompts: from nine blocks per SM on (3200 tokens x 32 heads, 5.4 per SM, 111 | 129, 3600
+// x 40, 7.8, 182 | 197, 4096 x 32, 6.9, 178 | 187, 6000 x 32, 10.2, 387 | 385, 8192 x 32, 13.8, 709 | 683).
+//   More prompts, whose single blocks come out uneven from a fixed deal: from five (three of 900 x 32, 5.2, 66 |
+// 58).  The items have to be three quarters full (93 of 128 tokens x 32: one block each, 111 | 135; 31 of 384: two
+// items for three, 124 | 134).  Single blocks take the query heads of a group together in sweep 2, and the fixed
+// deal evens out with many items, so grouped heads also need streamed tiles in an item: two on average below
+// seven blocks per SM, two and a half below 24, else five (six of 400 x 32 on 8, three tiles, 5.2 per SM, 53 | 49, 40
+// of them, 35 per SM, 219 | 246; 46 of 256, two tiles, 20 per SM, 100 | 114; 15 of 700, four tiles, 169 | 159).
+//   Four blocks, one prompt: from four items per SM (9000 x 32, 3.9, 846 with two | 843, 8192 x 40, 4.3, 862 | 844,
+// 16384 x 32, 6.9, 2662 | 2583).  More: from eight, with six streamed tiles each on average (five of 2000 x 32,
+// 4.3 items, 257 | 276; 15 of 700, 6.5, 155 | 178; 32 of 33 to 2918 x 16, 11.4, 605 | 594).
+int sweep_blocks(const Plan& pl, long long sms) {
+    const auto shape = [&](int k, long long& sets, long long& streamed) {
+        sets = streamed = 0;
+        for (const Req& q : pl.reqs) {
+            const long long n = (q.nblk + k - 1) / k;
+            sets += n;
+            streamed += n * q.nblk - k * n * (n - 1) / 2;            // a set streams the tiles from its first block on
+        }
+    };
+    const bool one = pl.n_req == 1;
+    long long blocks, sets, streamed;
+    shape(1, blocks, streamed);
+    shape(4, sets, streamed);
+    if (sets * pl.n_q_heads >= (one ? 4 : 8) * sms && (one || streamed >= 6 * sets)) return 4;
+    shape(2, sets, streamed);
+    const long long all = blocks * pl.n_q_heads;
+    const int half_tiles = pl.group == 1 ? 0 : all < 7 * sms ? 4 : all < 24 * sms ? 5 : 10;
+    return all >= (pl.n_req <= 2 ? 9 : 5) * sms && 100 * blocks >= 76 * 2 * sets && 2 * streamed >= half_tiles * sets ? 2 : 1;
+}
 // The kTailSets shortest items of all prompts come last: with each prompt's items in a row the last
 // prompt's longest ones would end the sweep.  Scores of eight prompts of 4000 to 6000 tokens x 16 heads
 // (8.6 items per SM) 1122 -> 1094 us, four of 1000 to 12000 x 8 603 -> 590, three of 2000 to 3000 x 32 291 ->
@@ -83,9 +105,7 @@ void plan_splits(Plan& pl) {
     const long long mean = std::max<long long>(1, tiles * pl.n_q_heads / sms);
     for (int s = 0; s < 2; ++s) {
         const long long longest = (long long)pl.reqs[0].nblk * (s ? pl.group : 1);
-        const long long quad = pl.reqs[0].nblk == pl.reqs.back().nblk ? kQuadItemsPerSm : kRaggedQuadItemsPerSm;
-        if (blocks >= kPairBlocksPerSm * sms) pl.blocks[s] = 2;
-        if (blocks >= 4 * quad * sms) pl.blocks[s] = 4;
+        pl.blocks[s] = sweep_blocks(pl, sms);
         if (pl.blocks[s] > 1 && blocks < kTailItemsPerSm * pl.blocks[s] * sms)
             pl.tail_sets[s] = std::min(kTailSets, (pl.reqs.back().nblk + pl.blocks[s] - 1) / pl.blocks[s]);
         if (pl.blocks[s] == 1 && 2 * longest > 3 * mean && longest >= mean + 10)

@@ -134,10 +134,12 @@ def test_scores_of_items_cut_into_ranges(B, lens, Hq, Hkv):
 
 @pytest.mark.parametrize("lens,Hq,Hkv", [([1665], 64, 64), ([1664], 64, 64), ([1500, 129, 1, 800, 128], 72, 24), ([200] * 16, 32, 16),
                                          ([600, 513, 512, 640, 1, 129, 300, 900], 96, 96), ([1300, 1300, 770], 192, 48), ([2000, 1700], 40, 8),
-                                         ([600, 513, 512, 640, 1, 129, 300, 900], 128, 128)])
+                                         ([600, 513, 512, 640, 1, 129, 300, 900], 128, 128),
+                                         ([1665], 96, 96), ([1664], 112, 56), ([1665], 160, 160), ([2100], 128, 32),
+                                         ([1300, 1300, 770, 1500, 129], 128, 128), ([1300, 1301, 770, 1409], 128, 32)])
 def test_scores_of_items_of_two_or_four_blocks(B, lens, Hq, Hkv):
-    """Enough heads for items of two blocks (in sweep 1 alone with 24 KV heads) or four (128 and 192
-    query heads): one to four blocks in the last item of a prompt, requests of one block, a last block of one
+    """Enough heads for items of two blocks or four (the last four of the list), each query head of a group an
+    item of its own: one to four blocks in the last item of a prompt, requests of one block, a last block of one
     row; logits rise along the prompts."""
     import torch
     T = sum(lens)
@@ -169,7 +171,7 @@ def test_scores_of_items_of_two_or_four_blocks(B, lens, Hq, Hkv):
         assert np.allclose(lse[qs, a:a + n].cpu().numpy().reshape(len(heads), g, n), lse_o, rtol=1e-6, atol=2e-5)
 
 
-@pytest.mark.parametrize("Hq,Hkv", [(4, 2), (16, 16), (40, 8), (64, 32)])
+@pytest.mark.parametrize("Hq,Hkv", [(4, 2), (16, 16), (40, 8), (64, 32), (64, 64)])
 def test_scores_of_many_short_prompts_of_one_to_three_blocks(B, Hq, Hkv):
     """Items in which some epilogue groups have no tile, one after another: which group adds up a block
     changes from item to item and nothing but the barriers of the combination orders them.  More requests
