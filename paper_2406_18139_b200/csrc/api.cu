@@ -38,13 +38,13 @@ struct Plan {
     std::vector<int> out_len;               // caller order
     // workspace offsets (bytes)
     int splits[2] = {1, 1};                 // ranges of a sweep 1 / sweep 2 item's streamed tiles
-    int blocks[2] = {1, 1};                 // blocks per sweep item
-    int tail_sets[2] = {0, 0};              // several blocks per item: shortest sets that every request keeps
-    int tail_begin[2] = {0, 0};             // for the end, and the first item of these
+    int blocks = 1;                         // blocks per sweep item
+    int tail_sets = 0, tail_begin = 0;      // several blocks per item: shortest sets that every request keeps
+                                            // for the end, and the first item of these
     size_t n_arrived[2] = {0, 0};           // their arrival counters
     size_t clear_words = 64;                // status word and arrival counters
     size_t o_status, o_reqs, o_lse, o_lse_split, o_scores, o_rank, o_rnorm_all, o_kept, o_evict, o_kept_keys,
-        o_rnorm_kept, o_assign, o_sim, o_row_ptr, o_entries, o_units, o_slot_cnt, o_parts, o_sort_a, o_sort_b,
+        o_rnorm_kept, o_assign, o_sim, o_row_begin, o_entries, o_units, o_slot_cnt, o_parts, o_sort_a, o_sort_b,
         total;
 };
 
@@ -103,12 +103,15 @@ void plan_splits(Plan& pl) {
         blocks += (long long)q.nblk * pl.n_q_heads;
     }
     const long long mean = std::max<long long>(1, tiles * pl.n_q_heads / sms);
+    pl.blocks = sweep_blocks(pl, sms);
+    if (pl.blocks > 1) {
+        if (blocks < kTailItemsPerSm * pl.blocks * sms)
+            pl.tail_sets = std::min(kTailSets, (pl.reqs.back().nblk + pl.blocks - 1) / pl.blocks);
+        return;
+    }
     for (int s = 0; s < 2; ++s) {
         const long long longest = (long long)pl.reqs[0].nblk * (s ? pl.group : 1);
-        pl.blocks[s] = sweep_blocks(pl, sms);
-        if (pl.blocks[s] > 1 && blocks < kTailItemsPerSm * pl.blocks[s] * sms)
-            pl.tail_sets[s] = std::min(kTailSets, (pl.reqs.back().nblk + pl.blocks[s] - 1) / pl.blocks[s]);
-        if (pl.blocks[s] == 1 && 2 * longest > 3 * mean && longest >= mean + 10)
+        if (2 * longest > 3 * mean && longest >= mean + 10)
             pl.splits[s] = (int)std::min<long long>(kMaxSplits, (longest + mean - 1) / mean);
     }
     // (sweep 1's partial results, 8 bytes per range, query head and token, have room where the kept keys go)
@@ -201,19 +204,18 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
         const bool merges = q.mode != LOOKM_MERGE_NONE;
         const long long n_units = merges ? (q.L + unit_entries - 1) / unit_entries : 0;
         units += (long long)pl.n_kv_heads * n_units;
-        it0 += (long long)((q.nblk + pl.blocks[0] - 1) / pl.blocks[0] - pl.tail_sets[0]) * pl.n_q_heads * pl.splits[0];
+        const long long sets = (q.nblk + pl.blocks - 1) / pl.blocks - pl.tail_sets;
+        it0 += sets * pl.n_q_heads * pl.splits[0];
         // (several blocks per item: the query heads of a group are items of their own in sweep 2 too)
-        it1 += (long long)((q.nblk + pl.blocks[1] - 1) / pl.blocks[1] - pl.tail_sets[1]) *
-               (pl.blocks[1] > 1 ? pl.n_q_heads : pl.n_kv_heads) * pl.splits[1];
+        it1 += sets * (pl.blocks > 1 ? pl.n_q_heads : pl.n_kv_heads) * pl.splits[1];
         // match items: blocks of 128 entries of every head's evicted list
         it2 += (q.E > 0 && merges) ? (long long)((q.E + kTile - 1) / kTile) * pl.n_kv_heads : 0;
         slots += (long long)q.B * pl.n_kv_heads;
     }
     pl.total_units = units;
-    pl.tail_begin[0] = (int)it0;
-    pl.tail_begin[1] = (int)it1;
-    pl.n_items[kSweep1] = (int)(it0 + (long long)pl.tail_sets[0] * n_req * pl.n_q_heads);
-    pl.n_items[kSweep2] = (int)(it1 + (long long)pl.tail_sets[1] * n_req * pl.n_q_heads);
+    pl.tail_begin = (int)it0;                       // (the same in both sweeps: see above)
+    pl.n_items[kSweep1] = (int)(it0 + (long long)pl.tail_sets * n_req * pl.n_q_heads);
+    pl.n_items[kSweep2] = (int)(it1 + (long long)pl.tail_sets * n_req * pl.n_q_heads);
     pl.n_items[kMatch] = (int)it2;
 
     size_t o = 0;
@@ -223,7 +225,7 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
     // head) and over how the sweeps are cut, so the carving depends only on the prompt lengths and head
     // counts and never shrinks with more query heads: a size computed for a layout also serves the entry
     // points that know its KV heads alone.
-    const size_t score_parts = pl.blocks[1] > 1 ? pl.group : pl.splits[1];       // partial column sums of sweep 2
+    const size_t score_parts = pl.blocks > 1 ? pl.group : pl.splits[1];       // partial column sums of sweep 2
     for (int s = 0; s < 2; ++s)
         if (pl.splits[s] > 1 || (s && score_parts > 1)) pl.n_arrived[s] = 4 * (size_t)tiles * (s ? Hkv : Hq);
     pl.clear_words += pl.n_arrived[0] + pl.n_arrived[1];
@@ -242,7 +244,7 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
     pl.o_rnorm_kept = carve(4 * Hkv * T);
     pl.o_assign = carve(4 * Hkv * T);
     pl.o_sim = carve(4 * Hkv * T);
-    pl.o_row_ptr = carve(4 * (Hkv * T + Hkv * (size_t)n_req));
+    pl.o_row_begin = carve(4 * (Hkv * T + Hkv * (size_t)n_req));
     pl.o_entries = carve(8 * Hkv * T);
     pl.o_units = carve(16 * (size_t)pl.total_units);
     pl.o_slot_cnt = carve(4 * Hkv * T);
@@ -391,6 +393,9 @@ TileParams tile_params(const Plan& pl, void* ws, const lookm_layout* lay) {
     p.T = pl.T;
     p.scale_log2 = scale_log2(lay);
     p.status = at<int>(ws, pl.o_status);
+    p.blocks = pl.blocks;
+    p.tail_begin = pl.tail_begin;
+    p.tail_sets = pl.tail_sets;
     return p;
 }
 
@@ -408,10 +413,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     p.scores = scores;
     if (!lse_is_input) {
         p.n_items = pl.n_items[kSweep1];
-        p.blocks = pl.blocks[0];
         p.next_item = p.status + 16 + kSweep1;
-        p.tail_begin = pl.tail_begin[0];
-        p.tail_sets = pl.tail_sets[0];
         p.splits = pl.splits[0];
         p.parts1 = at<float2>(ws, pl.o_kept_keys);
         p.arrived = p.status + 64;
@@ -423,10 +425,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     }
     mark_stage(1, st);
     p.n_items = pl.n_items[kSweep2];
-    p.blocks = pl.blocks[1];
     p.next_item = p.status + 16 + kSweep2;
-    p.tail_begin = pl.tail_begin[1];
-    p.tail_sets = pl.tail_sets[1];
     p.splits = pl.splits[1];
     p.parts2 = at<float>(ws, pl.o_kept_keys);
     p.arrived = p.status + 64 + pl.n_arrived[0];
@@ -480,7 +479,7 @@ constexpr int kInvMinShare = 512;
 cudaError_t run_inversion(const Plan& pl, const DeviceInfo& di, const int* kept_idx, const int* evict_idx, const int* assign,
                           const float* sim, void* ws, cudaStream_t st) {
     const Req* reqs = at<Req>(ws, pl.o_reqs);
-    int *status = at<int>(ws, pl.o_status), *row_ptr = at<int>(ws, pl.o_row_ptr);
+    int *status = at<int>(ws, pl.o_status), *row_begin = at<int>(ws, pl.o_row_begin);
     int2* entries = at<int2>(ws, pl.o_entries);
     int4* units = at<int4>(ws, pl.o_units);
     int* slot_cnt = at<int>(ws, pl.o_slot_cnt);
@@ -497,7 +496,7 @@ cudaError_t run_inversion(const Plan& pl, const DeviceInfo& di, const int* kept_
     int ctas = ctas_per_head(std::min(kInvCtasPerSm, std::max(1ll, kInvSmemPerSm / slot_bytes)));
     if (pl.max_B <= kCountMaxSlots && pl.max_E <= ctas * kCountWarps * kCountSeg) {
         const int max_slots = ctas * (((pl.max_B + ctas - 1) / ctas + 3) / 4 * 4);
-        return launch_invert_counting(assign, kept_idx, evict_idx, sim, reqs, pl.n_req, pl.n_kv_heads, ctas, max_slots, pl.T, row_ptr,
+        return launch_invert_counting(assign, kept_idx, evict_idx, sim, reqs, pl.n_req, pl.n_kv_heads, ctas, max_slots, pl.T,
                                       entries, units, slot_cnt, status, st);
     }
     // counter width and widest digit over the requests of the call
@@ -509,7 +508,7 @@ cudaError_t run_inversion(const Plan& pl, const DeviceInfo& di, const int* kept_
         invert_digits(r.B, wide ? kInvDigitBits32 : kInvDigitBits16, n_pass, dbits);
         digit_bits = std::max(digit_bits, dbits);
     }
-    return launch_invert_assignment(assign, kept_idx, evict_idx, sim, reqs, pl.n_req, pl.n_kv_heads, ctas, pl.T, wide, digit_bits, row_ptr,
+    return launch_invert_assignment(assign, kept_idx, evict_idx, sim, reqs, pl.n_req, pl.n_kv_heads, ctas, pl.T, wide, digit_bits, row_begin,
                                     entries, units, slot_cnt, at<unsigned>(ws, pl.o_sort_a), at<unsigned>(ws, pl.o_sort_b),
                                     status, st);
 }
@@ -534,11 +533,10 @@ int run_merge(const Plan& pl, const lookm_layout* lay, const void* k, const void
                                           pl.out_stride_head, out_k, out_v, status, di.sms, st));
         else
             LOOKM_CUDA(launch_merge(k, v, lay->kv_stride_tok, lay->kv_stride_head, reqs, pl.n_req,
-                                    pl.n_kv_heads, pl.T, pl.total_units, at<int>(ws, pl.o_row_ptr),
-                                    at<int2>(ws, pl.o_entries),
+                                    pl.n_kv_heads, pl.T, pl.total_units, at<int2>(ws, pl.o_entries),
                                     at<int4>(ws, pl.o_units), at<int>(ws, pl.o_slot_cnt),
                                     at<float>(ws, pl.o_parts), varlen_output, pl.out_stride_head, out_k,
-                                    out_v, status, di.sms, st));
+                                    out_v, di.sms, st));
         ++g_launches;
     }
     if (pl.n_none > 0) {
@@ -906,7 +904,7 @@ extern "C" int lookm_merge_noalloc(const void* k, const void* v, const int* kept
     pl.clear_words = 64;
     pl.o_status = carve(256);
     pl.o_reqs = carve(sizeof(Req) * (size_t)n_requests);
-    pl.o_row_ptr = carve(4 * (units + (size_t)pl.n_kv_heads * (size_t)n_requests));
+    pl.o_row_begin = carve(4 * (units + (size_t)pl.n_kv_heads * (size_t)n_requests));
     pl.o_entries = carve(8 * units);
     pl.o_units = carve(16 * (size_t)pl.total_units);
     pl.o_slot_cnt = carve(4 * (size_t)pl.total_slots);

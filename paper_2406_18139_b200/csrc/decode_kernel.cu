@@ -352,6 +352,8 @@ constexpr int kMmaRows = 16;                         // rows per warp and step
 constexpr int kMmaRing = 3;                          // steps in a warp's ring (all but one in flight)
 constexpr int kMmaStepBytes = 2 * kMmaRows * kDecRowBytes;         // [K|V][row][256 B]
 constexpr int kMmaRingBytes = kMmaWarps * kMmaRing * kMmaStepBytes;
+static_assert(kMmaRingBytes * (kDecodeMaxCtasPerSm + 1) > (228 << 10) && kDecRingBytes * (kDecodeMaxCtasPerSm + 1) > (228 << 10),
+              "the workspace has room for the splits of kDecodeMaxCtasPerSm CTAs per SM");
 constexpr float kMmaSlack = 8.f;                     // log2 by which a logit may exceed the reference
 
 __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {

@@ -52,8 +52,8 @@ struct Req {
     long long kept_off;   // n_kv_heads * out_begin          (start of this request's kept lists)
     long long ev_off;     // n_kv_heads * sum of E before    (start of this request's evicted lists)
     long long sim_off;    // n_kv_heads * sum of E*B before  (start of its similarity blocks)
-    long long rp_off;     // kept_off + n_kv_heads * (caller index): start of its row_ptr blocks,
-                          // which hold B + 1 entries per head
+    long long rp_off;     // kept_off + n_kv_heads * (caller index): start of its scratch of the sorting
+                          // inversion, B + 1 words per head
     int item_begin[3];    // first work item of this request in sweep 1 / sweep 2 / match order
     int slot_begin;       // first (head, slot) row of this request in merge order (table order)
     int unit_entries;     // entries read per merge work unit: chosen per call so that every warp
@@ -135,13 +135,13 @@ cudaError_t launch_write_table(const ReqChunk& chunk, int count, Req* dst, int* 
 
 cudaError_t launch_invert_assignment(const int* assign, const int* kept_idx, const int* evict_idx,
                                      const float* sim, const Req* reqs, int n_req, int n_kv_heads, int ctas,
-                                     long long T, bool wide_counts, int digit_bits, int* row_ptr,
+                                     long long T, bool wide_counts, int digit_bits, int* row_begin,
                                      int2* entries, int4* unit_first, int* slot_cnt,
                                      unsigned* sort_a, unsigned* sort_b, int* status,
                                      cudaStream_t stream);
 
 cudaError_t launch_invert_counting(const int* assign, const int* kept_idx, const int* evict_idx, const float* sim, const Req* reqs,
-                                   int n_req, int n_kv_heads, int ctas, int max_slots, long long T, int* row_ptr, int2* entries,
+                                   int n_req, int n_kv_heads, int ctas, int max_slots, long long T, int2* entries,
                                    int4* unit_first, int* slot_cnt, int* status, cudaStream_t stream);
 
 // Inversion and merge in one launch; every request has at most kMergeShortMax tokens.
@@ -155,10 +155,10 @@ int merge_warps_per_sm();
 
 cudaError_t launch_merge(const void* k, const void* v, long long stride_tok, long long stride_head,
                          const Req* reqs, int n_req, int n_kv_heads, long long T,
-                         long long total_units, const int* row_ptr, const int2* entries,
+                         long long total_units, const int2* entries,
                          const int4* unit_first, int* slot_cnt, float* parts,
                          int varlen_output, long long out_stride_head, void* out_k, void* out_v,
-                         int* status, int num_sms, cudaStream_t stream);
+                         int num_sms, cudaStream_t stream);
 
 // Kept K and V rows of the requests whose mode is LOOKM_MERGE_NONE copied to the output cache
 // (eviction alone, Eq. 6-7); requests with another mode are left to the merge kernel.
@@ -187,7 +187,7 @@ struct DecodeBatch { int n_req; int pad; DecodeReq r[kDecodeChunk]; };
 #define LOOKM_DEC_THREADS 256
 #endif
 constexpr int kDecodeThreads = LOOKM_DEC_THREADS;             // threads per CTA of the decode kernel
-constexpr int kDecodeMaxCtasPerSm = 2048 / kDecodeThreads;    // what an SM's thread limit allows
+constexpr int kDecodeMaxCtasPerSm = 2048 / kDecodeThreads;    // more than the kernels' rings let an SM hold
 constexpr int kDecodeMaxCluster = 8;     // splits of a (KV head, pass) that one thread-block cluster adds up
 int decode_ctas_per_sm(int gt, bool mma);    // resident CTAs per SM of the kernel (0: unknown)
 

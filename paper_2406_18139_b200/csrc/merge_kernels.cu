@@ -156,9 +156,9 @@ argmax_rows_kernel(const float* __restrict__ sim_matrix, const Req* __restrict__
 
 // ---------------------------------------------------------------------------------------------
 // Inversion of the assignment: for each (request, head) a stable sort of the evicted ranks by
-// their kept slot gives, per kept row, its members in ascending position, as CSR
-// (row_ptr [B + 1 per (request, head)], member positions and weights [E]).  A cluster of CTAs per
-// (request, head); stable LSD radix sort: every warp of the cluster owns a contiguous segment of the
+// their kept slot gives, per kept row, its members in ascending position; the result is the merge
+// kernel's entry list (position and weight of every kept row and, behind it, of its members).  A cluster
+// of CTAs per (request, head); stable LSD radix sort: every warp of the cluster owns a contiguous segment of the
 // list, ranks equal digits inside a 32-element step with ballots, and adds the counts of earlier steps,
 // of earlier warps and, read from their shared memory, of earlier CTAs.
 // What bounds it is the chain of dependent steps, not the bytes: a list of 26214 evicted tokens is 100
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(kInvThreads, 2)
 invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__ kept_idx,
                          const int* __restrict__ evict_idx,
                          const float* __restrict__ sim, const Req* __restrict__ reqs,
-                         int n_kv_heads, int ctas, long long T, int* row_ptr,
+                         int n_kv_heads, int ctas, long long T, int* row_begin,
                          int2* __restrict__ entries,
                          int4* __restrict__ unit_first, int* __restrict__ slot_cnt,
                          unsigned* sort_a, unsigned* sort_b, int* status) {
@@ -228,7 +228,7 @@ invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__
     const int h = blockIdx.x / ctas, cta = blockIdx.x % ctas;     // the cluster: the CTAs of one head
     const int E = rq.E, B = rq.B;
     const long long ev_base = rq.ev_off + (long long)h * E;
-    int* rp = row_ptr + rq.rp_off + (long long)h * (B + 1);
+    int* rp = row_begin + rq.rp_off + (long long)h * (B + 1);     // scratch of several passes: first member of a slot
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
     const int thread = cta * kInvThreads + threadIdx.x, n_threads = ctas * kInvThreads;   // of the cluster
@@ -241,7 +241,6 @@ invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__
     const int* kept_idx_head = kept_idx + rq.kept_off + (long long)h * B;
     const bool weighted = (rq.mode == LOOKM_MERGE_WEIGHTED);
     if (E == 0) {
-        for (int c = thread; c <= B; c += n_threads) rp[c] = 0;
         for (int c = thread; c < B; c += n_threads) kept.write(c, kept_idx_head[c], 0, 0);
         return;
     }
@@ -403,12 +402,11 @@ invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__
     }
     if (n_pass == 1) {
         // digit = slot: digit_begin[c] is the first sorted index whose slot is >= c
-        auto row_begin = [&](int c) { return c < nd ? digit_begin[c] : E; };
-        for (int c = thread; c <= B; c += n_threads) rp[c] = row_begin(c);
-        for (int c = thread; c < B; c += n_threads) kept.write(c, kept_idx_head[c], row_begin(c), row_begin(c + 1) - row_begin(c));
+        auto begin = [&](int c) { return c < nd ? digit_begin[c] : E; };
+        for (int c = thread; c < B; c += n_threads) kept.write(c, kept_idx_head[c], begin(c), begin(c + 1) - begin(c));
         return;
     }
-    // row boundaries: row_ptr[c] = first sorted index whose slot is >= c
+    // row boundaries: rp[c] = first sorted index whose slot is >= c
     const unsigned* fin_k = key_buf[(n_pass - 1) & 1];
     for (int i0 = thread; i0 < E; i0 += n_threads * kInvBatch) {
         int cur[kInvBatch], prev[kInvBatch];
@@ -451,7 +449,7 @@ __device__ __forceinline__ int bytes_sum(const uint4& v, const uint4& m) {
 __global__ void __launch_bounds__(kInvThreads, 2)
 invert_counting_kernel(const int* __restrict__ assign, const int* __restrict__ kept_idx, const int* __restrict__ evict_idx,
                        const float* __restrict__ sim, const Req* __restrict__ reqs, int n_kv_heads, int ctas, int max_slots,
-                       long long T, int* __restrict__ row_ptr, int2* __restrict__ entries,
+                       long long T, int2* __restrict__ entries,
                        int4* __restrict__ unit_first, int* __restrict__ slot_cnt, int* status) {
     extern __shared__ __align__(16) unsigned char inv_smem[];
     __shared__ int warp_sums[kInvWarps];
@@ -473,7 +471,6 @@ invert_counting_kernel(const int* __restrict__ assign, const int* __restrict__ k
     const KeptEntries kept = {ent, unit_first + rq.unit_begin, slot_cnt + rq.kept_off + (long long)h * B, status,
                               rq.L, rq.unit_entries, h, n_kv_heads};
     const int* kept_idx_head = kept_idx + rq.kept_off + (long long)h * B;
-    int* rp = row_ptr + rq.rp_off + (long long)h * (B + 1);
 
     // the warp's elements
     const int seg = (E + ctas * kInvThreads - 1) / (ctas * kInvThreads) * 32;
@@ -591,12 +588,9 @@ invert_counting_kernel(const int* __restrict__ assign, const int* __restrict__ k
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            if (d0 + j >= B) continue;
-            rp[d0 + j] = first[j];
-            kept.write(d0 + j, pc[j], first[j], all[j]);
+            if (d0 + j < B) kept.write(d0 + j, pc[j], first[j], all[j]);
         }
     }
-    if (cta == 0 && threadIdx.x == 0) rp[B] = E;
     sync();
 
     const auto before = [&](int v) {                     // ones in the bytes of word v that belong to earlier warps
@@ -661,11 +655,10 @@ __device__ __forceinline__ float4 ld_cg_f4(const float* p) { return __ldcg(reint
 __global__ void __launch_bounds__(kMergeWarps * 32)
 merge_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
              long long stride_tok, long long stride_head, const Req* __restrict__ reqs, int n_req,
-             int n_kv_heads, long long T, long long total_units, const int* __restrict__ row_ptr,
-             const int2* __restrict__ entries,
+             int n_kv_heads, long long T, long long total_units, const int2* __restrict__ entries,
              const int4* __restrict__ unit_first, int* __restrict__ slot_cnt, float* __restrict__ parts,
              int varlen_output, long long out_stride_head, __nv_bfloat16* __restrict__ out_k,
-             __nv_bfloat16* __restrict__ out_v, int* status) {
+             __nv_bfloat16* __restrict__ out_v) {
     extern __shared__ uint8_t merge_smem_raw[];
     MergeShared& sh = *reinterpret_cast<MergeShared*>(
         (reinterpret_cast<uintptr_t>(merge_smem_raw) + 127) & ~static_cast<uintptr_t>(127));
@@ -860,7 +853,6 @@ merge_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
                             __shfl_sync(0xffffffffu, u1, which), __shfl_sync(0xffffffffu, n, which));
         }
     }
-    (void)status;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1126,7 +1118,7 @@ cudaError_t launch_gather_kept(const void* k, long long stride_tok, long long st
 
 cudaError_t launch_invert_assignment(const int* assign, const int* kept_idx, const int* evict_idx,
                                      const float* sim, const Req* reqs, int n_req, int n_kv_heads, int ctas,
-                                     long long T, bool wide_counts, int digit_bits, int* row_ptr,
+                                     long long T, bool wide_counts, int digit_bits, int* row_begin,
                                      int2* entries, int4* unit_first, int* slot_cnt,
                                      unsigned* sort_a, unsigned* sort_b, int* status,
                                      cudaStream_t stream) {
@@ -1143,11 +1135,11 @@ cudaError_t launch_invert_assignment(const int* assign, const int* kept_idx, con
     if (err != cudaSuccess) return err;
     return launch_chained_clusters(wide_counts ? wide : narrow, dim3((unsigned)(n_kv_heads * ctas), (unsigned)n_req), dim3(kInvThreads),
                                    (unsigned)ctas, bytes(wide_counts ? 4 : 2, digit_bits), stream, assign, kept_idx, evict_idx, sim,
-                                   reqs, n_kv_heads, ctas, T, row_ptr, entries, unit_first, slot_cnt, sort_a, sort_b, status);
+                                   reqs, n_kv_heads, ctas, T, row_begin, entries, unit_first, slot_cnt, sort_a, sort_b, status);
 }
 
 cudaError_t launch_invert_counting(const int* assign, const int* kept_idx, const int* evict_idx, const float* sim, const Req* reqs,
-                                   int n_req, int n_kv_heads, int ctas, int max_slots, long long T, int* row_ptr, int2* entries,
+                                   int n_req, int n_kv_heads, int ctas, int max_slots, long long T, int2* entries,
                                    int4* unit_first, int* slot_cnt, int* status, cudaStream_t stream) {
     static unsigned long long configured = 0;
     cudaError_t err = once_per_device(configured, [&]() {
@@ -1157,17 +1149,17 @@ cudaError_t launch_invert_counting(const int* assign, const int* kept_idx, const
     if (err != cudaSuccess) return err;
     return launch_chained_clusters(invert_counting_kernel, dim3((unsigned)(n_kv_heads * ctas), (unsigned)n_req), dim3(kInvThreads),
                                    (unsigned)ctas, (size_t)max_slots * kCountSlotBytes, stream, assign, kept_idx, evict_idx, sim,
-                                   reqs, n_kv_heads, ctas, max_slots, T, row_ptr, entries, unit_first, slot_cnt, status);
+                                   reqs, n_kv_heads, ctas, max_slots, T, entries, unit_first, slot_cnt, status);
 }
 
 int merge_warps_per_sm() { return kMergeWarps; }
 
 cudaError_t launch_merge(const void* k, const void* v, long long stride_tok, long long stride_head,
                          const Req* reqs, int n_req, int n_kv_heads, long long T,
-                         long long total_units, const int* row_ptr, const int2* entries,
+                         long long total_units, const int2* entries,
                          const int4* unit_first, int* slot_cnt, float* parts,
                          int varlen_output, long long out_stride_head, void* out_k, void* out_v,
-                         int* status, int num_sms, cudaStream_t stream) {
+                         int num_sms, cudaStream_t stream) {
     if (total_units <= 0) return cudaSuccess;
     if (stride_tok <= 0 || stride_tok >= (1ll << 31)) return cudaErrorInvalidValue;   // byte stride kept in 32 bits
     const int smem = (int)sizeof(MergeShared) + 128;
@@ -1180,9 +1172,8 @@ cudaError_t launch_merge(const void* k, const void* v, long long stride_tok, lon
     if (blocks > num_sms) blocks = num_sms;              // persistent: one CTA per SM
     return launch_chained(merge_kernel, dim3((unsigned)blocks), dim3(kMergeWarps * 32), (size_t)smem, stream,
                           (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, stride_tok, stride_head, reqs,
-                          n_req, n_kv_heads, T, total_units, row_ptr, entries, unit_first, slot_cnt,
-                          parts, varlen_output, out_stride_head, (__nv_bfloat16*)out_k, (__nv_bfloat16*)out_v,
-                          status);
+                          n_req, n_kv_heads, T, total_units, entries, unit_first, slot_cnt,
+                          parts, varlen_output, out_stride_head, (__nv_bfloat16*)out_k, (__nv_bfloat16*)out_v);
 }
 
 // Parts per (request, head): about two CTAs per SM, at least eight slots each.

@@ -52,18 +52,8 @@ namespace {
 constexpr int kStages = LOOKM_TILE_STAGES;       // ring of streamed tiles
 constexpr int kABuf = LOOKM_TILE_ABUF;           // buffers of the stationary tile (2: the next item's is
                                                  // loaded while this item's is in use)
-#ifndef LOOKM_TILE_GROUPS
-#define LOOKM_TILE_GROUPS 4
-#endif
 constexpr int kAccum = 4;                        // TMEM accumulators (128 fp32 columns each)
-#ifndef LOOKM_TILE_HALVES
-#define LOOKM_TILE_HALVES 1
-#endif
-constexpr int kGroups = LOOKM_TILE_GROUPS;       // epilogue groups; tile g goes to group g mod kGroups
-constexpr int kHalves = LOOKM_TILE_HALVES;       // a group is kHalves PARTS of four warps; part p of a group
-                                                 // reads columns [p, p + 1) * kCols of the group's accumulators
-constexpr int kParts = kGroups * kHalves;        // four-warp units of the epilogue (each keeps partial results)
-constexpr int kCols = kTile / kHalves;           // accumulator columns per part
+constexpr int kGroups = 4;                       // epilogue groups of four warps; tile g goes to group g mod kGroups
 // "Accumulator filled" barriers form a ring twice as long as the accumulators: tile g uses barrier
 // g mod kFullRing in phase g / kFullRing.  A group may reach tile g while tile g - kAccum (same
 // accumulator, other group, other issuing thread) is still being multiplied; with one barrier per
@@ -73,15 +63,15 @@ constexpr int kCols = kTile / kHalves;           // accumulator columns per part
 constexpr int kFullRing = 2 * kAccum;
 constexpr int kIssuers = 2;                      // MMA-issuing threads (tiles alternate between them)
 constexpr int kEpiWarp0 = 2;                     // first epilogue warp
-constexpr int kGatherWarp = kEpiWarp0 + kParts * 4 + 1;    // match: gathers the evicted rows of the A tiles
+constexpr int kGatherWarp = kEpiWarp0 + kGroups * 4 + 1;    // match: gathers the evicted rows of the A tiles
 // Match: items of at most so many tiles wait for their stationary rows, so the gather warp sends all its
 // copies at once; with longer items, one ahead of the MMAs, it reads positions and sends copies in eights,
 // which leaves the streamed tiles more room.  Match in us, in eights and at once: 2 tiles an item (700
 // tokens x 32 heads) 16.4 and 14.3, 4 tiles (7777 x 8 at 5 %) 32.7 and 26.6, (2048 x 32) 24.6 and 20.5, 7
 // tiles (4096 x 32) 47 and 57, 13 tiles (8192 x 32) 126 and 155.
 constexpr int kBurstTiles = 4;
-// producer warp, MMA warp, kParts x 4 epilogue warps, second MMA warp (+ the gather warp of the match)
-__host__ __device__ constexpr int threads_of(int kind) { return 64 + kParts * 128 + 32 + (kind == kMatch ? 32 : 0); }
+// producer warp, MMA warp, kGroups x 4 epilogue warps, second MMA warp (+ the gather warp of the match)
+__host__ __device__ constexpr int threads_of(int kind) { return 64 + kGroups * 128 + 32 + (kind == kMatch ? 32 : 0); }
 constexpr int kHalfBytes = kTile * 64 * 2;       // one TMA box: 128 rows x 64 bf16 (128 B rows)
 constexpr int kTileBytes = 2 * kHalfBytes;       // 128 x 128 bf16
 constexpr int kSplitBytes = kTile * 16 * 2;      // 128 rows x 16 bf16 (32-byte rows, 32-byte swizzle)
@@ -94,15 +84,15 @@ constexpr float kLn2 = 0.6931471805599453f;
 template <int KIND>
 struct __align__(1024) Shared {
     static constexpr int kXStages = (KIND == kSweep2) ? kStages : 1;   // only sweep 2 streams companions
-    static constexpr int kPlanes = (KIND == kSweep2) ? 1 : 2;          // values per row and part to combine
+    static constexpr int kPlanes = (KIND == kSweep2) ? 1 : 2;          // values per row and group to combine
     uint8_t a[kABuf][kTileBytes];                // stationary tiles
     uint8_t b[kStages][kTileBytes];              // streamed tiles
     uint8_t bx[kXStages][kSplitBytes];           // sweep 2: the streamed tiles' 16-column companions
     union {
-        float side[kParts][2][kCols];            // match: per epilogue part, double-buffered column data
+        float side[kGroups][2][kTile];            // match: per epilogue group, double-buffered column data
         uint8_t ax[kSplitBytes];                 // sweep 2: constant ones tile that multiplies bx
     };
-    float comb[2][kParts][kPlanes][kTile];       // partial results of the parts, double-buffered
+    float comb[2][kGroups][kPlanes][kTile];       // partial results of the groups, double-buffered
     Req reqs[kReqCache];                         // copy of the request table (when it fits)
     unsigned long long a_full[kABuf], a_empty[kABuf];
     unsigned long long b_full[kStages], b_empty[kStages];
@@ -314,10 +304,10 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         }
         for (int i = 0; i < kFullRing; ++i) ptx::mbar_init(ptx::smem_u32(&sh.t_full[i]), 1);
         for (int i = 0; i < kAccum; ++i)
-            ptx::mbar_init(ptx::smem_u32(&sh.t_empty[i]), 4 * kHalves);   // one arrival per epilogue warp of a group
+            ptx::mbar_init(ptx::smem_u32(&sh.t_empty[i]), 4);   // one arrival per epilogue warp of a group
         for (int i = 0; i < 2; ++i) {
-            ptx::mbar_init(ptx::smem_u32(&sh.comb_full[i]), (kParts - 1) * 4);    // warps of the other parts
-            ptx::mbar_init(ptx::smem_u32(&sh.comb_free[i]), 4);                   // warps of the combining part
+            ptx::mbar_init(ptx::smem_u32(&sh.comb_full[i]), (kGroups - 1) * 4);    // warps of the other groups
+            ptx::mbar_init(ptx::smem_u32(&sh.comb_free[i]), 4);                   // warps of the combining group
         }
         ptx::mbar_init(ptx::smem_u32(&sh.mma_done), kIssuers);
         sh.abort_flag = 0;
@@ -476,7 +466,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.a_full[ab]));
         }
-    } else if (warp == 1 || warp == kEpiWarp0 + kParts * 4) {
+    } else if (warp == 1 || warp == kEpiWarp0 + kGroups * 4) {
         // ------------------------------------------------------------ MMA issuers -----------
         // One thread spends about as long on the waits, fences, commits and loop bookkeeping of a
         // tile as the tensor core needs for its eight MMAs, and it is blocked while they are
@@ -540,9 +530,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         }
     } else {
         // ------------------------------------------------------------ epilogue --------------
-        const int part = (warp - kEpiWarp0) >> 2;            // four-warp unit of the epilogue
-        const int wg = part / kHalves;                       // its group
-        const int col0 = (part % kHalves) * kCols;           // first accumulator column it reads
+        const int wg = (warp - kEpiWarp0) >> 2;              // group of the epilogue
         const int quarter = warp & 3;                        // TMEM lane quarter this warp may read
         const int row = quarter * 32 + lane;                 // row of the stationary tile
         const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
@@ -562,8 +550,8 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             float best = -INFINITY;                          // match
             int best_slot = 0x7fffffff;
             // match: 1 / |k| of this thread's evicted row takes two dependent loads (its position, then
-            // the norm).  They are requested here and after the part's first tile, not in the combine
-            // at the item's end, where the part that combines would sit out both round trips while
+            // the norm).  They are requested here and after the group's first tile, not in the combine
+            // at the item's end, where the group that combines would sit out both round trips while
             // its next accumulator stays full.
             int row_at = 0;
             float row_rnorm = 0.f;
@@ -581,7 +569,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             for (int t = 0; t < it.nt; ++t, ++gb) {
                 if ((int)(gb % kGroups) != wg) continue;
                 const int buf = (int)(gb % kAccum);
-                float* side = sh.side[part][lt & 1];
+                float* side = sh.side[wg][lt & 1];
                 bool diag = false;                           // tile crosses the causal diagonal
                 int col_limit = kTile;                       // valid columns of the tile (match, sweep 2)
                 int diag_from = 0;                           // sweep 2: first column this row may use
@@ -595,12 +583,10 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                     diag = (ib == it.blk) || (col_limit < kTile);
                     diag_from = (ib == it.blk) ? row : 0;
                 } else {
-                    if (row < kCols) {
-                        const int slot = t * kTile + col0 + row;
-                        side[row] = (slot < it.B) ? p.rnorm_kept[it.kept_row0 + slot] : 0.f;
-                    }
+                    const int slot = t * kTile + row;
+                    side[row] = (slot < it.B) ? p.rnorm_kept[it.kept_row0 + slot] : 0.f;
                     col_limit = min(kTile, it.B - t * kTile);
-                    ptx::named_barrier_sync(1 + part, 128);
+                    ptx::named_barrier_sync(1 + wg, 128);
                 }
                 ++lt;
                 ptx::mbar_wait(ptx::smem_u32(&sh.t_full[gb % kFullRing]), (gb / kFullRing) & 1, abort_flag);
@@ -612,7 +598,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                     // beats the running best is its first column looked up, so a strict comparison
                     // in ascending slot order keeps the lowest slot.
                     auto columns16 = [&](const uint32_t (&r)[16], int c0) {      // c0: column of the tile
-                        const float4* sd = reinterpret_cast<const float4*>(side + (c0 - col0));
+                        const float4* sd = reinterpret_cast<const float4*>(side + c0);
                         float v[16];
 #pragma unroll
                         for (int c4 = 0; c4 < 4; ++c4) {
@@ -642,15 +628,15 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         }
                     };
                     uint32_t ra[16], rb[16];
-                    const uint32_t tbase = lane_addr + buf * kTile + col0;
+                    const uint32_t tbase = lane_addr + buf * kTile;
                     ptx::tmem_ld_32x16(tbase, ra);
 #pragma unroll
-                    for (int k = 0; k < kCols / 32; ++k) {
+                    for (int k = 0; k < kTile / 32; ++k) {
                         ptx::tmem_ld_wait16(ra);
                         ptx::tmem_ld_32x16(tbase + (2 * k + 1) * 16, rb, ra);
-                        columns16(ra, col0 + 2 * k * 16);
+                        columns16(ra, 2 * k * 16);
                         ptx::tmem_ld_wait16(rb);
-                        if (k < kCols / 32 - 1) {
+                        if (k < kTile / 32 - 1) {
                             ptx::tmem_ld_32x16(tbase + (2 * k + 2) * 16, ra, rb);
                         } else {
                             // everything is in registers: hand the accumulator back
@@ -658,7 +644,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                             __syncwarp();
                             if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.t_empty[buf]));
                         }
-                        columns16(rb, col0 + (2 * k + 1) * 16);
+                        columns16(rb, (2 * k + 1) * 16);
                     }
                     if (!rnorm_asked) ask_rnorm();
                     continue;
@@ -680,14 +666,14 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                     __syncwarp();
                     if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.t_empty[buf]));
                 };
-                const uint32_t tbase = lane_addr + buf * kTile + col0;
+                const uint32_t tbase = lane_addr + buf * kTile;
 #pragma unroll 1
-                for (int ch = 0; ch < kCols / 32; ++ch) {
+                for (int ch = 0; ch < kTile / 32; ++ch) {
                     uint32_t raw[32];
                     ptx::tmem_ld_32x32(tbase + ch * 32, raw);
                     ptx::tmem_ld_wait();
-                    if (ch == kCols / 32 - 1) release();
-                    process(raw, col0 + ch * 32);
+                    if (ch == kTile / 32 - 1) release();
+                    process(raw, ch * 32);
                 }
             }
 
@@ -697,59 +683,59 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             // item without waiting for anybody.  Values are always combined in group order.
             const int cslot = n & 1;
             const uint32_t cuse = static_cast<uint32_t>(n) >> 1;         // earlier uses of this buffer
-            const int combiner = static_cast<int>((gb - 1u) % kGroups) * kHalves + (kHalves - 1);
+            const int combiner = static_cast<int>((gb - 1u) % kGroups);
             float (*cb)[Shared<KIND>::kPlanes][kTile] = sh.comb[cslot];
             constexpr int kP1 = Shared<KIND>::kPlanes - 1;       // second value of a row (not in sweep 2)
-            // The buffer's previous contents (two items ago) have been read.  The combining part waits for
+            // The buffer's previous contents (two items ago) have been read.  The combining group waits for
             // this too: the parity of comb_full tells one use from the next only once the use before is
             // over, and a warp may come here ahead of others that have yet to arrive for that one (groups
             // without a tile in short items hold nobody back).
             ptx::mbar_wait(ptx::smem_u32(&sh.comb_free[cslot]), (cuse & 1u) ^ 1u, abort_flag);
-            if (part != combiner) {
-                if (KIND == kSweep1) { cb[part][0][row] = m_run; cb[part][kP1][row] = l_run; }
-                else if (KIND == kSweep2) { cb[part][0][row] = (acc[0] + acc[1]) + (acc[2] + acc[3]); }
-                else { cb[part][0][row] = best; cb[part][kP1][row] = __int_as_float(best_slot); }
+            if (wg != combiner) {
+                if (KIND == kSweep1) { cb[wg][0][row] = m_run; cb[wg][kP1][row] = l_run; }
+                else if (KIND == kSweep2) { cb[wg][0][row] = (acc[0] + acc[1]) + (acc[2] + acc[3]); }
+                else { cb[wg][0][row] = best; cb[wg][kP1][row] = __int_as_float(best_slot); }
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.comb_full[cslot]));
             } else {
                 ptx::mbar_wait(ptx::smem_u32(&sh.comb_full[cslot]), cuse & 1u, abort_flag);
                 if (pos < (KIND == kMatch ? it.E : it.L) && !*abort_flag) {
                     if (KIND == kSweep1) {
-                        float mg[kParts], lg[kParts];
+                        float mg[kGroups], lg[kGroups];
 #pragma unroll
-                        for (int g = 0; g < kParts; ++g) {
-                            mg[g] = (g == part) ? m_run : cb[g][0][row];
-                            lg[g] = (g == part) ? l_run : cb[g][kP1][row];
+                        for (int g = 0; g < kGroups; ++g) {
+                            mg[g] = (g == wg) ? m_run : cb[g][0][row];
+                            lg[g] = (g == wg) ? l_run : cb[g][kP1][row];
                         }
                         float m = mg[0];
 #pragma unroll
-                        for (int g = 1; g < kParts; ++g) m = fmaxf(m, mg[g]);
+                        for (int g = 1; g < kGroups; ++g) m = fmaxf(m, mg[g]);
                         float l = lg[0] * ptx::ex2((mg[0] - m) * c2);
 #pragma unroll
-                        for (int g = 1; g < kParts; ++g) l += lg[g] * ptx::ex2((mg[g] - m) * c2);
+                        for (int g = 1; g < kGroups; ++g) l += lg[g] * ptx::ex2((mg[g] - m) * c2);
                         if (kSplits && it.n_splits > 1)
                             __stcg(p.parts1 + ((long long)it.split * p.n_q_heads + it.head) * p.T + it.tok_begin + pos, make_float2(m, l));
                         else
                             store_lse(p, it.head, it.tok_begin + pos, m, l);
                     } else if (KIND == kSweep2) {
                         const float own = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-                        float a = (part == 0) ? own : cb[0][0][row];
+                        float a = (wg == 0) ? own : cb[0][0][row];
 #pragma unroll
-                        for (int g = 1; g < kParts; ++g) a += (g == part) ? own : cb[g][0][row];
+                        for (int g = 1; g < kGroups; ++g) a += (g == wg) ? own : cb[g][0][row];
                         if (kSplits && it.n_splits > 1)
                             __stcg(p.parts2 + ((long long)it.split * p.n_kv_heads + it.head) * p.T + it.tok_begin + pos, a);
                         else
                             p.scores[(long long)it.head * p.T + it.tok_begin + pos] = a;
                     } else {
-                        if (!rnorm_asked) ask_rnorm();           // a part without a tile in this item
+                        if (!rnorm_asked) ask_rnorm();           // a group without a tile in this item
                         const int e = pos;
                         {
-                            float bb = (part == 0) ? best : cb[0][0][row];
-                            int bs = (part == 0) ? best_slot : __float_as_int(cb[0][kP1][row]);
+                            float bb = (wg == 0) ? best : cb[0][0][row];
+                            int bs = (wg == 0) ? best_slot : __float_as_int(cb[0][kP1][row]);
 #pragma unroll
-                            for (int g = 1; g < kParts; ++g) {
-                                const float b1 = (g == part) ? best : cb[g][0][row];
-                                const int s1 = (g == part) ? best_slot : __float_as_int(cb[g][kP1][row]);
+                            for (int g = 1; g < kGroups; ++g) {
+                                const float b1 = (g == wg) ? best : cb[g][0][row];
+                                const int s1 = (g == wg) ? best_slot : __float_as_int(cb[g][kP1][row]);
                                 if (b1 > bb || (b1 == bb && s1 < bs)) { bb = b1; bs = s1; }
                             }
                             p.assign[it.ev0 + e] = bs;
@@ -862,7 +848,7 @@ struct __align__(1024) MultiShared {
 static_assert(sizeof(MultiShared<kSweep1, 2>) + 1024 <= 232448 && sizeof(MultiShared<kSweep2, 2>) + 1024 <= 232448 &&
               sizeof(MultiShared<kSweep1, 4>) + 1024 <= 232448 && sizeof(MultiShared<kSweep2, 4>) + 1024 <= 232448,
               "shared memory of the multi-block sweeps exceeds 227 KB");
-static_assert(kAccum == 4 && kGroups == 4 && kHalves == 1 && kIssuers == 2, "the paired sweeps assume this layout");
+static_assert(kAccum == 4 && kGroups == 4 && kIssuers == 2, "the paired sweeps assume this layout");
 
 struct MultiItem {
     int tok_begin, L, blk, head, nt;
@@ -1272,7 +1258,7 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
         return e;
     });
     if (err != cudaSuccess) return err;
-    if (p.blocks > 1)
+    if (p.blocks > 1 && kind != kMatch)
         return launch_chained(multi[kind][p.blocks == 4], dim3(grid), dim3(threads_of(kSweep1)), multi_smem[kind][p.blocks == 4],
                               stream, map_a, map_b, mx, p);
     return launch_chained(kernels[kind][p.splits > 1], dim3(grid), dim3(threads_of(kind)), smem_of[kind], stream, map_a, map_b, mx, p);
