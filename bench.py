@@ -581,7 +581,8 @@ def run_ours(args):
                 "target": 0.50, "target_met": bool(512.0 / clocks_per_tile >= 0.50)}
     cap = captured_traffic()
     traffic = cap[dom] * (L * Hq) / (cap["tokens"] * cap["heads"]) if cap else None
-    roofline = {"kernel": "tile_kernel<%s>" % dom, "bound": "tensor", "achieved": stages[dom]["tflops"],
+    roofline = {"kernel": "%s (multi_kernel; tile_kernel at reduced sizes)" % dom, "bound": "tensor",
+                "achieved": stages[dom]["tflops"],
                 "peak": tf_peak, "peak_source": "%s (cuBLAS bf16, %s: timed region %.2f s, reasons %s)"
                 % (peaks["source"], regime, ms_total * 1e-3, clocks["reasons"]),
                 "unit": "TFLOP/s", "frac": stages[dom]["frac"], "frac_of_burst": stages[dom]["frac_of_burst"],

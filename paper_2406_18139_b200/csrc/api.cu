@@ -85,15 +85,16 @@ int sweep_blocks(const Plan& pl, long long sms) {
 }
 // The kTailSets shortest items of all prompts come last: with each prompt's items in a row the last
 // prompt's longest ones would end the sweep.  Scores of eight prompts of 4000 to 6000 tokens x 16 heads
-// (8.6 items per SM) 1122 -> 1094 us, four of 1000 to 12000 x 8 603 -> 590, three of 2000 to 3000 x 32 291 ->
-// 285.  Neighbouring CTAs then share no tiles in L2, which costs more where there are many items: 16 prompts
-// of 1000 to 3000 x 32 (14 per SM) 937 -> 944.
+// (8.6 items per SM), in rows | last: 1122 us | 1094, eight of 5000 x 16 1152 | 1051, four of 1000 to 12000 x 8
+// 603 | 590, three of 2000 to 3000 x 32 291 | 285.  Neighbouring CTAs then share no tiles in L2, which costs more
+// where there are many items: 16 prompts of 1000 to 3000 x 32 (14 per SM) 937 | 944, from 20 per SM no difference
+// beyond the scatter.
 constexpr int kTailSets = 6, kTailItemsPerSm = 12;
 // Splits of the sweep items: as many as bring the longest item down to what an SM has on average, if it
-// is more than one and a half times that and ten tiles longer.  Both sweeps together, us: 5000 tokens
-// with 2 heads 63.5 -> 38, 12000 with 2 query on 1 KV head 188 -> 110, 2048 with 32 on 8 78 -> 63, 700
-// with 32 on 8 35 -> 25; below ten tiles the partial results cost more than they save (2048 tokens with
-// 8 heads, 16 tiles against 7: 33 -> 37).
+// is more than one and a half times that and ten tiles longer.  Both sweeps together, us, whole | cut: 5000
+// tokens with 2 heads 63.5 | 38, 12000 with 2 query on 1 KV head 188 | 110, 2048 with 32 on 8 78 | 63, 700
+// with 32 on 8 35 | 25; ten tiles longer: 1300 x 1 23 | 18, 1300 x 4 23.7 | 22.3.  Nine: 1600 x 8 27 | 33, 2048 x 8 30 |
+// 36, 2600 x 8 38 | 42: the partial results cost more than they save.
 void plan_splits(Plan& pl) {
     DeviceInfo di;
     const long long sms = (device_info(di) == LOOKM_OK && di.sms > 0) ? di.sms : 148;
@@ -1005,9 +1006,10 @@ DecodeWay decode_way(const lookm_cache_layout* lay, int n_req, const int* lens, 
     // before two share one, smaller ones seven eighths: 16 heads x 8 took 5.7 us where 12 x 8 took
     // 3.1).  Worth it while a split is short, or at any length if the CTAs cover nearly all SMs (one
     // request of 32 heads x 4 or 64 x 2: 119 to 129 CTAs);
-    // us per step, two launches -> one: 32 heads x 4 splits 409 rows 4.6 -> 3.8, 8192 rows
-    // 24.4 -> 23.2; 12 x 8 1638 rows 5.3 -> 4.9, 8192 rows 12.6 -> 13.0; 16 x 4 800 rows 4.6 -> 4.7
-    // (5.8 instead of 8.0 with the launches issued one by one), 3000 rows 7.0 -> 9.1.
+    // us per step, two launches | one: 32 heads x 4 splits 409 rows 4.6 | 3.8, 3000 rows 10.2 | 9.2, 32768 rows
+    // 78.9 | 79.9; 31 x 4 8192 rows 23.3 | 22.1; 60 x 2 8192 rows 41.2 | 39.8; 64 x 2 32768 rows 165 | 159; 12 x 8
+    // 1638 rows 5.3 | 4.9, 8192 rows 12.6 | 13.0; 16 x 4 800 rows 4.6 | 4.7 (8.0 | 5.8 with the launches issued one
+    // by one), 3000 rows 6.9 | 9.0.
     int c = kDecodeMaxCluster;
     while (c > 1 && n_req * units * c > (c == 8 ? sms * 2 / 3 : sms * 7 / 8)) c /= 2;
     const long long rows = (longest + c - 1) / c;

@@ -162,8 +162,8 @@ argmax_rows_kernel(const float* __restrict__ sim_matrix, const Req* __restrict__
 // list, ranks equal digits inside a 32-element step with ballots, and adds the counts of earlier steps,
 // of earlier warps and, read from their shared memory, of earlier CTAs.
 // What bounds it is the chain of dependent steps, not the bytes: a list of 26214 evicted tokens is 100
-// KB.  One CTA of 32 warps per list -> up to eight of 16: 26214 evicted tokens x 8 heads into 6554 slots
-// 164 -> 43 us, 13107 x 40 into 3277 92 -> 46, 7388 x 8 into 389 22 -> 16.
+// KB.  One CTA of 32 warps per list | up to eight of 16: 26214 evicted tokens x 8 heads into 6554 slots
+// 164 | 43 us, 13107 x 40 into 3277 92 | 46, 7388 x 8 into 389 22 | 16.
 // ---------------------------------------------------------------------------------------------
 constexpr int kInvThreads = 512;
 constexpr int kInvWarps = kInvThreads / 32;
@@ -857,14 +857,15 @@ merge_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
 
 // ---------------------------------------------------------------------------------------------
 // Inversion, merge and compaction in one launch, for short prompts.  There the two kernels above are
-// chains of round trips (table -> lists -> sort -> entry list in memory -> metadata -> rows -> records
-// -> counters) and a launch, not bandwidth.  A CTA owns the slots [c0, c1) of one (request, head): it
+// chains of round trips (table, lists, sort, entry list in memory, metadata, rows, records, counters) and a launch, not bandwidth.  A CTA owns the slots [c0, c1) of one (request, head): it
 // sorts the evicted tokens of its slots by slot (stable, counters in shared memory), keeps the entry
 // list in shared memory, and its warps walk equal shares of that list.  A slot whose entries straddle
 // shares is summed piecewise through shared memory, pieces in share order.
-// lookm_merge as a whole, two kernels -> one (us, graph replay): 700 tokens x 32 heads 26.7 -> 16.4,
-// 2048 x 8 28.7 -> 14.7, 2048 x 32 30.1 -> 23.0, 4096 x 8 30.8 -> 20.5, 4096 x 32 37.4 -> 34.9.  Every
-// CTA of a head sorts the whole evicted list, so the gain is gone soon after kMergeShortMax.
+// lookm_merge as a whole, two kernels | one (us, graph replay): 700 tokens x 32 heads 26.7 | 16.4,
+// 2048 x 8 28.7 | 14.7, 2048 x 32 30.1 | 23.0, 4096 x 8 30.8 | 20.5, 4096 x 32 37.4 | 34.9; batches, where one CTA
+// has a whole head: 200 prompts of 100 x 32 466 | 200, 16 of 1000 x 32 166 | 89, 64 of 1000 x 8 171 | 94, 16 of 4000
+// x 32 364 | 334.  Every CTA of a head sorts the whole evicted list, so the gain is gone soon after
+// kMergeShortMax.
 // ---------------------------------------------------------------------------------------------
 constexpr int kFuseThreads = 512;
 constexpr int kFuseWarps = kFuseThreads / 32;

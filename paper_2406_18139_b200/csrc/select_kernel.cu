@@ -10,15 +10,15 @@
 // Either way one class is kept wholesale or not at all and the other needs an exact top-k.  The k-th
 // largest key (order-preserving 32-bit image of the score) is found by bisection between the smallest
 // and the largest one: a step counts the keys at or above the middle, with the keys in registers and
-// one block barrier.  Ties at the threshold go to the lowest positions.  An ordered pass over the same
+// one block barrier.  (Prompts too long for the registers count 2048 parts of that range instead, see
+// select_kernel.)  Ties at the threshold go to the lowest positions.  An ordered pass over the same
 // registers writes the kept and evicted lists in ascending position: ballots number a warp's tokens, one
 // block scan the warps.
 //
 // The kernel is bound by the latency of one CTA's barriers and round trips.  A four-pass radix select
 // over a shared-memory histogram (its first digits nearly equal for all scores, so that the atomics
-// collide), two block scans and a second reading of the scores for the lists took, lookm_select with
-// 32 heads and in us, 14.4 at 700 tokens, 18.5 at 4096 and 22.6 at 8192; this takes 9.3, 12.3 and 14.4 (32768
-// tokens x 8 heads with the norms: 80 -> 50).
+// collide), two block scans and a second reading of the scores for the lists | this, lookm_select with 32
+// heads, us: 2048 tokens 14.4 | 8.9, 8192 18.4 | 15.0, 16384 30.7 | 25.4, 32768 55 | 44, 65536 122 | 89, 262144 513 | 386.
 //
 // The selection occupies only n_requests * n_kv_heads CTAs, so the same launch carries, in further
 // CTAs, work that does not depend on it and is needed next: 1 / |k| of every key row (the cosine
@@ -71,8 +71,8 @@ __device__ __forceinline__ float sum_squares(const uint4& u) {
 // r / n_kv_heads of head r % n_kv_heads; quotient, remainder and address are carried along instead of
 // computed every time.  The four rows are added up together, each ending in a quarter of the half-warp,
 // so that one root and one division serve all of them (with four sums over the half-warp and four of
-// these the loop was bound by instructions; the launch takes, before and after, 28.6 and 20.5 us with 8192
-// tokens x 32 heads, 66.6 and 49.6 with 16384 x 40, 437 and 317 with 16 prompts, 158314 tokens x 32).
+// these the loop is bound by instructions; the launch takes then | now 28.6 us | 20.5 with 8192 tokens x 32
+// heads, 66.6 | 49.6 with 16384 x 40).
 template <int kThreads>
 __device__ __forceinline__ void key_norms(const __nv_bfloat16* __restrict__ k, long long stride_tok,
                                           long long stride_head, int n_kv_heads, long long T,

@@ -66,9 +66,9 @@ constexpr int kEpiWarp0 = 2;                     // first epilogue warp
 constexpr int kGatherWarp = kEpiWarp0 + kGroups * 4 + 1;    // match: gathers the evicted rows of the A tiles
 // Match: items of at most so many tiles wait for their stationary rows, so the gather warp sends all its
 // copies at once; with longer items, one ahead of the MMAs, it reads positions and sends copies in eights,
-// which leaves the streamed tiles more room.  Match in us, in eights and at once: 2 tiles an item (700
-// tokens x 32 heads) 16.4 and 14.3, 4 tiles (7777 x 8 at 5 %) 32.7 and 26.6, (2048 x 32) 24.6 and 20.5, 7
-// tiles (4096 x 32) 47 and 57, 13 tiles (8192 x 32) 126 and 155.
+// which leaves the streamed tiles more room.  Match in us, in eights | at once: 2 tiles an item (700
+// tokens x 32 heads) 16.4 | 14.3, 4 tiles (2048 x 32) 24.6 | 20.5, 5 tiles (2048 x 32) 34 | 39, (4096 x 32) 58 |
+// 76, (16384 x 8) 59 | 77, (4096 x 8) 24.5 | 22.2, 7 tiles (4096 x 32) 60 | 71, 13 tiles (8192 x 32) 126 | 155.
 constexpr int kBurstTiles = 4;
 // producer warp, MMA warp, kGroups x 4 epilogue warps, second MMA warp (+ the gather warp of the match)
 __host__ __device__ constexpr int threads_of(int kind) { return 64 + kGroups * 128 + 32 + (kind == kMatch ? 32 : 0); }
@@ -790,10 +790,9 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 // The sweeps of large problems: an item owns kBlocks = 2 or 4 adjacent stationary blocks and every
 // streamed tile is multiplied with all of them, so a tile is brought into shared memory once per two or
 // four products.  These sweeps run at the board's power limit, where time is energy, and a tenth of that
-// goes into moving tiles from L2 (a build without the loads ran 9-11 % faster).  Whole layers in a row,
-// one block per item -> two -> four: 16384 tokens x 40 heads 4.45 -> 4.10 -> 3.92 ms, 32768 x 32 query
-// heads on 8 11.2 -> 10.6 -> 10.4 ms, 16 ragged prompts x 32 heads 24.4 -> 23.4 -> 22.5 ms, 8192 x 32
-// 0.918 -> 0.886 (four blocks: 0.93).
+// goes into moving tiles from L2 (a build without the loads ran 9-11 % faster).  Whole layers in a row, ms,
+// one block per item | two | four: 16384 tokens x 40 heads 4.45 | 4.10 | 3.92, 32768 x 32 query heads on 8
+// 11.2 | 10.6 | 10.4, 8192 x 32 0.918 | 0.886 | 0.93 (the rule: sweep_blocks in api.cu).
 // Two blocks: streamed tile g of the CTA goes to accumulators 2 (g mod 2) + block, and each accumulator
 // has one issuing thread (g mod 2) and one epilogue group, which works on one block and on the tiles of
 // one parity; the two groups of a block are combined at the item's end like the four of tile_kernel.
@@ -801,11 +800,10 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 // tile skips the blocks it lies above (sweep 1) or below (sweep 2).
 // A CTA starts with the item of its own index and takes further ones from a counter in global memory,
 // one ahead of need; the producer passes them on to the other roles through a ring in shared memory.
-// Prompts of different lengths come out uneven from a fixed deal (three prompts of 4655, 4945 and 1831
-// tokens x 32 heads: the fullest CTA 1.17 times the average): their scores took 597 us and take 567,
-// the batch of 16 prompts 22.7 -> 22.0 ms, 8192 x 32 901 -> 889 us.  Which CTA takes an item changes no
-// result: a block's tiles are added in their order, two blocks per item in the two parities of the
-// tile's index in the item.
+// Prompts of different lengths come out uneven from a fixed deal (the fullest CTA had 1.17 times the average
+// of three prompts of 1800 to 5000 tokens x 32 heads: scores dealt 597 us, by counter 567; 8192 x 32 901 | 889).
+// Which CTA takes an item changes no result: a block's tiles are added in their order, two blocks per
+// item in the two parities of the tile's index in the item.
 // ------------------------------------------------------------------------------------------------
 // Items announced to the roles of a CTA, -1: no more.
 struct ItemRing {

@@ -270,7 +270,7 @@ def test_select_is_bit_exact_on_oracle_scores(B, L, budget, window, n_text):
 @pytest.mark.parametrize("L,budget,window,n_text", [(2048, 400, 32, 300), (2049, 410, 31, 2049), (8192, 2000, 16, 900),
                                                      (8193, 1, 0, 50), (32768, 3000, 64, 5000), (32777, 32000, 64, 20000)])
 def test_select_at_the_edges_of_what_stays_in_registers(B, L, budget, window, n_text):
-    """256 or 1024 threads, one or four passes of keys in registers, keys read again beyond those;
+    """512 or 1024 threads, eight to 32 keys per thread in registers, keys read again beyond those;
     scores over 40 orders of magnitude, some zero or negative, some equal."""
     Hkv = 2
     s32 = np.exp(synth.normal(synth.stream_key(76, L), Hkv * L) * 15).astype(np.float32).reshape(Hkv, L)
