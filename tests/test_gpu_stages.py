@@ -138,7 +138,7 @@ def test_scores_of_items_cut_into_ranges(B, lens, Hq, Hkv):
                                          ([1665], 96, 96), ([1664], 112, 56), ([1665], 160, 160), ([2100], 128, 32),
                                          ([1300, 1300, 770, 1500, 129], 128, 128), ([1300, 1301, 770, 1409], 128, 32)])
 def test_scores_of_items_of_two_or_four_blocks(B, lens, Hq, Hkv):
-    """Enough heads for items of two blocks or four (the last four of the list), each query head of a group an
+    """Enough heads for items of two blocks or four (192 heads, and the last four of the list), each query head of a group an
     item of its own: one to four blocks in the last item of a prompt, requests of one block, a last block of one
     row; logits rise along the prompts."""
     import torch
