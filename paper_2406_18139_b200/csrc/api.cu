@@ -467,7 +467,7 @@ int run_match(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     p.rnorm_kept = rnorm_kept;
     p.assign = assign;
     p.sim = sim;
-    LOOKM_CUDA(launch_tile_kernel(kMatch, map_c, map_c, nullptr, p, di.sms, st));
+    LOOKM_CUDA(launch_match(map_c, p, di.sms, st));
     ++g_launches;
     mark_stage(5, st);
     return LOOKM_OK;

@@ -101,6 +101,9 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
                                const CUtensorMap* map_x, const TileParams& p, int num_sms,
                                cudaStream_t stream);
 
+// Matching of the evicted rows with the compacted kept keys (match_kernel.cu).
+cudaError_t launch_match(const CUtensorMap& map_kept, const TileParams& p, int num_sms, cudaStream_t stream);
+
 // lse_split from a given lse (for callers that supply their own log-sum-exp)
 cudaError_t launch_lse_split(const float* lse, int n_q_heads, long long T, float scale_log2,
                              unsigned short* lse_split, cudaStream_t stream);

@@ -1,7 +1,6 @@
-// Tensor-core kernels of the path: the two sweeps of the cumulative attention score (Eq. 4) and
-// the cosine matching with fused row argmax (Eq. 9).
+// The two sweeps of the cumulative attention score (Eq. 4).
 //
-// All three are the same persistent, warp-specialised pipeline over 128 x 128 x 128 bf16 tiles:
+// Both are the same persistent, warp-specialised pipeline over 128 x 128 x 128 bf16 tiles:
 //   - a work item owns one STATIONARY 128-row tile (the A operand, rows on the 128 TMEM lanes)
 //     and streams a sequence of 128-row tiles (the B operand) against it;
 //   - warp 0 (one thread) issues the TMA loads, warps 1 and 18 (one thread each, tiles taken
@@ -10,9 +9,9 @@
 //     owns accumulator w and takes the tiles whose running index is w mod 4, so each SM
 //     sub-partition always has four epilogue warps to switch between;
 //   - each epilogue thread owns one row of the stationary tile, so every reduction over the
-//     streamed axis (row maximum and sum, column-sum of probabilities for one key, running
-//     arg-max) stays in that thread's registers; the four groups are combined through shared
-//     memory once per item.  No L x L matrix is ever stored.
+//     streamed axis (row maximum and sum, column-sum of probabilities for one key) stays in
+//     that thread's registers; the four groups are combined through shared memory once per
+//     item.  No L x L matrix is ever stored.
 //
 //   sweep 1: A = 128 queries of one query head, B = key tiles 0..diagonal.  Online softmax
 //            statistics per query row  ->  lse[i] = log sum_{j<=i} exp(s_ij).
@@ -22,10 +21,6 @@
 //            three bf16 terms in a 16-column companion of the query tensor, and a ninth MMA per
 //            tile multiplies it with a constant tile of ones, so the accumulator already holds
 //            s_ij - lse_i / scale and the epilogue needs no per-column data at all.
-//   match  : A = 128 EVICTED key rows in the order of the evicted list, gathered by a warp of its
-//            own with 16-byte cp.async copies into the 128-byte-swizzled layout the tensor core
-//            expects; B = tiles of the compacted kept keys.  Thread keeps the largest
-//            s_ij / |k_j| and its slot.
 //
 // A small problem has fewer or more uneven sweep items than the CTAs can share.  Then the streamed tiles of an item are cut into
 // p.splits ranges, items of their own that leave partial results in memory; the one that arrives last
@@ -63,15 +58,8 @@ constexpr int kGroups = 4;                       // epilogue groups of four warp
 constexpr int kFullRing = 2 * kAccum;
 constexpr int kIssuers = 2;                      // MMA-issuing threads (tiles alternate between them)
 constexpr int kEpiWarp0 = 2;                     // first epilogue warp
-constexpr int kGatherWarp = kEpiWarp0 + kGroups * 4 + 1;    // match: gathers the evicted rows of the A tiles
-// Match: items of at most so many tiles wait for their stationary rows, so the gather warp sends all its
-// copies at once; with longer items, one ahead of the MMAs, it reads positions and sends copies in eights,
-// which leaves the streamed tiles more room.  Match in us, in eights | at once: 2 tiles an item (700
-// tokens x 32 heads) 16.4 | 14.3, 4 tiles (2048 x 32) 24.6 | 20.5, 5 tiles (2048 x 32) 34 | 39, (4096 x 32) 58 |
-// 76, (16384 x 8) 59 | 77, (4096 x 8) 24.5 | 22.2, 7 tiles (4096 x 32) 60 | 71, 13 tiles (8192 x 32) 126 | 155.
-constexpr int kBurstTiles = 4;
-// producer warp, MMA warp, kGroups x 4 epilogue warps, second MMA warp (+ the gather warp of the match)
-__host__ __device__ constexpr int threads_of(int kind) { return 64 + kGroups * 128 + 32 + (kind == kMatch ? 32 : 0); }
+// producer warp, MMA warp, kGroups x 4 epilogue warps, second MMA warp
+constexpr int kThreads = 64 + kGroups * 128 + 32;
 constexpr int kHalfBytes = kTile * 64 * 2;       // one TMA box: 128 rows x 64 bf16 (128 B rows)
 constexpr int kTileBytes = 2 * kHalfBytes;       // 128 x 128 bf16
 constexpr int kSplitBytes = kTile * 16 * 2;      // 128 rows x 16 bf16 (32-byte rows, 32-byte swizzle)
@@ -88,10 +76,7 @@ struct __align__(1024) Shared {
     uint8_t a[kABuf][kTileBytes];                // stationary tiles
     uint8_t b[kStages][kTileBytes];              // streamed tiles
     uint8_t bx[kXStages][kSplitBytes];           // sweep 2: the streamed tiles' 16-column companions
-    union {
-        float side[kGroups][2][kTile];            // match: per epilogue group, double-buffered column data
-        uint8_t ax[kSplitBytes];                 // sweep 2: constant ones tile that multiplies bx
-    };
+    uint8_t ax[kSplitBytes];                     // sweep 2: constant ones tile that multiplies bx
     float comb[2][kGroups][kPlanes][kTile];       // partial results of the groups, double-buffered
     Req reqs[kReqCache];                         // copy of the request table (when it fits)
     unsigned long long a_full[kABuf], a_empty[kABuf];
@@ -102,8 +87,8 @@ struct __align__(1024) Shared {
     uint32_t tmem_base;
     int abort_flag;
 };
-static_assert(sizeof(Shared<kSweep1>) + 1024 <= 232448 && sizeof(Shared<kSweep2>) + 1024 <= 232448 &&
-              sizeof(Shared<kMatch>) + 1024 <= 232448, "shared memory of the tile kernels exceeds 227 KB");
+static_assert(sizeof(Shared<kSweep1>) + 1024 <= 232448 && sizeof(Shared<kSweep2>) + 1024 <= 232448,
+              "shared memory of the tile kernels exceeds 227 KB");
 
 // The softmax epilogues are bound by the special-function unit (16 ex2 per clock and SM), so one
 // column in kPolyEvery is exponentiated on the FMA pipe instead.
@@ -213,12 +198,10 @@ __device__ __forceinline__ void write_ones_row(uint8_t* ax, int r) {
 }
 
 struct Item {
-    int tok_begin, L, B, E, blk, head, nt;
+    int tok_begin, L, blk, head, nt;
     int t0;                   // first streamed tile of the item (the sweeps' splits)
     int split, n_splits;      // which range of the block's tiles, of how many
     int tile;                 // index of the block over the whole batch
-    long long kept_row0;      // match: first row of this (request, head) in the kept-key matrix
-    long long ev0;            // match: start of its evicted list
 };
 
 template <int KIND, bool kSplits>
@@ -233,38 +216,27 @@ __device__ __forceinline__ Item decode_item(const TileParams& p, const Req* tbl,
     Item it;
     it.tok_begin = rq.tok_begin;
     it.L = rq.L;
-    it.B = rq.B;
-    it.E = rq.E;
     it.t0 = 0;
     it.split = 0;
     it.n_splits = 1;
-    it.kept_row0 = 0;
-    it.ev0 = 0;
-    if (KIND != kMatch) {                        // heaviest first: last query block, first key block
-        const int heads = (KIND == kSweep1 ? p.n_q_heads : p.n_kv_heads) * (kSplits ? p.splits : 1);
-        const int b = u / heads, v = u % heads;
-        it.blk = KIND == kSweep1 ? rq.nblk - 1 - b : b;
-        it.nt = KIND == kSweep1 ? it.blk + 1 : (rq.nblk - it.blk) * p.group;
-        it.head = v;
-        if (kSplits) {
-            it.head = v / p.splits;
-            it.split = v % p.splits;
-            it.n_splits = min(p.splits, it.nt);
-            it.tile = rq.tile_begin + it.blk;
-            const int all = it.nt;
-            if (it.split < it.n_splits) {
-                it.t0 = all * it.split / it.n_splits;
-                it.nt = all * (it.split + 1) / it.n_splits - it.t0;
-            } else {
-                it.nt = 0;                       // no tile: every role passes over the item
-            }
+    // heaviest first: last query block, first key block
+    const int heads = (KIND == kSweep1 ? p.n_q_heads : p.n_kv_heads) * (kSplits ? p.splits : 1);
+    const int b = u / heads, v = u % heads;
+    it.blk = KIND == kSweep1 ? rq.nblk - 1 - b : b;
+    it.nt = KIND == kSweep1 ? it.blk + 1 : (rq.nblk - it.blk) * p.group;
+    it.head = v;
+    if (kSplits) {
+        it.head = v / p.splits;
+        it.split = v % p.splits;
+        it.n_splits = min(p.splits, it.nt);
+        it.tile = rq.tile_begin + it.blk;
+        const int all = it.nt;
+        if (it.split < it.n_splits) {
+            it.t0 = all * it.split / it.n_splits;
+            it.nt = all * (it.split + 1) / it.n_splits - it.t0;
+        } else {
+            it.nt = 0;                           // no tile: every role passes over the item
         }
-    } else {                                     // blk: block of 128 entries of the evicted list
-        it.blk = u / p.n_kv_heads;
-        it.head = u % p.n_kv_heads;
-        it.nt = (rq.B + kTile - 1) / kTile;
-        it.kept_row0 = rq.kept_off + (long long)it.head * rq.B;
-        it.ev0 = rq.ev_off + (long long)it.head * rq.E;
     }
     return it;
 }
@@ -283,7 +255,7 @@ __device__ __forceinline__ int item_of_round(int round, int cta, int n_cta) {
 }
 
 template <int KIND, bool kSplits>
-__global__ void __launch_bounds__(threads_of(KIND), 1)
+__global__ void __launch_bounds__(kThreads, 1)
 tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
             const __grid_constant__ CUtensorMap map_x, const TileParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -321,7 +293,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     grid_dependency_wait();
     const Req* tbl = p.reqs;
     if (p.n_req <= kReqCache) {                  // the table is read once per item by every role
-        for (int i = threadIdx.x; i < p.n_req * (int)(sizeof(Req) / 4); i += threads_of(KIND))
+        for (int i = threadIdx.x; i < p.n_req * (int)(sizeof(Req) / 4); i += kThreads)
             reinterpret_cast<int*>(sh.reqs)[i] = reinterpret_cast<const int*>(p.reqs)[i];
         tbl = sh.reqs;
     }
@@ -350,16 +322,13 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 const Item it = decode_item<KIND, kSplits>(p, tbl, item);
                 if (kSplits && it.nt == 0) { --n; continue; }
                 const int ab = n % kABuf;
-                if (KIND != kMatch) {                    // the match's stationary tiles come from the gather warp
-                    if (!ptx::mbar_wait(ptx::smem_u32(&sh.a_empty[ab]), ((n / kABuf) & 1) ^ 1, abort_flag)) break;
-                    const uint32_t abar = ptx::smem_u32(&sh.a_full[ab]);
-                    ptx::mbar_arrive_expect_tx(abar, kTileBytes);
-                    const uint32_t adst = ptx::smem_u32(&sh.a[ab][0]);
-                    const int a_head = it.head;
-                    const int a_row = it.tok_begin + it.blk * kTile;
-                    ptx::tma_load_3d(adst, &map_a, 0, a_head, a_row, abar);
-                    ptx::tma_load_3d(adst + kHalfBytes, &map_a, 64, a_head, a_row, abar);
-                }
+                if (!ptx::mbar_wait(ptx::smem_u32(&sh.a_empty[ab]), ((n / kABuf) & 1) ^ 1, abort_flag)) break;
+                const uint32_t abar = ptx::smem_u32(&sh.a_full[ab]);
+                ptx::mbar_arrive_expect_tx(abar, kTileBytes);
+                const uint32_t adst = ptx::smem_u32(&sh.a[ab][0]);
+                const int a_row = it.tok_begin + it.blk * kTile;
+                ptx::tma_load_3d(adst, &map_a, 0, it.head, a_row, abar);
+                ptx::tma_load_3d(adst + kHalfBytes, &map_a, 64, it.head, a_row, abar);
                 for (int t = 0; t < it.nt; ++t, ++gb) {
                     const int s = gb % kStages;
                     if (!ptx::mbar_wait(ptx::smem_u32(&sh.b_empty[s]), ((gb / kStages) & 1) ^ 1, abort_flag)) {
@@ -374,16 +343,12 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         const int h = it.head / p.group;
                         ptx::tma_load_3d(bdst, &map_b, 0, h, row, bbar);
                         ptx::tma_load_3d(bdst + kHalfBytes, &map_b, 64, h, row, bbar);
-                    } else if (KIND == kSweep2) {
+                    } else {
                         const int row = it.tok_begin + (it.blk + (it.t0 + t) / p.group) * kTile;
                         const int h = it.head * p.group + (it.t0 + t) % p.group;
                         ptx::tma_load_3d(bdst, &map_b, 0, h, row, bbar);
                         ptx::tma_load_3d(bdst + kHalfBytes, &map_b, 64, h, row, bbar);
                         ptx::tma_load_3d(ptx::smem_u32(&sh.bx[s % Shared<KIND>::kXStages][0]), &map_x, 0, h, row, bbar);
-                    } else {
-                        const int row = (int)(it.kept_row0 + (long long)t * kTile);
-                        ptx::tma_load_2d(bdst, &map_b, 0, row, bbar);
-                        ptx::tma_load_2d(bdst + kHalfBytes, &map_b, 64, row, bbar);
                     }
                 }
             }
@@ -398,73 +363,9 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 for (uint32_t g = (gb > (uint32_t)kStages ? gb - kStages : 0); g < gb; ++g)
                     ptx::mbar_wait(ptx::smem_u32(&sh.b_full[g % kStages]), (g / kStages) & 1, &ignore,
                                    200000000ull);
-                if (KIND != kMatch)
-                    for (int m = (n > kABuf ? n - kABuf : 0); m < n; ++m)
-                        ptx::mbar_wait(ptx::smem_u32(&sh.a_full[m % kABuf]), (m / kABuf) & 1, &ignore, 200000000ull);
+                for (int m = (n > kABuf ? n - kABuf : 0); m < n; ++m)
+                    ptx::mbar_wait(ptx::smem_u32(&sh.a_full[m % kABuf]), (m / kABuf) & 1, &ignore, 200000000ull);
             }
-        }
-    } else if (KIND == kMatch && warp == kGatherWarp) {
-        // ------------------------------------------------------------ gather warp (match) ---
-        // Stationary tile of an item: rows e0 .. e0 + 127 of the head's evicted list, i.e. the key
-        // rows at positions evict_idx[e].  Lane l copies 16-byte chunk (l mod 16) of two rows per
-        // step (half a warp per 256-byte row), 64 steps per tile, into the layout a TMA box pair
-        // with the 128-byte swizzle would have produced: 64 features (128 bytes) per row and box,
-        // chunk c of row r at r * 128 + ((c xor (r mod 8)) * 16).  Rows past the end of the list are
-        // zero-filled.  The copies are waited for and published to the tensor core's proxy before
-        // the tile is announced, one item ahead of the MMAs.
-        const int l16 = lane & 15;
-        const int box = l16 >> 3, c8 = l16 & 7;
-        int n = 0;
-        for (int round = 0;; ++round, ++n) {
-            const int item = item_of_round(round, blockIdx.x, n_cta);
-            if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; --n; continue; }
-            const Item it = decode_item<KIND, kSplits>(p, tbl, item);
-            const int ab = n % kABuf;
-            int free_now = 1;                            // one lane waits, the warp follows its verdict
-            if (lane == 0)
-                free_now = ptx::mbar_wait(ptx::smem_u32(&sh.a_empty[ab]), ((n / kABuf) & 1) ^ 1, abort_flag) ? 1 : 0;
-            if (!__shfl_sync(0xffffffffu, free_now, 0)) break;
-            const uint32_t adst = ptx::smem_u32(&sh.a[ab][0]) + box * kHalfBytes;
-            const int* ev = p.evict_idx + it.ev0 + it.blk * kTile;
-            const int n_rows = min(kTile, it.E - it.blk * kTile);
-            const char* src0 = reinterpret_cast<const char*>(p.k_rows) +
-                               2 * ((long long)it.tok_begin * p.k_stride_tok + (long long)it.head * p.k_stride_head) + l16 * 16;
-            const auto copy_rows = [&](int st, int pos) {            // rows 2 st and 2 st + 1
-                const int r = 2 * st + (lane >> 4);
-                const char* src = src0 + 2 * (long long)pos * p.k_stride_tok;
-                const uint32_t dst = adst + r * 128 + ((c8 ^ (r & 7)) << 4);
-                const int nbytes = r < n_rows ? 16 : 0;
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(nbytes) : "memory");
-            };
-            const auto checked = [&](int pos) {
-                if (pos >= 0 && pos < it.L) return pos;
-                atomicExch(p.status, (int)LOOKM_ERR_DEVICE_BAD_INDEX);
-                return 0;
-            };
-            if (it.nt <= kBurstTiles) {
-                // all positions first, four per lane, so that all the copies go out together
-                int at[kTile / 32];
-#pragma unroll
-                for (int j = 0; j < kTile / 32; ++j) at[j] = j * 32 + lane < n_rows ? __ldg(ev + j * 32 + lane) : 0;
-#pragma unroll
-                for (int j = 0; j < kTile / 32; ++j) {
-                    const int mine = checked(at[j]);
-#pragma unroll
-                    for (int st = 16 * j; st < 16 * j + 16; ++st)
-                        copy_rows(st, __shfl_sync(0xffffffffu, mine, (2 * st + (lane >> 4)) & 31));
-                }
-            } else {
-#pragma unroll 8
-                for (int st = 0; st < kTile / 2; ++st) {
-                    const int r = 2 * st + (lane >> 4);
-                    copy_rows(st, checked(r < n_rows ? __ldg(ev + r) : 0));
-                }
-            }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-            ptx::fence_proxy_async_shared();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.a_full[ab]));
         }
     } else if (warp == 1 || warp == kEpiWarp0 + kGroups * 4) {
         // ------------------------------------------------------------ MMA issuers -----------
@@ -536,125 +437,40 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
         const float c2 = p.scale_log2;
         uint32_t gb = 0;
-        uint32_t lt = 0;                                     // tiles taken by this group
         int n = 0;
         for (int round = 0;; ++round, ++n) {
             const int item = item_of_round(round, blockIdx.x, n_cta);
             if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; --n; continue; }
             const Item it = decode_item<KIND, kSplits>(p, tbl, item);
             if (kSplits && it.nt == 0) { --n; continue; }
-            const int pos = it.blk * kTile + row;            // position of this thread's row (match: its
-                                                             // index in the evicted list)
+            const int pos = it.blk * kTile + row;            // position of this thread's row
             float m_run = -INFINITY, l_run = 0.f;            // sweep 1
             float acc[4] = {0.f, 0.f, 0.f, 0.f};             // sweep 2
-            float best = -INFINITY;                          // match
-            int best_slot = 0x7fffffff;
-            // match: 1 / |k| of this thread's evicted row takes two dependent loads (its position, then
-            // the norm).  They are requested here and after the group's first tile, not in the combine
-            // at the item's end, where the group that combines would sit out both round trips while
-            // its next accumulator stays full.
-            int row_at = 0;
-            float row_rnorm = 0.f;
-            bool rnorm_asked = false;
-            if (KIND == kMatch && pos < it.E) row_at = ptx::ld_nc_s32(p.evict_idx + it.ev0 + pos);
-            auto ask_rnorm = [&]() {
-                if (pos < it.E) {
-                    int at = row_at;
-                    if (at < 0 || at >= it.L) at = 0;       // reported by the gather warp
-                    row_rnorm = ptx::ld_nc_f32(p.rnorm_all + (long long)it.head * p.T + it.tok_begin + at);
-                }
-                rnorm_asked = true;
-            };
 
             for (int t = 0; t < it.nt; ++t, ++gb) {
                 if ((int)(gb % kGroups) != wg) continue;
                 const int buf = (int)(gb % kAccum);
-                float* side = sh.side[wg][lt & 1];
                 bool diag = false;                           // tile crosses the causal diagonal
-                int col_limit = kTile;                       // valid columns of the tile (match, sweep 2)
+                int col_limit = kTile;                       // sweep 2: valid columns of the tile
                 int diag_from = 0;                           // sweep 2: first column this row may use
                 if (KIND == kSweep1) {
                     diag = (it.t0 + t == it.blk);
-                } else if (KIND == kSweep2) {
+                } else {
                     const int ib = it.blk + (it.t0 + t) / p.group;
                     // columns to mask: below the diagonal in the item's first query block, and past
                     // the end of the request in its last one (rows of the next request or zeros)
                     col_limit = min(kTile, it.L - ib * kTile);
                     diag = (ib == it.blk) || (col_limit < kTile);
                     diag_from = (ib == it.blk) ? row : 0;
-                } else {
-                    const int slot = t * kTile + row;
-                    side[row] = (slot < it.B) ? p.rnorm_kept[it.kept_row0 + slot] : 0.f;
-                    col_limit = min(kTile, it.B - t * kTile);
-                    ptx::named_barrier_sync(1 + wg, 128);
                 }
-                ++lt;
                 ptx::mbar_wait(ptx::smem_u32(&sh.t_full[gb % kFullRing]), (gb / kFullRing) & 1, abort_flag);
                 ptx::tc_fence_after_sync();
-                if (KIND == kMatch) {
-                    // running arg-max of dot / |kept key| over kept slots, 16 columns at a time with
-                    // the next 16 already on their way from TMEM (a load takes about as long as
-                    // the work on 32 columns).  The maximum of the 16 is taken first; only when it
-                    // beats the running best is its first column looked up, so a strict comparison
-                    // in ascending slot order keeps the lowest slot.
-                    auto columns16 = [&](const uint32_t (&r)[16], int c0) {      // c0: column of the tile
-                        const float4* sd = reinterpret_cast<const float4*>(side + c0);
-                        float v[16];
-#pragma unroll
-                        for (int c4 = 0; c4 < 4; ++c4) {
-                            const float4 r4 = sd[c4];
-                            v[c4 * 4 + 0] = __uint_as_float(r[c4 * 4 + 0]) * r4.x;
-                            v[c4 * 4 + 1] = __uint_as_float(r[c4 * 4 + 1]) * r4.y;
-                            v[c4 * 4 + 2] = __uint_as_float(r[c4 * 4 + 2]) * r4.z;
-                            v[c4 * 4 + 3] = __uint_as_float(r[c4 * 4 + 3]) * r4.w;
-                        }
-                        if (col_limit < kTile) {           // last tile of the kept list only
-#pragma unroll
-                            for (int c = 0; c < 16; ++c)
-                                if (c0 + c >= col_limit) v[c] = -INFINITY;
-                        }
-                        const float m0 = ptx::fmax3(v[0], v[1], v[2]);
-                        const float m1 = ptx::fmax3(v[3], v[4], v[5]);
-                        const float m2 = ptx::fmax3(v[6], v[7], v[8]);
-                        const float m3 = ptx::fmax3(v[9], v[10], v[11]);
-                        const float m4 = ptx::fmax3(v[12], v[13], v[14]);
-                        const float mx = fmaxf(ptx::fmax3(m0, m1, m2), ptx::fmax3(m3, m4, v[15]));
-                        if (mx > best) {
-                            best = mx;
-                            int idx = 15;
-#pragma unroll
-                            for (int c = 14; c >= 0; --c) if (v[c] == mx) idx = c;
-                            best_slot = t * kTile + c0 + idx;
-                        }
-                    };
-                    uint32_t ra[16], rb[16];
-                    const uint32_t tbase = lane_addr + buf * kTile;
-                    ptx::tmem_ld_32x16(tbase, ra);
-#pragma unroll
-                    for (int k = 0; k < kTile / 32; ++k) {
-                        ptx::tmem_ld_wait16(ra);
-                        ptx::tmem_ld_32x16(tbase + (2 * k + 1) * 16, rb, ra);
-                        columns16(ra, 2 * k * 16);
-                        ptx::tmem_ld_wait16(rb);
-                        if (k < kTile / 32 - 1) {
-                            ptx::tmem_ld_32x16(tbase + (2 * k + 2) * 16, ra, rb);
-                        } else {
-                            // everything is in registers: hand the accumulator back
-                            ptx::tc_fence_before_sync();
-                            __syncwarp();
-                            if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.t_empty[buf]));
-                        }
-                        columns16(rb, (2 * k + 1) * 16);
-                    }
-                    if (!rnorm_asked) ask_rnorm();
-                    continue;
-                }
                 // work on 32 columns of the accumulator, c0 = first column of the chunk
                 auto process = [&](const uint32_t (&raw)[32], int c0) {
                     if (KIND == kSweep1) {
                         if (diag) sweep1_diagonal(raw, c0, row, c2, m_run, l_run);
                         else sweep1_columns(raw, c2, m_run, l_run);
-                    } else if (KIND == kSweep2) {
+                    } else {
                         if (diag) sweep2_diagonal(raw, c0, diag_from, col_limit, c2, acc);
                         else sweep2_columns(raw, c2, acc);
                     }
@@ -693,13 +509,12 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             ptx::mbar_wait(ptx::smem_u32(&sh.comb_free[cslot]), (cuse & 1u) ^ 1u, abort_flag);
             if (wg != combiner) {
                 if (KIND == kSweep1) { cb[wg][0][row] = m_run; cb[wg][kP1][row] = l_run; }
-                else if (KIND == kSweep2) { cb[wg][0][row] = (acc[0] + acc[1]) + (acc[2] + acc[3]); }
-                else { cb[wg][0][row] = best; cb[wg][kP1][row] = __int_as_float(best_slot); }
+                else { cb[wg][0][row] = (acc[0] + acc[1]) + (acc[2] + acc[3]); }
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.comb_full[cslot]));
             } else {
                 ptx::mbar_wait(ptx::smem_u32(&sh.comb_full[cslot]), cuse & 1u, abort_flag);
-                if (pos < (KIND == kMatch ? it.E : it.L) && !*abort_flag) {
+                if (pos < it.L && !*abort_flag) {
                     if (KIND == kSweep1) {
                         float mg[kGroups], lg[kGroups];
 #pragma unroll
@@ -717,7 +532,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                             __stcg(p.parts1 + ((long long)it.split * p.n_q_heads + it.head) * p.T + it.tok_begin + pos, make_float2(m, l));
                         else
                             store_lse(p, it.head, it.tok_begin + pos, m, l);
-                    } else if (KIND == kSweep2) {
+                    } else {
                         const float own = (acc[0] + acc[1]) + (acc[2] + acc[3]);
                         float a = (wg == 0) ? own : cb[0][0][row];
 #pragma unroll
@@ -726,21 +541,6 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                             __stcg(p.parts2 + ((long long)it.split * p.n_kv_heads + it.head) * p.T + it.tok_begin + pos, a);
                         else
                             p.scores[(long long)it.head * p.T + it.tok_begin + pos] = a;
-                    } else {
-                        if (!rnorm_asked) ask_rnorm();           // a group without a tile in this item
-                        const int e = pos;
-                        {
-                            float bb = (wg == 0) ? best : cb[0][0][row];
-                            int bs = (wg == 0) ? best_slot : __float_as_int(cb[0][kP1][row]);
-#pragma unroll
-                            for (int g = 1; g < kGroups; ++g) {
-                                const float b1 = (g == wg) ? best : cb[g][0][row];
-                                const int s1 = (g == wg) ? best_slot : __float_as_int(cb[g][kP1][row]);
-                                if (b1 > bb || (b1 == bb && s1 < bs)) { bb = b1; bs = s1; }
-                            }
-                            p.assign[it.ev0 + e] = bs;
-                            p.sim[it.ev0 + e] = bb * row_rnorm;
-                        }
                     }
                 }
                 __syncwarp();
@@ -914,7 +714,7 @@ __device__ __forceinline__ MultiItem decode_multi(const TileParams& p, const Req
 }
 
 template <int KIND, int kBlocks>
-__global__ void __launch_bounds__(threads_of(kSweep1), 1)
+__global__ void __launch_bounds__(kThreads, 1)
 multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
             const __grid_constant__ CUtensorMap map_x, const TileParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -957,7 +757,7 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
     grid_dependency_wait();
     const Req* tbl = p.reqs;
     if (p.n_req <= kReqCache) {
-        for (int i = threadIdx.x; i < p.n_req * (int)(sizeof(Req) / 4); i += threads_of(kSweep1))
+        for (int i = threadIdx.x; i < p.n_req * (int)(sizeof(Req) / 4); i += kThreads)
             reinterpret_cast<int*>(sh.reqs)[i] = reinterpret_cast<const int*>(p.reqs)[i];
         tbl = sh.reqs;
     }
@@ -1232,10 +1032,9 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
                                cudaStream_t stream) {
     if (p.n_items <= 0) return cudaSuccess;
     typedef void (*Kernel)(CUtensorMap, CUtensorMap, CUtensorMap, TileParams);
-    static const Kernel kernels[3][2] = {{tile_kernel<kSweep1, false>, tile_kernel<kSweep1, true>},
-                                         {tile_kernel<kSweep2, false>, tile_kernel<kSweep2, true>},
-                                         {tile_kernel<kMatch, false>, tile_kernel<kMatch, false>}};
-    const size_t smem_of[3] = {sizeof(Shared<kSweep1>) + 1024, sizeof(Shared<kSweep2>) + 1024, sizeof(Shared<kMatch>) + 1024};
+    static const Kernel kernels[2][2] = {{tile_kernel<kSweep1, false>, tile_kernel<kSweep1, true>},
+                                         {tile_kernel<kSweep2, false>, tile_kernel<kSweep2, true>}};
+    const size_t smem_of[2] = {sizeof(Shared<kSweep1>) + 1024, sizeof(Shared<kSweep2>) + 1024};
     const int grid = p.n_items < num_sms ? p.n_items : num_sms;
     const CUtensorMap& mx = map_x ? *map_x : map_b;      // only sweep 2 uses it
     static const Kernel multi[2][2] = {{multi_kernel<kSweep1, 2>, multi_kernel<kSweep1, 4>},
@@ -1249,17 +1048,17 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
             for (int j = 0; j < 2; ++j)
                 if (e == cudaSuccess)
                     e = cudaFuncSetAttribute(multi[i][j], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)multi_smem[i][j]);
-        for (int i = 0; i < 3; ++i)
+        for (int i = 0; i < 2; ++i)
             for (int j = 0; j < 2; ++j)
                 if (e == cudaSuccess)
                     e = cudaFuncSetAttribute(kernels[i][j], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of[i]);
         return e;
     });
     if (err != cudaSuccess) return err;
-    if (p.blocks > 1 && kind != kMatch)
-        return launch_chained(multi[kind][p.blocks == 4], dim3(grid), dim3(threads_of(kSweep1)), multi_smem[kind][p.blocks == 4],
+    if (p.blocks > 1)
+        return launch_chained(multi[kind][p.blocks == 4], dim3(grid), dim3(kThreads), multi_smem[kind][p.blocks == 4],
                               stream, map_a, map_b, mx, p);
-    return launch_chained(kernels[kind][p.splits > 1], dim3(grid), dim3(threads_of(kind)), smem_of[kind], stream, map_a, map_b, mx, p);
+    return launch_chained(kernels[kind][p.splits > 1], dim3(grid), dim3(kThreads), smem_of[kind], stream, map_a, map_b, mx, p);
 }
 
 cudaError_t launch_lse_split(const float* lse, int n_q_heads, long long T, float scale_log2,

@@ -442,6 +442,36 @@ def test_match_whole_blocks_single_rows_and_strided_keys(B, L, budget):
             assert S[e, a_ref[e]] - S[e, a_got[h, e]] <= 1e-4
 
 
+@pytest.mark.parametrize("budget", [512, 513, 640, 1100])
+def test_match_starts_in_the_middle_and_the_lower_slot_wins(B, budget):
+    """Items of more than four tiles start with the tile around their own positions: of identical kept keys
+    the one in the lower slot wins although its tile comes later (or in another group)."""
+    import torch
+    L, Hkv = 1500, 2
+    kb = synth.f32_to_bf16_bits(synth.normal(synth.stream_key(98), L * Hkv * 128).reshape(L, Hkv, 128).astype(np.float32))
+    kept_np = np.sort((np.arange(budget) * L) // budget).astype(np.int32)
+    ev_np = np.setdiff1d(np.arange(L, dtype=np.int32), kept_np)
+    pairs = [(s, budget - 1 - s) for s in range(3, 60)]               # kept slots with equal keys, far apart ...
+    for i, (lo, hi) in enumerate(pairs):
+        kb[kept_np[hi]] = kb[kept_np[lo]]
+        kb[ev_np[len(ev_np) - 2 - 6 * i]] = kb[kept_np[lo]]           # ... and evicted rows equal to both
+    k, kf = to_dev(kb), synth.bf16_to_f32(kb)
+    kept, ev = (torch.from_numpy(np.tile(x, Hkv)).cuda() for x in (kept_np, ev_np))
+    assign, sim = torch.full_like(ev, -7), torch.full((ev.numel(),), -7.0, device="cuda")
+    lay = B.make_layout(None, k)
+    ws = B.alloc_workspace(lay, [L])
+    B.check(B.lookm_match(k, kept, ev, [0, L], [budget], lay, assign, sim, ws))
+    assert B.lookm_device_status(ws) == B.OK
+    a_got, s_got = assign.cpu().numpy().reshape(Hkv, -1), sim.cpu().numpy().reshape(Hkv, -1).astype(np.float64)
+    for h in range(Hkv):
+        a_ref, s_ref, S = orc.match(kf, h, kept_np, ev_np, want_matrix=True)
+        assert np.allclose(s_got[h], s_ref, atol=2e-6, rtol=0)
+        for e in np.where(a_got[h] != a_ref)[0]:
+            assert S[e, a_ref[e]] - S[e, a_got[h, e]] <= 1e-4
+        for i, (lo, _) in enumerate(pairs):
+            assert a_got[h, len(ev_np) - 2 - 6 * i] == lo
+
+
 def test_match_of_many_short_prompts_one_kept_tile_each(B):
     """Items of a single tile: three of the four epilogue groups have no tile in an item and may run ahead
     of the one that has; every repetition must give the same bits, and no wait may run out."""
