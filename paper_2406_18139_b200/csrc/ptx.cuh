@@ -224,6 +224,55 @@ __device__ __forceinline__ float ex2_fma(float x) {
     p = fmaf(p, f, 1.000000119e+00f);
     return __int_as_float(__float_as_int(p) + (__float_as_int(r) << 23));
 }
+// ---- two fp32 numbers at a time (the even-numbered register of a pair is .x) ----------------------
+typedef uint64_t f32x2;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+    f32x2 v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(__float_as_uint(x)), "r"(__float_as_uint(y)));
+    return v;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    uint32_t x, y;
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(x), "=r"(y) : "l"(v));
+    return make_float2(__uint_as_float(x), __uint_as_float(y));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// ex2_fma of both numbers, without its upper limit: arguments must not exceed 127.
+__device__ __forceinline__ f32x2 ex2_fma2(f32x2 x) {
+    const float2 v = unpack2(x);
+    x = pack2(fmaxf(v.x, -125.f), fmaxf(v.y, -125.f));
+    const f32x2 magic = pack2(12582912.f, 12582912.f);
+    const f32x2 r = add2(x, magic);
+    const f32x2 f = sub2(x, sub2(r, magic));
+    f32x2 p = pack2(1.327647245e-03f, 1.327647245e-03f);
+    p = fma2(p, f, pack2(9.675540961e-03f, 9.675540961e-03f));
+    p = fma2(p, f, pack2(5.550713092e-02f, 5.550713092e-02f));
+    p = fma2(p, f, pack2(2.402212024e-01f, 2.402212024e-01f));
+    p = fma2(p, f, pack2(6.931469440e-01f, 6.931469440e-01f));
+    p = fma2(p, f, pack2(1.000000119e+00f, 1.000000119e+00f));
+    const float2 n = unpack2(r), q = unpack2(p);
+    return pack2(__int_as_float(__float_as_int(q.x) + (__float_as_int(n.x) << 23)),
+                 __int_as_float(__float_as_int(q.y) + (__float_as_int(n.y) << 23)));
+}
 __device__ __forceinline__ float lg2(float x) {
     float y;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

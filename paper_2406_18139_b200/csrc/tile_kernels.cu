@@ -67,6 +67,7 @@ constexpr int kItemRing = 4;                     // items announced to the roles
 constexpr int kReqCache = 16;                    // request-table entries cached in shared memory
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kReferenceSlack = 1.152921504606847e18f;   // 2^60: largest chunk sum kept against a stale reference
+constexpr float kReferenceSlackLog2 = 60.f;
 constexpr float kLn2 = 0.6931471805599453f;
 
 template <int KIND>
@@ -90,8 +91,21 @@ struct __align__(1024) Shared {
 static_assert(sizeof(Shared<kSweep1>) + 1024 <= 232448 && sizeof(Shared<kSweep2>) + 1024 <= 232448,
               "shared memory of the tile kernels exceeds 227 KB");
 
-// The softmax epilogues are bound by the special-function unit (16 ex2 per clock and SM), so one
-// column in kPolyEvery is exponentiated on the FMA pipe instead.
+// The softmax epilogues are bound by the special-function unit (16 ex2 per clock and SM) and by issue
+// slots, so some columns are exponentiated on the FMA pipe instead: on full tiles kPolyPairs of the sixteen pairs
+// of a chunk, two numbers per instruction, with one test of the chunk's largest logit in place of an upper limit on
+// every argument (which took two instructions a pair more).  A two-wide multiply-add takes two issue
+// slots, so it is the limit's instructions that are saved.  Scores in us, one column in six one by one | 2, 3, 5, 6 and 7
+// pairs: 8192 tokens x 32 heads 678 | 676, 669, 684, 700, 726; 4096 x 32 191.3 | 189.4, 190.4, 195.9, 202.8, 210.5; three
+// prompts of 1800 to 5000 x 32 on 8 552 | 549, 548, 567, 583, 605.
+constexpr int kPolyPairs = 3;
+__host__ __device__ constexpr bool poly_pair(int i) { return ((i + 1) * kPolyPairs) / 16 != (i * kPolyPairs) / 16; }
+__device__ __forceinline__ ptx::f32x2 exp2_pair(int i, ptx::f32x2 x) {
+    if (poly_pair(i)) return ptx::ex2_fma2(x);
+    const float2 v = ptx::unpack2(x);
+    return ptx::pack2(ptx::ex2(v.x), ptx::ex2(v.y));
+}
+// Diagonal tiles: one column in kPolyEvery.
 constexpr int kPolyEvery = 6;
 __device__ __forceinline__ float exp2_mixed(int column, float x) {
     return (column % kPolyEvery == kPolyEvery - 1) ? ptx::ex2_fma(x) : ptx::ex2(x);
@@ -130,14 +144,18 @@ __device__ __forceinline__ void sweep1_columns(const uint32_t (&raw)[32], float 
 #pragma unroll 1
     for (int round2 = 0;; ++round2) {
         const float mc = ref * c2;
-        float s0 = 0.f, s1 = 0.f;
+        const ptx::f32x2 scale = ptx::pack2(c2, c2), shift = ptx::pack2(-mc, -mc);
+        ptx::f32x2 s[2] = {0ull, 0ull};
+        float high = -INFINITY;                          // largest logit that the polynomial met
 #pragma unroll
-        for (int c = 0; c < 32; c += 2) {
-            s0 += exp2_mixed(c, fmaf(__uint_as_float(raw[c]), c2, -mc));
-            s1 += exp2_mixed(c + 1, fmaf(__uint_as_float(raw[c + 1]), c2, -mc));
+        for (int i = 0; i < 16; ++i) {
+            const float a = __uint_as_float(raw[2 * i]), b = __uint_as_float(raw[2 * i + 1]);
+            if (poly_pair(i)) high = ptx::fmax3(high, a, b);
+            s[i & 1] = ptx::add2(s[i & 1], exp2_pair(i, ptx::fma2(ptx::pack2(a, b), scale, shift)));
         }
-        sum = s0 + s1;
-        if (sum < kReferenceSlack || round2) break;
+        const float2 t = ptx::unpack2(ptx::add2(s[0], s[1]));
+        sum = t.x + t.y;
+        if ((sum < kReferenceSlack && fmaf(high, c2, -mc) < kReferenceSlackLog2) || round2) break;
         float mx = ref;
 #pragma unroll
         for (int c = 0; c < 32; c += 2) mx = ptx::fmax3(mx, __uint_as_float(raw[c]), __uint_as_float(raw[c + 1]));
@@ -157,8 +175,20 @@ __device__ __forceinline__ void sweep2_diagonal(const uint32_t (&raw)[32], int c
     }
 }
 __device__ __forceinline__ void sweep2_columns(const uint32_t (&raw)[32], float c2, float (&acc)[4]) {
+    const ptx::f32x2 scale = ptx::pack2(c2, c2);
+    ptx::f32x2 s[2] = {ptx::pack2(acc[0], acc[1]), ptx::pack2(acc[2], acc[3])};
+    float high = -INFINITY;
 #pragma unroll
-    for (int c = 0; c < 32; ++c) acc[c & 3] += exp2_mixed(c, __uint_as_float(raw[c]) * c2);
+    for (int i = 0; i < 16; ++i) {
+        const float a = __uint_as_float(raw[2 * i]), b = __uint_as_float(raw[2 * i + 1]);
+        if (poly_pair(i)) high = ptx::fmax3(high, a, b);
+        s[i & 1] = ptx::add2(s[i & 1], exp2_pair(i, ptx::mul2(ptx::pack2(a, b), scale)));
+    }
+    const float2 u = ptx::unpack2(s[0]), v = ptx::unpack2(s[1]);
+    acc[0] = high * c2 > 127.f ? INFINITY : u.x;         // (probabilities beyond 2^127: a caller's log-sum-exp is not one)
+    acc[1] = u.y;
+    acc[2] = v.x;
+    acc[3] = v.y;
 }
 
 // -lse / scale of one query row as three bf16 terms (their sum carries 24 bits) and 13 zeros:

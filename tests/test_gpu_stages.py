@@ -101,6 +101,37 @@ def test_scores_logits_that_grow_along_the_prompt(B):
     assert np.allclose(got.sum(axis=1), L, rtol=1e-5)
 
 
+@pytest.mark.parametrize("rise", [50.0, 62.0, 126.0, 130.0, 400.0])
+@pytest.mark.parametrize("cols", [(11,), (12,), (20, 30)])
+def test_scores_one_logit_far_above_the_reference(B, cols, rise):
+    """A single column of a chunk leaves the row's reference by 2^rise, be it one that the special-function unit
+    exponentiates (12) or one that the polynomial does (10, 11, 20, 21, 30, 31), whose sum alone would not
+    show it: the row's log-sum-exp is right either way."""
+    import torch
+    L, scale = 600, 0.125
+    qn = np.zeros((L, 1, 128), dtype=np.float32)
+    kn = synth.normal(synth.stream_key(143), L * 128).reshape(L, 1, 128).astype(np.float32) * 0.25
+    qn[:, 0, 0] = 16.0
+    qn[:, 0, 1] = 0.5
+    kn[:, 0, 0] = 0.0
+    for c in cols:
+        kn[256 + c, 0, 0] = rise / np.log2(np.e) / (16.0 * scale)     # logit of `rise` in base 2
+    qb, kb = synth.f32_to_bf16_bits(qn), synth.f32_to_bf16_bits(kn)
+    qf, kf = synth.bf16_to_f32(qb), synth.bf16_to_f32(kb)
+    q, k = to_dev(qb), to_dev(kb)
+    lay = B.make_layout(q, k, softmax_scale=scale)
+    ws = B.alloc_workspace(lay, [L])
+    scores = torch.zeros(1, L, dtype=torch.float32, device="cuda")
+    lse = torch.zeros(1, L, dtype=torch.float32, device="cuda")
+    B.check(B.lookm_score(q, k, [0, L], lay, scores, lse, False, ws))
+    assert B.lookm_device_status(ws) == B.OK
+    A, lse_o = orc.scores(qf, kf, scale=scale, want_lse=True)
+    # one fp32 rounding of arguments up to 400 / 1.44 on top of the sums
+    assert np.allclose(lse.cpu().numpy().reshape(1, 1, L), lse_o, rtol=1e-6, atol=2e-5)
+    got = scores.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(got - A) <= 1e-4 * A + 1e-30)
+
+
 @pytest.mark.parametrize("lens,Hq,Hkv", [([1900, 1, 130, 640], 4, 1), ([1409], 1, 1), ([2100, 2100], 2, 2)])
 def test_scores_of_items_cut_into_ranges(B, lens, Hq, Hkv):
     """Few heads: both sweeps cut their items into up to four ranges (fewer where an item has fewer
