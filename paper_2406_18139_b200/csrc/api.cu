@@ -4,7 +4,9 @@
 #include <cmath>
 #include <cstring>
 #include <initializer_list>
+#include <functional>
 #include <mutex>
+#include <queue>
 #include <vector>
 
 #include <cudaTypedefs.h>
@@ -944,6 +946,7 @@ struct DecodeWay {
     bool mma = false;
     long long rows_per_split = 64;
     int cluster = 1;                        // > 1: so many splits everywhere, added up inside the launch
+    bool shares = false;                    // the CTAs take equal shares of all rows (one query head at a time)
     double us = 0.;                         // estimated time
 };
 struct DecodePlan {
@@ -966,6 +969,31 @@ struct DecodeCost { double launch, step, wave, combine, splits16; };
 constexpr DecodeCost kCostOneHead = {0.9, 0.59, 1.0, 2.4, 0.7}, kCostTwoHeads = {1.25, 0.78, 1.4, 2.6, 0.7},
                      kCostMma = {1.9, 1.33, 1.35, 2.7, 0.85};
 constexpr double kMmaStepAlone = 1.9;       // of a CTA that has its SM to itself and waits for each of its steps
+
+// Most rows that an SM gets when whole splits (of s rows at most) go in order to whichever of `wave` SMs is free
+// first: SMs with the same load, as (load, how many), move on together.
+long long most_rows(const int* lens, int n_req, long long units, long long s, long long wave) {
+    typedef std::pair<long long, long long> Load;
+    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> free;
+    free.push({0, wave});
+    long long most = 0;
+    const auto give = [&](long long rows, long long pieces) {
+        while (pieces > 0) {
+            Load l = free.top();
+            free.pop();
+            const long long n = std::min(pieces, l.second);
+            if (l.second > n) free.push({l.first, l.second - n});
+            free.push({l.first + rows, n});
+            most = std::max(most, l.first + rows);
+            pieces -= n;
+        }
+    };
+    for (int r = 0; r < n_req; ++r) {
+        const long long rows = (long long)lens[r] + 1;
+        give(std::min(s, rows), units * ((rows + s - 1) / s));
+    }
+    return most;
+}
 
 DecodeWay decode_way(const lookm_cache_layout* lay, int n_req, const int* lens, int gt, bool mma, int sms) {
     DecodeWay w;
@@ -1024,6 +1052,33 @@ DecodeWay decode_way(const lookm_cache_layout* lay, int n_req, const int* lens, 
     const DecodeCost& cost = mma ? kCostMma : gt == 2 ? kCostTwoHeads : kCostOneHead;
     w.us = cost.launch + waves * steps * (mma && ctas <= sms ? kMmaStepAlone : cost.step) + (waves - 1.) * cost.wave;
     if (w.cluster == 1 && splits > 1) w.us += cost.combine + cost.splits16 * std::max<long long>(0, splits - 16) / 16.;
+    if (gt == 1 && !mma) {
+        // Equal shares?  Whole splits take as long as memory needs for all rows, or as long as an SM needs for the
+        // most rows that it gets, with a start per further wave.  Shares cost a little per unit in one and nearly
+        // always the second launch.  (The constants fit 32 steps of 1 to 64 requests, 41 to 32768 rows and 8 to 40 heads;
+        // of these the slower way is picked by 3 % at most.)  us, whole | shares: 4 requests of 1000 to 8000 rows x 32
+        // heads 78 | 63.7, 16 of 4000 to 8000 x 32 293 | 266, 64 of 40 x 32 37 | 17, one of 32768 x 40 115 | 107; one of 8192 x 32
+        // 22.6 | 25.2, of 20000 x 8 16.7 | 19.1, 8 of 300 to 2000 x 40 33 | 35.2, 7 of 100 to 8000 x 32 80 | 86.8.
+        constexpr double kRowUs = 7.8e-5, kSmRowUs = 1e-2, kStartUs = 2., kWaveUs = 1.5, kCombineUs = 1.5, kShareUs = 4.5, kUnitUs = 1.3;
+        const double share_ctas = (double)std::min<long long>((long long)sms * kDecodeShareCtasPerSm, total_rows / kDecodeShareRows + 1);
+        const double shares = std::max((double)total_rows * kRowUs, (double)total_rows / share_ctas * kDecodeShareCtasPerSm * kSmRowUs) +
+                              (double)(n_req * units) / share_ctas * kUnitUs + kShareUs;
+        const double later_waves = std::max(0., (double)ctas / (double)wave - 1.);
+        const auto whole_with = [&](double most) {
+            return std::max(most * kSmRowUs + later_waves * kWaveUs, (double)total_rows * kRowUs) + kStartUs +
+                   (w.cluster == 1 && splits > 1 ? kCombineUs : 0.);
+        };
+        // (most rows of an SM: between the mean and that plus a split; the order in which SMs come free only counts in between)
+        const double mean = (double)total_rows / (double)wave, piece = (double)std::min<long long>(s, longest);
+        double whole = whole_with(ctas <= wave ? piece : mean);
+        if (ctas > wave && shares >= 0.95 * whole && shares < 0.95 * whole_with(mean + piece))
+            whole = whole_with((double)most_rows(lens, n_req, units, s, wave));
+        w.shares = shares < 0.95 * whole;
+        if (w.shares) {
+            w.cluster = 1;
+            w.us += shares - whole;
+        }
+    }
     return w;
 }
 
@@ -1077,8 +1132,7 @@ int build_decode_plan(DecodePlan& dp, const lookm_cache_layout* lay, int n_req, 
             q.index = r;
             q.n_splits = dp.way.cluster > 1 ? dp.way.cluster : (int)(((long long)lens[r] + 1 + s - 1) / s);
             q.cta_begin = 0;
-            q.part_begin = (int)parts;
-            q.pad = 0;
+            q.part_begin = parts;
             parts += (long long)q.n_splits * lay->n_kv_heads * dp.way.n_pass * dp.way.gt;
         }
     }
@@ -1110,13 +1164,25 @@ int decode_common(const void* q, const void* k_new, const void* v_new, void* cac
         DecodeBatch batch;
         std::memset(&batch, 0, sizeof(batch));
         batch.n_req = std::min(kDecodeChunk, n_req - base);
-        long long ctas = 0;
+        long long ctas = 0, steps = 0;
         bool split = false;
         for (int i = 0; i < batch.n_req; ++i) {
             batch.r[i] = dp.reqs[base + i];
             batch.r[i].cta_begin = (int)ctas;
             ctas += (long long)batch.r[i].n_splits * units;
             split = split || (batch.r[i].n_splits > 1 && dp.way.cluster == 1);
+            if (dp.way.shares) {
+                const int unit = batch.r[i].len / kDecodeShareRows + 1;
+                batch.r[i].step_begin = steps;
+                steps += unit * units;
+                split = split || unit > 1;
+            }
+        }
+        if (dp.way.shares) {
+            ctas = std::min<long long>((long long)di.sms * kDecodeShareCtasPerSm, steps);
+            if (steps / ctas >= (1ll << 30)) return LOOKM_ERR_UNSUPPORTED;
+            batch.share = (int)(steps / ctas);
+            batch.longer = (int)(steps % ctas);
         }
         if (ctas >= (1ll << 31)) return LOOKM_ERR_UNSUPPORTED;
         LOOKM_CUDA(launch_decode(batch, (int)ctas, dp.way.gt, dp.way.mma, dp.way.cluster, q, k_new, v_new, cache_k, cache_v,

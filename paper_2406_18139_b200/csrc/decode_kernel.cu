@@ -17,11 +17,15 @@
 // behind the first, adds the splits in split order.  No CTA waits for another and the order of
 // additions never depends on timing, so results are reproducible bit for bit.
 //
+// Batches whose caches differ much in length, or have few rows, and head counts that leave SMs without a split
+// go to decode_shared_kernel below, whose CTAs take equal shares of the rows of all units.
+//
 // Several query heads that share a KV head can go to decode_mma_kernel below, which has the same structure;
 // the planner compares (decode_way in api.cu).
 #include <cuda_bf16.h>
 #include <float.h>
 #include <math.h>
+#include <type_traits>
 
 #include "internal.h"
 #include "ptx.cuh"
@@ -110,104 +114,43 @@ struct DecShared {
     float o[kDecWarps][GT][kHeadDim];
 };
 
-// GT = 1 or 2 query heads of the group are handled per pass over the rows.
-template <int GT, bool kClustered>
-__global__ void __launch_bounds__(kDecThreads)
-decode_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __restrict__ q,
-              const __nv_bfloat16* __restrict__ k_new, const __nv_bfloat16* __restrict__ v_new,
-              __nv_bfloat16* __restrict__ cache_k, __nv_bfloat16* __restrict__ cache_v,
-              long long stride_row, long long stride_head, int n_q_heads, int n_kv_heads, int group,
-              int rows_per_split, float scale_log2, float* __restrict__ parts, float* __restrict__ out) {
-    __shared__ DecShared<GT> sh;
-    __shared__ ClusterShared<GT> cs;
-    extern __shared__ __align__(128) uint8_t dec_ring[];         // [warp][ring step][half][row][K|V][256 B]
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int hw = threadIdx.x >> 4, l16 = lane & 15;
+// Asks for the first rows of a CTA's split while the kernel before this one drains: rows already in the cache
+// may not be read before that kernel is over, but they may be brought into L2.  Long splits only (us per step):
+// 32768 rows with 32 heads on 8 28.4 -> 27.1, 8192 x 32 23.8 -> 23.3, 20000 x 8 18.4 -> 17.6; with 256 rows nothing is
+// left of it, with 512 it costs 1 us.
+constexpr int kPrefetchRows = 96, kPrefetchFrom = 384;
+__device__ __forceinline__ void prefetch_rows(const __nv_bfloat16* cache_k, const __nv_bfloat16* cache_v, long long first,
+                                              long long stride_row, int rows) {
+    if (rows < kPrefetchFrom) return;
+    for (int i = threadIdx.x; i < kPrefetchRows * 2; i += blockDim.x) {
+        const long long at = first + (long long)(i >> 1) * stride_row + (i & 1) * 64;
+        ptx::prefetch_l2(cache_k + at);
+        ptx::prefetch_l2(cache_v + at);
+    }
+}
 
-    // which (request, KV head, pass, split) this CTA owns: requests are found by their first CTA
-    int r = 0;
-    {
-        int lo = 0, hi = batch.n_req - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (batch.r[mid].cta_begin <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
+// A half-warp's query features and running softmax statistics (reference, sum, weighted V sum); a lane has 8
+// features.
+template <int GT>
+struct DecState {
+    float qv[GT][8], m[GT], l[GT], o[GT][8];
+    __device__ __forceinline__ void reset() {
+#pragma unroll
+        for (int g = 0; g < GT; ++g) {
+            m[g] = -INFINITY;
+            l[g] = 0.f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) o[g][i] = 0.f;
         }
-        r = lo;
     }
-    const DecodeReq rq = batch.r[r];
-    const int n_pass = group / GT;
-    const int local = (int)blockIdx.x - rq.cta_begin;            // [head][pass][split]
-    const int split = local % rq.n_splits;
-    const int pass = (local / rq.n_splits) % n_pass;
-    const int h = local / (rq.n_splits * n_pass);
-    const int n_rows = rq.len + 1;                               // cached rows + the new one
-    const int row0 = split * rows_per_split, row1 = min(n_rows, row0 + rows_per_split);
-    const int qh0 = h * group + pass * GT;                       // first query head of this pass
-
-    grid_dependency_wait();
-
-    // this lane's 8 features of the GT query rows
-    float qv[GT][8];
+    // q: this lane's features of the pass's first head
+    __device__ __forceinline__ void load_query(const __nv_bfloat16* q) {
 #pragma unroll
-    for (int g = 0; g < GT; ++g) {
-        const uint4 u = *reinterpret_cast<const uint4*>(q + ((long long)rq.index * n_q_heads + qh0 + g) * kHeadDim + l16 * 8);
-        unpack_bf16x8(u, qv[g]);
+        for (int g = 0; g < GT; ++g) unpack_bf16x8(*reinterpret_cast<const uint4*>(q + g * kHeadDim), qv[g]);
     }
-    const long long head_off = (long long)h * stride_head + l16 * 8;
-    const __nv_bfloat16* ck = cache_k + rq.begin * stride_row + head_off;
-    const __nv_bfloat16* cv = cache_v + rq.begin * stride_row + head_off;
-    const __nv_bfloat16* nk = k_new + ((long long)rq.index * n_kv_heads + h) * kHeadDim + l16 * 8;
-    const __nv_bfloat16* nv = v_new + ((long long)rq.index * n_kv_heads + h) * kHeadDim + l16 * 8;
-
-    float m[GT], l[GT], o[GT][8];
-#pragma unroll
-    for (int g = 0; g < GT; ++g) {
-        m[g] = -INFINITY;
-        l[g] = 0.f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) o[g][i] = 0.f;
-    }
-
-    // The appended row (Eq. 2) is read from k_new / v_new by whoever owns it; the CTA that owns it
-    // on the group's first pass also writes it into the cache (nobody reads cache row `len` in this
-    // step, so the write races with nothing).
-    if (pass == 0 && rq.len >= row0 && rq.len < row1 && warp == 0) {
-        const __nv_bfloat16* src = lane < 16 ? nk : nv;
-        __nv_bfloat16* dst = (lane < 16 ? cache_k : cache_v) + rq.begin * stride_row + head_off +
-                             (long long)rq.len * stride_row;
-        *reinterpret_cast<uint4*>(dst) = __ldg(reinterpret_cast<const uint4*>(src));
-    }
-
-    // Copies of one step: K and V of kDecFlight rows per half-warp, 16 bytes per lane and row,
-    // straight into this warp's ring.  Rows past the split are zero-filled (a copy of 0 source
-    // bytes), so that they contribute exact zeros.  One commit group per step, also past the end.
-    const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(dec_ring) + warp * (kDecRing * kDecStepBytes) +
-                           ((lane >> 4) * kDecFlight * 2) * kDecRowBytes + l16 * 16;
-    auto issue = [&](int step) {
-        const int base = row0 + step * (kDecHalfWarps * kDecFlight);
-        const uint32_t dst = ring0 + (uint32_t)(step % kDecRing) * kDecStepBytes;
-        if (base < row1) {
-#pragma unroll
-            for (int f = 0; f < kDecFlight; ++f) {
-                const int row = base + f * kDecHalfWarps + hw;
-                const bool is_new = (row == rq.len);
-                const bool valid = row < row1;
-                const __nv_bfloat16* kp = (is_new || !valid) ? nk : ck + (long long)row * stride_row;
-                const __nv_bfloat16* vp = (is_new || !valid) ? nv : cv + (long long)row * stride_row;
-                const int nbytes = valid ? 16 : 0;
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
-                             ::"r"(dst + (2 * f) * kDecRowBytes), "l"(kp), "r"(nbytes) : "memory");
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
-                             ::"r"(dst + (2 * f + 1) * kDecRowBytes), "l"(vp), "r"(nbytes) : "memory");
-            }
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    // Softmax statistics and weighted V sums of one step's rows (online softmax against the running
-    // maximum of this half-warp).
-    auto consume = [&](int step) {
-        const int base = row0 + step * (kDecHalfWarps * kDecFlight);
-        const uint32_t src = ring0 + (uint32_t)(step % kDecRing) * kDecStepBytes;
+    // One step's rows, K and V alternating from shared address src on, the f-th of them at position row + f *
+    // kDecHalfWarps: online softmax against the running maximum of this half-warp.  Rows from row1 on don't count.
+    __device__ __forceinline__ void take(uint32_t src, int row, int row1, float scale_log2) {
         uint4 ku[kDecFlight], vu[kDecFlight];
 #pragma unroll
         for (int f = 0; f < kDecFlight; ++f) {
@@ -221,7 +164,7 @@ decode_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __
         float s[kDecFlight][GT];
 #pragma unroll
         for (int f = 0; f < kDecFlight; ++f) {
-            const bool valid = base + f * kDecHalfWarps + hw < row1;
+            const bool valid = row + f * kDecHalfWarps < row1;
             float kx[8];
             unpack_bf16x8(ku[f], kx);
 #pragma unroll
@@ -259,8 +202,131 @@ decode_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __
                 for (int i = 0; i < 8; ++i) o[g][i] = fmaf(p[f], vx[i], o[g][i]);
             }
         }
-    };
+    }
+    // Combines the two half-warps of a warp and leaves the result for the CTA.
+    __device__ __forceinline__ void leave(DecShared<GT>& sh, int warp, int lane, float scale_log2) {
+#pragma unroll
+        for (int g = 0; g < GT; ++g) {
+            const float m_o = __shfl_xor_sync(0xffffffffu, m[g], 16);
+            const float l_o = __shfl_xor_sync(0xffffffffu, l[g], 16);
+            const float mx = fmaxf(m[g], m_o);
+            // lower half-warp first, whichever half this lane is in
+            const bool low = lane < 16;
+            const float a_me = (mx == -INFINITY) ? 0.f : dec_ex2((m[g] - mx) * scale_log2);
+            const float a_ot = (mx == -INFINITY) ? 0.f : dec_ex2((m_o - mx) * scale_log2);
+            const float l_lo = low ? l[g] * a_me : l_o * a_ot, l_hi = low ? l_o * a_ot : l[g] * a_me;
+            l[g] = l_lo + l_hi;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float o_o = __shfl_xor_sync(0xffffffffu, o[g][i], 16);
+                const float o_lo = low ? o[g][i] * a_me : o_o * a_ot, o_hi = low ? o_o * a_ot : o[g][i] * a_me;
+                o[g][i] = o_lo + o_hi;
+            }
+            m[g] = mx;
+            if (lane == 0) { sh.m[warp][g] = m[g]; sh.l[warp][g] = l[g]; }
+            if (low) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) sh.o[warp][g][(lane & 15) * 8 + i] = o[g][i];
+            }
+        }
+    }
+};
+// The warps' results of query head g in warp order: reference, sum and weighted V sum of feature t.
+template <int GT>
+__device__ __forceinline__ void add_warps(const DecShared<GT>& sh, int g, int t, float scale_log2, float& mx, float& lsum, float& osum) {
+    mx = -INFINITY;
+#pragma unroll
+    for (int w = 0; w < kDecWarps; ++w) mx = fmaxf(mx, sh.m[w][g]);
+    lsum = osum = 0.f;
+#pragma unroll
+    for (int w = 0; w < kDecWarps; ++w) {
+        const float a = mx == -INFINITY ? 0.f : dec_ex2((sh.m[w][g] - mx) * scale_log2);   // 0 for an idle warp
+        lsum = fmaf(sh.l[w][g], a, lsum);
+        osum = fmaf(sh.o[w][g][t], a, osum);
+    }
+}
 
+// GT = 1 or 2 query heads of the group are handled per pass over the rows.
+template <class Batch, int GT, bool kClustered>
+__global__ void __launch_bounds__(kDecThreads)
+decode_kernel(const __grid_constant__ Batch batch, const __nv_bfloat16* __restrict__ q,
+              const __nv_bfloat16* __restrict__ k_new, const __nv_bfloat16* __restrict__ v_new,
+              __nv_bfloat16* __restrict__ cache_k, __nv_bfloat16* __restrict__ cache_v,
+              long long stride_row, long long stride_head, int n_q_heads, int n_kv_heads, int group,
+              int rows_per_split, float scale_log2, float* __restrict__ parts, float* __restrict__ out) {
+    __shared__ DecShared<GT> sh;
+    __shared__ ClusterShared<GT> cs;
+    extern __shared__ __align__(128) uint8_t dec_ring[];         // [warp][ring step][half][row][K|V][256 B]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int hw = threadIdx.x >> 4, l16 = lane & 15;
+
+    // which (request, KV head, pass, split) this CTA owns: requests are found by their first CTA
+    int r = 0;
+    {
+        int lo = 0, hi = batch.n_req - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (batch.r[mid].cta_begin <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
+        }
+        r = lo;
+    }
+    const DecodeReq rq = batch.r[r];
+    const int n_pass = group / GT;
+    const int local = (int)blockIdx.x - rq.cta_begin;            // [head][pass][split]
+    const int split = local % rq.n_splits;
+    const int pass = (local / rq.n_splits) % n_pass;
+    const int h = local / (rq.n_splits * n_pass);
+    const int n_rows = rq.len + 1;                               // cached rows + the new one
+    const int row0 = split * rows_per_split, row1 = min(n_rows, row0 + rows_per_split);
+    const int qh0 = h * group + pass * GT;                       // first query head of this pass
+
+    prefetch_rows(cache_k, cache_v, (rq.begin + row0) * stride_row + h * stride_head, stride_row, min(row1, rq.len) - row0);
+    grid_dependency_wait();
+
+    DecState<GT> state;
+    state.load_query(q + ((long long)rq.index * n_q_heads + qh0) * kHeadDim + l16 * 8);
+    state.reset();
+    const long long head_off = (long long)h * stride_head + l16 * 8;
+    const __nv_bfloat16* ck = cache_k + rq.begin * stride_row + head_off;
+    const __nv_bfloat16* cv = cache_v + rq.begin * stride_row + head_off;
+    const __nv_bfloat16* nk = k_new + ((long long)rq.index * n_kv_heads + h) * kHeadDim + l16 * 8;
+    const __nv_bfloat16* nv = v_new + ((long long)rq.index * n_kv_heads + h) * kHeadDim + l16 * 8;
+
+    // The appended row (Eq. 2) is read from k_new / v_new by whoever owns it; the CTA that owns it
+    // on the group's first pass also writes it into the cache (nobody reads cache row `len` in this
+    // step, so the write races with nothing).
+    if (pass == 0 && rq.len >= row0 && rq.len < row1 && warp == 0) {
+        const __nv_bfloat16* src = lane < 16 ? nk : nv;
+        __nv_bfloat16* dst = (lane < 16 ? cache_k : cache_v) + rq.begin * stride_row + head_off +
+                             (long long)rq.len * stride_row;
+        *reinterpret_cast<uint4*>(dst) = __ldg(reinterpret_cast<const uint4*>(src));
+    }
+
+    // Copies of one step: K and V of kDecFlight rows per half-warp, 16 bytes per lane and row,
+    // straight into this warp's ring.  Rows past the split are zero-filled (a copy of 0 source
+    // bytes), so that they contribute exact zeros.  One commit group per step, also past the end.
+    const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(dec_ring) + warp * (kDecRing * kDecStepBytes) +
+                           ((lane >> 4) * kDecFlight * 2) * kDecRowBytes + l16 * 16;
+    auto issue = [&](int step) {
+        const int base = row0 + step * (kDecHalfWarps * kDecFlight);
+        const uint32_t dst = ring0 + (uint32_t)(step % kDecRing) * kDecStepBytes;
+        if (base < row1) {
+#pragma unroll
+            for (int f = 0; f < kDecFlight; ++f) {
+                const int row = base + f * kDecHalfWarps + hw;
+                const bool is_new = (row == rq.len);
+                const bool valid = row < row1;
+                const __nv_bfloat16* kp = (is_new || !valid) ? nk : ck + (long long)row * stride_row;
+                const __nv_bfloat16* vp = (is_new || !valid) ? nv : cv + (long long)row * stride_row;
+                const int nbytes = valid ? 16 : 0;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                             ::"r"(dst + (2 * f) * kDecRowBytes), "l"(kp), "r"(nbytes) : "memory");
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                             ::"r"(dst + (2 * f + 1) * kDecRowBytes), "l"(vp), "r"(nbytes) : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
     // the step count does not depend on the half-warp, so both halves of a warp reach the shuffles
     const int n_steps = (row1 - row0 + kDecHalfWarps * kDecFlight - 1) / (kDecHalfWarps * kDecFlight);
 #pragma unroll
@@ -269,34 +335,11 @@ decode_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __
         // the buffer refilled here was read into registers one iteration ago
         issue(st + kDecRing - 1);
         asm volatile("cp.async.wait_group %0;" ::"n"(kDecRing - 1) : "memory");
-        consume(st);
+        state.take(ring0 + (uint32_t)(st % kDecRing) * kDecStepBytes, row0 + st * (kDecHalfWarps * kDecFlight) + hw, row1, scale_log2);
     }
 
     // ---- combine: the two half-warps of a warp in registers, then the warps in warp order -------
-#pragma unroll
-    for (int g = 0; g < GT; ++g) {
-        const float m_o = __shfl_xor_sync(0xffffffffu, m[g], 16);
-        const float l_o = __shfl_xor_sync(0xffffffffu, l[g], 16);
-        const float mx = fmaxf(m[g], m_o);
-        // lower half-warp first, whichever half this lane is in
-        const bool low = lane < 16;
-        const float a_me = (mx == -INFINITY) ? 0.f : dec_ex2((m[g] - mx) * scale_log2);
-        const float a_ot = (mx == -INFINITY) ? 0.f : dec_ex2((m_o - mx) * scale_log2);
-        const float l_lo = low ? l[g] * a_me : l_o * a_ot, l_hi = low ? l_o * a_ot : l[g] * a_me;
-        l[g] = l_lo + l_hi;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float o_o = __shfl_xor_sync(0xffffffffu, o[g][i], 16);
-            const float o_lo = low ? o[g][i] * a_me : o_o * a_ot, o_hi = low ? o_o * a_ot : o[g][i] * a_me;
-            o[g][i] = o_lo + o_hi;
-        }
-        m[g] = mx;
-        if (lane == 0) { sh.m[warp][g] = m[g]; sh.l[warp][g] = l[g]; }
-        if (low) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) sh.o[warp][g][l16 * 8 + i] = o[g][i];
-        }
-    }
+    state.leave(sh, warp, lane, scale_log2);
     __syncthreads();
     // thread t < 128 owns feature t of every query head of the pass
     const int n_splits = rq.n_splits;
@@ -306,16 +349,8 @@ decode_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __
         const int t = threadIdx.x;
 #pragma unroll
         for (int g = 0; g < GT; ++g) {
-            float mx = -INFINITY;
-#pragma unroll
-            for (int w = 0; w < kDecWarps; ++w) mx = fmaxf(mx, sh.m[w][g]);
-            float lsum = 0.f, osum = 0.f;
-#pragma unroll
-            for (int w = 0; w < kDecWarps; ++w) {
-                const float a = mx == -INFINITY ? 0.f : dec_ex2((sh.m[w][g] - mx) * scale_log2);   // 0 for an idle warp
-                lsum = fmaf(sh.l[w][g], a, lsum);
-                osum = fmaf(sh.o[w][g][t], a, osum);
-            }
+            float mx, lsum, osum;
+            add_warps(sh, g, t, scale_log2, mx, lsum, osum);
             if (kClustered) {
                 if (t == 0) { cs.m[g] = mx; cs.l[g] = lsum; }
                 cs.o[g][t] = osum;
@@ -330,6 +365,179 @@ decode_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __
     }
     if (kClustered)
         cluster_combine(cs, n_splits, GT, scale_log2, out + ((long long)rq.index * n_q_heads + qh0) * kHeadDim);
+}
+
+// ---------------------------------------------------------------------------------------------
+// One query head at a time, equal shares.  The rows of all units ((request, query head), a unit's rows in steps of
+// 64) form one sequence, and every CTA takes the same number of steps of it, two CTAs to an SM: a CTA may
+// end one unit and begin the next, and its copies run ahead into the next unit while it combines.  A unit that
+// lies in several CTAs' shares is added up by decode_combine_kernel; a CTA leaves at most two partial results
+// (of the unit its share begins in and of the one it ends in).
+// us per step, whole splits | shares: four caches of 1000 to 8000 rows x 32 heads 82 | 66, 64 of 40 rows x 32 37 | 21,
+// twelve of 200 to 6000 x 8 36.5 | 30, one of 32768 x 40 118 | 109; but sixteen of 400 to 3300 x 32 78 | 80, 20000 x 8 18.4 |
+// 20.8: a share's second unit costs about 1 us (the planner compares: decode_way in api.cu).
+// ---------------------------------------------------------------------------------------------
+constexpr int kShareRing = 3;                        // steps in the ring of a warp: two CTAs to an SM
+constexpr int kShareRingBytes = kDecWarps * kShareRing * kDecStepBytes;
+constexpr int kShareRows = kDecHalfWarps * kDecFlight;
+static_assert(kShareRows == kDecodeShareRows, "the planner counts these steps");
+static_assert(kShareRingBytes * (kDecodeShareCtasPerSm + 1) > (228 << 10) && 2 * kDecodeShareCtasPerSm <= kDecodeMaxCtasPerSm,
+              "the workspace has room for two partial results of every CTA");
+
+// A CTA's way through its share.
+struct Walk {
+    int r, h;                                        // request; query head
+    int row, row1;                                   // next row; end of the share's part of the unit
+    int left;                                        // the CTA's steps from here on
+};
+__device__ __forceinline__ int unit_steps(const DecodeReq& rq) { return rq.len / kShareRows + 1; }       // of len + 1 rows
+__device__ __forceinline__ long long divide(long long x, int y) { return x >> 31 ? x / y : (int)x / y; }
+// First step of CTA c's share, and the CTA that has a given step: every share has batch.share steps, the first
+// batch.longer shares one more.
+template <class Batch>
+__device__ __forceinline__ long long share_begin(const Batch& batch, int c) {
+    return (long long)c * batch.share + min(c, batch.longer);
+}
+template <class Batch>
+__device__ __forceinline__ int share_of(const Batch& batch, long long step) {
+    const long long in_longer = (long long)batch.longer * (batch.share + 1);
+    return step < in_longer ? (int)divide(step, batch.share + 1) : batch.longer + (int)divide(step - in_longer, batch.share);
+}
+template <class Batch>
+__device__ __forceinline__ Walk start_walk(const Batch& batch) {
+    const long long s0 = share_begin(batch, blockIdx.x);
+    int lo = 0, hi = batch.n_req - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (batch.r[mid].step_begin <= s0) lo = mid; else hi = mid - 1;
+    }
+    const DecodeReq& rq = batch.r[lo];
+    const int n = unit_steps(rq);
+    Walk w;
+    w.r = lo;
+    w.h = (int)divide(s0 - rq.step_begin, n);
+    const int st = (int)(s0 - rq.step_begin - (long long)w.h * n);
+    w.left = batch.share + ((int)blockIdx.x < batch.longer ? 1 : 0);
+    w.row = st * kShareRows;
+    w.row1 = w.left >= n - st ? rq.len + 1 : (st + w.left) * kShareRows;
+    return w;
+}
+// On to the next step; true if it belongs to another unit.
+template <class Batch>
+__device__ __forceinline__ bool next_step(Walk& w, const Batch& batch, int n_q_heads) {
+    --w.left;
+    w.row += kShareRows;
+    if (w.row < w.row1 || w.left == 0) return false;
+    if (++w.h == n_q_heads) { w.h = 0; ++w.r; }
+    const DecodeReq& rq = batch.r[w.r];
+    w.row = 0;
+    w.row1 = w.left >= unit_steps(rq) ? rq.len + 1 : w.left * kShareRows;
+    return true;
+}
+
+template <class Batch>
+__global__ void __launch_bounds__(kDecThreads)
+decode_shared_kernel(const __grid_constant__ Batch batch, const __nv_bfloat16* __restrict__ q,
+                     const __nv_bfloat16* __restrict__ k_new, const __nv_bfloat16* __restrict__ v_new,
+                     __nv_bfloat16* __restrict__ cache_k, __nv_bfloat16* __restrict__ cache_v,
+                     long long stride_row, long long stride_head, int n_q_heads, int n_kv_heads, int group,
+                     float scale_log2, float* __restrict__ parts, float* __restrict__ out) {
+    __shared__ DecShared<1> shared_parts[2];         // of the last part of a unit and the one before
+    extern __shared__ __align__(128) uint8_t dec_ring[];         // [warp][ring step][half][row][K|V][256 B]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int hw = threadIdx.x >> 4, l16 = lane & 15;
+
+    Walk ahead = start_walk(batch);                  // the copies' way
+    {
+        const DecodeReq& rq = batch.r[ahead.r];
+        prefetch_rows(cache_k, cache_v, (rq.begin + ahead.row) * stride_row + (long long)(ahead.h / group) * stride_head, stride_row,
+                      min(ahead.row1, rq.len) - ahead.row);
+    }
+    grid_dependency_wait();
+
+    const __nv_bfloat16 *ck, *cv, *nk, *nv;
+    int len;
+    const auto enter = [&]() {
+        const DecodeReq& rq = batch.r[ahead.r];
+        const int kvh = ahead.h / group;
+        const long long off = rq.begin * stride_row + (long long)kvh * stride_head + l16 * 8;
+        const long long row_new = ((long long)rq.index * n_kv_heads + kvh) * kHeadDim + l16 * 8;
+        ck = cache_k + off;
+        cv = cache_v + off;
+        nk = k_new + row_new;
+        nv = v_new + row_new;
+        len = rq.len;
+    };
+    enter();
+    // copies of one step, as in decode_kernel
+    const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(dec_ring) + warp * (kShareRing * kDecStepBytes) +
+                           ((lane >> 4) * kDecFlight * 2) * kDecRowBytes + l16 * 16;
+    const auto issue = [&](int step) {
+        const uint32_t dst = ring0 + (uint32_t)(step % kShareRing) * kDecStepBytes;
+        if (ahead.left > 0) {
+#pragma unroll
+            for (int f = 0; f < kDecFlight; ++f) {
+                const int row = ahead.row + f * kDecHalfWarps + hw;
+                const bool is_new = (row == len);
+                const bool valid = row < ahead.row1;
+                const __nv_bfloat16* kp = (is_new || !valid) ? nk : ck + (long long)row * stride_row;
+                const __nv_bfloat16* vp = (is_new || !valid) ? nv : cv + (long long)row * stride_row;
+                ptx::cp_async_16(dst + (2 * f) * kDecRowBytes, kp, valid ? 16 : 0);
+                ptx::cp_async_16(dst + (2 * f + 1) * kDecRowBytes, vp, valid ? 16 : 0);
+            }
+            if (next_step(ahead, batch, n_q_heads)) enter();
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    Walk here = ahead;                               // the arithmetic's way
+#pragma unroll
+    for (int st = 0; st < kShareRing - 1; ++st) issue(st);
+
+    DecState<1> state;
+    const auto begin_part = [&]() {
+        const DecodeReq& rq = batch.r[here.r];
+        state.load_query(q + ((long long)rq.index * n_q_heads + here.h) * kHeadDim + l16 * 8);
+        state.reset();
+        // whoever owns the appended row for the group's first head also writes it into the cache
+        if (here.h % group == 0 && rq.len >= here.row && rq.len < here.row1 && warp == 0) {
+            const long long from = ((long long)rq.index * n_kv_heads + here.h / group) * kHeadDim + l16 * 8;
+            const long long to = (rq.begin + rq.len) * stride_row + (long long)(here.h / group) * stride_head + l16 * 8;
+            *reinterpret_cast<uint4*>((lane < 16 ? cache_k : cache_v) + to) =
+                __ldg(reinterpret_cast<const uint4*>((lane < 16 ? k_new : v_new) + from));
+        }
+    };
+    begin_part();
+    bool from_start = here.row == 0;                 // the part begins with its unit
+    int part = 0;                                    // parts of units so far
+    for (int st = 0; here.left > 0; ++st) {
+        issue(st + kShareRing - 1);                  // the buffer refilled here was read into registers one iteration ago
+        asm volatile("cp.async.wait_group %0;" ::"n"(kShareRing - 1) : "memory");
+        state.take(ring0 + (uint32_t)(st % kShareRing) * kDecStepBytes, here.row + hw, here.row1, scale_log2);
+        const Walk done = here;
+        const bool other = next_step(here, batch, n_q_heads);
+        if (!other && here.left > 0) continue;
+        // ---- end of a part: combined like a split of decode_kernel.  One barrier: a warp that is a part ahead
+        // writes to the other buffer.
+        DecShared<1>& sh = shared_parts[part & 1];
+        state.leave(sh, warp, lane, scale_log2);
+        __syncthreads();
+        if (threadIdx.x < kHeadDim) {
+            const int t = threadIdx.x;
+            const DecodeReq& rq = batch.r[done.r];
+            float mx, lsum, osum;
+            add_warps(sh, 0, t, scale_log2, mx, lsum, osum);
+            if (from_start && done.row1 == rq.len + 1) {
+                out[((long long)rq.index * n_q_heads + done.h) * kHeadDim + t] = osum / lsum;
+            } else {
+                float* rec = parts + (2ll * blockIdx.x + (part > 0)) * (kHeadDim + 2);
+                if (t == 0) { rec[0] = mx; rec[1] = lsum; }
+                rec[2 + t] = osum;
+            }
+        }
+        ++part;
+        if (other) begin_part();
+        from_start = true;
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -387,9 +595,9 @@ struct MmaShared {
 };
 
 // gt <= GP query heads of the group are handled per pass over the rows.
-template <int GP, bool kClustered>
+template <class Batch, int GP, bool kClustered>
 __global__ void __launch_bounds__(kMmaThreads)
-decode_mma_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16* __restrict__ q,
+decode_mma_kernel(const __grid_constant__ Batch batch, const __nv_bfloat16* __restrict__ q,
                   const __nv_bfloat16* __restrict__ k_new, const __nv_bfloat16* __restrict__ v_new,
                   __nv_bfloat16* __restrict__ cache_k, __nv_bfloat16* __restrict__ cache_v,
                   long long stride_row, long long stride_head, int n_q_heads, int n_kv_heads, int group, int gt,
@@ -417,6 +625,7 @@ decode_mma_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16
     const int row0 = split * rows_per_split, row1 = min(n_rows, row0 + rows_per_split);
     const int qh0 = h * group + pass * gt;                       // first query head of this pass
 
+    prefetch_rows(cache_k, cache_v, (rq.begin + row0) * stride_row + h * stride_head, stride_row, min(row1, rq.len) - row0);
     grid_dependency_wait();
 
     const long long head_off = (long long)h * stride_head;
@@ -617,24 +826,41 @@ decode_mma_kernel(const __grid_constant__ DecodeBatch batch, const __nv_bfloat16
 // (the kernel is bound by the latency of these loads).  Launched
 // behind decode_kernel with programmatic stream serialisation: no counters, no atomics, nothing in
 // the workspace has to be cleared, and the order of additions is fixed.
+template <class Batch>
 __global__ void __launch_bounds__(kHeadDim)
-decode_combine_kernel(const __grid_constant__ DecodeBatch batch, int gt, int n_pass, int n_q_heads, int group,
+decode_combine_kernel(const __grid_constant__ Batch batch, int gt, int n_pass, int n_q_heads, int group,
                       float scale_log2, const float* __restrict__ parts, float* __restrict__ out) {
     const DecodeReq rq = batch.r[blockIdx.y];
-    const int n_splits = rq.n_splits;
     const int g = (int)blockIdx.x % gt, unit = (int)blockIdx.x / gt;     // unit = h * n_pass + pass
     const int pass = unit % n_pass, h = unit / n_pass;
     const int t = threadIdx.x;
-    grid_dependency_wait();
-    if (n_splits == 1) return;                                   // decode_kernel wrote the output itself
     const long long part_stride = kHeadDim + 2;
-    const float* base = parts + ((long long)rq.part_begin + (long long)unit * n_splits * gt + g) * part_stride;
-    const long long step = (long long)gt * part_stride;          // between the records of two splits
+    int n_splits;                                                // partial results of the unit,
+    const float* base;                                           // the first of them (but see `skip`),
+    long long step, skip = 0;                                    // and from one to the next
+    if (batch.share > 0) {
+        // the CTAs whose shares hold the unit's first and last step.  The unit is the first CTA's last one, in
+        // its second record, unless the share begins with it; it is the others' first.
+        const int steps = unit_steps(rq);
+        const long long s0 = rq.step_begin + (long long)unit * steps;
+        const int c0 = share_of(batch, s0);
+        n_splits = share_of(batch, s0 + steps - 1) - c0 + 1;
+        base = parts + 2ll * c0 * part_stride;
+        step = 2 * part_stride;
+        skip = share_begin(batch, c0) == s0 ? 0 : part_stride;
+    } else {
+        n_splits = rq.n_splits;
+        base = parts + (rq.part_begin + (long long)unit * n_splits * gt + g) * part_stride;
+        step = (long long)gt * part_stride;
+    }
+    grid_dependency_wait();
+    if (n_splits == 1) return;                                   // the output is already written
+    const auto record = [&](int i) { return base + i * step + (i == 0 ? skip : 0); };
     // largest reference value over the splits: thread t looks at splits t, t + 128, ...; one round
     // trip for up to 128 splits, then a block-wide maximum
     __shared__ float warp_max[kHeadDim / 32];
     float mx = -INFINITY;
-    for (int sp = t; sp < n_splits; sp += kHeadDim) mx = fmaxf(mx, __ldcg(base + sp * step));
+    for (int sp = t; sp < n_splits; sp += kHeadDim) mx = fmaxf(mx, __ldcg(record(sp)));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if ((t & 31) == 0) warp_max[t >> 5] = mx;
@@ -648,7 +874,7 @@ decode_combine_kernel(const __grid_constant__ DecodeBatch batch, int gt, int n_p
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
             const bool in = s0 + j < n_splits;
-            const float* rec = base + (s0 + j) * step;
+            const float* rec = record(s0 + j);
             mv[j] = in ? __ldcg(rec) : -INFINITY;
             lv[j] = in ? __ldcg(rec + 1) : 0.f;
             ov[j] = in ? __ldcg(rec + 2 + t) : 0.f;
@@ -667,31 +893,55 @@ decode_combine_kernel(const __grid_constant__ DecodeBatch batch, int gt, int n_p
 
 namespace {
 
-typedef void (*MmaKernel)(DecodeBatch, const __nv_bfloat16*, const __nv_bfloat16*, const __nv_bfloat16*, __nv_bfloat16*,
-                          __nv_bfloat16*, long long, long long, int, int, int, int, int, float, float*, float*);
-MmaKernel mma_kernel(int gt, bool clustered) {
-    if (clustered)
-        return gt > 4 ? decode_mma_kernel<8, true> : gt > 2 ? decode_mma_kernel<4, true> : decode_mma_kernel<2, true>;
-    return gt > 4 ? decode_mma_kernel<8, false> : gt > 2 ? decode_mma_kernel<4, false> : decode_mma_kernel<2, false>;
-}
+template <class Batch>
+struct Kernels {
+    typedef void (*Scalar)(Batch, const __nv_bfloat16*, const __nv_bfloat16*, const __nv_bfloat16*, __nv_bfloat16*,
+                           __nv_bfloat16*, long long, long long, int, int, int, int, float, float*, float*);
+    typedef void (*Mma)(Batch, const __nv_bfloat16*, const __nv_bfloat16*, const __nv_bfloat16*, __nv_bfloat16*,
+                        __nv_bfloat16*, long long, long long, int, int, int, int, int, float, float*, float*);
+    static Scalar scalar(int gt, bool clustered) {
+        return gt == 2 ? (clustered ? decode_kernel<Batch, 2, true> : decode_kernel<Batch, 2, false>)
+                       : (clustered ? decode_kernel<Batch, 1, true> : decode_kernel<Batch, 1, false>);
+    }
+    static Mma mma(int gt, bool clustered) {
+        if (clustered)
+            return gt > 4 ? decode_mma_kernel<Batch, 8, true> : gt > 2 ? decode_mma_kernel<Batch, 4, true> : decode_mma_kernel<Batch, 2, true>;
+        return gt > 4 ? decode_mma_kernel<Batch, 8, false> : gt > 2 ? decode_mma_kernel<Batch, 4, false> : decode_mma_kernel<Batch, 2, false>;
+    }
+    static cudaError_t configure() {
+        cudaError_t e = cudaFuncSetAttribute(decode_shared_kernel<Batch>, cudaFuncAttributeMaxDynamicSharedMemorySize, kShareRingBytes);
+        for (bool clustered : {false, true}) {
+            for (int gt : {1, 2})
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute(scalar(gt, clustered), cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
+            for (int gt : {2, 4, 8})
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute(mma(gt, clustered), cudaFuncAttributeMaxDynamicSharedMemorySize, kMmaRingBytes);
+        }
+        return e;
+    }
+};
 
 // The rings need more dynamic shared memory than the default limit: raised once per device.
 cudaError_t configure_decode() {
     static unsigned long long configured = 0;
     return once_per_device(configured, []() {
-        cudaError_t e = cudaFuncSetAttribute(decode_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(decode_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(decode_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(decode_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecRingBytes);
-        for (int gt : {2, 4, 8})
-            for (bool clustered : {false, true})
-                if (e == cudaSuccess)
-                    e = cudaFuncSetAttribute(mma_kernel(gt, clustered), cudaFuncAttributeMaxDynamicSharedMemorySize, kMmaRingBytes);
-        return e;
+        const cudaError_t e = Kernels<DecodeBatch>::configure();
+        return e != cudaSuccess ? e : Kernels<DecodeBatchOf<1>>::configure();
     });
+}
+
+// f(batch), with the smaller argument where there is one request
+template <class F>
+cudaError_t with_batch(const DecodeBatch& batch, F f) {
+    if (batch.n_req != 1) return f(batch);
+    DecodeBatchOf<1> one;
+    one.n_req = 1;
+    one.share = batch.share;
+    one.longer = batch.longer;
+    one.pad = 0;
+    one.r[0] = batch.r[0];
+    return f(one);
 }
 
 }  // namespace
@@ -706,16 +956,15 @@ int decode_ctas_per_sm(int gt, bool mma) {
     int v = __atomic_load_n(&cache[dev][idx], __ATOMIC_ACQUIRE);
     if (v > 0) return v;
     if (configure_decode() != cudaSuccess) { cudaGetLastError(); return 0; }
-    cudaError_t err;
-    if (mma) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, mma_kernel(gt, false), kMmaThreads, kMmaRingBytes);
-    else if (gt == 2) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, decode_kernel<2, false>, kDecThreads, kDecRingBytes);
-    else err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, decode_kernel<1, false>, kDecThreads, kDecRingBytes);
+    typedef Kernels<DecodeBatch> K;
+    const cudaError_t err = mma ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, K::mma(gt, false), kMmaThreads, kMmaRingBytes)
+                                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, K::scalar(gt, false), kDecThreads, kDecRingBytes);
     if (err != cudaSuccess || v <= 0) { cudaGetLastError(); return 0; }
     __atomic_store_n(&cache[dev][idx], v, __ATOMIC_RELEASE);
     return v;
 }
 
-cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, bool mma, int cluster, const void* q,
+cudaError_t launch_decode(const DecodeBatch& all, int total_ctas, int gt, bool mma, int cluster, const void* q,
                           const void* k_new, const void* v_new, void* cache_k, void* cache_v,
                           long long stride_row, long long stride_head, int n_q_heads, int n_kv_heads,
                           int rows_per_split, float scale_log2, float* parts, float* out,
@@ -725,26 +974,34 @@ cudaError_t launch_decode(const DecodeBatch& batch, int total_ctas, int gt, bool
     cudaError_t err = configure_decode();
     if (err != cudaSuccess) return err;
     const bool clustered = cluster > 1;
-    if (mma)
-        return launch_chained_clusters(mma_kernel(gt, clustered), dim3((unsigned)total_ctas), dim3(kMmaThreads), (unsigned)cluster,
-                                       (size_t)kMmaRingBytes, stream, batch, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_new,
-                                       (const __nv_bfloat16*)v_new, (__nv_bfloat16*)cache_k, (__nv_bfloat16*)cache_v, stride_row,
-                                       stride_head, n_q_heads, n_kv_heads, group, gt, rows_per_split, scale_log2, parts, out);
-    const auto scalar = gt == 2 ? (clustered ? decode_kernel<2, true> : decode_kernel<2, false>)
-                                : (clustered ? decode_kernel<1, true> : decode_kernel<1, false>);
-    return launch_chained_clusters(scalar, dim3((unsigned)total_ctas),
-                                   dim3(kDecThreads), (unsigned)cluster, (size_t)kDecRingBytes, stream, batch, (const __nv_bfloat16*)q,
-                                   (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, (__nv_bfloat16*)cache_k,
-                                   (__nv_bfloat16*)cache_v, stride_row, stride_head, n_q_heads, n_kv_heads, group,
-                                   rows_per_split, scale_log2, parts, out);
+    const dim3 grid((unsigned)total_ctas);
+    const auto *qb = (const __nv_bfloat16*)q, *kb = (const __nv_bfloat16*)k_new, *vb = (const __nv_bfloat16*)v_new;
+    auto *ck = (__nv_bfloat16*)cache_k, *cv = (__nv_bfloat16*)cache_v;
+    return with_batch(all, [&](const auto& batch) {
+        typedef Kernels<typename std::decay<decltype(batch)>::type> K;
+        typedef typename std::decay<decltype(batch)>::type Batch;
+        if (batch.share > 0)
+            return launch_chained(decode_shared_kernel<Batch>, grid, dim3(kDecThreads), (size_t)kShareRingBytes, stream, batch, qb, kb, vb,
+                                  ck, cv, stride_row, stride_head, n_q_heads, n_kv_heads, group, scale_log2, parts, out);
+        if (mma)
+            return launch_chained_clusters(K::mma(gt, clustered), grid, dim3(kMmaThreads), (unsigned)cluster, (size_t)kMmaRingBytes, stream,
+                                           batch, qb, kb, vb, ck, cv, stride_row, stride_head, n_q_heads, n_kv_heads, group, gt,
+                                           rows_per_split, scale_log2, parts, out);
+        return launch_chained_clusters(K::scalar(gt, clustered), grid, dim3(kDecThreads), (unsigned)cluster, (size_t)kDecRingBytes, stream,
+                                       batch, qb, kb, vb, ck, cv, stride_row, stride_head, n_q_heads, n_kv_heads, group, rows_per_split,
+                                       scale_log2, parts, out);
+    });
 }
 
-cudaError_t launch_decode_combine(const DecodeBatch& batch, int gt, int n_q_heads, int n_kv_heads,
+cudaError_t launch_decode_combine(const DecodeBatch& all, int gt, int n_q_heads, int n_kv_heads,
                                   float scale_log2, const float* parts, float* out, cudaStream_t stream) {
     const int group = n_q_heads / n_kv_heads;
     const int n_pass = group / gt;
-    return launch_chained(decode_combine_kernel, dim3((unsigned)(n_kv_heads * n_pass * gt), (unsigned)batch.n_req),
-                          dim3(kHeadDim), 0, stream, batch, gt, n_pass, n_q_heads, group, scale_log2, parts, out);
+    return with_batch(all, [&](const auto& batch) {
+        return launch_chained(decode_combine_kernel<typename std::decay<decltype(batch)>::type>,
+                              dim3((unsigned)(n_kv_heads * n_pass * gt), (unsigned)batch.n_req), dim3(kHeadDim), 0, stream, batch, gt,
+                              n_pass, n_q_heads, group, scale_log2, parts, out);
+    });
 }
 
 }  // namespace lookm

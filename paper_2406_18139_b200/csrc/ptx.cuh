@@ -182,6 +182,10 @@ __device__ __forceinline__ void tmem_ld_wait() {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// Brings the 128 bytes at p into L2; a hint that changes nothing else.
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
 // Read-only global loads that stay where they are written (the compiler may not sink them to their
 // first use): for values requested long before they are needed.
 __device__ __forceinline__ int ld_nc_s32(const int* p) {

@@ -170,6 +170,47 @@ def test_batches_of_grouped_queries_at_the_edges_of_sixteen_row_steps(B, group):
         assert torch.equal(dk[a + n], kn[r]) and torch.equal(dv[a + n], vn[r])
 
 
+@pytest.mark.parametrize("lens,heads,group,ranked", [
+    ([0, 1, 31, 40, 62, 63, 64, 65, 126, 127, 128, 129] * 9, 24, 1, False),      # more requests than one launch carries
+    ([40] * 64, 32, 1, True),                            # units of one step: none is shared
+    ([7000, 63, 64, 2000], 32, 1, False),                # units that many CTAs share beside units of a single step
+    ([20031], 40, 1, True),                              # a head per 7.4 CTAs
+    ([5000, 100, 5000], 20, 2, False)])
+def test_equal_shares_of_all_rows(B, lens, heads, group, ranked):
+    """CTAs whose shares begin and end anywhere in a unit: units of less than a step to hundreds of steps, the
+    appended row in the last step or in one of its own; `heads` KV heads, [heads, rows, 128] or packed."""
+    import torch
+    f, n_req, hq = synth.bf16_to_f32, len(lens), heads * group
+    begins = np.concatenate([[0], np.cumsum([n + 1 for n in lens])]).tolist()
+    shape = (heads, begins[-1], 128) if ranked else (begins[-1], heads, 128)
+    gen = torch.Generator(device="cuda").manual_seed(len(lens) + heads)
+    dk, dv, q, kn, vn = (torch.randn(*s_, 128, generator=gen, device="cuda").bfloat16()
+                         for s_ in (shape[:2], shape[:2], (n_req, hq), (n_req, heads), (n_req, heads)))
+    lay = B.CacheLayout(hq, heads, 128, *((128, begins[-1] * 128) if ranked else (heads * 128, 128)), 0.0)
+    ws = B.alloc_decode_workspace(lay, n_req)
+    outs = []
+    by_head = lambda t: t if ranked else t.transpose(0, 1)
+    before_k, before_v = dk.clone(), dv.clone()
+    for _ in range(3):
+        ws.random_(0, 255)                               # nothing in the workspace counts
+        out = torch.full((n_req, hq, 128), np.nan, device="cuda")
+        B.check(B.lookm_decode_step_varlen(q, kn, vn, dk, dv, begins[:-1], lens, lay, out, ws))
+        outs.append(out)
+    torch.cuda.synchronize()
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+    K, V = by_head(dk).double(), by_head(dv).double()
+    untouched = torch.ones(begins[-1], dtype=torch.bool, device="cuda")
+    for r, n in enumerate(lens):
+        a = begins[r]
+        assert torch.equal(by_head(dk)[:, a + n], kn[r]) and torch.equal(by_head(dv)[:, a + n], vn[r])
+        untouched[a + n] = False
+        s_ = torch.einsum("hgd,hnd->hgn", q[r].double().view(heads, group, 128), K[:, a:a + n + 1]) / 128 ** 0.5
+        ref = torch.einsum("hgn,hnd->hgd", s_.softmax(-1), V[:, a:a + n + 1]).reshape(hq, 128)
+        assert ((outs[0][r].double() - ref).abs() <= 1e-3 * ref.abs() + 1e-5).all(), (r, n)
+    assert torch.equal(by_head(dk)[:, untouched], by_head(before_k)[:, untouched])
+    assert torch.equal(by_head(dv)[:, untouched], by_head(before_v)[:, untouched])
+
+
 def test_long_cache_is_cut_into_many_splits(B):
     # 2 KV heads x 20001 rows: about 150 splits per head, combined by the last CTA to arrive
     run_step(B, 8, 2, 20000, 20001, False, seed=701)
