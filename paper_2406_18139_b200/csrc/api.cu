@@ -362,12 +362,18 @@ int make_map_2d(CUtensorMap* map, const void* base, long long rows) {
         if (st_ != LOOKM_OK) return st_;  \
     } while (0)
 
+// A call of one prompt that begins with sweep 1 of whole single blocks needs no table writer: its launches
+// carry the request, and that sweep clears the words that later ones count in.
+bool sweep_clears(const Plan& pl) { return pl.n_req == 1 && pl.blocks == 1 && pl.splits[0] == 1; }
+
 template <class T>
 T* at(void* ws, size_t off) { return reinterpret_cast<T*>(static_cast<char*>(ws) + off); }
 
-// Clears the status word and the arrival counters and writes the request table into the workspace.
-int begin_call(const Plan& pl, void* ws, cudaStream_t st) {
+// Clears the status word and the arrival counters and writes the request table into the workspace (unless the
+// call's sweep 1 does what is needed of that: see sweep_clears).
+int begin_call(const Plan& pl, void* ws, cudaStream_t st, bool with_sweep1 = false) {
     g_launches = 0;
+    if (with_sweep1 && sweep_clears(pl)) return LOOKM_OK;
     for (int base = 0; base < pl.n_req; base += kReqChunk) {
         ReqChunk chunk;
         const int cnt = std::min(kReqChunk, pl.n_req - base);
@@ -385,11 +391,18 @@ float scale_log2(const lookm_layout* lay) {
     return s * 1.4426950408889634f;
 }
 
+ReqTable req_table(const Plan& pl, void* ws) {
+    ReqTable t;
+    t.rows = at<Req>(ws, pl.o_reqs);
+    t.n = pl.n_req;
+    t.only = pl.reqs[0];
+    return t;
+}
+
 TileParams tile_params(const Plan& pl, void* ws, const lookm_layout* lay) {
     TileParams p;
     std::memset(&p, 0, sizeof(p));
-    p.reqs = at<Req>(ws, pl.o_reqs);
-    p.n_req = pl.n_req;
+    p.reqs = req_table(pl, ws);
     p.n_q_heads = pl.n_q_heads;
     p.n_kv_heads = pl.n_kv_heads;
     p.group = pl.group;
@@ -416,6 +429,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     p.scores = scores;
     if (!lse_is_input) {
         p.n_items = pl.n_items[kSweep1];
+        p.n_clear = sweep_clears(pl) ? (int)pl.clear_words : 0;
         p.next_item = p.status + 16 + kSweep1;
         p.splits = pl.splits[0];
         p.parts1 = at<float2>(ws, pl.o_kept_keys);
@@ -446,13 +460,13 @@ int run_match(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     float* rnorm_all = at<float>(ws, pl.o_rnorm_all);
     float* rnorm_kept = at<float>(ws, pl.o_rnorm_kept);
     void* kept_keys = at<void>(ws, pl.o_kept_keys);
-    const Req* reqs = at<Req>(ws, pl.o_reqs);
+    const ReqTable reqs = req_table(pl, ws);
     if (!norms_done) {
         LOOKM_CUDA(launch_key_norms(k, lay->kv_stride_tok, lay->kv_stride_head, pl.n_kv_heads, pl.T,
                                     rnorm_all, st));
         ++g_launches;
     }
-    LOOKM_CUDA(launch_gather_kept(k, lay->kv_stride_tok, lay->kv_stride_head, reqs, pl.n_req,
+    LOOKM_CUDA(launch_gather_kept(k, lay->kv_stride_tok, lay->kv_stride_head, reqs,
                                   pl.n_kv_heads, pl.T, pl.total_slots, kept_idx, rnorm_all,
                                   kept_keys, rnorm_kept, at<int>(ws, pl.o_status), st));
     ++g_launches;
@@ -481,7 +495,7 @@ constexpr long long kInvCtasPerSm = 2, kInvSmemPerSm = 220 << 10;
 constexpr int kInvMinShare = 512;
 cudaError_t run_inversion(const Plan& pl, const DeviceInfo& di, const int* kept_idx, const int* evict_idx, const int* assign,
                           const float* sim, void* ws, cudaStream_t st) {
-    const Req* reqs = at<Req>(ws, pl.o_reqs);
+    const ReqTable reqs = req_table(pl, ws);
     int *status = at<int>(ws, pl.o_status), *row_begin = at<int>(ws, pl.o_row_begin);
     int2* entries = at<int2>(ws, pl.o_entries);
     int4* units = at<int4>(ws, pl.o_units);
@@ -499,7 +513,7 @@ cudaError_t run_inversion(const Plan& pl, const DeviceInfo& di, const int* kept_
     int ctas = ctas_per_head(std::min(kInvCtasPerSm, std::max(1ll, kInvSmemPerSm / slot_bytes)));
     if (pl.max_B <= kCountMaxSlots && pl.max_E <= ctas * kCountWarps * kCountSeg) {
         const int max_slots = ctas * (((pl.max_B + ctas - 1) / ctas + 3) / 4 * 4);
-        return launch_invert_counting(assign, kept_idx, evict_idx, sim, reqs, pl.n_req, pl.n_kv_heads, ctas, max_slots, pl.T,
+        return launch_invert_counting(assign, kept_idx, evict_idx, sim, reqs, pl.n_kv_heads, ctas, max_slots, pl.T,
                                       entries, units, slot_cnt, status, st);
     }
     // counter width and widest digit over the requests of the call
@@ -511,7 +525,7 @@ cudaError_t run_inversion(const Plan& pl, const DeviceInfo& di, const int* kept_
         invert_digits(r.B, wide ? kInvDigitBits32 : kInvDigitBits16, n_pass, dbits);
         digit_bits = std::max(digit_bits, dbits);
     }
-    return launch_invert_assignment(assign, kept_idx, evict_idx, sim, reqs, pl.n_req, pl.n_kv_heads, ctas, pl.T, wide, digit_bits, row_begin,
+    return launch_invert_assignment(assign, kept_idx, evict_idx, sim, reqs, pl.n_kv_heads, ctas, pl.T, wide, digit_bits, row_begin,
                                     entries, units, slot_cnt, at<unsigned>(ws, pl.o_sort_a), at<unsigned>(ws, pl.o_sort_b),
                                     status, st);
 }
@@ -519,7 +533,7 @@ cudaError_t run_inversion(const Plan& pl, const DeviceInfo& di, const int* kept_
 int run_merge(const Plan& pl, const lookm_layout* lay, const void* k, const void* v,
               const int* kept_idx, const int* evict_idx, const int* assign, const float* sim,
               int varlen_output, void* out_k, void* out_v, void* ws, cudaStream_t st) {
-    const Req* reqs = at<Req>(ws, pl.o_reqs);
+    const ReqTable reqs = req_table(pl, ws);
     int* status = at<int>(ws, pl.o_status);
     const bool short_merge = pl.max_L <= kMergeShortMax;
     DeviceInfo di;
@@ -532,10 +546,10 @@ int run_merge(const Plan& pl, const lookm_layout* lay, const void* k, const void
     if (pl.n_none < pl.n_req) {
         if (short_merge)
             LOOKM_CUDA(launch_merge_short(k, v, lay->kv_stride_tok, lay->kv_stride_head, assign, kept_idx, evict_idx, sim,
-                                          reqs, pl.n_req, pl.n_kv_heads, pl.max_L, pl.max_E, pl.max_B, varlen_output,
+                                          reqs, pl.n_kv_heads, pl.max_L, pl.max_E, pl.max_B, varlen_output,
                                           pl.out_stride_head, out_k, out_v, status, di.sms, st));
         else
-            LOOKM_CUDA(launch_merge(k, v, lay->kv_stride_tok, lay->kv_stride_head, reqs, pl.n_req,
+            LOOKM_CUDA(launch_merge(k, v, lay->kv_stride_tok, lay->kv_stride_head, reqs,
                                     pl.n_kv_heads, pl.T, pl.total_units, at<int2>(ws, pl.o_entries),
                                     at<int4>(ws, pl.o_units), at<int>(ws, pl.o_slot_cnt),
                                     at<float>(ws, pl.o_parts), varlen_output, pl.out_stride_head, out_k,
@@ -544,7 +558,7 @@ int run_merge(const Plan& pl, const lookm_layout* lay, const void* k, const void
     }
     if (pl.n_none > 0) {
         // eviction alone: the kept rows of those requests go straight to the output
-        LOOKM_CUDA(launch_compact_kept(k, v, lay->kv_stride_tok, lay->kv_stride_head, reqs, pl.n_req,
+        LOOKM_CUDA(launch_compact_kept(k, v, lay->kv_stride_tok, lay->kv_stride_head, reqs,
                                        pl.n_kv_heads, pl.total_slots, kept_idx, varlen_output,
                                        pl.out_stride_head, out_k, out_v, status, st));
         ++g_launches;
@@ -601,7 +615,7 @@ int compress_common(const void* q, const void* k, const void* v, const uint8_t* 
         out_cu[0] = 0;
         for (int r = 0; r < n_req; ++r) out_cu[r + 1] = out_cu[r] + pl.out_len[r];
     }
-    LOOKM_TRY(begin_call(pl, ws, st));
+    LOOKM_TRY(begin_call(pl, ws, st, !lse_in));
     mark_stage(0, st);
     float* scores = at<float>(ws, pl.o_scores);
     int* kept = at<int>(ws, pl.o_kept);
@@ -614,7 +628,7 @@ int compress_common(const void* q, const void* k, const void* v, const uint8_t* 
     LOOKM_TRY(run_score(pl, di, lay, q, k, scores, lse, lse_in != nullptr, ws, st));
     // the selection launch also computes the key norms that the matching needs
     const bool need_match = pl.n_items[kMatch] > 0;
-    LOOKM_CUDA(launch_select(scores, text_prior ? mask : nullptr, at<Req>(ws, pl.o_reqs), pl.n_req,
+    LOOKM_CUDA(launch_select(scores, text_prior ? mask : nullptr, req_table(pl, ws),
                              pl.n_kv_heads, pl.T, pl.max_L, kept, evict, rank, need_match ? k : nullptr,
                              lay->kv_stride_tok, lay->kv_stride_head, at<float>(ws, pl.o_rnorm_all),
                              di.sms, st));
@@ -716,7 +730,7 @@ int lookm_score(const void* q, const void* k, const int* cu_seqlens_host, int n_
     DeviceInfo di;
     LOOKM_TRY(device_info(di));
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    LOOKM_TRY(begin_call(pl, workspace, st));
+    LOOKM_TRY(begin_call(pl, workspace, st, !lse_is_input));
     float* lse_buf = lse ? lse : at<float>(workspace, pl.o_lse);
     return run_score(pl, di, layout, q, k, scores, lse_buf, lse_is_input != 0, workspace, st);
 }
@@ -737,7 +751,7 @@ int lookm_select(const float* scores, const uint8_t* modality_mask, const int* c
     LOOKM_TRY(check_workspace(pl, workspace, workspace_bytes));
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     LOOKM_TRY(begin_call(pl, workspace, st));
-    LOOKM_CUDA(launch_select(scores, modality_mask, at<Req>(workspace, pl.o_reqs), pl.n_req,
+    LOOKM_CUDA(launch_select(scores, modality_mask, req_table(pl, workspace),
                              pl.n_kv_heads, pl.T, pl.max_L, kept_idx, evict_idx, rank, nullptr, 0, 0, nullptr, 0, st));
     ++g_launches;
     return LOOKM_OK;
@@ -774,7 +788,7 @@ int lookm_match_from_sim(const float* sim_matrix, const int* cu_seqlens_host, in
     LOOKM_TRY(check_workspace(pl, workspace, workspace_bytes));
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     LOOKM_TRY(begin_call(pl, workspace, st));
-    LOOKM_CUDA(launch_argmax_rows(sim_matrix, at<Req>(workspace, pl.o_reqs), pl.n_req, pl.n_kv_heads,
+    LOOKM_CUDA(launch_argmax_rows(sim_matrix, req_table(pl, workspace), pl.n_kv_heads,
                                   pl.max_E, assign, sim, st));
     ++g_launches;
     return LOOKM_OK;

@@ -63,12 +63,26 @@ struct Req {
     int tile_begin;       // 128-row blocks of the requests before this one (table order)
 };
 
+// The requests of a call as its launches get them.  A single request travels with every launch: fetching
+// it from the table in the workspace would be the first of the dependent loads that a short prompt's kernels
+// consist of.
+struct ReqTable {
+    const Req* rows;      // in the workspace; not written where `only` is all that the launches need
+    int n;
+    Req only;             // n == 1
+#ifdef __CUDACC__
+    __device__ __forceinline__ Req get(int i) const {
+        if (n == 1) return only;
+        return rows[i];
+    }
+#endif
+};
+
 enum TileKind { kSweep1 = 0, kSweep2 = 1, kMatch = 2 };
 
 constexpr int kMaxSplits = 4;
 struct TileParams {
-    const Req* reqs;
-    int n_req;
+    ReqTable reqs;
     int n_items;
     int n_q_heads, n_kv_heads, group;
     long long T;                 // total packed tokens
@@ -93,6 +107,7 @@ struct TileParams {
     int* assign;                 // evicted-list layout  (match)
     float* sim;                  // evicted-list layout  (match)
     int* status;                 // device status word
+    int n_clear;                 // words from the status word on that sweep 1 has to clear
 };
 
 // ---- launchers (each enqueues on `stream` and returns the CUDA error of the launch) -----------
@@ -112,7 +127,7 @@ cudaError_t launch_lse_split(const float* lse, int n_q_heads, long long T, float
 // nobody arrives at; on expiry it writes LOOKM_ERR_DEVICE_TIMEOUT to *status like they do.
 cudaError_t launch_wait_probe(unsigned long long limit_ns, int* status, cudaStream_t stream);
 
-cudaError_t launch_select(const float* scores, const uint8_t* mask, const Req* reqs, int n_req,
+cudaError_t launch_select(const float* scores, const uint8_t* mask, const ReqTable& reqs,
                           int n_kv_heads, long long T, int max_L, int* kept_idx, int* evict_idx, int* rank,
                           const void* k_for_norms, long long stride_tok, long long stride_head,
                           float* rnorm_all, int num_sms, cudaStream_t stream);
@@ -121,12 +136,12 @@ cudaError_t launch_key_norms(const void* k, long long stride_tok, long long stri
                              int n_kv_heads, long long T, float* rnorm_all, cudaStream_t stream);
 
 cudaError_t launch_gather_kept(const void* k, long long stride_tok, long long stride_head,
-                               const Req* reqs, int n_req, int n_kv_heads, long long T,
+                               const ReqTable& reqs, int n_kv_heads, long long T,
                                long long total_kept_rows, const int* kept_idx,
                                const float* rnorm_all, void* kept_keys, float* rnorm_kept,
                                int* status, cudaStream_t stream);
 
-cudaError_t launch_argmax_rows(const float* sim_matrix, const Req* reqs, int n_req, int n_kv_heads,
+cudaError_t launch_argmax_rows(const float* sim_matrix, const ReqTable& reqs, int n_kv_heads,
                                int max_evicted, int* assign, float* sim, cudaStream_t stream);
 
 // Copies up to kReqChunk table entries, passed by value as a kernel argument, into the workspace;
@@ -137,27 +152,27 @@ struct ReqChunk { Req r[kReqChunk]; };
 cudaError_t launch_write_table(const ReqChunk& chunk, int count, Req* dst, int* clear, size_t n_clear, cudaStream_t stream);
 
 cudaError_t launch_invert_assignment(const int* assign, const int* kept_idx, const int* evict_idx,
-                                     const float* sim, const Req* reqs, int n_req, int n_kv_heads, int ctas,
+                                     const float* sim, const ReqTable& reqs, int n_kv_heads, int ctas,
                                      long long T, bool wide_counts, int digit_bits, int* row_begin,
                                      int2* entries, int4* unit_first, int* slot_cnt,
                                      unsigned* sort_a, unsigned* sort_b, int* status,
                                      cudaStream_t stream);
 
-cudaError_t launch_invert_counting(const int* assign, const int* kept_idx, const int* evict_idx, const float* sim, const Req* reqs,
-                                   int n_req, int n_kv_heads, int ctas, int max_slots, long long T, int2* entries,
+cudaError_t launch_invert_counting(const int* assign, const int* kept_idx, const int* evict_idx, const float* sim, const ReqTable& reqs,
+                                   int n_kv_heads, int ctas, int max_slots, long long T, int2* entries,
                                    int4* unit_first, int* slot_cnt, int* status, cudaStream_t stream);
 
 // Inversion and merge in one launch; every request has at most kMergeShortMax tokens.
 constexpr int kMergeShortMax = 4096;
 cudaError_t launch_merge_short(const void* k, const void* v, long long stride_tok, long long stride_head, const int* assign,
-                               const int* kept_idx, const int* evict_idx, const float* sim, const Req* reqs, int n_req,
+                               const int* kept_idx, const int* evict_idx, const float* sim, const ReqTable& reqs,
                                int n_kv_heads, int max_L, int max_E, int max_B, int varlen_output, long long out_stride_head,
                                void* out_k, void* out_v, int* status, int num_sms, cudaStream_t stream);
 
 int merge_warps_per_sm();
 
 cudaError_t launch_merge(const void* k, const void* v, long long stride_tok, long long stride_head,
-                         const Req* reqs, int n_req, int n_kv_heads, long long T,
+                         const ReqTable& reqs, int n_kv_heads, long long T,
                          long long total_units, const int2* entries,
                          const int4* unit_first, int* slot_cnt, float* parts,
                          int varlen_output, long long out_stride_head, void* out_k, void* out_v,
@@ -166,7 +181,7 @@ cudaError_t launch_merge(const void* k, const void* v, long long stride_tok, lon
 // Kept K and V rows of the requests whose mode is LOOKM_MERGE_NONE copied to the output cache
 // (eviction alone, Eq. 6-7); requests with another mode are left to the merge kernel.
 cudaError_t launch_compact_kept(const void* k, const void* v, long long stride_tok,
-                                long long stride_head, const Req* reqs, int n_req, int n_kv_heads,
+                                long long stride_head, const ReqTable& reqs, int n_kv_heads,
                                 long long total_kept_rows, const int* kept_idx, int varlen_output,
                                 long long out_stride_head, void* out_k, void* out_v, int* status,
                                 cudaStream_t stream);

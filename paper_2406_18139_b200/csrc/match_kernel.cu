@@ -67,7 +67,7 @@ struct Item {
     long long ev0;                               // start of its evicted list
 };
 __device__ __forceinline__ Item decode_item(const TileParams& p, const Req* tbl, int item) {
-    int lo = 0, hi = p.n_req - 1;
+    int lo = 0, hi = p.reqs.n - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (tbl[mid].item_begin[kMatch] <= item) lo = mid; else hi = mid - 1;
@@ -168,13 +168,13 @@ match_kernel(const __grid_constant__ CUtensorMap map_b, const TileParams p) {
         sh.abort_flag = 0;
         ptx::fence_mbar_init();
     }
+    if (p.reqs.n == 1 && threadIdx.x < sizeof(Req) / 4)          // a single request came with the launch
+        reinterpret_cast<int*>(sh.reqs)[threadIdx.x] = reinterpret_cast<const int*>(&p.reqs.only)[threadIdx.x];
     grid_dependency_wait();
-    const Req* tbl = p.reqs;
-    if (p.n_req <= kReqCache) {                  // the table is read once per item by every role
-        for (int i = threadIdx.x; i < p.n_req * (int)(sizeof(Req) / 4); i += kMatchThreads)
-            reinterpret_cast<int*>(sh.reqs)[i] = reinterpret_cast<const int*>(p.reqs)[i];
-        tbl = sh.reqs;
-    }
+    const Req* tbl = p.reqs.n <= kReqCache ? sh.reqs : p.reqs.rows;      // the table is read once per item by every role
+    if (p.reqs.n > 1 && p.reqs.n <= kReqCache)
+        for (int i = threadIdx.x; i < p.reqs.n * (int)(sizeof(Req) / 4); i += kMatchThreads)
+            reinterpret_cast<int*>(sh.reqs)[i] = reinterpret_cast<const int*>(p.reqs.rows)[i];
     if (warp == 0) {
         ptx::tmem_alloc(ptx::smem_u32(&sh.tmem_base), 512);
         ptx::tmem_relinquish();

@@ -35,13 +35,14 @@ __device__ __forceinline__ uint4 pack8(const Row8& r) {
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-__device__ __forceinline__ const Req& find_req_by_slot(const Req* reqs, int n_req, long long g) {
-    int lo = 0, hi = n_req - 1;
+__device__ __forceinline__ Req find_req_by_slot(const ReqTable& reqs, long long g) {
+    if (reqs.n == 1) return reqs.only;
+    int lo = 0, hi = reqs.n - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if ((long long)reqs[mid].slot_begin <= g) lo = mid; else hi = mid - 1;
+        if ((long long)reqs.rows[mid].slot_begin <= g) lo = mid; else hi = mid - 1;
     }
-    return reqs[lo];
+    return reqs.rows[lo];
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -75,7 +76,7 @@ key_norms_kernel(const __nv_bfloat16* __restrict__ k, long long stride_tok, long
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
 gather_kept_kernel(const __nv_bfloat16* __restrict__ k, long long stride_tok, long long stride_head,
-                   const Req* __restrict__ reqs, int n_req, int n_kv_heads, long long T,
+                   const __grid_constant__ ReqTable reqs, int n_kv_heads, long long T,
                    long long total_rows, const int* __restrict__ kept_idx,
                    const float* __restrict__ rnorm_all, __nv_bfloat16* __restrict__ kept_keys,
                    float* __restrict__ rnorm_kept, int* status) {
@@ -83,11 +84,11 @@ gather_kept_kernel(const __nv_bfloat16* __restrict__ k, long long stride_tok, lo
     const int half = threadIdx.x >> 4, l16 = threadIdx.x & 15;
     const long long g = (long long)blockIdx.x * 16 + half;
     if (g >= total_rows) return;
-    const Req& rq = find_req_by_slot(reqs, n_req, g);
+    const Req rq = find_req_by_slot(reqs, g);
     if (rq.mode == LOOKM_MERGE_NONE) return;             // nothing is matched against its kept keys
-    const long long u = g - rq.slot_begin;
-    const int h = (int)(u / rq.B), slot = (int)(u % rq.B);
-    const long long dst = rq.kept_off + (long long)h * rq.B + slot;
+    const int u = (int)(g - rq.slot_begin);              // (there are fewer than 2^31 kept rows in all)
+    const int h = u / rq.B;
+    const long long dst = rq.kept_off + u;
     int pos = kept_idx[dst];
     if (pos < 0 || pos >= rq.L) { if (l16 == 0) atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); pos = 0; }
     const long long tok = rq.tok_begin + pos;
@@ -102,7 +103,7 @@ gather_kept_kernel(const __nv_bfloat16* __restrict__ k, long long stride_tok, lo
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
 compact_kept_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
-                    long long stride_tok, long long stride_head, const Req* __restrict__ reqs, int n_req,
+                    long long stride_tok, long long stride_head, const __grid_constant__ ReqTable reqs,
                     int n_kv_heads, long long total_rows, const int* __restrict__ kept_idx,
                     int varlen_output, long long out_stride_head, __nv_bfloat16* __restrict__ out_k,
                     __nv_bfloat16* __restrict__ out_v, int* status) {
@@ -110,7 +111,7 @@ compact_kept_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __
     const int lane = threadIdx.x & 31, l16 = lane & 15;
     const long long g = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (g >= total_rows) return;
-    const Req& rq = find_req_by_slot(reqs, n_req, g);
+    const Req rq = find_req_by_slot(reqs, g);
     if (rq.mode != LOOKM_MERGE_NONE) return;
     const long long u = g - rq.slot_begin;
     const int h = (int)(u / rq.B), slot = (int)(u % rq.B);
@@ -128,9 +129,9 @@ compact_kept_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __
 // Row arg-max of given similarity blocks (one warp per evicted row); lowest slot wins ties.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
-argmax_rows_kernel(const float* __restrict__ sim_matrix, const Req* __restrict__ reqs,
+argmax_rows_kernel(const float* __restrict__ sim_matrix, const __grid_constant__ ReqTable reqs,
                    int n_kv_heads, int* __restrict__ assign, float* __restrict__ sim) {
-    const Req rq = reqs[blockIdx.z];
+    const Req rq = reqs.get(blockIdx.z);
     const int h = blockIdx.y;
     const int e = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -214,7 +215,7 @@ template <typename CountT, int kMaxBits>
 __global__ void __launch_bounds__(kInvThreads, 2)
 invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__ kept_idx,
                          const int* __restrict__ evict_idx,
-                         const float* __restrict__ sim, const Req* __restrict__ reqs,
+                         const float* __restrict__ sim, const __grid_constant__ ReqTable reqs,
                          int n_kv_heads, int ctas, long long T, int* row_begin,
                          int2* __restrict__ entries,
                          int4* __restrict__ unit_first, int* __restrict__ slot_cnt,
@@ -223,7 +224,7 @@ invert_assignment_kernel(const int* __restrict__ assign, const int* __restrict__
     extern __shared__ __align__(16) unsigned char inv_smem[];
     __shared__ int warp_sums[kInvWarps];
     grid_dependency_wait();
-    const Req rq = reqs[blockIdx.y];
+    const Req rq = reqs.get(blockIdx.y);
     if (rq.mode == LOOKM_MERGE_NONE) return;             // its kept rows are copied, nothing is merged
     const int h = blockIdx.x / ctas, cta = blockIdx.x % ctas;     // the cluster: the CTAs of one head
     const int E = rq.E, B = rq.B;
@@ -448,7 +449,7 @@ __device__ __forceinline__ int bytes_sum(const uint4& v, const uint4& m) {
 
 __global__ void __launch_bounds__(kInvThreads, 2)
 invert_counting_kernel(const int* __restrict__ assign, const int* __restrict__ kept_idx, const int* __restrict__ evict_idx,
-                       const float* __restrict__ sim, const Req* __restrict__ reqs, int n_kv_heads, int ctas, int max_slots,
+                       const float* __restrict__ sim, const __grid_constant__ ReqTable reqs, int n_kv_heads, int ctas, int max_slots,
                        long long T, int2* __restrict__ entries,
                        int4* __restrict__ unit_first, int* __restrict__ slot_cnt, int* status) {
     extern __shared__ __align__(16) unsigned char inv_smem[];
@@ -459,7 +460,7 @@ invert_counting_kernel(const int* __restrict__ assign, const int* __restrict__ k
     int* off = reinterpret_cast<int*>(inv_smem + (size_t)max_slots * 16);             // [slot]
     unsigned short* tot = reinterpret_cast<unsigned short*>(off + max_slots);         // [slot]
     grid_dependency_wait();
-    const Req rq = reqs[blockIdx.y];
+    const Req rq = reqs.get(blockIdx.y);
     if (rq.mode == LOOKM_MERGE_NONE) return;             // its kept rows are copied, nothing is merged
     const int h = blockIdx.x / ctas, cta = blockIdx.x % ctas;     // the cluster: the CTAs of one head
     const int E = rq.E, B = rq.B;
@@ -641,20 +642,21 @@ struct MergeShared {
     alignas(128) uint8_t rows[kMergeWarps][kRing][kChunk][2 * kRowBytes];   // [warp][buffer][entry][K|V]
 };
 
-__device__ __forceinline__ const Req& find_req_by_unit(const Req* reqs, int n_req, long long g) {
-    int lo = 0, hi = n_req - 1;
+__device__ __forceinline__ Req find_req_by_unit(const ReqTable& reqs, long long g) {
+    if (reqs.n == 1) return reqs.only;
+    int lo = 0, hi = reqs.n - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if ((long long)reqs[mid].unit_begin <= g) lo = mid; else hi = mid - 1;
+        if ((long long)reqs.rows[mid].unit_begin <= g) lo = mid; else hi = mid - 1;
     }
-    return reqs[lo];
+    return reqs.rows[lo];
 }
 
 __device__ __forceinline__ float4 ld_cg_f4(const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }
 
 __global__ void __launch_bounds__(kMergeWarps * 32)
 merge_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
-             long long stride_tok, long long stride_head, const Req* __restrict__ reqs, int n_req,
+             long long stride_tok, long long stride_head, const __grid_constant__ ReqTable reqs,
              int n_kv_heads, long long T, long long total_units, const int2* __restrict__ entries,
              const int4* __restrict__ unit_first, int* __restrict__ slot_cnt, float* __restrict__ parts,
              int varlen_output, long long out_stride_head, __nv_bfloat16* __restrict__ out_k,
@@ -673,7 +675,7 @@ merge_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
 
     for (long long g = (long long)blockIdx.x * kMergeWarps + warp; g < total_units;
          g += (long long)gridDim.x * kMergeWarps) {
-        const Req& rq = find_req_by_unit(reqs, n_req, g);
+        const Req rq = find_req_by_unit(reqs, g);
         const int L = rq.L, B = rq.B, mode = rq.mode, ue = rq.unit_entries;
         const long long ul = g - rq.unit_begin;
         // heads vary fastest: warps running at the same time then read the same token range of
@@ -886,7 +888,7 @@ template <int kSteps>
 __global__ void __launch_bounds__(kFuseThreads, 2)
 merge_short_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, long long stride_tok,
                    long long stride_head, const int* __restrict__ assign, const int* __restrict__ kept_idx,
-                   const int* __restrict__ evict_idx, const float* __restrict__ sim, const Req* __restrict__ reqs,
+                   const int* __restrict__ evict_idx, const float* __restrict__ sim, const __grid_constant__ ReqTable reqs,
                    int n_kv_heads, int max_slots, int varlen_output, long long out_stride_head,
                    __nv_bfloat16* __restrict__ out_k, __nv_bfloat16* __restrict__ out_v, int* status) {
     extern __shared__ __align__(16) unsigned char fuse_raw[];
@@ -897,7 +899,7 @@ merge_short_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __r
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
     grid_dependency_wait();
-    const Req rq = reqs[blockIdx.z];
+    const Req rq = reqs.get(blockIdx.z);
     if (rq.mode == LOOKM_MERGE_NONE) return;
     const int h = blockIdx.y;
     const int E = rq.E, B = rq.B, mode = rq.mode;
@@ -923,6 +925,8 @@ merge_short_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __r
             if (mode == LOOKM_MERGE_WEIGHTED) wgt[q] = sim[ev_base + i];
         }
     }
+    // (the kept rows' positions, the first of a thread's, too)
+    const int kept_at = (int)threadIdx.x < n_slots ? kept_idx[kept_base + c0 + threadIdx.x] : 0;
     for (int i = threadIdx.x; i < kFuseWarps * n_slots; i += kFuseThreads) cnt[i] = 0;
     __syncthreads();
     // ---- rank of every token among its warp's tokens of the same slot ----
@@ -988,7 +992,7 @@ merge_short_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __r
     if (threadIdx.x == 0) first[n_slots] = n_ent;
     __syncthreads();
     for (int c = threadIdx.x; c < n_slots; c += kFuseThreads) {
-        int pc = kept_idx[kept_base + c0 + c];
+        int pc = c < kFuseThreads ? kept_at : kept_idx[kept_base + c0 + c];
         if (pc < 0 || pc >= rq.L) { atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); pc = 0; }
         ent[first[c]] = make_int2(pc | (int)0x80000000, c);
     }
@@ -1105,20 +1109,20 @@ cudaError_t launch_key_norms(const void* k, long long stride_tok, long long stri
 }
 
 cudaError_t launch_gather_kept(const void* k, long long stride_tok, long long stride_head,
-                               const Req* reqs, int n_req, int n_kv_heads, long long T,
+                               const ReqTable& reqs, int n_kv_heads, long long T,
                                long long total_kept_rows, const int* kept_idx,
                                const float* rnorm_all, void* kept_keys, float* rnorm_kept,
                                int* status, cudaStream_t stream) {
     if (total_kept_rows <= 0) return cudaSuccess;
     const long long blocks = (total_kept_rows + 15) / 16;
     return launch_chained(gather_kept_kernel, dim3((unsigned)blocks), dim3(256), 0, stream,
-                          (const __nv_bfloat16*)k, stride_tok, stride_head, reqs, n_req, n_kv_heads, T,
+                          (const __nv_bfloat16*)k, stride_tok, stride_head, reqs, n_kv_heads, T,
                           total_kept_rows, kept_idx, rnorm_all, (__nv_bfloat16*)kept_keys, rnorm_kept,
                           status);
 }
 
 cudaError_t launch_invert_assignment(const int* assign, const int* kept_idx, const int* evict_idx,
-                                     const float* sim, const Req* reqs, int n_req, int n_kv_heads, int ctas,
+                                     const float* sim, const ReqTable& reqs, int n_kv_heads, int ctas,
                                      long long T, bool wide_counts, int digit_bits, int* row_begin,
                                      int2* entries, int4* unit_first, int* slot_cnt,
                                      unsigned* sort_a, unsigned* sort_b, int* status,
@@ -1134,13 +1138,13 @@ cudaError_t launch_invert_assignment(const int* assign, const int* kept_idx, con
         return e != cudaSuccess ? e : cudaFuncSetAttribute(wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(4, kInvDigitBits32));
     });
     if (err != cudaSuccess) return err;
-    return launch_chained_clusters(wide_counts ? wide : narrow, dim3((unsigned)(n_kv_heads * ctas), (unsigned)n_req), dim3(kInvThreads),
+    return launch_chained_clusters(wide_counts ? wide : narrow, dim3((unsigned)(n_kv_heads * ctas), (unsigned)reqs.n), dim3(kInvThreads),
                                    (unsigned)ctas, bytes(wide_counts ? 4 : 2, digit_bits), stream, assign, kept_idx, evict_idx, sim,
                                    reqs, n_kv_heads, ctas, T, row_begin, entries, unit_first, slot_cnt, sort_a, sort_b, status);
 }
 
-cudaError_t launch_invert_counting(const int* assign, const int* kept_idx, const int* evict_idx, const float* sim, const Req* reqs,
-                                   int n_req, int n_kv_heads, int ctas, int max_slots, long long T, int2* entries,
+cudaError_t launch_invert_counting(const int* assign, const int* kept_idx, const int* evict_idx, const float* sim, const ReqTable& reqs,
+                                   int n_kv_heads, int ctas, int max_slots, long long T, int2* entries,
                                    int4* unit_first, int* slot_cnt, int* status, cudaStream_t stream) {
     static unsigned long long configured = 0;
     cudaError_t err = once_per_device(configured, [&]() {
@@ -1148,7 +1152,7 @@ cudaError_t launch_invert_counting(const int* assign, const int* kept_idx, const
                                     (kCountMaxSlots + 4 * kInvMaxCluster) * kCountSlotBytes);
     });
     if (err != cudaSuccess) return err;
-    return launch_chained_clusters(invert_counting_kernel, dim3((unsigned)(n_kv_heads * ctas), (unsigned)n_req), dim3(kInvThreads),
+    return launch_chained_clusters(invert_counting_kernel, dim3((unsigned)(n_kv_heads * ctas), (unsigned)reqs.n), dim3(kInvThreads),
                                    (unsigned)ctas, (size_t)max_slots * kCountSlotBytes, stream, assign, kept_idx, evict_idx, sim,
                                    reqs, n_kv_heads, ctas, max_slots, T, entries, unit_first, slot_cnt, status);
 }
@@ -1156,7 +1160,7 @@ cudaError_t launch_invert_counting(const int* assign, const int* kept_idx, const
 int merge_warps_per_sm() { return kMergeWarps; }
 
 cudaError_t launch_merge(const void* k, const void* v, long long stride_tok, long long stride_head,
-                         const Req* reqs, int n_req, int n_kv_heads, long long T,
+                         const ReqTable& reqs, int n_kv_heads, long long T,
                          long long total_units, const int2* entries,
                          const int4* unit_first, int* slot_cnt, float* parts,
                          int varlen_output, long long out_stride_head, void* out_k, void* out_v,
@@ -1173,16 +1177,16 @@ cudaError_t launch_merge(const void* k, const void* v, long long stride_tok, lon
     if (blocks > num_sms) blocks = num_sms;              // persistent: one CTA per SM
     return launch_chained(merge_kernel, dim3((unsigned)blocks), dim3(kMergeWarps * 32), (size_t)smem, stream,
                           (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, stride_tok, stride_head, reqs,
-                          n_req, n_kv_heads, T, total_units, entries, unit_first, slot_cnt,
+                          n_kv_heads, T, total_units, entries, unit_first, slot_cnt,
                           parts, varlen_output, out_stride_head, (__nv_bfloat16*)out_k, (__nv_bfloat16*)out_v);
 }
 
 // Parts per (request, head): about two CTAs per SM, at least eight slots each.
 cudaError_t launch_merge_short(const void* k, const void* v, long long stride_tok, long long stride_head, const int* assign,
-                               const int* kept_idx, const int* evict_idx, const float* sim, const Req* reqs, int n_req,
+                               const int* kept_idx, const int* evict_idx, const float* sim, const ReqTable& reqs,
                                int n_kv_heads, int max_L, int max_E, int max_B, int varlen_output, long long out_stride_head,
                                void* out_k, void* out_v, int* status, int num_sms, cudaStream_t stream) {
-    const long long heads = (long long)n_kv_heads * n_req;
+    const long long heads = (long long)n_kv_heads * reqs.n;
     long long parts = 2ll * num_sms / heads;             // one wave: two CTAs fit on an SM
     if (parts < 1) parts = 1;
     if (parts > (max_B + 7) / 8) parts = (max_B + 7) / 8;
@@ -1197,14 +1201,14 @@ cudaError_t launch_merge_short(const void* k, const void* v, long long stride_to
     });
     if (err != cudaSuccess) return err;
     auto kernel = max_E <= 2 * kFuseThreads ? merge_short_kernel<2> : merge_short_kernel<8>;
-    return launch_chained(kernel, dim3((unsigned)parts, (unsigned)n_kv_heads, (unsigned)n_req), dim3(kFuseThreads), smem, stream,
+    return launch_chained(kernel, dim3((unsigned)parts, (unsigned)n_kv_heads, (unsigned)reqs.n), dim3(kFuseThreads), smem, stream,
                           (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, stride_tok, stride_head, assign, kept_idx, evict_idx,
                           sim, reqs, n_kv_heads, max_slots, varlen_output, out_stride_head, (__nv_bfloat16*)out_k,
                           (__nv_bfloat16*)out_v, status);
 }
 
 cudaError_t launch_compact_kept(const void* k, const void* v, long long stride_tok,
-                                long long stride_head, const Req* reqs, int n_req, int n_kv_heads,
+                                long long stride_head, const ReqTable& reqs, int n_kv_heads,
                                 long long total_kept_rows, const int* kept_idx, int varlen_output,
                                 long long out_stride_head, void* out_k, void* out_v, int* status,
                                 cudaStream_t stream) {
@@ -1212,15 +1216,15 @@ cudaError_t launch_compact_kept(const void* k, const void* v, long long stride_t
     const long long blocks = (total_kept_rows + 7) / 8;
     return launch_chained(compact_kept_kernel, dim3((unsigned)blocks), dim3(256), 0, stream,
                           (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, stride_tok, stride_head, reqs,
-                          n_req, n_kv_heads, total_kept_rows, kept_idx, varlen_output, out_stride_head,
+                          n_kv_heads, total_kept_rows, kept_idx, varlen_output, out_stride_head,
                           (__nv_bfloat16*)out_k, (__nv_bfloat16*)out_v, status);
 }
 
-cudaError_t launch_argmax_rows(const float* sim_matrix, const Req* reqs, int n_req,
+cudaError_t launch_argmax_rows(const float* sim_matrix, const ReqTable& reqs,
                                     int n_kv_heads, int max_evicted, int* assign, float* sim,
                                     cudaStream_t stream) {
     if (max_evicted <= 0) return cudaSuccess;
-    dim3 grid((max_evicted + 7) / 8, n_kv_heads, n_req);
+    dim3 grid((max_evicted + 7) / 8, n_kv_heads, reqs.n);
     argmax_rows_kernel<<<grid, 256, 0, stream>>>(sim_matrix, reqs, n_kv_heads, assign, sim);
     return cudaGetLastError();
 }

@@ -130,7 +130,7 @@ constexpr int kParts = 2048;
 template <int kThreads, int kSteps, bool kLong>
 __global__ void __launch_bounds__(kThreads)
 select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask,
-              const Req* __restrict__ reqs, int n_select_blocks, int n_kv_heads, long long T,
+              const __grid_constant__ ReqTable reqs, int n_select_blocks, int n_kv_heads, long long T,
               int* __restrict__ kept_idx, int* __restrict__ evict_idx, int* __restrict__ rank,
               const __nv_bfloat16* __restrict__ keys, long long stride_tok, long long stride_head,
               float* __restrict__ rnorm_all) {
@@ -147,7 +147,7 @@ select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask
         return;
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const Req rq = reqs[blockIdx.x / n_kv_heads];
+    const Req rq = reqs.get(blockIdx.x / n_kv_heads);
     const int h = blockIdx.x % n_kv_heads;
     const float* s = scores + (long long)h * T + rq.tok_begin;
     const uint8_t* msk = mask ? mask + rq.tok_begin : nullptr;
@@ -345,17 +345,17 @@ select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask
 
 }  // namespace
 
-cudaError_t launch_select(const float* scores, const uint8_t* mask, const Req* reqs, int n_req,
+cudaError_t launch_select(const float* scores, const uint8_t* mask, const ReqTable& reqs,
                           int n_kv_heads, long long T, int max_L, int* kept_idx, int* evict_idx, int* rank,
                           const void* k_for_norms, long long stride_tok, long long stride_head,
                           float* rnorm_all, int num_sms, cudaStream_t stream) {
-    const int n_select = n_kv_heads * n_req;
+    const int n_select = n_kv_heads * reqs.n;
     // Cheaper barriers with fewer threads, a shorter chain of steps with more: a layer of 2048 tokens x 8
     // heads takes 67.0 us with 256 threads, 64.9 with 512 and 65.8 with 1024, 2048 x 32 123, 119.5 and
     // 119.5, 3000 x 8 85.1 with 512 and 84.2 with 1024.  Registers hold up to 32768 tokens, in variants of 8, 16 and
     // 32 per thread (the last spills: 16384 tokens x 8 heads 32.8 us with 32, 21.3 with 16); beyond, sixteen are
     // held and the rest is read again (65536 tokens x 8 heads 88 us; bisected with 32 held 179).
-    typedef void (*Kernel)(const float*, const uint8_t*, const Req*, int, int, long long, int*, int*, int*, const __nv_bfloat16*,
+    typedef void (*Kernel)(const float*, const uint8_t*, ReqTable, int, int, long long, int*, int*, int*, const __nv_bfloat16*,
                            long long, long long, float*);
     struct Variant { int threads, most; Kernel kernel; };
     static const Variant variants[] = {{512, 512 * 4, select_kernel<512, 8, false>}, {1024, 1024 * 8, select_kernel<1024, 8, false>},

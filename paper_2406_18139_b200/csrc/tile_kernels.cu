@@ -236,7 +236,7 @@ struct Item {
 
 template <int KIND, bool kSplits>
 __device__ __forceinline__ Item decode_item(const TileParams& p, const Req* tbl, int item) {
-    int lo = 0, hi = p.n_req - 1;
+    int lo = 0, hi = p.reqs.n - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (tbl[mid].item_begin[KIND] <= item) lo = mid; else hi = mid - 1;
@@ -320,13 +320,15 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     }
     // everything above touches only this CTA's shared memory; from here on global memory written
     // by the kernel before this one is read
+    if (p.reqs.n == 1 && threadIdx.x < sizeof(Req) / 4)          // a single request came with the launch
+        reinterpret_cast<int*>(sh.reqs)[threadIdx.x] = reinterpret_cast<const int*>(&p.reqs.only)[threadIdx.x];
     grid_dependency_wait();
-    const Req* tbl = p.reqs;
-    if (p.n_req <= kReqCache) {                  // the table is read once per item by every role
-        for (int i = threadIdx.x; i < p.n_req * (int)(sizeof(Req) / 4); i += kThreads)
-            reinterpret_cast<int*>(sh.reqs)[i] = reinterpret_cast<const int*>(p.reqs)[i];
-        tbl = sh.reqs;
-    }
+    const Req* tbl = p.reqs.n <= kReqCache ? sh.reqs : p.reqs.rows;      // the table is read once per item by every role
+    if (p.reqs.n > 1 && p.reqs.n <= kReqCache)
+        for (int i = threadIdx.x; i < p.reqs.n * (int)(sizeof(Req) / 4); i += kThreads)
+            reinterpret_cast<int*>(sh.reqs)[i] = reinterpret_cast<const int*>(p.reqs.rows)[i];
+    if (KIND == kSweep1 && !kSplits)             // no table writer went before
+        for (int i = blockIdx.x * kThreads + threadIdx.x; i < p.n_clear; i += gridDim.x * kThreads) p.status[i] = 0;
     if (warp == 0) {
         ptx::tmem_alloc(ptx::smem_u32(&sh.tmem_base), 512);
         ptx::tmem_relinquish();
@@ -718,7 +720,7 @@ __device__ __forceinline__ MultiItem decode_multi(const TileParams& p, const Req
     const int heads = p.n_q_heads;
     int r, set;
     if (item < p.tail_begin) {
-        int lo = 0, hi = p.n_req - 1;
+        int lo = 0, hi = p.reqs.n - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
             if (tbl[mid].item_begin[KIND] <= item) lo = mid; else hi = mid - 1;
@@ -727,8 +729,8 @@ __device__ __forceinline__ MultiItem decode_multi(const TileParams& p, const Req
         set = (item - tbl[r].item_begin[KIND]) / heads;
     } else {
         const int v = (item - p.tail_begin) / heads;                          // [set][request]
-        r = v % p.n_req;
-        set = (tbl[r].nblk + kBlocks - 1) / kBlocks - p.tail_sets + v / p.n_req;
+        r = v % p.reqs.n;
+        set = (tbl[r].nblk + kBlocks - 1) / kBlocks - p.tail_sets + v / p.reqs.n;
     }
     const Req& rq = tbl[r];
     const int n_sets = (rq.nblk + kBlocks - 1) / kBlocks;
@@ -784,13 +786,13 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         ptx::fence_mbar_init();
     }
     if (KIND == kSweep2 && threadIdx.x < kTile) write_ones_row(sh.ax, threadIdx.x);
+    if (p.reqs.n == 1 && threadIdx.x < sizeof(Req) / 4)          // a single request came with the launch
+        reinterpret_cast<int*>(sh.reqs)[threadIdx.x] = reinterpret_cast<const int*>(&p.reqs.only)[threadIdx.x];
     grid_dependency_wait();
-    const Req* tbl = p.reqs;
-    if (p.n_req <= kReqCache) {
-        for (int i = threadIdx.x; i < p.n_req * (int)(sizeof(Req) / 4); i += kThreads)
-            reinterpret_cast<int*>(sh.reqs)[i] = reinterpret_cast<const int*>(p.reqs)[i];
-        tbl = sh.reqs;
-    }
+    const Req* tbl = p.reqs.n <= kReqCache ? sh.reqs : p.reqs.rows;      // the table is read once per item by every role
+    if (p.reqs.n > 1 && p.reqs.n <= kReqCache)
+        for (int i = threadIdx.x; i < p.reqs.n * (int)(sizeof(Req) / 4); i += kThreads)
+            reinterpret_cast<int*>(sh.reqs)[i] = reinterpret_cast<const int*>(p.reqs.rows)[i];
     if (warp == 0) {
         ptx::tmem_alloc(ptx::smem_u32(&sh.tmem_base), 512);
         ptx::tmem_relinquish();
