@@ -362,18 +362,19 @@ int make_map_2d(CUtensorMap* map, const void* base, long long rows) {
         if (st_ != LOOKM_OK) return st_;  \
     } while (0)
 
-// A call of one prompt that begins with sweep 1 of whole single blocks needs no table writer: its launches
-// carry the request, and that sweep clears the words that later ones count in.
-bool sweep_clears(const Plan& pl) { return pl.n_req == 1 && pl.blocks == 1 && pl.splits[0] == 1; }
+// A whole-path call of one prompt in single blocks needs no table writer: its launches carry the request, and the
+// first of them (sweep 1, or the one that takes its place) clears the words that later ones count in.
+// (Eviction alone keeps it: its number of launches is pinned.)
+bool first_launch_clears(const Plan& pl) { return pl.n_req == 1 && pl.blocks == 1 && pl.splits[0] == 1 && pl.n_none == 0; }
 
 template <class T>
 T* at(void* ws, size_t off) { return reinterpret_cast<T*>(static_cast<char*>(ws) + off); }
 
 // Clears the status word and the arrival counters and writes the request table into the workspace (unless the
-// call's sweep 1 does what is needed of that: see sweep_clears).
-int begin_call(const Plan& pl, void* ws, cudaStream_t st, bool with_sweep1 = false) {
+// call's first launch does what is needed of that).
+int begin_call(const Plan& pl, void* ws, cudaStream_t st, bool first_clears = false) {
     g_launches = 0;
-    if (with_sweep1 && sweep_clears(pl)) return LOOKM_OK;
+    if (first_clears) return LOOKM_OK;
     for (int base = 0; base < pl.n_req; base += kReqChunk) {
         ReqChunk chunk;
         const int cnt = std::min(kReqChunk, pl.n_req - base);
@@ -416,7 +417,7 @@ TileParams tile_params(const Plan& pl, void* ws, const lookm_layout* lay) {
 }
 
 int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, const void* q,
-              const void* k, float* scores, float* lse, bool lse_is_input, void* ws, cudaStream_t st) {
+              const void* k, float* scores, float* lse, bool lse_is_input, bool clears, void* ws, cudaStream_t st) {
     CUtensorMap map_q, map_k;
     LOOKM_TRY(make_map_3d(&map_q, q, pl.T, pl.n_q_heads, lay->q_stride_tok, lay->q_stride_head));
     LOOKM_TRY(make_map_3d(&map_k, k, pl.T, pl.n_kv_heads, lay->kv_stride_tok, lay->kv_stride_head));
@@ -429,7 +430,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     p.scores = scores;
     if (!lse_is_input) {
         p.n_items = pl.n_items[kSweep1];
-        p.n_clear = sweep_clears(pl) ? (int)pl.clear_words : 0;
+        p.n_clear = clears ? (int)pl.clear_words : 0;
         p.next_item = p.status + 16 + kSweep1;
         p.splits = pl.splits[0];
         p.parts1 = at<float2>(ws, pl.o_kept_keys);
@@ -437,7 +438,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
         LOOKM_CUDA(launch_tile_kernel(kSweep1, map_q, map_k, nullptr, p, di.sms, st));
         ++g_launches;
     } else {
-        LOOKM_CUDA(launch_lse_split(lse, pl.n_q_heads, pl.T, p.scale_log2, split, st));
+        LOOKM_CUDA(launch_lse_split(lse, pl.n_q_heads, pl.T, p.scale_log2, split, p.status, clears ? (int)pl.clear_words : 0, st));
         ++g_launches;
     }
     mark_stage(1, st);
@@ -615,7 +616,8 @@ int compress_common(const void* q, const void* k, const void* v, const uint8_t* 
         out_cu[0] = 0;
         for (int r = 0; r < n_req; ++r) out_cu[r + 1] = out_cu[r] + pl.out_len[r];
     }
-    LOOKM_TRY(begin_call(pl, ws, st, !lse_in));
+    const bool clears = first_launch_clears(pl);
+    LOOKM_TRY(begin_call(pl, ws, st, clears));
     mark_stage(0, st);
     float* scores = at<float>(ws, pl.o_scores);
     int* kept = at<int>(ws, pl.o_kept);
@@ -625,7 +627,7 @@ int compress_common(const void* q, const void* k, const void* v, const uint8_t* 
     float* sim = at<float>(ws, pl.o_sim);
     // a caller's log-sum-exp (read only) replaces the first sweep
     float* lse = lse_in ? const_cast<float*>(lse_in) : at<float>(ws, pl.o_lse);
-    LOOKM_TRY(run_score(pl, di, lay, q, k, scores, lse, lse_in != nullptr, ws, st));
+    LOOKM_TRY(run_score(pl, di, lay, q, k, scores, lse, lse_in != nullptr, clears, ws, st));
     // the selection launch also computes the key norms that the matching needs
     const bool need_match = pl.n_items[kMatch] > 0;
     LOOKM_CUDA(launch_select(scores, text_prior ? mask : nullptr, req_table(pl, ws),
@@ -730,9 +732,10 @@ int lookm_score(const void* q, const void* k, const int* cu_seqlens_host, int n_
     DeviceInfo di;
     LOOKM_TRY(device_info(di));
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    LOOKM_TRY(begin_call(pl, workspace, st, !lse_is_input));
+    const bool clears = !lse_is_input && first_launch_clears(pl);
+    LOOKM_TRY(begin_call(pl, workspace, st, clears));
     float* lse_buf = lse ? lse : at<float>(workspace, pl.o_lse);
-    return run_score(pl, di, layout, q, k, scores, lse_buf, lse_is_input != 0, workspace, st);
+    return run_score(pl, di, layout, q, k, scores, lse_buf, lse_is_input != 0, clears, workspace, st);
 }
 
 int lookm_select(const float* scores, const uint8_t* modality_mask, const int* cu_seqlens_host,

@@ -119,9 +119,9 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
 // Matching of the evicted rows with the compacted kept keys (match_kernel.cu).
 cudaError_t launch_match(const CUtensorMap& map_kept, const TileParams& p, int num_sms, cudaStream_t stream);
 
-// lse_split from a given lse (for callers that supply their own log-sum-exp)
+// lse_split from a given lse (for callers that supply their own log-sum-exp); clears n_clear words
 cudaError_t launch_lse_split(const float* lse, int n_q_heads, long long T, float scale_log2,
-                             unsigned short* lse_split, cudaStream_t stream);
+                             unsigned short* lse_split, int* clear, int n_clear, cudaStream_t stream);
 
 // One CTA that waits, with the tile kernels' own bounded wait and the given limit, on an mbarrier
 // nobody arrives at; on expiry it writes LOOKM_ERR_DEVICE_TIMEOUT to *status like they do.

@@ -210,8 +210,9 @@ __device__ __forceinline__ void store_lse_split(unsigned short* row16, float lse
 }
 
 __global__ void lse_split_kernel(const float* __restrict__ lse, int n_q_heads, long long T,
-                                 float scale_log2, unsigned short* __restrict__ lse_split) {
+                                 float scale_log2, unsigned short* __restrict__ lse_split, int* clear, int n_clear) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // over [head][token]
+    for (long long j = i; j < n_clear; j += (long long)gridDim.x * blockDim.x) clear[j] = 0;
     if (i >= T * n_q_heads) return;
     const long long h = i / T, tok = i % T;
     store_lse_split(lse_split + (tok * n_q_heads + h) * 16, lse[i], scale_log2);
@@ -1094,10 +1095,10 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
 }
 
 cudaError_t launch_lse_split(const float* lse, int n_q_heads, long long T, float scale_log2,
-                             unsigned short* lse_split, cudaStream_t stream) {
+                             unsigned short* lse_split, int* clear, int n_clear, cudaStream_t stream) {
     const long long n = T * n_q_heads;
     if (n <= 0) return cudaSuccess;
-    lse_split_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(lse, n_q_heads, T, scale_log2, lse_split);
+    lse_split_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(lse, n_q_heads, T, scale_log2, lse_split, clear, n_clear);
     return cudaGetLastError();
 }
 
