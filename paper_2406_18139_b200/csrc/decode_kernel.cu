@@ -926,22 +926,26 @@ struct Kernels {
 cudaError_t configure_decode() {
     static unsigned long long configured = 0;
     return once_per_device(configured, []() {
-        const cudaError_t e = Kernels<DecodeBatch>::configure();
-        return e != cudaSuccess ? e : Kernels<DecodeBatchOf<1>>::configure();
+        cudaError_t e = Kernels<DecodeBatch>::configure();
+        if (e == cudaSuccess) e = Kernels<DecodeBatchOf<1>>::configure();
+        return e != cudaSuccess ? e : Kernels<DecodeBatchOf<kDecodeFew>>::configure();
     });
 }
 
-// f(batch), with the smaller argument where there is one request
+// f(batch), in the smallest argument that holds its requests
+template <int kRequests, class F>
+cudaError_t with_copy(const DecodeBatch& batch, F f) {
+    DecodeBatchOf<kRequests> few;
+    few.n_req = batch.n_req;
+    few.share = batch.share;
+    few.longer = batch.longer;
+    few.pad = 0;
+    for (int i = 0; i < kRequests; ++i) few.r[i] = batch.r[i];          // (those past the last are zeros)
+    return f(few);
+}
 template <class F>
 cudaError_t with_batch(const DecodeBatch& batch, F f) {
-    if (batch.n_req != 1) return f(batch);
-    DecodeBatchOf<1> one;
-    one.n_req = 1;
-    one.share = batch.share;
-    one.longer = batch.longer;
-    one.pad = 0;
-    one.r[0] = batch.r[0];
-    return f(one);
+    return batch.n_req == 1 ? with_copy<1>(batch, f) : batch.n_req <= kDecodeFew ? with_copy<kDecodeFew>(batch, f) : f(batch);
 }
 
 }  // namespace

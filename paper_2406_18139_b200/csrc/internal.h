@@ -201,7 +201,9 @@ struct DecodeReq {
     };
 };
 // What a launch gets by value: one request takes 56 bytes, any number up to kDecodeChunk 3.9 KB, which costs
-// 0.45 us more to launch (409 rows x 32 heads, calls in a row from Python: 6.1 | 5.65 us).
+// 0.45 us more to launch (409 rows x 32 heads, calls in a row from Python: 6.1 | 5.65 us); up to sixteen take 656
+// bytes.
+constexpr int kDecodeFew = 16;
 constexpr int kDecodeChunk = 96;
 template <int kRequests>
 struct DecodeBatchOf {

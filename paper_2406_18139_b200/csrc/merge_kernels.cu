@@ -925,8 +925,6 @@ merge_short_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __r
             if (mode == LOOKM_MERGE_WEIGHTED) wgt[q] = sim[ev_base + i];
         }
     }
-    // (the kept rows' positions, the first of a thread's, too)
-    const int kept_at = (int)threadIdx.x < n_slots ? kept_idx[kept_base + c0 + threadIdx.x] : 0;
     for (int i = threadIdx.x; i < kFuseWarps * n_slots; i += kFuseThreads) cnt[i] = 0;
     __syncthreads();
     // ---- rank of every token among its warp's tokens of the same slot ----
@@ -992,7 +990,7 @@ merge_short_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __r
     if (threadIdx.x == 0) first[n_slots] = n_ent;
     __syncthreads();
     for (int c = threadIdx.x; c < n_slots; c += kFuseThreads) {
-        int pc = c < kFuseThreads ? kept_at : kept_idx[kept_base + c0 + c];
+        int pc = kept_idx[kept_base + c0 + c];
         if (pc < 0 || pc >= rq.L) { atomicExch(status, (int)LOOKM_ERR_DEVICE_BAD_INDEX); pc = 0; }
         ent[first[c]] = make_int2(pc | (int)0x80000000, c);
     }

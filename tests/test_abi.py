@@ -4,6 +4,9 @@ import ctypes as C
 import os
 import re
 
+import numpy as np
+import pytest
+
 from paper_2406_18139_b200 import binding as B, build
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -155,3 +158,12 @@ def test_the_binding_loads_the_in_tree_library_only():
     B.lib()
     mapped = [l.split()[-1] for l in open("/proc/self/maps") if "liblookm" in l]
     assert mapped and all(os.path.samefile(m, here) for m in mapped)
+
+
+@pytest.mark.parametrize("seq", [[3, 1, 2], (5,), range(4), np.array([7, 8], dtype=np.int64), [np.int32(4), True], [2.0, 3.7], ["6"],
+                                 [2 ** 31], bytes([1, 2]), []])
+def test_binding_passes_host_integers_as_it_always_did(seq):
+    """Every sequence whose elements int() takes, with ctypes' own wrap-around beyond 32 bits."""
+    expected = [int(x) for x in seq]
+    for got, ctype in ((B._ints(seq), C.c_int), (B._c_array(C.c_longlong, "q", seq), C.c_longlong)):
+        assert list(got) == list((ctype * len(expected))(*expected)) and got._type_ is ctype
