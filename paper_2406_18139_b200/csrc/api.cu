@@ -363,7 +363,8 @@ int make_map_2d(CUtensorMap* map, const void* base, long long rows) {
     } while (0)
 
 // A whole-path call of one prompt in single blocks needs no table writer: its launches carry the request, and the
-// first of them (sweep 1, or the one that takes its place) clears the words that later ones count in.
+// first of them (sweep 1, or the one that takes its place) clears the words that later ones count in and writes the
+// request to its row, for the launch that reads it there.
 // (Eviction alone keeps it: its number of launches is pinned.)
 bool first_launch_clears(const Plan& pl) { return pl.n_req == 1 && pl.blocks == 1 && pl.splits[0] == 1 && pl.n_none == 0; }
 
@@ -438,7 +439,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
         LOOKM_CUDA(launch_tile_kernel(kSweep1, map_q, map_k, nullptr, p, di.sms, st));
         ++g_launches;
     } else {
-        LOOKM_CUDA(launch_lse_split(lse, pl.n_q_heads, pl.T, p.scale_log2, split, p.status, clears ? (int)pl.clear_words : 0, st));
+        LOOKM_CUDA(launch_lse_split(lse, pl.n_q_heads, pl.T, p.scale_log2, split, p.reqs, p.status, clears ? (int)pl.clear_words : 0, st));
         ++g_launches;
     }
     mark_stage(1, st);

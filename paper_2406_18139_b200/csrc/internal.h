@@ -67,7 +67,7 @@ struct Req {
 // it from the table in the workspace would be the first of the dependent loads that a short prompt's kernels
 // consist of.
 struct ReqTable {
-    const Req* rows;      // in the workspace; not written where `only` is all that the launches need
+    const Req* rows;      // in the workspace
     int n;
     Req only;             // n == 1
 #ifdef __CUDACC__
@@ -107,7 +107,8 @@ struct TileParams {
     int* assign;                 // evicted-list layout  (match)
     float* sim;                  // evicted-list layout  (match)
     int* status;                 // device status word
-    int n_clear;                 // words from the status word on that sweep 1 has to clear
+    int n_clear;                 // words from the status word on that sweep 1 has to clear; if any, it also writes the
+                                 // single request to its row
 };
 
 // ---- launchers (each enqueues on `stream` and returns the CUDA error of the launch) -----------
@@ -119,9 +120,10 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
 // Matching of the evicted rows with the compacted kept keys (match_kernel.cu).
 cudaError_t launch_match(const CUtensorMap& map_kept, const TileParams& p, int num_sms, cudaStream_t stream);
 
-// lse_split from a given lse (for callers that supply their own log-sum-exp); clears n_clear words
+// lse_split from a given lse (for callers that supply their own log-sum-exp); clears n_clear words from `clear` on and,
+// if there are any, writes the single request to its row
 cudaError_t launch_lse_split(const float* lse, int n_q_heads, long long T, float scale_log2,
-                             unsigned short* lse_split, int* clear, int n_clear, cudaStream_t stream);
+                             unsigned short* lse_split, const ReqTable& reqs, int* clear, int n_clear, cudaStream_t stream);
 
 // One CTA that waits, with the tile kernels' own bounded wait and the given limit, on an mbarrier
 // nobody arrives at; on expiry it writes LOOKM_ERR_DEVICE_TIMEOUT to *status like they do.

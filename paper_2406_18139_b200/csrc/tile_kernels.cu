@@ -209,10 +209,18 @@ __device__ __forceinline__ void store_lse_split(unsigned short* row16, float lse
     dst[1] = make_uint4(0u, 0u, 0u, 0u);
 }
 
+// The single request of a call without a table writer, for the launches that read it from the table.
+__device__ __forceinline__ void write_single_request(const ReqTable& reqs) {
+    if (blockIdx.x == 0 && threadIdx.x < sizeof(Req) / 4)
+        reinterpret_cast<int*>(const_cast<Req*>(reqs.rows))[threadIdx.x] = reinterpret_cast<const int*>(&reqs.only)[threadIdx.x];
+}
+
 __global__ void lse_split_kernel(const float* __restrict__ lse, int n_q_heads, long long T,
-                                 float scale_log2, unsigned short* __restrict__ lse_split, int* clear, int n_clear) {
+                                 float scale_log2, unsigned short* __restrict__ lse_split,
+                                 const __grid_constant__ ReqTable reqs, int* clear, int n_clear) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // over [head][token]
     for (long long j = i; j < n_clear; j += (long long)gridDim.x * blockDim.x) clear[j] = 0;
+    if (n_clear > 0) write_single_request(reqs);
     if (i >= T * n_q_heads) return;
     const long long h = i / T, tok = i % T;
     store_lse_split(lse_split + (tok * n_q_heads + h) * 16, lse[i], scale_log2);
@@ -328,8 +336,10 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     if (p.reqs.n > 1 && p.reqs.n <= kReqCache)
         for (int i = threadIdx.x; i < p.reqs.n * (int)(sizeof(Req) / 4); i += kThreads)
             reinterpret_cast<int*>(sh.reqs)[i] = reinterpret_cast<const int*>(p.reqs.rows)[i];
-    if (KIND == kSweep1 && !kSplits)             // no table writer went before
+    if (KIND == kSweep1 && !kSplits && p.n_clear > 0) {          // no table writer went before
         for (int i = blockIdx.x * kThreads + threadIdx.x; i < p.n_clear; i += gridDim.x * kThreads) p.status[i] = 0;
+        write_single_request(p.reqs);
+    }
     if (warp == 0) {
         ptx::tmem_alloc(ptx::smem_u32(&sh.tmem_base), 512);
         ptx::tmem_relinquish();
@@ -734,7 +744,6 @@ __device__ __forceinline__ MultiItem decode_multi(const TileParams& p, const Req
         set = (tbl[r].nblk + kBlocks - 1) / kBlocks - p.tail_sets + v / p.reqs.n;
     }
     const Req& rq = tbl[r];
-    const int n_sets = (rq.nblk + kBlocks - 1) / kBlocks;
     MultiItem it;
     it.tok_begin = rq.tok_begin;
     it.L = rq.L;
@@ -1095,10 +1104,10 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
 }
 
 cudaError_t launch_lse_split(const float* lse, int n_q_heads, long long T, float scale_log2,
-                             unsigned short* lse_split, int* clear, int n_clear, cudaStream_t stream) {
+                             unsigned short* lse_split, const ReqTable& reqs, int* clear, int n_clear, cudaStream_t stream) {
     const long long n = T * n_q_heads;
     if (n <= 0) return cudaSuccess;
-    lse_split_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(lse, n_q_heads, T, scale_log2, lse_split, clear, n_clear);
+    lse_split_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(lse, n_q_heads, T, scale_log2, lse_split, reqs, clear, n_clear);
     return cudaGetLastError();
 }
 
