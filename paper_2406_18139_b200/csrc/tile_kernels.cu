@@ -747,9 +747,13 @@ __device__ __forceinline__ MultiItem decode_multi(const TileParams& p, const Req
     MultiItem it;
     it.tok_begin = rq.tok_begin;
     it.L = rq.L;
-    it.blk = kBlocks * (KIND == kSweep1 ? n_sets - 1 - set : set);
+    // Sets are counted from the request's longest blocks on, so that the one that is not full is the shortest.
+    // (From the first block on, sweep 1's longest item had a single block where their number is odd. Scores: 2900
+    // tokens x 40 heads 130.4 | 127.6 us, 9100 x 32 851 | 844, 12400 x 32 on 8 1482 | 1473, three ragged prompts 548 | 542.)
+    const int rest = rq.nblk - kBlocks * set;                                 // blocks from this set on
+    it.n = min(kBlocks, rest);
+    it.blk = KIND == kSweep1 ? rest - it.n : kBlocks * set;
     it.head = item % heads;          // (the items of a request, and those of the tail, begin at a multiple of it)
-    it.n = min(kBlocks, rq.nblk - it.blk);
     it.tile = rq.tile_begin + it.blk;
     it.nt = KIND == kSweep1 ? it.blk + it.n : rq.nblk - it.blk;
     return it;
