@@ -130,7 +130,7 @@ constexpr int kParts = 2048;
 template <int kThreads, int kSteps, bool kLong>
 __global__ void __launch_bounds__(kThreads)
 select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask,
-              const __grid_constant__ ReqTable reqs, int n_select_blocks, int n_kv_heads, long long T,
+              const Req* __restrict__ reqs, int n_select_blocks, int n_kv_heads, long long T,
               int* __restrict__ kept_idx, int* __restrict__ evict_idx, int* __restrict__ rank,
               const __nv_bfloat16* __restrict__ keys, long long stride_tok, long long stride_head,
               float* __restrict__ rnorm_all) {
@@ -147,7 +147,9 @@ select_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ mask
         return;
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const Req rq = reqs.get(blockIdx.x / n_kv_heads);
+    // (from the table, also of a single prompt: by value 700 tokens x 32 heads 8.7 | 9.5 us, 131072 x 8 187.3 | 189,
+    // a layer of 700 x 32 52.7 either way)
+    const Req rq = reqs[blockIdx.x / n_kv_heads];
     const int h = blockIdx.x % n_kv_heads;
     const float* s = scores + (long long)h * T + rq.tok_begin;
     const uint8_t* msk = mask ? mask + rq.tok_begin : nullptr;
@@ -355,7 +357,7 @@ cudaError_t launch_select(const float* scores, const uint8_t* mask, const ReqTab
     // 119.5, 3000 x 8 85.1 with 512 and 84.2 with 1024.  Registers hold up to 32768 tokens, in variants of 8, 16 and
     // 32 per thread (the last spills: 16384 tokens x 8 heads 32.8 us with 32, 21.3 with 16); beyond, sixteen are
     // held and the rest is read again (65536 tokens x 8 heads 88 us; bisected with 32 held 179).
-    typedef void (*Kernel)(const float*, const uint8_t*, ReqTable, int, int, long long, int*, int*, int*, const __nv_bfloat16*,
+    typedef void (*Kernel)(const float*, const uint8_t*, const Req*, int, int, long long, int*, int*, int*, const __nv_bfloat16*,
                            long long, long long, float*);
     struct Variant { int threads, most; Kernel kernel; };
     static const Variant variants[] = {{512, 512 * 4, select_kernel<512, 8, false>}, {1024, 1024 * 8, select_kernel<1024, 8, false>},
@@ -375,7 +377,7 @@ cudaError_t launch_select(const float* scores, const uint8_t* mask, const ReqTab
         n_norm = (int)std::min<long long>(want, (long long)per_sm * (n_select < num_sms / 2 ? num_sms - n_select : num_sms));
     }
     return launch_chained(use->kernel, dim3(n_select + n_norm), dim3(threads), 0, stream,
-                          scores, mask, reqs, n_select, n_kv_heads, T, kept_idx, evict_idx, rank,
+                          scores, mask, reqs.rows, n_select, n_kv_heads, T, kept_idx, evict_idx, rank,
                           (const __nv_bfloat16*)k_for_norms, stride_tok, stride_head, rnorm_all);
 }
 
