@@ -55,11 +55,14 @@ int device_info(DeviceInfo& out);
 
 // Blocks per sweep item, from the scores of some 370 problems with one, two and four blocks per item (us).
 // Several blocks pay where there are enough items and the items are full.
-//   Two blocks, one prompt: from 6.4 blocks per SM on (3200 tokens x 32 heads, 5.4 per SM, 118 | 120, 2600 x 40, 5.7, 108 |
-// 111, 3500 x 32, 6.1, 148 | 143, but a whole layer of it 221.8 | 223, at a higher clock, of 2800 x 40 189 | 196; 3800 x 32,
-// 6.5, 165.8 | 162.2, 4096 x 32, 6.9, 189 | 184, 5000 x 32, 8.6, 290 | 278, 20000 x 8, 8.5, 991 | 952, 8192 x 32, 13.8, 714 | 672),
-// with grouped heads from five (3000 x 32 on 8, 5.2, 120 | 115).  Two prompts: from nine (layers of 2250 on average x 32, 7.6,
-// 232 | 236).
+//   Two blocks, one prompt whose items stream 13 tiles on average, 16 with grouped heads: from 6.4 blocks per SM on (3200
+// tokens x 32 heads, 5.4 per SM, 118 | 120, 2600 x 40, 5.7, 108 | 111, 3500 x 32, 6.1, 148 | 143, but a whole layer of it 221.8 | 223, at a
+// higher clock, of 2800 x 40 189 | 196; 3800 x 32, 6.5, 165.8 | 162.2, 4096 x 32, 6.9, 189 | 184, 5000 x 32, 8.6, 290 |
+// 278, 20000 x 8, 8.5, 991 | 952, 8192 x 32, 13.8, 714 | 672; grouped heads, layers: 6000 x 16 on 4, 5.1, 244 | 255, 4000 x 24
+// on 6, 5.2, 180 | 183, 3300 x 40 on 10, 13.5 tiles, 7.0, 193 | 199, 3000 x 40 on 8, 12.5, 6.5, 183 | 172, 5000 x 24 on 6, 6.5,
+// 255 | 251, 8000 x 16 on 4, 6.8, 388 | 372, 5000 x 32 on 8, 8.6, 324 | 314).
+// Shorter ones and two prompts: from nine (256 x 512, two tiles, 6.9, 36 | 42, 1000 x 128, five, 6.9, 67 | 70, 1200 x 96 on
+// 48, six, 6.5, 71 | 78; layers of two of 2250 on average x 32, 7.6, 232 | 236).
 //   More prompts, whose single blocks come out uneven from a fixed deal: from five (three of 900 x 32, 5.2, 66 |
 // 58).  The items have to be three quarters full (93 of 128 tokens x 32: one block each, 111 | 135; 31 of 384: two
 // items for three, 124 | 134).  Single blocks take the query heads of a group together in sweep 2, and the fixed
@@ -86,7 +89,7 @@ int sweep_blocks(const Plan& pl, long long sms) {
     shape(2, sets, streamed);
     const long long all = blocks * pl.n_q_heads;
     const int half_tiles = pl.group == 1 ? 0 : all < 7 * sms ? 4 : all < 24 * sms ? 5 : 10;
-    const bool many = 10 * all >= (one ? (pl.group == 1 ? 64 : 50) : pl.n_req == 2 ? 90 : 50) * sms;
+    const bool many = 10 * all >= (one && streamed >= (pl.group == 1 ? 13 : 16) * sets ? 64 : pl.n_req <= 2 ? 90 : 50) * sms;
     return many && 100 * blocks >= 76 * 2 * sets && 2 * streamed >= half_tiles * sets ? 2 : 1;
 }
 // The kTailSets shortest items of all prompts come last: with each prompt's items in a row the last
