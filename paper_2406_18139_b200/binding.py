@@ -115,14 +115,14 @@ def _c_array(ctype, code, seq):
     """`seq` as a C array.  Through array.array, which takes sixteen lengths in 1.0 us where a conversion one by
     one takes 2.6 (a generation step of sixteen short caches is launched in ten); what that does not
     take as integers is converted one by one."""
-    if not isinstance(seq, (bytes, bytearray, str)):
-        try:
-            values = array(code, seq)
-            return (ctype * len(values)).from_buffer(values)
-        except (TypeError, OverflowError, ValueError):
-            pass
-    values = [int(x) for x in seq]
-    return (ctype * len(values))(*values)
+    if not isinstance(seq, (list, tuple)):
+        seq = list(seq)                  # an iterator can be walked once only; bytes are their values here
+    try:
+        values = array(code, seq)
+        return (ctype * len(values)).from_buffer(values)
+    except (TypeError, OverflowError, ValueError):
+        values = [int(x) for x in seq]
+        return (ctype * len(values))(*values)
 
 
 def _ints(seq: Optional[Sequence[int]]):

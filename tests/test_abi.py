@@ -167,3 +167,13 @@ def test_binding_passes_host_integers_as_it_always_did(seq):
     expected = [int(x) for x in seq]
     for got, ctype in ((B._ints(seq), C.c_int), (B._c_array(C.c_longlong, "q", seq), C.c_longlong)):
         assert list(got) == list((ctype * len(expected))(*expected)) and got._type_ is ctype
+
+
+@pytest.mark.parametrize("make", [lambda: map(float, [5, 6, 7]), lambda: (x for x in [2.9, 3.0]), lambda: iter(["6", 7]),
+                                  lambda: (2 ** 31 + x for x in range(3)), lambda: iter([1, 2, 3.5])])
+def test_binding_passes_every_element_of_an_iterator(make):
+    """Also when an element is found not to be an integer of the C type: the library is told the count that the
+    caller's other lists have, and would read past a shorter array."""
+    expected = [int(x) for x in make()]
+    for got, ctype in ((B._ints(make()), C.c_int), (B._c_array(C.c_longlong, "q", make()), C.c_longlong)):
+        assert list(got) == list((ctype * len(expected))(*expected)) and got._type_ is ctype
