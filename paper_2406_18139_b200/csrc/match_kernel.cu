@@ -259,6 +259,7 @@ match_kernel(const __grid_constant__ CUtensorMap map_b, const TileParams p) {
             int free_now = 1;
             if (lane == 0) free_now = ptx::mbar_wait(ptx::smem_u32(&sh.a_empty[ab]), ((n >> 1) & 1) ^ 1, abort_flag) ? 1 : 0;
             if (!__shfl_sync(0xffffffffu, free_now, 0)) break;
+            __syncwarp();                        // the positions are there for all lanes (a shuffle orders no memory)
             ++n;
             const uint32_t adst = ptx::smem_u32(&sh.a[ab][0]) + lane_dst;
             const char* src0 = reinterpret_cast<const char*>(p.k_rows) +

@@ -503,6 +503,27 @@ def test_match_starts_in_the_middle_and_the_lower_slot_wins(B, budget):
             assert a_got[h, len(ev_np) - 2 - 6 * i] == lo
 
 
+@pytest.mark.parametrize("L,budget,Hkv", [(6000, 700, 8), (5000, 100, 16)])
+def test_match_gathers_block_after_block_from_positions_of_its_own(B, L, budget, Hkv):
+    """Every CTA gathers several blocks one after another through the same list of positions, which differ from
+    block to block and from head to head: every evicted row's cosine is that of its own key."""
+    import torch
+    gen = torch.Generator().manual_seed(L)
+    perm = torch.rand(Hkv, L, generator=gen).argsort(1).int()
+    kept, ev = perm[:, :budget].sort(1).values.contiguous().cuda(), perm[:, budget:].sort(1).values.contiguous().cuda()
+    k = torch.randn(L, Hkv, 128, generator=gen).bfloat16().cuda()
+    assign, sim = torch.full_like(ev, -7), torch.full(ev.shape, -7.0, device="cuda")
+    lay = B.make_layout(None, k)
+    ws = B.alloc_workspace(lay, [L])
+    B.check(B.lookm_match(k, kept, ev, [0, L], [budget], lay, assign, sim, ws))
+    assert B.lookm_device_status(ws) == B.OK
+    kn = torch.nn.functional.normalize(k.double(), dim=-1)
+    for h in range(Hkv):
+        S = kn[ev[h].long(), h] @ kn[kept[h].long(), h].t()
+        assert (sim[h].double() - S.max(1).values).abs().max() <= 2e-6
+        assert (S.gather(1, assign[h].long()[:, None])[:, 0] >= S.max(1).values - 1e-4).all()
+
+
 def test_match_of_many_short_prompts_one_kept_tile_each(B):
     """Items of a single tile: three of the four epilogue groups have no tile in an item and may run ahead
     of the one that has; every repetition must give the same bits, and no wait may run out."""
