@@ -205,6 +205,12 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
+// ... which is NaN if any of the three is
+__device__ __forceinline__ float fmax3_nan(float a, float b, float c) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -260,7 +266,8 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
-// ex2_fma of both numbers, without its upper limit: arguments must not exceed 127.
+// ex2_fma of both numbers, without its upper limit: right below 128 (there the exponent field is full when the
+// polynomial's value is below 1); of arguments from 128 on, and of NaN, the result means nothing.
 __device__ __forceinline__ f32x2 ex2_fma2(f32x2 x) {
     const float2 v = unpack2(x);
     x = pack2(fmaxf(v.x, -125.f), fmaxf(v.y, -125.f));

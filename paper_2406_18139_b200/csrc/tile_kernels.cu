@@ -93,8 +93,8 @@ static_assert(sizeof(Shared<kSweep1>) + 1024 <= 232448 && sizeof(Shared<kSweep2>
 
 // The softmax epilogues are bound by the special-function unit (16 ex2 per clock and SM) and by issue
 // slots, so some columns are exponentiated on the FMA pipe instead: on full tiles kPolyPairs of the sixteen pairs
-// of a chunk, two numbers per instruction, with one test of the chunk's largest logit in place of an upper limit on
-// every argument (which took two instructions a pair more).  A two-wide multiply-add takes two issue
+// of a chunk, two numbers per instruction, with one test of the largest logit (of a chunk in sweep 1, of a whole item in
+// sweep 2) in place of an upper limit on every argument (which took two instructions a pair more).  A two-wide multiply-add takes two issue
 // slots, so it is the limit's instructions that are saved.  Scores in us, one column in six one by one | 2, 3, 5, 6 and 7
 // pairs: 8192 tokens x 32 heads 678 | 676, 669, 684, 700, 726; 4096 x 32 191.3 | 189.4, 190.4, 195.9, 202.8, 210.5; three
 // prompts of 1800 to 5000 x 32 on 8 552 | 549, 548, 567, 583, 605.
@@ -146,11 +146,11 @@ __device__ __forceinline__ void sweep1_columns(const uint32_t (&raw)[32], float 
         const float mc = ref * c2;
         const ptx::f32x2 scale = ptx::pack2(c2, c2), shift = ptx::pack2(-mc, -mc);
         ptx::f32x2 s[2] = {0ull, 0ull};
-        float high = -INFINITY;                          // largest logit that the polynomial met
+        float high = -INFINITY;                          // largest logit that the polynomial met, or NaN
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const float a = __uint_as_float(raw[2 * i]), b = __uint_as_float(raw[2 * i + 1]);
-            if (poly_pair(i)) high = ptx::fmax3(high, a, b);
+            if (poly_pair(i)) high = ptx::fmax3_nan(high, a, b);
             s[i & 1] = ptx::add2(s[i & 1], exp2_pair(i, ptx::fma2(ptx::pack2(a, b), scale, shift)));
         }
         const float2 t = ptx::unpack2(ptx::add2(s[0], s[1]));
@@ -160,6 +160,7 @@ __device__ __forceinline__ void sweep1_columns(const uint32_t (&raw)[32], float 
 #pragma unroll
         for (int c = 0; c < 32; c += 2) mx = ptx::fmax3(mx, __uint_as_float(raw[c]), __uint_as_float(raw[c + 1]));
         l *= ptx::ex2(ref * c2 - mx * c2);
+        if (!(high < INFINITY)) l = high - high;         // NaN, as the other unit makes it of such a logit
         ref = mx;
     }
     l += sum;
@@ -174,21 +175,27 @@ __device__ __forceinline__ void sweep2_diagonal(const uint32_t (&raw)[32], int c
         acc[c & 3] += (c0 + c >= from && c0 + c < limit) ? e : 0.f;
     }
 }
-__device__ __forceinline__ void sweep2_columns(const uint32_t (&raw)[32], float c2, float (&acc)[4]) {
+// (high: the largest logit that the polynomial met, or NaN)
+__device__ __forceinline__ void sweep2_columns(const uint32_t (&raw)[32], float c2, float (&acc)[4], float& high) {
     const ptx::f32x2 scale = ptx::pack2(c2, c2);
     ptx::f32x2 s[2] = {ptx::pack2(acc[0], acc[1]), ptx::pack2(acc[2], acc[3])};
-    float high = -INFINITY;
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         const float a = __uint_as_float(raw[2 * i]), b = __uint_as_float(raw[2 * i + 1]);
-        if (poly_pair(i)) high = ptx::fmax3(high, a, b);
+        if (poly_pair(i)) high = ptx::fmax3_nan(high, a, b);
         s[i & 1] = ptx::add2(s[i & 1], exp2_pair(i, ptx::mul2(ptx::pack2(a, b), scale)));
     }
     const float2 u = ptx::unpack2(s[0]), v = ptx::unpack2(s[1]);
-    acc[0] = high * c2 > 127.f ? INFINITY : u.x;         // (probabilities beyond 2^127: a caller's log-sum-exp is not one)
+    acc[0] = u.x;
     acc[1] = u.y;
     acc[2] = v.x;
     acc[3] = v.y;
+}
+// A row's sum, given the largest logit that the polynomial met: infinite from a probability of 2^128 on (a caller's
+// log-sum-exp that is not one), of which the polynomial makes anything.
+__device__ __forceinline__ float sweep2_sum(float sum, float high, float c2) {
+    const float x = high * c2;
+    return x < 128.f ? sum : x >= 128.f ? INFINITY : x;
 }
 
 // -lse / scale of one query row as three bf16 terms (their sum carries 24 bits) and 13 zeros:
@@ -488,7 +495,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             if (kSplits && it.nt == 0) { --n; continue; }
             const int pos = it.blk * kTile + row;            // position of this thread's row
             float m_run = -INFINITY, l_run = 0.f;            // sweep 1
-            float acc[4] = {0.f, 0.f, 0.f, 0.f};             // sweep 2
+            float acc[4] = {0.f, 0.f, 0.f, 0.f}, high = -INFINITY;       // sweep 2
 
             for (int t = 0; t < it.nt; ++t, ++gb) {
                 if ((int)(gb % kGroups) != wg) continue;
@@ -515,7 +522,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         else sweep1_columns(raw, c2, m_run, l_run);
                     } else {
                         if (diag) sweep2_diagonal(raw, c0, diag_from, col_limit, c2, acc);
-                        else sweep2_columns(raw, c2, acc);
+                        else sweep2_columns(raw, c2, acc, high);
                     }
                 };
                 // the last columns are in registers: hand the accumulator back, so that the next
@@ -552,7 +559,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             ptx::mbar_wait(ptx::smem_u32(&sh.comb_free[cslot]), (cuse & 1u) ^ 1u, abort_flag);
             if (wg != combiner) {
                 if (KIND == kSweep1) { cb[wg][0][row] = m_run; cb[wg][kP1][row] = l_run; }
-                else { cb[wg][0][row] = (acc[0] + acc[1]) + (acc[2] + acc[3]); }
+                else { cb[wg][0][row] = sweep2_sum((acc[0] + acc[1]) + (acc[2] + acc[3]), high, c2); }
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh.comb_full[cslot]));
             } else {
@@ -576,7 +583,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         else
                             store_lse(p, it.head, it.tok_begin + pos, m, l);
                     } else {
-                        const float own = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+                        const float own = sweep2_sum((acc[0] + acc[1]) + (acc[2] + acc[3]), high, c2);
                         float a = (wg == 0) ? own : cb[0][0][row];
 #pragma unroll
                         for (int g = 1; g < kGroups; ++g) a += (g == wg) ? own : cb[g][0][row];
@@ -957,7 +964,7 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             const int t_first = KIND == kSweep2 ? half : 0;        // active tiles [t_first, t_end)
             const int t_end = KIND == kSweep1 ? blk + 1 : it.nt;
             float m_run = -INFINITY, l_run = 0.f;            // sweep 1
-            float total = 0.f;                               // sweep 2: sums of whole tiles (short chains of
+            float total = 0.f, high = -INFINITY;             // sweep 2: sums of whole tiles (short chains of
                                                              // additions, whatever the prompt's length)
             // tiles of this group: all of them, or the first one of its parity and every other one
             constexpr int kStep = kBlocks == 2 ? 2 : 1;
@@ -990,11 +997,12 @@ multi_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                         else sweep1_columns(raw, c2, m_run, l_run);
                     } else {
                         if (diag) sweep2_diagonal(raw, ch * 32, diag_from, col_limit, c2, acc);
-                        else sweep2_columns(raw, c2, acc);
+                        else sweep2_columns(raw, c2, acc, high);
                     }
                 }
                 if (KIND == kSweep2) total += (acc[0] + acc[1]) + (acc[2] + acc[3]);
             }
+            if (KIND == kSweep2) total = sweep2_sum(total, high, c2);
             if (kBlocks == 4) {                              // nobody else worked on the block
                 const bool mine = pos < it.L && !*abort_flag;
                 if (KIND == kSweep2) store_scores(p, it.head, it.tile + half, quarter, it.tok_begin + pos, mine, total);

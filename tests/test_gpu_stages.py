@@ -132,6 +132,51 @@ def test_scores_one_logit_far_above_the_reference(B, cols, rise):
     assert np.all(np.abs(got - A) <= 1e-4 * A + 1e-30)
 
 
+@pytest.mark.parametrize("L,H", [(600, 1), (4096, 32)])                  # single blocks, pairs
+@pytest.mark.parametrize("x", [126.5, 127.25, 127.75, 127.9999, 128.25, 200.0, 1e6, np.nan])
+@pytest.mark.parametrize("col", [10, 12, 21, 30])
+def test_scores_of_a_log_sum_exp_that_is_none(B, col, x, L, H):
+    """A caller's log-sum-exp far below the logits: a probability of 2^x is itself while fp32 holds it and else
+    infinite, and NaN stays NaN, on either unit (the polynomial takes columns 10, 11, 20, 21, 30 and 31 of 32)."""
+    import torch
+    q, k = (torch.zeros(L, H, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2))       # all logits are 0
+    lse = torch.full((H, L), 50.0, device="cuda")
+    lse[:, 256 + col] = -x * np.log(2.0)
+    scores = torch.zeros(H, L, device="cuda")
+    lay = B.make_layout(q, k)
+    ws = B.alloc_workspace(lay, [L])
+    B.check(B.lookm_score(q, k, [0, L], lay, scores, lse, True, ws))
+    assert B.lookm_device_status(ws) == B.OK
+    got = scores[:, :256].double()                       # the blocks that meet the column in a whole tile
+    if np.isnan(x):
+        assert got.isnan().all()
+    elif x >= 128:
+        assert (got == np.inf).all()
+    else:                                                # four roundings of the exponent: 4 * 128 * 2^-24 * ln 2
+        assert ((got / 2.0 ** x - 1).abs() <= 2.5e-5).all()
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("col", [5, 10, 12, 21, 31])
+def test_scores_of_a_key_that_is_no_number(B, col, value):
+    """Its logit makes the log-sum-exp of every query in the blocks behind it NaN, whichever unit takes its column;
+    the queries before it don't see it."""
+    import torch
+    L = 600
+    gen = torch.Generator(device="cuda").manual_seed(144)
+    q, k = (torch.randn(L, 1, 128, generator=gen, device="cuda").abs().bfloat16() for _ in range(2))
+    lay = B.make_layout(q, k)
+    ws = B.alloc_workspace(lay, [L])
+    lse = torch.zeros(2, 1, L, device="cuda")
+    scores = torch.zeros(1, L, device="cuda")
+    B.check(B.lookm_score(q, k, [0, L], lay, scores, lse[0], False, ws))
+    k[256 + col] = value
+    B.check(B.lookm_score(q, k, [0, L], lay, scores, lse[1], False, ws))
+    assert B.lookm_device_status(ws) == B.OK
+    assert torch.equal(lse[0, 0, :256 + col], lse[1, 0, :256 + col])
+    assert lse[1, 0, 384:].isnan().all()
+
+
 @pytest.mark.parametrize("lens,Hq,Hkv", [([1900, 1, 130, 640], 4, 1), ([1409], 1, 1), ([2100, 2100], 2, 2)])
 def test_scores_of_items_cut_into_ranges(B, lens, Hq, Hkv):
     """Few heads: both sweeps cut their items into up to four ranges (fewer where an item has fewer
