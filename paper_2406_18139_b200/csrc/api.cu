@@ -45,7 +45,7 @@ struct Plan {
                                             // for the end, and the first item of these
     size_t n_arrived[2] = {0, 0};           // their arrival counters
     size_t clear_words = 64;                // status word and arrival counters
-    size_t o_status, o_reqs, o_lse, o_lse_split, o_scores, o_rank, o_rnorm_all, o_kept, o_evict, o_kept_keys,
+    size_t o_status, o_verdicts, o_reqs, o_lse, o_lse_split, o_scores, o_rank, o_rnorm_all, o_kept, o_evict, o_kept_keys,
         o_rnorm_kept, o_assign, o_sim, o_row_begin, o_entries, o_units, o_slot_cnt, o_parts, o_sort_a, o_sort_b,
         total;
 };
@@ -240,6 +240,8 @@ int build_plan(Plan& pl, const lookm_layout* lay, int n_req, const int* cu_seqle
         if (pl.splits[s] > 1 || (s && score_parts > 1)) pl.n_arrived[s] = 4 * (size_t)tiles * (s ? Hkv : Hq);
     pl.clear_words += pl.n_arrived[0] + pl.n_arrived[1];
     pl.o_status = carve(4 * (64 + 4 * (size_t)tiles * (Hq + Hkv)));
+    // (where sweep 1 leaves verdicts, one per CTA and so at most tiles * Hq, its items are whole and need no counters)
+    pl.o_verdicts = pl.o_status + 4 * (64 + 4 * (size_t)tiles * Hkv);
     pl.o_reqs = carve(sizeof(Req) * n_req);
     pl.o_lse = carve(4 * Hq * T);
     pl.o_lse_split = carve(32 * Hq * T);
@@ -439,6 +441,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
     if (!lse_is_input) {
         p.n_items = pl.n_items[kSweep1];
         p.n_clear = clears ? (int)pl.clear_words : 0;
+        p.verdicts = at<int>(ws, pl.o_verdicts);
         p.next_item = p.status + 16 + kSweep1;
         p.splits = pl.splits[0];
         p.parts1 = at<float2>(ws, pl.o_kept_keys);
@@ -450,6 +453,7 @@ int run_score(const Plan& pl, const DeviceInfo& di, const lookm_layout* lay, con
         ++g_launches;
     }
     mark_stage(1, st);
+    p.n_verdicts = !lse_is_input && clears ? tile_grid(pl.n_items[kSweep1], di.sms) : 0;
     p.n_items = pl.n_items[kSweep2];
     p.next_item = p.status + 16 + kSweep2;
     p.splits = pl.splits[1];

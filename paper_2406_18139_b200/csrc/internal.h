@@ -109,7 +109,12 @@ struct TileParams {
     int* status;                 // device status word
     int n_clear;                 // words from the status word on that sweep 1 has to clear; if any, it also writes the
                                  // single request to its row
+    int* verdicts;               // then: one word per CTA of sweep 1, its status.  It can't go to the status word, which
+    int n_verdicts;              // another CTA may yet have to clear; sweep 2 passes on what its n_verdicts words say
 };
+
+// CTAs of a sweep
+inline int tile_grid(int n_items, int num_sms) { return n_items < num_sms ? n_items : num_sms; }
 
 // ---- launchers (each enqueues on `stream` and returns the CUDA error of the launch) -----------
 // map_x: the lse_split tensor (sweep 2 only; NULL otherwise)

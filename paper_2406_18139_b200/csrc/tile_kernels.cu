@@ -346,6 +346,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     if (KIND == kSweep1 && !kSplits && p.n_clear > 0) {          // no table writer went before
         for (int i = blockIdx.x * kThreads + threadIdx.x; i < p.n_clear; i += gridDim.x * kThreads) p.status[i] = 0;
         write_single_request(p.reqs);
+        if (threadIdx.x == kThreads - 1) p.verdicts[blockIdx.x] = LOOKM_OK;  // (a store at the end would hold the launch up)
     }
     if (warp == 0) {
         ptx::tmem_alloc(ptx::smem_u32(&sh.tmem_base), 512);
@@ -481,6 +482,9 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         }
     } else {
         // ------------------------------------------------------------ epilogue --------------
+        if (KIND == kSweep2 && blockIdx.x == gridDim.x - 1)  // (not the CTA with the longest item, and its last group first)
+            for (int i = 32 * (kEpiWarp0 + 4 * kGroups) - 1 - threadIdx.x; i < p.n_verdicts; i += kGroups * 128)
+                if (p.verdicts[i] != LOOKM_OK) atomicExch(p.status, p.verdicts[i]);
         const int wg = (warp - kEpiWarp0) >> 2;              // group of the epilogue
         const int quarter = warp & 3;                        // TMEM lane quarter this warp may read
         const int row = quarter * 32 + lane;                 // row of the stationary tile
@@ -633,7 +637,8 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc(tmem_base, 512);
     }
-    if (threadIdx.x == 0 && sh.abort_flag) atomicExch(p.status, (int)LOOKM_ERR_DEVICE_TIMEOUT);
+    if (threadIdx.x == 0 && sh.abort_flag)
+        atomicExch(KIND == kSweep1 && !kSplits && p.n_clear > 0 ? p.verdicts + blockIdx.x : p.status, (int)LOOKM_ERR_DEVICE_TIMEOUT);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1089,7 +1094,7 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
     static const Kernel kernels[2][2] = {{tile_kernel<kSweep1, false>, tile_kernel<kSweep1, true>},
                                          {tile_kernel<kSweep2, false>, tile_kernel<kSweep2, true>}};
     const size_t smem_of[2] = {sizeof(Shared<kSweep1>) + 1024, sizeof(Shared<kSweep2>) + 1024};
-    const int grid = p.n_items < num_sms ? p.n_items : num_sms;
+    const int grid = tile_grid(p.n_items, num_sms);
     const CUtensorMap& mx = map_x ? *map_x : map_b;      // only sweep 2 uses it
     static const Kernel multi[2][2] = {{multi_kernel<kSweep1, 2>, multi_kernel<kSweep1, 4>},
                                        {multi_kernel<kSweep2, 2>, multi_kernel<kSweep2, 4>}};

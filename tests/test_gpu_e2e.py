@@ -206,3 +206,28 @@ def test_batch_of_many_short_requests(B):
 def test_gqa_scores_are_summed_over_the_group(B):
     w = synth.tiny(700, 8, 2, 140, 16, 1, image_spans=[(50, 600)], seed=77)
     run_layer(B, w, threads=4)
+
+
+@pytest.mark.parametrize("L,Hq,Hkv", [(1, 1, 1), (129, 2, 1), (700, 32, 8), (1500, 20, 20), (2048, 8, 8)])
+def test_one_prompt_on_a_workspace_full_of_anything(B, L, Hq, Hkv):
+    """A prompt in single blocks has no launch before its first sweep, which clears the status word while its own
+    CTAs leave a verdict each in words of their own: nothing that lay there before reaches the status or a result."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    q, k, v = (torch.randn(L, h, 128, generator=gen, device="cuda").bfloat16() for h in (Hq, Hkv, Hkv))
+    mask = torch.zeros(L, dtype=torch.uint8, device="cuda")
+    budget, blocks = max(1, L // 5), (L + 127) // 128
+    lay = B.make_layout(q, k)
+    ws = B.alloc_workspace(lay, [L])
+    outs = []
+    for fill in (0, 255, 3):
+        ws.fill_(fill)
+        out = torch.zeros(2, Hkv, budget, 128, dtype=torch.bfloat16, device="cuda")
+        st, _ = B.lookm_compress_layer(q, k, v, mask, L, budget, 1, B.MERGE_PIVOTAL, lay, out[0], out[1], ws)
+        B.check(st)
+        assert B.lookm_device_status(ws) == B.OK
+        outs.append(out)
+        verdicts = ws.view(torch.int32)[64 + 4 * blocks * Hkv:]
+        ctas = min(blocks * Hq, torch.cuda.get_device_properties(0).multi_processor_count)
+        assert (verdicts[:ctas] == 0).all() and fill == ws[256 + 16 * blocks * Hkv + 4 * ctas]
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
