@@ -107,7 +107,8 @@ def test_grouped_queries_are_as_precise_as_single_ones(B, Hq, Hkv, n, q_scale):
     assert err[0] <= 1.5 * err[1], err / 4
 
 
-@pytest.mark.parametrize("Hq,Hkv,n", [(2, 2, 300), (2, 1, 300), (4, 1, 300), (8, 1, 300), (12, 2, 3000), (4, 2, 9000), (16, 4, 40)])
+@pytest.mark.parametrize("Hq,Hkv,n", [(2, 2, 300), (2, 1, 300), (4, 1, 300), (8, 1, 300), (12, 2, 3000), (4, 2, 9000), (16, 4, 40),
+                                      (76, 76, 1600)])
 def test_logits_of_minus_infinity_and_infinite_values(B, Hq, Hkv, n):
     """Rows whose logits overflow to -inf count nothing, also where a warp meets them first; an infinite
     value makes its feature infinite and leaves the others alone.  One query head or several per row."""
@@ -170,13 +171,38 @@ def test_batches_of_grouped_queries_at_the_edges_of_sixteen_row_steps(B, group):
         assert torch.equal(dk[a + n], kn[r]) and torch.equal(dv[a + n], vn[r])
 
 
-@pytest.mark.parametrize("lens,heads,group,ranked", [
-    ([0, 1, 31, 40, 62, 63, 64, 65, 126, 127, 128, 129] * 9, 24, 1, False),      # more requests than one launch carries
-    ([40] * 64, 32, 1, True),                            # units of one step: none is shared
-    ([7000, 63, 64, 2000], 32, 1, False),                # units that many CTAs share beside units of a single step
-    ([20031], 40, 1, True),                              # a head per 7.4 CTAs
-    ([5000, 100, 5000], 20, 2, False)])
-def test_equal_shares_of_all_rows(B, lens, heads, group, ranked):
+def records_of_shares(lens, q_heads, sms):
+    """Partial results that the CTAs of a step in equal shares leave behind, by their place in the workspace: the
+    steps of 64 rows of all (request, query head), in a row, are dealt to two CTAs per SM; a CTA whose share holds
+    a unit in part writes the first of its two records if the share begins with the unit or inside it, else the second."""
+    records = set()
+    for chunk in range(0, len(lens), 96):                # requests that one launch carries
+        units = [n // 64 + 1 for n in lens[chunk:chunk + 96] for _ in range(q_heads)]
+        ends = np.cumsum(units)
+        ctas = min(2 * sms, int(ends[-1]))
+        shares = np.concatenate([[0], np.cumsum([int(ends[-1]) // ctas + (c < int(ends[-1]) % ctas) for c in range(ctas)])])
+        for end, steps in zip(ends.tolist(), units):
+            first, last = (int(np.searchsorted(shares, x, side="right")) - 1 for x in (end - steps, end - 1))
+            if first < last:
+                records |= {2 * c + int(c == first and shares[c] < end - steps) for c in range(first, last + 1)}
+    return records
+
+
+# (The planner goes by estimated times: where a refit of these sends a case another way, `shared` tells.)
+@pytest.mark.parametrize("lens,heads,group,ranked,shared", [
+    ([0, 1, 31, 40, 62, 63, 64, 65, 126, 127, 128, 129] * 9, 24, 1, False, True),      # more requests than one launch carries
+    ([40] * 64, 32, 1, True, True),                      # units of one step: none is divided
+    ([40] * 63 + [200], 32, 1, True, True),
+    ([7000, 63, 64, 2000], 32, 1, False, True),          # units that many CTAs share beside units of a single step
+    ([1600], 76, 1, True, True),                         # one request, a head per 3.9 CTAs
+    ([4000], 76, 1, False, True),
+    ([628, 52, 10], 4, 11, False, True),                 # grouped queries, one head at a time
+    ([3166, 307], 5, 11, True, True),
+    ([20, 728, 3], 16, 3, False, True),
+    ([13, 13, 32, 874], 6, 5, True, True),
+    ([20031], 40, 1, True, False),                       # whole splits
+    ([5000, 100, 5000], 20, 2, False, False)])           # two heads at a time, or tensor cores
+def test_equal_shares_of_all_rows(B, lens, heads, group, ranked, shared):
     """CTAs whose shares begin and end anywhere in a unit: units of less than a step to hundreds of steps, the
     appended row in the last step or in one of its own; `heads` KV heads, [heads, rows, 128] or packed."""
     import torch
@@ -191,13 +217,18 @@ def test_equal_shares_of_all_rows(B, lens, heads, group, ranked):
     outs = []
     by_head = lambda t: t if ranked else t.transpose(0, 1)
     before_k, before_v = dk.clone(), dv.clone()
-    for _ in range(3):
-        ws.random_(0, 255)                               # nothing in the workspace counts
+    for last in (False, False, True):
+        ws.fill_(255) if last else ws.random_(0, 255)    # nothing in the workspace counts
         out = torch.full((n_req, hq, 128), np.nan, device="cuda")
         B.check(B.lookm_decode_step_varlen(q, kn, vn, dk, dv, begins[:-1], lens, lay, out, ws))
         outs.append(out)
     torch.cuda.synchronize()
     assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+    words = ws.view(torch.int32)
+    records = words[:words.numel() // 130 * 130].view(-1, 130)           # reference, sum and 128 features
+    written = set((records != -1).any(1).nonzero()[:, 0].tolist())
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert (written == records_of_shares(lens, hq, sms)) == shared, "another kernel took the step"
     K, V = by_head(dk).double(), by_head(dv).double()
     untouched = torch.ones(begins[-1], dtype=torch.bool, device="cuda")
     for r, n in enumerate(lens):
