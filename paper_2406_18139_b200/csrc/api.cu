@@ -1003,7 +1003,9 @@ constexpr double kMmaStepAlone = 1.9;       // of a CTA that has its SM to itsel
 // first: SMs with the same load, as (load, how many), move on together.
 long long most_rows(const int* lens, int n_req, long long units, long long s, long long wave) {
     typedef std::pair<long long, long long> Load;
-    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> free;
+    std::vector<Load> room;
+    room.reserve(128);
+    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> free(std::greater<Load>(), std::move(room));
     free.push({0, wave});
     long long most = 0;
     const auto give = [&](long long rows, long long pieces) {
@@ -1022,6 +1024,37 @@ long long most_rows(const int* lens, int n_req, long long units, long long s, lo
         give(std::min(s, rows), units * ((rows + s - 1) / s));
     }
     return most;
+}
+
+// Time of the slowest CTA of each launch in equal shares: so much per step of 64 rows, while two CTAs work on an SM, per
+// unit, and per further launch.  A share has most units where it begins with a request or ends with one (the shares lie where
+// they lie: this is up to a unit off); the walk costs 0.1 us per eight requests, one over the CTAs' shares 1 to 2 us.
+constexpr double kShareStepUs = 1.3, kShareUnitUs = 0.86, kShareLaunchUs = 4.2;
+double slowest_share(const int* lens, int n_req, long long units, int sms) {
+    double us = -kShareLaunchUs;
+    for (int base = 0; base < n_req; base += kDecodeChunk) {
+        const int n = std::min(kDecodeChunk, n_req - base);
+        long long per[kDecodeChunk], steps = 0;                       // steps of a unit
+        for (int r = 0; r < n; ++r) {
+            per[r] = lens[base + r] / kDecodeShareRows + 1;
+            steps += per[r] * units;
+        }
+        const long long ctas = std::min<long long>((long long)sms * kDecodeShareCtasPerSm, steps), share = (steps + ctas - 1) / ctas;
+        long long most = 1;
+        for (int step : {1, -1})
+            for (int from = 0; from < n; ++from) {
+                if (from > 0 && from < n - 1 && per[from] >= per[from - step]) continue;          // (denser units lie before it)
+                long long left = share, count = 0;
+                for (int r = from; r >= 0 && r < n && left > 0; r += step) {
+                    const long long here = std::min(left, per[r] * units);
+                    count += here == left ? (here + per[r] - 1) / per[r] : units;
+                    left -= here;
+                }
+                most = std::max(most, count);
+            }
+        us += kShareLaunchUs + (double)share * kShareStepUs + (double)most * kShareUnitUs;
+    }
+    return us;
 }
 
 DecodeWay decode_way(const lookm_cache_layout* lay, int n_req, const int* lens, int gt, bool mma, int sms) {
@@ -1083,30 +1116,36 @@ DecodeWay decode_way(const lookm_cache_layout* lay, int n_req, const int* lens, 
     if (w.cluster == 1 && splits > 1) w.us += cost.combine + cost.splits16 * std::max<long long>(0, splits - 16) / 16.;
     if (gt == 1 && !mma) {
         // Equal shares?  Whole splits take as long as memory needs for all rows, or as long as an SM needs for the
-        // most rows that it gets, with a start per further wave.  Shares cost a little per unit in one and nearly
-        // always the second launch.  (The constants fit 32 steps of 1 to 64 requests, 41 to 32768 rows and 8 to 40 heads;
-        // of these the slower way is picked by 3 % at most.)  us, whole | shares: 4 requests of 1000 to 8000 rows x 32
-        // heads 78 | 63.7, 16 of 4000 to 8000 x 32 293 | 266, 64 of 40 x 32 37 | 17, one of 32768 x 40 115 | 107; one of 8192 x 32
-        // 22.6 | 25.2, of 20000 x 8 16.7 | 19.1, 8 of 300 to 2000 x 40 33 | 35.2, 7 of 100 to 8000 x 32 80 | 86.8.
-        constexpr double kRowUs = 7.8e-5, kSmRowUs = 1e-2, kStartUs = 2., kWaveUs = 1.5, kCombineUs = 1.5, kShareUs = 4.5, kUnitUs = 1.3;
-        const double share_ctas = (double)std::min<long long>((long long)sms * kDecodeShareCtasPerSm, total_rows / kDecodeShareRows + 1);
-        const double shares = std::max((double)total_rows * kRowUs, (double)total_rows / share_ctas * kDecodeShareCtasPerSm * kSmRowUs) +
-                              (double)(n_req * units) / share_ctas * kUnitUs + kShareUs;
-        const double later_waves = std::max(0., (double)ctas / (double)wave - 1.);
+        // most rows that it gets, with a start per further wave and mostly a second launch.  Shares, nearly always two launches,
+        // take as long as the CTA whose steps and units together take longest: a share of many short units lasts longer
+        // than the others.  Fitted to 350 steps of 1 to 150 requests, 10 to 32768 rows and 1 to 100 heads, both ways; from 8 us on
+        // the estimates are 5 % off.  Of 1200 steps that follow this rule, half of them in shares, one in shares takes 8 %
+        // longer than in whole splits and seven 3 to 5.  us, whole | shares: 4 requests of 1000 to 8000 rows x 32 heads 76 | 47,
+        // 14 of 2000 to 6000 x 8 47.6 | 38.9, 64 of 40 x 32 38 | 18, one of 32768 x 40 117 | 108; left whole: nine of 61 to
+        // 4390 x 32, the 61 in one share, 60.7 | 86.5, 33 of 54 to 1168 x 8 18.3 | 21.3, 36 of 22 to 1088 x 16 34.7 | 43.4, one of
+        // 8990 x 16 15.1 | 17.1.
+        constexpr double kRowUs = 7.9e-5, kSmRowUs = 9.6e-3, kStartUs = 2.8, kWaveUs = 2.1, kCombineUs = 1.3, kShareUs = 3.7,
+                         kLaunchUs = 0.5;
+        const bool combined = w.cluster == 1 && splits > 1;
+        // (the heads of a group find their rows in L2)
+        const double from_memory = (double)total_rows / (double)w.n_pass * kRowUs, later_waves = std::max(0., (double)ctas / (double)wave - 1.);
         const auto whole_with = [&](double most) {
-            return std::max(most * kSmRowUs + later_waves * kWaveUs, (double)total_rows * kRowUs) + kStartUs +
-                   (w.cluster == 1 && splits > 1 ? kCombineUs : 0.);
+            return std::max(most * kSmRowUs + later_waves * kWaveUs, from_memory) + kStartUs + (combined ? kCombineUs : 0.);
         };
-        // (most rows of an SM: between the mean and that plus a split; the order in which SMs come free only counts in between)
+        // The most rows of an SM are no fewer than the mean and a split's, and no more than both together; worked out only where
+        // that leaves it open.  (A launch more also takes the host longer.)
         const double mean = (double)total_rows / (double)wave, piece = (double)std::min<long long>(s, longest);
-        double whole = whole_with(ctas <= wave ? piece : mean);
-        if (ctas > wave && shares >= 0.95 * whole && shares < 0.95 * whole_with(mean + piece))
-            whole = whole_with((double)most_rows(lens, n_req, units, s, wave));
-        w.shares = shares < 0.95 * whole;
-        if (w.shares) {
-            w.cluster = 1;
-            w.us += shares - whole;
+        double whole = whole_with(ctas <= wave ? piece : std::max(mean, piece));
+        const double slower = ctas <= wave ? whole : whole_with(mean + piece);
+        if (slower > kShareUs + kShareStepUs + kShareUnitUs) {               // (no share is shorter)
+            const double shares = std::max(slowest_share(lens, n_req, units, sms), from_memory) + kShareUs +
+                                  (!combined && longest > kDecodeShareRows ? kLaunchUs : 0.);
+            const auto pays = [&](double whole) { return shares + std::min(0.06 * whole, 1.6) < whole; };
+            if (!pays(whole) && pays(slower)) whole = whole_with((double)most_rows(lens, n_req, units, s, wave));
+            w.shares = pays(whole);
+            if (w.shares) w.us += shares - whole;
         }
+        if (w.shares) w.cluster = 1;
     }
     return w;
 }
@@ -1138,7 +1177,9 @@ int build_decode_plan(DecodePlan& dp, const lookm_cache_layout* lay, int n_req, 
         // on 1, 13.4, 9.5 and 4.4; 32 heads on 8 with 409 rows 3.7, 4.0 and 4.3, with 8192 20.6, 16.0 and 11.4.
         dp.way = decode_way(lay, n_req, lens, 1, false, sms);
         if (group > 1) {
-            const auto better = [&](const DecodeWay& w) { if (w.us < dp.way.us) dp.way = w; };
+            // (shares of single heads by a clear margin only: of one cache of 28811 rows, 96 heads on 32, 184 us estimated
+            // against 217 on the tensor cores were 165 against 160)
+            const auto better = [&](const DecodeWay& w) { if (w.us < (dp.way.shares ? 1.25 : 1.) * dp.way.us) dp.way = w; };
             if (group % 2 == 0) better(decode_way(lay, n_req, lens, 2, false, sms));
             if (widest > 1) better(decode_way(lay, n_req, lens, widest, true, sms));
         }

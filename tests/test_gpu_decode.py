@@ -196,12 +196,17 @@ def records_of_shares(lens, q_heads, sms):
     ([7000, 63, 64, 2000], 32, 1, False, True),          # units that many CTAs share beside units of a single step
     ([1600], 76, 1, True, True),                         # one request, a head per 3.9 CTAs
     ([4000], 76, 1, False, True),
-    ([628, 52, 10], 4, 11, False, True),                 # grouped queries, one head at a time
-    ([3166, 307], 5, 11, True, True),
-    ([20, 728, 3], 16, 3, False, True),
+    ([32768], 40, 1, True, True),                        # a head per 7.4 CTAs
+    ([3166, 307], 5, 11, True, True),                    # grouped queries, one head at a time
+    ([700, 3000, 64], 3, 13, False, True),
     ([13, 13, 32, 874], 6, 5, True, True),
-    ([20031], 40, 1, True, False),                       # whole splits
-    ([5000, 100, 5000], 20, 2, False, False)])           # two heads at a time, or tensor cores
+    # whole splits, where a share of short units would last longest or two launches would take longer
+    ([61, 1582, 4390, 3260, 2685, 2120, 3375, 841, 2736], 32, 1, True, False),
+    ([968, 54, 847, 280, 513, 756, 184, 867, 453, 106, 997, 399, 1168, 641, 613, 119, 850], 8, 1, False, False),
+    ([20031], 40, 1, True, False),
+    ([628, 52, 10], 4, 11, False, False),
+    ([8000], 32, 3, False, False),                       # tensor cores
+    ([5000, 100, 5000], 20, 2, False, False)])
 def test_equal_shares_of_all_rows(B, lens, heads, group, ranked, shared):
     """CTAs whose shares begin and end anywhere in a unit: units of less than a step to hundreds of steps, the
     appended row in the last step or in one of its own; `heads` KV heads, [heads, rows, 128] or packed."""
