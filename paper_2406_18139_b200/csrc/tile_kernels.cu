@@ -250,9 +250,9 @@ struct Item {
     int tile;                 // index of the block over the whole batch
 };
 
-template <int KIND, bool kSplits>
+template <int KIND, bool kSplits, bool kOne>
 __device__ __forceinline__ Item decode_item(const TileParams& p, const Req* tbl, int item) {
-    int lo = 0, hi = p.reqs.n - 1;
+    int lo = 0, hi = kOne ? 0 : p.reqs.n - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (tbl[mid].item_begin[KIND] <= item) lo = mid; else hi = mid - 1;
@@ -300,7 +300,9 @@ __device__ __forceinline__ int item_of_round(int round, int cta, int n_cta) {
     return round * n_cta + ((round & 1) ? (n_cta - 1 - cta) : cta);
 }
 
-template <int KIND, bool kSplits>
+// kOne: of a single request, which comes with the launch and may have no launch before it.  (Variants of their own: that code in
+// the sweeps of batches cost 0.2 to 0.5 us a call, scores of four prompts of 134 to 1009 tokens x 16 heads 32.49 | 32.95.)
+template <int KIND, bool kSplits, bool kOne>
 __global__ void __launch_bounds__(kThreads, 1)
 tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
             const __grid_constant__ CUtensorMap map_x, const TileParams p) {
@@ -336,14 +338,15 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     }
     // everything above touches only this CTA's shared memory; from here on global memory written
     // by the kernel before this one is read
-    if (p.reqs.n == 1 && threadIdx.x < sizeof(Req) / 4)          // a single request came with the launch
+    if (kOne && threadIdx.x < sizeof(Req) / 4)
         reinterpret_cast<int*>(sh.reqs)[threadIdx.x] = reinterpret_cast<const int*>(&p.reqs.only)[threadIdx.x];
     grid_dependency_wait();
-    const Req* tbl = p.reqs.n <= kReqCache ? sh.reqs : p.reqs.rows;      // the table is read once per item by every role
-    if (p.reqs.n > 1 && p.reqs.n <= kReqCache)
+    const Req* tbl = kOne || p.reqs.n <= kReqCache ? sh.reqs : p.reqs.rows;      // the table is read once per item by every role
+    if (!kOne && p.reqs.n <= kReqCache)
+#pragma unroll 1
         for (int i = threadIdx.x; i < p.reqs.n * (int)(sizeof(Req) / 4); i += kThreads)
             reinterpret_cast<int*>(sh.reqs)[i] = reinterpret_cast<const int*>(p.reqs.rows)[i];
-    if (KIND == kSweep1 && !kSplits && p.n_clear > 0) {          // no table writer went before
+    if (KIND == kSweep1 && !kSplits && kOne && p.n_clear > 0) {          // no table writer went before
         for (int i = blockIdx.x * kThreads + threadIdx.x; i < p.n_clear; i += gridDim.x * kThreads) p.status[i] = 0;
         write_single_request(p.reqs);
         if (threadIdx.x == kThreads - 1) p.verdicts[blockIdx.x] = LOOKM_OK;  // (a store at the end would hold the launch up)
@@ -370,7 +373,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             for (int round = 0; !stop; ++round, ++n) {
                 const int item = item_of_round(round, blockIdx.x, n_cta);
                 if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; --n; continue; }
-                const Item it = decode_item<KIND, kSplits>(p, tbl, item);
+                const Item it = decode_item<KIND, kSplits, kOne>(p, tbl, item);
                 if (kSplits && it.nt == 0) { --n; continue; }
                 const int ab = n % kABuf;
                 if (!ptx::mbar_wait(ptx::smem_u32(&sh.a_empty[ab]), ((n / kABuf) & 1) ^ 1, abort_flag)) break;
@@ -433,7 +436,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             for (int round = 0; !stop; ++round, ++n) {
                 const int item = item_of_round(round, blockIdx.x, n_cta);
                 if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; --n; continue; }
-                const Item it = decode_item<KIND, kSplits>(p, tbl, item);
+                const Item it = decode_item<KIND, kSplits, kOne>(p, tbl, item);
                 if (kSplits && it.nt == 0) { --n; continue; }
                 const int ab = n % kABuf;
                 if (!ptx::mbar_wait(ptx::smem_u32(&sh.a_full[ab]), (n / kABuf) & 1, abort_flag)) break;
@@ -482,7 +485,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         }
     } else {
         // ------------------------------------------------------------ epilogue --------------
-        if (KIND == kSweep2 && blockIdx.x == gridDim.x - 1)  // (not the CTA with the longest item, and its last group first)
+        if (KIND == kSweep2 && kOne && blockIdx.x == gridDim.x - 1)  // (not the CTA with the longest item, and its last group first)
             for (int i = 32 * (kEpiWarp0 + 4 * kGroups) - 1 - threadIdx.x; i < p.n_verdicts; i += kGroups * 128)
                 if (p.verdicts[i] != LOOKM_OK) atomicExch(p.status, p.verdicts[i]);
         const int wg = (warp - kEpiWarp0) >> 2;              // group of the epilogue
@@ -495,7 +498,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         for (int round = 0;; ++round, ++n) {
             const int item = item_of_round(round, blockIdx.x, n_cta);
             if (item >= p.n_items) { if (round * n_cta >= p.n_items) break; --n; continue; }
-            const Item it = decode_item<KIND, kSplits>(p, tbl, item);
+            const Item it = decode_item<KIND, kSplits, kOne>(p, tbl, item);
             if (kSplits && it.nt == 0) { --n; continue; }
             const int pos = it.blk * kTile + row;            // position of this thread's row
             float m_run = -INFINITY, l_run = 0.f;            // sweep 1
@@ -638,7 +641,7 @@ tile_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         ptx::tmem_dealloc(tmem_base, 512);
     }
     if (threadIdx.x == 0 && sh.abort_flag)
-        atomicExch(KIND == kSweep1 && !kSplits && p.n_clear > 0 ? p.verdicts + blockIdx.x : p.status, (int)LOOKM_ERR_DEVICE_TIMEOUT);
+        atomicExch(KIND == kSweep1 && !kSplits && kOne && p.n_clear > 0 ? p.verdicts + blockIdx.x : p.status, (int)LOOKM_ERR_DEVICE_TIMEOUT);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1091,8 +1094,10 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
                                cudaStream_t stream) {
     if (p.n_items <= 0) return cudaSuccess;
     typedef void (*Kernel)(CUtensorMap, CUtensorMap, CUtensorMap, TileParams);
-    static const Kernel kernels[2][2] = {{tile_kernel<kSweep1, false>, tile_kernel<kSweep1, true>},
-                                         {tile_kernel<kSweep2, false>, tile_kernel<kSweep2, true>}};
+    static const Kernel kernels[2][2][2] = {{{tile_kernel<kSweep1, false, false>, tile_kernel<kSweep1, false, true>},
+                                             {tile_kernel<kSweep1, true, false>, tile_kernel<kSweep1, true, true>}},
+                                            {{tile_kernel<kSweep2, false, false>, tile_kernel<kSweep2, false, true>},
+                                             {tile_kernel<kSweep2, true, false>, tile_kernel<kSweep2, true, true>}}};
     const size_t smem_of[2] = {sizeof(Shared<kSweep1>) + 1024, sizeof(Shared<kSweep2>) + 1024};
     const int grid = tile_grid(p.n_items, num_sms);
     const CUtensorMap& mx = map_x ? *map_x : map_b;      // only sweep 2 uses it
@@ -1109,15 +1114,16 @@ cudaError_t launch_tile_kernel(int kind, const CUtensorMap& map_a, const CUtenso
                     e = cudaFuncSetAttribute(multi[i][j], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)multi_smem[i][j]);
         for (int i = 0; i < 2; ++i)
             for (int j = 0; j < 2; ++j)
-                if (e == cudaSuccess)
-                    e = cudaFuncSetAttribute(kernels[i][j], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of[i]);
+                for (int one = 0; one < 2; ++one)
+                    if (e == cudaSuccess)
+                        e = cudaFuncSetAttribute(kernels[i][j][one], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of[i]);
         return e;
     });
     if (err != cudaSuccess) return err;
     if (p.blocks > 1)
         return launch_chained(multi[kind][p.blocks == 4], dim3(grid), dim3(kThreads), multi_smem[kind][p.blocks == 4],
                               stream, map_a, map_b, mx, p);
-    return launch_chained(kernels[kind][p.splits > 1], dim3(grid), dim3(kThreads), smem_of[kind], stream, map_a, map_b, mx, p);
+    return launch_chained(kernels[kind][p.splits > 1][p.reqs.n == 1], dim3(grid), dim3(kThreads), smem_of[kind], stream, map_a, map_b, mx, p);
 }
 
 cudaError_t launch_lse_split(const float* lse, int n_q_heads, long long T, float scale_log2,
