@@ -60,7 +60,9 @@ int device_info(DeviceInfo& out);
 // higher clock, of 2800 x 40 189 | 196; 3800 x 32, 6.5, 165.8 | 162.2, 4096 x 32, 6.9, 189 | 184, 5000 x 32, 8.6, 290 |
 // 278, 20000 x 8, 8.5, 991 | 952, 8192 x 32, 13.8, 714 | 672; grouped heads, layers: 6000 x 16 on 4, 5.1, 244 | 255, 4000 x 24
 // on 6, 5.2, 180 | 183, 3300 x 40 on 10, 13.5 tiles, 7.0, 193 | 199, 3000 x 40 on 8, 12.5, 6.5, 183 | 172, 5000 x 24 on 6, 6.5,
-// 255 | 251, 8000 x 16 on 4, 6.8, 388 | 372, 5000 x 32 on 8, 8.6, 324 | 314).
+// 255 | 251, 8000 x 16 on 4, 6.8, 388 | 372, 5000 x 32 on 8, 8.6, 324 | 314).  Calls in a row for some tenths of a second, which
+// settle at the power limit: a few calls on a cool GPU are up to 4 % faster in single blocks from 6.4 to 8 per SM (layers, 12 ms | 500
+// ms in a row, single - pairs: 17707 x 8, 7.5, 957 - 983 | 976 - 950, 4453 x 32 on 8, 7.6, 252 - 262 | 262 - 263).
 // Shorter ones and two prompts: from nine (256 x 512, two tiles, 6.9, 36 | 42, 1000 x 128, five, 6.9, 67 | 70, 1200 x 96 on
 // 48, six, 6.5, 71 | 78; layers of two of 2250 on average x 32, 7.6, 232 | 236).
 //   More prompts, whose single blocks come out uneven from a fixed deal: from five (three of 900 x 32, 5.2, 66 |
@@ -374,7 +376,7 @@ int make_map_2d(CUtensorMap* map, const void* base, long long rows) {
 // A whole-path call of one prompt in single blocks needs no table writer: its launches carry the request, and the
 // first of them (sweep 1, or the one that takes its place) clears the words that later ones count in and writes the
 // request to its row, for the launch that reads it there.
-// (Eviction alone keeps it: its number of launches is pinned.)
+// (Eviction alone, and scores from a given log-sum-exp by themselves, keep it: their callers count five and three launches.)
 bool first_launch_clears(const Plan& pl) { return pl.n_req == 1 && pl.blocks == 1 && pl.splits[0] == 1 && pl.n_none == 0; }
 
 template <class T>

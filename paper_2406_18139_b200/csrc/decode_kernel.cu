@@ -115,9 +115,11 @@ struct DecShared {
 };
 
 // Asks for the first rows of a CTA's split while the kernel before this one drains: rows already in the cache
-// may not be read before that kernel is over, but they may be brought into L2.  Long splits only (us per step):
-// 32768 rows with 32 heads on 8 28.4 -> 27.1, 8192 x 32 23.8 -> 23.3, 20000 x 8 18.4 -> 17.6; with 256 rows nothing is
-// left of it, with 512 it costs 1 us.
+// may not be read before that kernel is over, but they may be brought into L2.  It helps behind a kernel that lets its
+// dependents start early (this library's do) and is within the scatter behind one that does not.  Caches in rotation, us per
+// step without | with, step after step and with a framework's elementwise kernel before each: 8192 rows x 32 heads 23.7 | 23.3,
+// 27.4 | 27.4; 32768 x 32 on 8 27.6 | 27.1, 30.9 | 30.9; 20000 x 8 18.2 | 17.6, 21.6 | 21.2; 1638 x 32 8.2 | 7.8, 11.7 | 12.0.
+// Of splits of 384 rows and more, 96 rows: asking for 256 of them gains nothing, for 512 costs 1 us.
 constexpr int kPrefetchRows = 96, kPrefetchFrom = 384;
 __device__ __forceinline__ void prefetch_rows(const __nv_bfloat16* cache_k, const __nv_bfloat16* cache_v, long long first,
                                               long long stride_row, int rows) {
@@ -373,9 +375,9 @@ decode_kernel(const __grid_constant__ Batch batch, const __nv_bfloat16* __restri
 // end one unit and begin the next, and its copies run ahead into the next unit while it combines.  A unit that
 // lies in several CTAs' shares is added up by decode_combine_kernel; a CTA leaves at most two partial results
 // (of the unit its share begins in and of the one it ends in).
-// us per step, whole splits | shares: four caches of 1000 to 8000 rows x 32 heads 82 | 66, 64 of 40 rows x 32 37 | 21,
-// twelve of 200 to 6000 x 8 36.5 | 30, one of 32768 x 40 118 | 109; but sixteen of 400 to 3300 x 32 78 | 80, 20000 x 8 18.4 |
-// 20.8: a share's second unit costs about 1 us (the planner compares: decode_way in api.cu).
+// us per step, whole splits | shares: four caches of 1000 to 8000 rows x 32 heads 75.7 | 47.5, 64 of 40 rows x 32 38.0 | 18.3,
+// one of 32768 x 40 117 | 108, one of 4000 x 76 38.7 | 29.5; but 20000 x 8 18.4 | 20.8, and nine of 61 to 4390 x 32 60.7 | 86.5:
+// a share's units cost some 0.9 us each beside their rows (the planner compares: decode_way in api.cu).
 // ---------------------------------------------------------------------------------------------
 constexpr int kShareRing = 3;                        // steps in the ring of a warp: two CTAs to an SM
 constexpr int kShareRingBytes = kDecWarps * kShareRing * kDecStepBytes;

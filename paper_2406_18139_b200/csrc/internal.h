@@ -207,9 +207,9 @@ struct DecodeReq {
         long long step_begin;   // shares: steps of the launch before the request's
     };
 };
-// What a launch gets by value: one request takes 56 bytes, any number up to kDecodeChunk 3.9 KB, which costs
-// 0.45 us more to launch (409 rows x 32 heads, calls in a row from Python: 6.1 | 5.65 us); up to sixteen take 656
-// bytes.
+// What a launch gets by value: one request takes 48 bytes, any number up to kDecodeChunk 3088, which costs
+// 0.45 us more to launch (409 rows x 32 heads, calls in a row from Python: 6.1 | 5.65 us); up to sixteen, a batch whose
+// step may still be as short as its launch, take 528.
 constexpr int kDecodeFew = 16;
 constexpr int kDecodeChunk = 96;
 template <int kRequests>
@@ -221,6 +221,7 @@ struct DecodeBatchOf {
     DecodeReq r[kRequests];
 };
 typedef DecodeBatchOf<kDecodeChunk> DecodeBatch;
+static_assert(sizeof(DecodeBatchOf<1>) == 48 && sizeof(DecodeBatchOf<kDecodeFew>) == 528 && sizeof(DecodeBatch) == 3088, "see above");
 constexpr int kDecodeShareRows = 64;         // rows of a step
 constexpr int kDecodeShareCtasPerSm = 2;
 

@@ -919,7 +919,7 @@ merge_short_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __r
     if (n_slots <= 0) return;
     const long long ev_base = rq.ev_off + (long long)h * E, kept_base = rq.kept_off + (long long)h * B;
 
-    // ---- all lists are requested at once ----
+    // ---- the evicted tokens' lists are requested at once (the kept positions when the entries are written) ----
     const int seg = ((E + kFuseWarps * 32 - 1) / (kFuseWarps * 32)) * 32;
     const int s_begin = warp * seg;
     int key[kSteps], pos[kSteps];
